@@ -402,7 +402,8 @@ BMU_API int bmu_search_static(const float *W, int64_t D, int64_t M, const int32_
  *   listed feature f, num[f*M + bmu[i]] += 1 (a repeated id counts twice).
  *   num uint32 [D][M] and cnt uint32 [M] are accumulated into: zero them at the
  *   start of an epoch, call once per corpus batch.  Exact integer counters.
- *   bmu[i] must lie in [0, M) (unchecked, like colidx).
+ *   bmu[i] must lie in [0, M) (unchecked, like colidx); M == 0 with documents is
+ *   BMU_ERR_INVALID_ARG.
  * bmu_update_blur: num_blur[f][j] = sum_k h(j, k) * num[f][k] and cnt_blur[j] =
  *   sum_k h(j, k) * cnt[k] in fp32, h(j, k) = exp(-(dx^2 + dy^2) / (2 sigma^2))
  *   for |dx|, |dy| <= ceil(3 sigma) and 0 beyond (no wrap-around, no

@@ -1448,6 +1448,7 @@ int bmu_update_scatter(const int32_t *rowptr, const int32_t *colidx, int64_t N, 
         set_error("null pointer argument");
         return BMU_ERR_INVALID_ARG;
     }
+    if (M == 0) { set_error("empty map: its documents have no unit"); return BMU_ERR_INVALID_ARG; }
     return launch_update_scatter(rowptr, colidx, N, bmu, D, M, num, cnt, static_cast<cudaStream_t>(stream));
 }
 

@@ -69,6 +69,14 @@ def test_argument_checks_need_no_gpu(lib):
                              ctypes.byref(o), None, 0, None) == 1
 
 
+def test_an_empty_map_is_refused_before_any_launch(lib):
+    """Documents have no unit on a map without units: refused like a search against an empty codebook."""
+    p = ctypes.c_void_p(256)                          # never looked at
+    assert lib.bmu_update_scatter(p, p, 5, 10, p, 16, 0, p, p, None) == 1
+    assert b"empty map" in lib.bmu_last_error()
+    assert lib.bmu_update_scatter(p, p, 0, 0, p, 16, 0, p, p, None) == 0       # no documents: nothing to do
+
+
 def test_describe_search_needs_no_gpu_and_names_the_kernel(lib):
     """bmu_describe_search is host logic: the benchmark shapes route as documented (large
     sweeps take the tensor-core sweep, the small one the planned kernel) and the launch count
