@@ -245,6 +245,8 @@ screen_collect_kernel(const VerifyArgs a)
         // a list that would overflow: drop what is out of the window by now
         const bool full = joining && n + n_new > (uint32_t)SC_LIST;
         if (__any_sync(0xffffffffu, full)) {
+            // (the entries change lanes through global memory: what other lanes appended before, what they read below)
+            __syncwarp();
             uint32_t kept = 0;
             for (int r = 0; r < (SC_LIST + 3) / 4; ++r) {
                 const uint32_t e = r * 4 + k;
@@ -254,6 +256,7 @@ screen_collect_kernel(const VerifyArgs a)
                 const uint32_t bs = mine ? lb[e] : 0u;
                 const bool keep = mine && v <= limit;
                 const uint32_t who = __ballot_sync(0xffffffffu, keep) & seg;
+                __syncwarp();                                // read by all before any of them is overwritten
                 if (keep) {                                  // entries move towards the front only
                     const uint32_t to = kept + __popc(who & ((1u << lane) - 1u));
                     lv[to] = v; lm[to] = mk; lb[to] = bs;

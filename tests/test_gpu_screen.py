@@ -112,6 +112,34 @@ def test_second_best_half_precision_and_plan(bmu):
     assert torch.equal(hb, b1) and torch.equal(hd, d1) and torch.equal(hb2, b2) and torch.equal(hd2, d2)
 
 
+@pytest.mark.parametrize("kind,M", [("const", 4096), ("dupes", 4096), ("ramp", 2304), ("steps", 4096)])
+def test_lists_that_fill_over_many_launches(bmu, kind, M):
+    """Launches of two slabs: a document's list fills up, is compacted when its minimum falls from
+    launch to launch (ramp, steps), and overflows where nothing falls out of the window (const, dupes).
+    Best and second-best unit and the half-precision codebook carry their minima between the launches."""
+    cfg = synth.CONFIGS["cfg1"]
+    rowptr, colidx = synth.make_corpus(cfg, n_docs=400)
+    if kind in ("ramp", "steps"):
+        # the same few features everywhere, a level that falls along the map
+        level = torch.linspace(0.5, 0.0, M) if kind == "ramp" else torch.floor(torch.arange(M) / 512.0) * -0.03 + 0.5
+        W = (0.2 * torch.rand((cfg.D, 1), generator=torch.Generator().manual_seed(9)) + level[None, :])
+    else:
+        W = synth.make_codebook(cfg.D, M, 67, kind=kind)
+    W = W.half().float().contiguous()
+    ob, od = check(bmu, W, rowptr, colidx, chunk_neurons=256)
+    Wd, rp, ci, o = W.cuda(), rowptr.cuda(), colidx.cuda(), opts_of(bmu, chunk_neurons=256)
+    args = (W.numpy(), rowptr.numpy(), colidx.numpy())
+    b1, d1, b2, d2 = bmu.bmu_search_top2_ws(Wd, rp, ci, opts=o)
+    parity.compare(b1.cpu().numpy(), d1.cpu().numpy(), *args)
+    np.testing.assert_allclose(d2.cpu().numpy(), oracle.bmu2(*args)[3], rtol=1e-5)
+    assert bool((b2 != b1).all())
+    if kind == "const":                              # exact ties: the two lowest units
+        assert int(b1.abs().max()) == 0 and int((b2 - 1).abs().max()) == 0
+    h1, e1, h2, e2 = bmu.bmu_search_f16_ws(Wd.half(), rp, ci, opts=o, top2=True)
+    parity.compare(h1.cpu().numpy(), e1.cpu().numpy(), *args)
+    np.testing.assert_allclose(e2.cpu().numpy(), d2.cpu().numpy(), rtol=1e-6)
+
+
 def test_batches_share_the_images_of_the_codebook(bmu):
     """Batches of one call: the second has lists that the images of the first are too fine for, the
     third lists other features, the fourth takes another route.  Every result as by itself."""
