@@ -177,6 +177,8 @@ BMU_API int bmu_codebook_norms(const float *W, int64_t D, int64_t M, float *norm
  * per-document running minimum merged across neuron chunks, the tiling plan,
  * the split image of the frequent rows (4 * head_rows bytes per neuron) and the
  * compact chunk copy of the tensor-core sweep).  `nnz` is the length of colidx.
+ * Never falls when N or nnz grow: a workspace for the largest batch serves all
+ * smaller ones (the other workspace queries likewise).
  */
 BMU_API size_t bmu_search_workspace_bytes(int64_t D, int64_t M, int64_t N, int64_t nnz,
                                   const bmu_opts *opts);

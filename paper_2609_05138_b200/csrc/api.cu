@@ -132,7 +132,7 @@ static Layout layout_for(int64_t D, int64_t M, int64_t N, int64_t nnz, int kerne
     l.tickets_off = l.slots_off = off;
     if (few) {                           // (the tickets behind the status word: cleared with it)
         off = align_up(off + (size_t)N * sizeof(uint32_t), 256);
-        l.slots_off = off; off = align_up(off + few_slots_bytes(M, N, top2, device_sms()), 256);
+        l.slots_off = off; off = align_up(off + few_slots_bytes(M, N, top2), 256);
     }
     l.norms_off = off; off = align_up(off + (size_t)M * sizeof(float), 256);
     l.state_off = off; off = align_up(off + (size_t)N * sizeof(u64), 256);
@@ -261,15 +261,29 @@ static Layout layout_of(const bmu_opts &o, int64_t D, int64_t M, int64_t N, int6
                       mma_repack_bytes(o, D, M, N, nnz, top2), plan_order(o, true));
 }
 
-// What the workspace queries answer: room for what layout_of says, and not less than the single-stage
-// kernels need -- a workspace sized once with default options serves the same sizes with others.
+// Could a search of no more documents and listings take the two-stage form?  Its model grows slower in the
+// listings than the others' and with the documents, theirs do not: most likely all listings in a single
+// document, or in the fewest that the line beside the model lets it have.
+static bool screen_within(const bmu_opts &o, int64_t D, int64_t M, int64_t N, int64_t nnz, bool f16 = false)
+{
+    return N > 0 && (screen_wanted(o, D, M, 1, nnz, f16) ||
+                     (N >= FEW_MAX_DOCS && screen_wanted(o, D, M, FEW_MAX_DOCS, nnz, f16)));
+}
+
+// What the workspace queries answer: room for every way that a search of these or smaller sizes may take
+// (N and nnz; D, M and the options the same), so that a workspace sized for the largest batch serves all,
+// and one sized with default options the same sizes with others.  Each part grows with N and with nnz.
 static size_t query_bytes(const bmu_opts &o, int64_t D, int64_t M, int64_t N, int64_t nnz, bool top2, bool plan)
 {
-    const size_t need = layout_of(o, D, M, N, nnz, top2, plan).total;
-    if (o.kernel != 0) return need;
-    const size_t single = layout_for(D, M, N, nnz, 0, top2, mma_head_rows(o, D),
-                                     mma_repack_bytes(o, D, M, N, nnz, top2), plan_order(o, true)).total;
-    return need > single ? need : single;
+    size_t need = layout_of(o, D, M, N, nnz, top2, plan).total;
+    auto room = [&](const Layout &l) { if (l.total > need) need = l.total; };
+    if (o.kernel == 0) {
+        room(layout_for(D, M, N, nnz, 0, top2, mma_head_rows(o, D), mma_repack_bytes(o, D, M, N, nnz, top2),
+                        plan_order(o, true)));
+        room(layout_for(D, M, N, nnz, plan ? 3 : 1, top2, 640, 0, 0, 0, true));
+    }
+    if (screen_within(o, D, M, N, nnz)) room(screen_layout_of(o, D, M, N, nnz, top2));
+    return need;
 }
 
 static int check_sizes(int64_t D, int64_t M, int64_t N, int64_t nnz)
@@ -937,6 +951,12 @@ static bool f16_route(const bmu_opts &o, int64_t D, int64_t M, int64_t nnz, bmu_
     return wide_ok;
 }
 
+static Layout f16_wide_layout(const bmu_opts &ow, int64_t D, int64_t M, int64_t N, int64_t nnz, bool top2)
+{
+    return layout_for(D, M, N, nnz, 6, top2, mma_head_rows(ow, D), mma_repack_bytes(ow, D, M, N, nnz, top2),
+                      plan_order(ow, true));
+}
+
 size_t bmu_search_f16_workspace_bytes(int64_t D, int64_t M, int64_t N, int64_t nnz,
                                       const bmu_opts *opts)
 {
@@ -944,10 +964,14 @@ size_t bmu_search_f16_workspace_bytes(int64_t D, int64_t M, int64_t N, int64_t n
     bmu_opts o, ow;
     memset(&o, 0, sizeof(o));
     if (opts) o = *opts;
-    if (screen_wanted(o, D, M, N, nnz, true)) return screen_layout_of(o, D, M, N, nnz, true).total;
     bool wide = false;
     f16_route(o, D, M, nnz, ow, wide);
-    return (wide ? layout_of(ow, D, M, N, nnz, true) : layout_for(D, M, N, nnz, 3, true)).total;
+    // (as query_bytes: for every way that these or smaller sizes may take)
+    size_t need = layout_for(D, M, N, nnz, 3, true).total;
+    auto room = [&](const Layout &l) { if (l.total > need) need = l.total; };
+    if (wide) room(f16_wide_layout(ow, D, M, N, nnz, true));
+    if (screen_within(o, D, M, N, nnz, true)) room(screen_layout_of(o, D, M, N, nnz, true));
+    return need;
 }
 
 int bmu_search_f16_ws(const void *W16, int64_t D, int64_t M, const float *norms,
@@ -1013,7 +1037,7 @@ int bmu_search_f16_ws(const void *W16, int64_t D, int64_t M, const float *norms,
                   "documents", MMA_SLAB, head);
         return BMU_ERR_UNSUPPORTED;
     }
-    const Layout l = wide ? layout_of(ow, D, M, N, nnz, top2) : layout_for(D, M, N, nnz, 3, top2);
+    const Layout l = wide ? f16_wide_layout(ow, D, M, N, nnz, top2) : layout_for(D, M, N, nnz, 3, top2);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255) != 0 || ws_bytes < l.total) {
         set_error("workspace missing, not 256-byte aligned, or smaller than %zu bytes", l.total);
         return BMU_ERR_WORKSPACE;

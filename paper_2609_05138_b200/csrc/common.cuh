@@ -182,7 +182,7 @@ struct FewArgs {
     int32_t *out_bmu, *out_bmu2;
     float *out_dist, *out_dist2;
 };
-size_t few_slots_bytes(int64_t M, int64_t N, bool top2, int sms);
+size_t few_slots_bytes(int64_t M, int64_t N, bool top2);
 int launch_sweep_few(FewArgs a, bool top2, int sms, cudaStream_t s);
 
 // ---- tiling plan (plan.cu) ---------------------------------------------------

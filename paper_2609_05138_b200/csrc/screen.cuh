@@ -105,7 +105,10 @@ struct VerifyArgs {
 void screen_layout(int64_t D, int64_t M, int64_t N, int head, int64_t chunk, bool top2, int sms,
                    ScreenLayout *l);
 void screen_shared_layout(int64_t D, int64_t M, int head, int64_t chunk, ScreenLayout *l);
+// blocks that share a launch's slabs, and the most that `blocks` or fewer sets of documents take of them in
+// all: a bound that grows with the blocks, unlike the splits, so that a workspace for many serves fewer
 int screen_splits(int64_t blocks, int64_t n_slabs, int sms);
+int64_t screen_split_blocks(int64_t blocks, int64_t n_slabs, int sms);
 // row ranges, scales, errors and the per-document windows: once per search (key: a document's gathered
 // ids, by its number in the corpus; the maxima behind `status` are zero).  codebook arrays at cb + cl;
 // `earlier`: the scalars of an earlier search of the same codebook and head, whose ranges still stand

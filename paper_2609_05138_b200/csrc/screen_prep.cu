@@ -33,9 +33,10 @@ void screen_layout(int64_t D, int64_t M, int64_t N, int head, int64_t chunk, boo
     const int64_t all = (M + SC_SLAB - 1) / SC_SLAB;
     l->chunk_slabs = chunk / SC_SLAB < all ? chunk / SC_SLAB : all;
     const int64_t launches = (all + l->chunk_slabs - 1) / l->chunk_slabs;
-    l->splits = screen_splits(l->n_pad / SC_DOCS, (all + launches - 1) / launches, sms);
+    const int64_t blocks = l->n_pad / SC_DOCS, slabs = (all + launches - 1) / launches;
+    l->splits = screen_splits(blocks, slabs, sms);
     const size_t n4 = (size_t)l->n_pad * 4;
-    const size_t stripes = (size_t)l->n_pad * 4 * (size_t)l->splits;
+    const size_t stripes = (size_t)screen_split_blocks(blocks, slabs, sms) * SC_DOCS * 4;
     codebook_layout(D, l->chunk_slabs, 1, take, l);
     l->window = take(n4);
     l->amin = take(n4); l->amin2 = top2 ? take(n4) : l->amin;

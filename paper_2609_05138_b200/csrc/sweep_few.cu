@@ -130,7 +130,10 @@ sweep_few_kernel(const FewArgs a)
 // How a search is cut: H = 2 (slabs of 256 neurons) once that still gives every SM sixteen warps,
 // else slabs of 128; pieces of one slab until there are four hundred warps per SM, longer ones
 // beyond (a warp's own set-up and merge are paid once per piece).  1000 documents on 65,536 units:
-// 1609 us with slabs of 128 and 64 warps per SM, 1087 so.
+// 1609 us with slabs of 128 and 64 warps per SM, 1087 so.  Never more than FEW_SLOTS keys beside one per
+// document (millions of units, or tens of thousands of nearly empty documents).
+static const int64_t FEW_SLOTS = 1 << 20;
+
 static void few_cut(int64_t M, int64_t N, bool vec, int sms, int &h, int64_t &piece)
 {
     h = vec && (M + 255) / 256 * N >= (int64_t)sms * 16 ? 2 : 1;
@@ -139,18 +142,16 @@ static void few_cut(int64_t M, int64_t N, bool vec, int sms, int &h, int64_t &pi
     if (per < 1) per = 1;
     if (per > 16) per = 16;
     if ((slabs + per - 1) / per > 65535) per = (slabs + 65534) / 65535;
+    if ((slabs + per - 1) / per * N > FEW_SLOTS + N) per = (slabs * N + FEW_SLOTS - 1) / FEW_SLOTS;
     piece = per * slab;
 }
 
-size_t few_slots_bytes(int64_t M, int64_t N, bool top2, int sms)
+// Room for any of its cuts: a bound that grows with the documents, unlike the cuts, so that a workspace
+// for many serves fewer.
+size_t few_slots_bytes(int64_t M, int64_t N, bool top2)
 {
-    int h;
-    int64_t piece, most = 0;
-    for (int vec = 0; vec < 2; ++vec) {          // (whether W is aligned is not known yet)
-        few_cut(M, N, vec, sms, h, piece);
-        if ((M + piece - 1) / piece > most) most = (M + piece - 1) / piece;
-    }
-    return (size_t)N * (size_t)most * sizeof(u64) * (top2 ? 2 : 1);
+    const int64_t all = (M + 127) / 128 * N, most = FEW_SLOTS + N;
+    return (size_t)(all < most ? all : most) * sizeof(u64) * (top2 ? 2 : 1);
 }
 
 template <bool VEC, int H>

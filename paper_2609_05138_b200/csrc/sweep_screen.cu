@@ -374,6 +374,14 @@ sweep_screen_kernel(const ScreenArgs a)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 
+int64_t screen_split_blocks(int64_t blocks, int64_t n_slabs, int sms)
+{
+    // what screen_splits takes beyond one block per set, at most (where it takes two: up to about
+    // 3/4 n_slabs * sms sets)
+    const int64_t most = (n_slabs < 16 ? n_slabs : 16) - 1, extra = 3 * (n_slabs + 4) * sms / 4;
+    return blocks + (most * blocks < extra ? most * blocks : extra);
+}
+
 // How many blocks share a launch's slabs for one set of documents, in units of a slab's time.  Each
 // block costs about half a slab to set up.  A few blocks per SM run in waves; with many, the longest
 // lists first and all blocks of a split in front of the next, the scheduler evens them out but for about
@@ -382,9 +390,10 @@ sweep_screen_kernel(const ScreenArgs a)
 // with four stretches per SM and 64.8 with one, against 56.9, on 512 x 512.)
 int screen_splits(int64_t blocks, int64_t n_slabs, int sms)
 {
+    const int64_t room = screen_split_blocks(blocks, n_slabs, sms);
     int best = 1;
     double least = 1e300;
-    for (int sp = 1; sp <= 16 && sp <= n_slabs; ++sp) {
+    for (int sp = 1; sp <= 16 && sp <= n_slabs && blocks * sp <= room; ++sp) {
         const int64_t waves = (blocks * sp + sms - 1) / sms;
         const double t = waves <= 4 ? (double)waves * ((double)((n_slabs + sp - 1) / sp) + 0.5)
                                     : (double)blocks * ((double)n_slabs + 0.5 * sp) / sms + (double)n_slabs / sp;

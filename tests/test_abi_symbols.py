@@ -53,6 +53,42 @@ def test_workspace_size_is_monotone(lib):
     assert a % 256 == 0 and b >= 262144 * 4 + 2_000_000 * 8
 
 
+def test_a_workspace_for_more_documents_serves_fewer(lib):
+    """The size queries never fall when documents or listings are added: a workspace allocated once for the
+    largest batch serves every smaller one, whichever kernel that takes."""
+    import random
+    from paper_2609_05138_b200 import Opts
+    rng = random.Random(7)
+    chunk, one, never = Opts(), Opts(), Opts()
+    chunk.chunk_neurons = 512
+    one.two_stage = 1
+    never.two_stage = 2
+
+    def log_int(lo, hi):
+        return int(round(lo * (hi / lo) ** rng.random()))
+
+    def size(which, D, M, N, nnz, o):
+        o = ctypes.byref(o) if o else None
+        if which == "plan":
+            return lib.bmu_plan_workspace_bytes(N, nnz, D, M, o)
+        return getattr(lib, "bmu_search_%sworkspace_bytes" % which)(D, M, N, nnz, o)
+
+    for trial in range(1500):
+        which = rng.choice(["", "top2_", "f16_", "plan"])
+        o = rng.choice([None, None, None, chunk, one, never])
+        D = rng.choice([1, 300, 4096, 16384, log_int(100, 65000)])
+        M = rng.choice([1024, 4096, 16384, 127 * 127, log_int(8, 300_000)])
+        M = max(256, M // 256 * 256) if which == "f16_" else M
+        N = log_int(1, 2_000_000)
+        nnz = int(N * rng.choice([0.0, 1.0, 30.0, 80.0, 80.0, 80.0, 400.0, 2000.0]))
+        need = size(which, D, M, N, nnz, o)
+        for _ in range(6):
+            n = rng.choice([N - 1, int(N * rng.uniform(0.9, 1.0)), int(N * rng.random()), rng.randint(0, min(N, 1500)), N])
+            n = max(0, n)
+            e = rng.choice([nnz, int(nnz * rng.random()), int(nnz * (n / N))])
+            assert size(which, D, M, n, e, o) <= need, (which, D, M, (N, nnz), (n, e))
+
+
 def test_argument_checks_need_no_gpu(lib):
     # sizes are checked before any CUDA call is made
     assert lib.bmu_codebook_norms(None, -1, 4, None, None) == 1

@@ -140,6 +140,24 @@ def test_lists_that_fill_over_many_launches(bmu, kind, M):
     np.testing.assert_allclose(e2.cpu().numpy(), d2.cpu().numpy(), rtol=1e-6)
 
 
+@pytest.mark.parametrize("n,fewer", [(45_500, 45_000), (45_500, 9_000), (2_500, 1_500), (2_500, 300)])
+def test_a_workspace_for_more_documents_serves_fewer(bmu, n, fewer):
+    """Best unit, second-best unit and half precision with the workspace of a larger search."""
+    cfg = synth.CONFIGS["cfg1"]
+    W = synth.make_codebook(cfg.D, 1024, 68, kind="scaled").half().float().cuda()
+    lens = synth.draw_nnz("poisson", 80.0, n, torch.Generator().manual_seed(4), "cpu")
+    rp, ci = (x.cuda() for x in synth.draw_corpus(n, cfg.D, 1.0, lens, 4, "cpu"))
+    small = (rp[:fewer + 1].contiguous(), ci[:int(rp[fewer])].contiguous())
+    lib = bmu.load()
+    for query, search, Wd in (("", bmu.bmu_search_ws, W), ("top2_", bmu.bmu_search_top2_ws, W),
+                              ("f16_", bmu.bmu_search_f16_ws, W.half())):
+        need = int(getattr(lib, "bmu_search_%sworkspace_bytes" % query)(cfg.D, 1024, n, ci.numel(), None))
+        ws = torch.empty(need + 256, dtype=torch.uint8, device="cuda")
+        got = [x.clone() for x in search(Wd, *small, workspace=ws)]
+        own = search(Wd, *small)
+        assert all(torch.equal(a, b) for a, b in zip(got, own))
+
+
 def test_batches_share_the_images_of_the_codebook(bmu):
     """Batches of one call: the second has lists that the images of the first are too fine for, the
     third lists other features, the fourth takes another route.  Every result as by itself."""
