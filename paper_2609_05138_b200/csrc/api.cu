@@ -152,7 +152,7 @@ static Layout layout_for(int64_t D, int64_t M, int64_t N, int64_t nnz, int kerne
     }
     l.plan_off = off;
     memset(&l.plan, 0, sizeof(l.plan));
-    if (kernel != 1 && D <= LANES_MAX_D) off += plan_bytes(N, nnz, head, D, cluster, &l.plan);
+    if (kernel != 1 && D <= LANES_MAX_D) off += plan_bytes(N, nnz, head, D, cluster, screen_chunk != 0, &l.plan);
     l.total = off;
     return l;
 }

@@ -260,7 +260,8 @@ int launch_sweep_mma2(const MmaArgs &a, const bmu_opts &o, cudaStream_t s);
 int launch_sweep_mma2_f16(const MmaArgs &a, const bmu_opts &o, cudaStream_t s);
 int launch_head_split2_f16(const void *W16, int64_t M, int64_t m_full, int head, const uint16_t *feat,
                            unsigned char *head_img, cudaStream_t s);
-size_t plan_bytes(int64_t N, int64_t nnz, int head, int64_t D, int cluster, PlanLayout *l);
+// quads: what launch_plan_screen makes and nothing else
+size_t plan_bytes(int64_t N, int64_t nnz, int head, int64_t D, int cluster, bool quads, PlanLayout *l);
 int launch_plan(const int32_t *rowptr, const int32_t *colidx, int64_t N, int64_t nnz,
                 int order_by_length, int head, int relabel, int64_t D, char *ws, const PlanLayout &l,
                 uint32_t *status, cudaStream_t s);

@@ -515,26 +515,27 @@ plan_tile_fill_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restr
     }
 }
 
-size_t plan_bytes(int64_t N, int64_t nnz, int head, int64_t D, int cluster, PlanLayout *l)
+size_t plan_bytes(int64_t N, int64_t nnz, int head, int64_t D, int cluster, bool quads, PlanLayout *l)
 {
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
     size_t off = 0;
     PlanLayout t;
     t.perm_off = off; off = up(off + (size_t)N * 4);
     t.docoff_off = off; off = up(off + (size_t)(N + 1) * 4);
-    t.ngroups_off = off; off = up(off + (size_t)(N + 1) * 4);
+    t.ngroups_off = off; if (!quads) off = up(off + (size_t)(N + 1) * 4);
     t.bins_off = off; off = up(off + (size_t)PLAN_BINS * 4 * 2 + 256);   // counters, cursors, aux
     t.id_groups_cap = (size_t)nnz / 8 + 2 * (size_t)N + 4;
-    t.ids_off = off; off = up(off + t.id_groups_cap * 16);
+    t.ids_off = off; if (!quads) off = up(off + t.id_groups_cap * 16);
     size_t scan_tmp = 0;
-    cub::DeviceScan::ExclusiveSum(nullptr, scan_tmp, (uint32_t *)nullptr, (uint32_t *)nullptr,
-                                  (int)(N + 1));
+    if (!quads)
+        cub::DeviceScan::ExclusiveSum(nullptr, scan_tmp, (uint32_t *)nullptr, (uint32_t *)nullptr,
+                                      (int)(N + 1));
     t.scan_off = off; t.scan_bytes = scan_tmp; off = up(off + scan_tmp);
     // tiles: with documents exactly length-ordered, the sum over tiles of the longest row
     // is at most nnz / 8 plus the spread of lengths (< 65536)
     const size_t n_tiles = ((size_t)N + 7) / 8;
     t.tilelen_off = off; off = up(off + (n_tiles + 1) * 4);
-    t.tilerows_off = off; off = up(off + (n_tiles + 1) * 4);
+    t.tilerows_off = off; if (!quads) off = up(off + (n_tiles + 1) * 4);
     t.tileoff_off = off; off = up(off + (n_tiles + 1) * 4);
     t.tilehead_off = off; off = up(off + n_tiles * 8 * 4 * (size_t)(head > 32 ? head / 32 : 1));
     t.tile_rows_cap = (size_t)nnz / 8 + 65536 + 4 * n_tiles;     // (rounded up to whole groups of four)
@@ -546,11 +547,14 @@ size_t plan_bytes(int64_t N, int64_t nnz, int head, int64_t D, int cluster, Plan
         const size_t d4 = up((size_t)D * 4), d2 = up((size_t)D * 2);
         t.rank_off = off; off += d2;
         t.feat_off = off; off += d2;
-        t.fsort_off = off; off += 4 * d4;            // counts, sorted counts, ids, sorted ids
-        size_t tmp = 0;
-        cub::DeviceRadixSort::SortPairsDescending(nullptr, tmp, (uint32_t *)nullptr, (uint32_t *)nullptr,
-                                                  (uint32_t *)nullptr, (uint32_t *)nullptr, (int)D);
-        t.fsort_tmp_off = off; t.fsort_tmp_bytes = tmp; off = up(off + tmp);
+        t.fsort_off = t.fsort_tmp_off = off;
+        if (!quads) {
+            off += 4 * d4;                           // counts, sorted counts, ids, sorted ids
+            size_t tmp = 0;
+            cub::DeviceRadixSort::SortPairsDescending(nullptr, tmp, (uint32_t *)nullptr, (uint32_t *)nullptr,
+                                                      (uint32_t *)nullptr, (uint32_t *)nullptr, (int)D);
+            t.fsort_tmp_off = off; t.fsort_tmp_bytes = tmp; off = up(off + tmp);
+        }
     }
     // ordering by content: 64-bit keys and document numbers, in and out, and the sort's scratch
     t.cluster_off = t.cluster_tmp_off = off;

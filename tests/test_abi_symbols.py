@@ -89,6 +89,16 @@ def test_a_workspace_for_more_documents_serves_fewer(lib):
             assert size(which, D, M, n, e, o) <= need, (which, D, M, (N, nnz), (n, e))
 
 
+def test_the_two_stage_form_reserves_one_copy_of_the_ids(lib):
+    """Its sweep walks 16-bit id lists by tile; the row lists of the other kernels are no part of it."""
+    from paper_2609_05138_b200 import Opts
+    o = Opts()
+    o.two_stage = 1
+    f = lambda nnz: lib.bmu_search_workspace_bytes(16384, 4096, 1_000_000, nnz, ctypes.byref(o))
+    o.kernel = 6                                      # (kernel 0 makes room for the other kernels too)
+    assert f(160_000_000) - f(80_000_000) <= 80_000_000 * 2 + 4096
+
+
 def test_argument_checks_need_no_gpu(lib):
     # sizes are checked before any CUDA call is made
     assert lib.bmu_codebook_norms(None, -1, 4, None, None) == 1
