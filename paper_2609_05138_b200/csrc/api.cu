@@ -501,6 +501,8 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
     v.lbase = reinterpret_cast<uint32_t *>(sb + l.screen.lbase);
     v.state = state; v.state2 = state2; v.status = status; v.splits = a.splits;
     v.out_bmu = out_bmu; v.out_dist = out_dist; v.out_bmu2 = out_bmu2; v.out_dist2 = out_dist2;
+    v.dense = reinterpret_cast<uint32_t *>(sb + l.screen.cval);         // (after the last launch)
+    v.dense_count = status + STATUS_DENSE;
     a.amin = v.amin; a.amin2 = v.amin2;
     // the slabs are dealt to the launches in turn, so that every launch sees the whole map: after
     // the first one a document's smallest value is near its final one and little joins its list
@@ -522,7 +524,8 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
         if ((rc = launch_sweep_screen(a, top2, s))) return rc;
         if ((rc = launch_screen_collect(v, top2, s))) return rc;
     }
-    return launch_screen_verify(v, top2, s);
+    if ((rc = launch_screen_verify(v, top2, s))) return rc;
+    return launch_screen_dense(v, top2, device_sms(), s);
 }
 
 static int search_impl(const float *W, int64_t D, int64_t M, const float *norms,

@@ -196,8 +196,10 @@ struct PlanLayout {
 static const int TILE_HEAD_ROWS = 32;    // ids below this are swept densely, once per tile
 static const int HEAD_ROWS_MAX = 2048;   // widest dense head (the tensor-core sweep's)
 // words behind the status word, zero when a search begins: the longest list, the tiles' cursor and the
-// ticket of the two-stage tiling pass; the codebook's maxima, eight copies each (screen_range_kernel)
-static const int STATUS_PLAN_MOST = 35, STATUS_TILE_CURSOR = 36, STATUS_KEY_TICKET = 37, STATUS_MAXIMA = 40;
+// ticket of the two-stage tiling pass; its documents to be evaluated whole; the codebook's maxima, eight
+// copies each (screen_range_kernel)
+static const int STATUS_PLAN_MOST = 35, STATUS_TILE_CURSOR = 36, STATUS_KEY_TICKET = 37, STATUS_DENSE = 38,
+                 STATUS_MAXIMA = 40;
 // status-word bit set when a scanned offset of the tiling pass exceeds its reserved room
 static const uint32_t PLAN_STATUS_OVERFLOW = 64u;
 int launch_plan_tiles(const int32_t *rowptr, int64_t N, int interleave, int head, int relabel,

@@ -9,7 +9,8 @@
 //            could be the best (or second-best) unit is in one of these groups.
 //   verify   the groups are evaluated exactly as the gathered kernels do it: fp32 sums over
 //            the fp32 (or widened fp16) weights of the caller's codebook, fp32 distances,
-//            lowest index on ties.  Only these numbers are ever returned.
+//            lowest index on ties.  Only these numbers are ever returned.  Documents that
+//            keep too many groups, or none, are evaluated whole (screen_dense.cu).
 //
 // The bound (screen_table_kernel and screen_window_kernel in screen_prep.cu compute it).  A
 // weight w of feature f is stored as q = round((w - c_f) / step_f), c_f the row's minimum, so
@@ -38,6 +39,7 @@ static const int SC_SCALARS = 16;
 // Candidates wait in a list per document until every unit has been screened: a launch's local
 // minimum says little before the document's own region of the map has been seen.
 static const int SC_LIST = 12;           // entries: smallest value, group mask, first group
+static const uint32_t SC_DENSE = 1u << 30;           // in a document's count: to be evaluated whole
 
 // Device arrays of one search: offsets into the workspace, relative to its screen part.
 struct ScreenLayout {
@@ -90,17 +92,38 @@ struct VerifyArgs {
     const float *cval2;
     const uint4 *cmask;
     float *amin, *amin2;                 // smallest (second) approximate value so far
-    uint32_t *lcount;                    // entries of the list; bit 31: state[] holds exact keys
+    uint32_t *lcount;                    // bits 0 .. 3: entries of the list; 4 .. 29: groups evaluated already;
+                                         // 30: to be evaluated whole; 31: state[] holds exact keys
     float *lval;
     uint4 *lmask;
     uint32_t *lbase;
     u64 *state, *state2;                 // exact keys of what did not fit a list
+    uint32_t *dense, *dense_count;       // planned documents to be evaluated whole
     int32_t *out_bmu, *out_bmu2;
     float *out_dist, *out_dist2;
     uint32_t *status;
     int64_t launch, launches;            // slab s of the launch is launch + s * launches of the map
     int32_t splits, first, f16;
 };
+
+// Rows are whole 16-byte pieces
+inline bool screen_vec(const VerifyArgs &a)
+{
+    return (reinterpret_cast<uintptr_t>(a.W) & 15) == 0 && a.M % (a.f16 ? 8 : 4) == 0;
+}
+
+// A document with more candidate groups than this, an eighth of the map, is evaluated whole: scattered
+// 32-byte sectors bring an update at an eighth to a quarter of the rate of whole rows (all of a map of
+// 4,096 units for 20,000 documents: 5.5 ms, 1.3).  Those that find no place in a list are evaluated before
+// it is known how many there will be: a quarter of that.
+__host__ __device__ __forceinline__ uint32_t screen_dense_groups(int64_t M)
+{
+    return M / 64 > 8 ? (uint32_t)(M / 64) : 8u;
+}
+__host__ __device__ __forceinline__ uint32_t screen_early_groups(int64_t M)
+{
+    return M / 256 > 8 ? (uint32_t)(M / 256) : 8u;
+}
 
 void screen_layout(int64_t D, int64_t M, int64_t N, int head, int64_t chunk, bool top2, int sms,
                    ScreenLayout *l);
@@ -124,10 +147,26 @@ int launch_screen_quantize(const void *W, int f16, int64_t D, int64_t M, const f
                            int64_t k, int64_t launches, int64_t n_slabs, int64_t slot, int head,
                            const uint16_t *feat, char *cb, const ScreenLayout &cl, const float *scalars,
                            bool expected, cudaStream_t s);
+// A launch that may begin under the end of the one before it on the stream, if that one's blocks allow it
+// (griddepcontrol.launch_dependents) and the kernel waits before it reads or writes (griddepcontrol.wait).
+struct ScreenLaunch {
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t c;
+    ScreenLaunch(unsigned blocks, unsigned threads, cudaStream_t s, bool early) : c()
+    {
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        c.gridDim = dim3(blocks); c.blockDim = dim3(threads);
+        c.stream = s; c.attrs = &attr; c.numAttrs = early ? 1 : 0;
+    }
+    ScreenLaunch(const ScreenLaunch &) = delete;
+};
 int launch_sweep_screen(const ScreenArgs &a, bool top2, cudaStream_t s);
 // after each launch: what it could not rule out, into the documents' lists
 int launch_screen_collect(const VerifyArgs &a, bool top2, cudaStream_t s);
 // after the last: the lists evaluated exactly, and the outputs
 int launch_screen_verify(const VerifyArgs &a, bool top2, cudaStream_t s);
+// directly behind it: the documents it handed over (none, as a rule)
+int launch_screen_dense(const VerifyArgs &a, bool top2, int sms, cudaStream_t s);
 
 }  // namespace bmu

@@ -4,11 +4,12 @@
 //          groups one lane of the sweep carried) in every split of the launch; stripes
 //          whose smallest approximate distance lies within the document's window of the smallest seen
 //          so far join the document's list.  A full list drops what the shrunken minimum has ruled
-//          out; what still does not fit is evaluated at once.
+//          out; what still does not fit is evaluated at once, up to screen_early_groups.
 // verify   after the last launch: the groups still within the window are evaluated exactly -- a 32-byte
 //          sector per row (16 bytes of fp16), sixteen (32) rows per instruction and four instructions
 //          in flight, as many fp32 sums per unit added in a fixed order -- and the outputs written.
-//          Exact keys are merged by their minimum, so the order never changes a result.
+//          Exact keys are merged by their minimum, so the order never changes a result.  Documents
+//          with more groups than screen_dense_groups, with none, or with an infinite window are handed on.
 //
 // Waiting for the last launch matters on trained maps: far from a document's own region the
 // distances lie close together, and evaluating every launch's local minimum took 11.4 ms of a
@@ -175,6 +176,7 @@ __device__ __forceinline__ void verify_merge(u64 &best, u64 &best2)
     }
 }
 
+__device__ __forceinline__ uint32_t popc4(const uint4 v) { return __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w); }
 __device__ __forceinline__ uint4 shfl4(const uint4 v, int src)
 {
     return make_uint4(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src),
@@ -188,11 +190,12 @@ screen_collect_kernel(const VerifyArgs a)
 {
     const int lane = threadIdx.x & 31, k = lane & 3;
     const int64_t p = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 8 + (lane >> 2);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // (the verify stage, after the last launch)
     // (one lane reads the status word for its warp: the lanes must stay together)
     if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(a.status), 0)) return;
     const bool there = p < a.N;
     const float win = there ? a.window[p] : 0.f;
-    const uint32_t seg = 15u << (lane & ~3);
+    const uint32_t seg = 15u << (lane & ~3), most = screen_early_groups(a.M);
     // pass 1: the document's smallest (and second smallest) approximate value so far.  The stripes of
     // a split bring the same second smallest, over all their groups and the earlier launches;
     // whatever a merge of such pairs leaves out only makes it larger, which keeps more.
@@ -215,8 +218,8 @@ screen_collect_kernel(const VerifyArgs a)
         v1 = fminf(v1, o1);
     }
     const float limit = (TOP2 ? v2 : v1) + win;
-    uint32_t count = there && !a.first ? a.lcount[p] : 0u, n = count & 0x7fffffffu;
-    bool touched = a.first;
+    uint32_t count = there && !a.first ? a.lcount[p] : 0u, n = count & 15u, done = count >> 4 & 0x3ffffffu;
+    bool touched = a.first, dense = (count & SC_DENSE) != 0u || win == CUDART_INF_F;
     float *lv = a.lval + (size_t)p * SC_LIST;
     uint4 *lm = a.lmask + (size_t)p * SC_LIST;
     uint32_t *lb = a.lbase + (size_t)p * SC_LIST;
@@ -226,7 +229,7 @@ screen_collect_kernel(const VerifyArgs a)
         const float2 cv = there ? a.cval[at] : make_float2(CUDART_INF_F, 0.f);
         const float own = cv.x;
         uint4 mask = make_uint4(0u, 0u, 0u, 0u);
-        if (there && own <= limit) {
+        if (there && !dense && own <= limit) {
             // words the block has written, slabs its minimum counts from
             const int from = __float_as_int(cv.y) & 255, to = __float_as_int(cv.y) >> 8;
             const uint32_t *words = reinterpret_cast<const uint32_t *>(a.cmask + at);
@@ -281,11 +284,16 @@ screen_collect_kernel(const VerifyArgs a)
             u64 best = KEY_WORST, best2 = KEY_WORST;
             for (uint32_t lanes = left_over; lanes; lanes &= lanes - 1) {
                 const int src = __ffs(lanes) - 1;
+                const uint4 groups = shfl4(mask, src);
+                const uint32_t more = popc4(groups) + __shfl_sync(0xffffffffu, done, src);
+                if (__shfl_sync(0xffffffffu, dense, src)) continue;
+                if (lane >> 2 == src >> 2) { dense = more > most; done = more; }
+                if (more > most) continue;
                 u64 k1 = KEY_WORST, k2 = KEY_WORST;
                 const int b0 = __shfl_sync(0xffffffffu, beg, src), e0 = __shfl_sync(0xffffffffu, end, src);
                 uint32_t ids[4];
                 if (VEC) VerifyVec<WT>::ids_of(a, b0, e0, ids);
-                verify_groups<WT, TOP2, VEC>(a, shfl4(mask, src), __shfl_sync(0xffffffffu, base, src), b0, e0, ids, k1, k2);
+                verify_groups<WT, TOP2, VEC>(a, groups, __shfl_sync(0xffffffffu, base, src), b0, e0, ids, k1, k2);
                 verify_merge<TOP2>(k1, k2);
                 if (lane >> 2 == src >> 2) {
                     if (TOP2) Best<true>::merge(best, best2, k1, k2);
@@ -310,7 +318,7 @@ screen_collect_kernel(const VerifyArgs a)
     if (there && k == 0) {
         a.amin[p] = v1;
         if (TOP2) a.amin2[p] = v2;
-        if (touched) a.lcount[p] = (count & 0x80000000u) | n;
+        if (touched) a.lcount[p] = (count & 0x80000000u) | (dense ? SC_DENSE : done << 4 | n);
     }
 }
 
@@ -319,7 +327,9 @@ template <typename WT, bool TOP2, bool VEC>
 __global__ void __launch_bounds__(256, 5)
 screen_verify_kernel(const VerifyArgs a)
 {
-    static_assert(SC_LIST <= 16, "a lane per entry");
+    static_assert(SC_LIST <= 15, "a lane per entry, four bits of the count");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // screen_dense_kernel waits for the rest
+    asm volatile("griddepcontrol.wait;" ::: "memory");                   // as this does for the last collection
     const int lane = threadIdx.x & 31, e = lane & 15;
     const int64_t p = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 2 + (lane >> 4);
     if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(a.status), 0)) return;
@@ -332,13 +342,18 @@ screen_verify_kernel(const VerifyArgs a)
         orig = a.perm[p];
         beg = __ldg(a.rowptr + orig);
         end = __ldg(a.rowptr + orig + 1);
-        if ((uint32_t)e < (count & 0x7fffffffu)) {
+        if ((uint32_t)e < (count & 15u)) {
             const float limit = (TOP2 ? a.amin2[p] : a.amin[p]) + a.window[p];
             if (a.lval[(size_t)p * SC_LIST + e] <= limit) todo = a.lmask[(size_t)p * SC_LIST + e];
             base = a.lbase[(size_t)p * SC_LIST + e];
         }
     }
-    __syncwarp();
+    // too many groups, or none (no distance of it is finite), or given up before
+    uint32_t groups = popc4(todo);
+#pragma unroll
+    for (int m = 8; m > 0; m >>= 1) groups += __shfl_xor_sync(0xffffffffu, groups, m);
+    const bool dense = (count & SC_DENSE) || groups > screen_dense_groups(a.M) || (groups == 0u && !(count & 0x80000000u));
+    if (dense) todo = make_uint4(0u, 0u, 0u, 0u);
     u64 best = KEY_WORST, best2 = KEY_WORST;
     const uint32_t entries = __ballot_sync(0xffffffffu, (todo.x | todo.y | todo.z | todo.w) != 0u);
 #pragma unroll 1
@@ -356,6 +371,15 @@ screen_verify_kernel(const VerifyArgs a)
         verify_merge<TOP2>(k1, k2);
         if (lane >> 4 == d) { best = k1; best2 = k2; }
     }
+    if (there && dense) {
+        if (e == 0) {
+            a.state[orig] = KEY_WORST;
+            if (TOP2) a.state2[orig] = KEY_WORST;
+            a.lcount[p] = 0u;                                // its ticket from here on
+            a.dense[atomicAdd(a.dense_count, 1u)] = (uint32_t)p;
+        }
+        return;
+    }
     if (there && (count & 0x80000000u)) {
         if (TOP2) Best<true>::merge(best, best2, a.state[orig], a.state2[orig]);
         else { const u64 old = a.state[orig]; best = old < best ? old : best; }
@@ -372,35 +396,25 @@ screen_verify_kernel(const VerifyArgs a)
     }
 }
 
-static bool verify_vec(const VerifyArgs &a)
-{
-    return (reinterpret_cast<uintptr_t>(a.W) & 15) == 0 && a.M % (a.f16 ? 8 : 4) == 0;
-}
-
-#define BMU_VERIFY(KERNEL, BLOCKS) \
-    do { \
-        const bool vec = verify_vec(a); \
-        if (a.f16) { \
-            if (top2) { if (vec) KERNEL<__half, true, true><<<BLOCKS, 256, 0, s>>>(a); else KERNEL<__half, true, false><<<BLOCKS, 256, 0, s>>>(a); } \
-            else { if (vec) KERNEL<__half, false, true><<<BLOCKS, 256, 0, s>>>(a); else KERNEL<__half, false, false><<<BLOCKS, 256, 0, s>>>(a); } \
-        } else { \
-            if (top2) { if (vec) KERNEL<float, true, true><<<BLOCKS, 256, 0, s>>>(a); else KERNEL<float, true, false><<<BLOCKS, 256, 0, s>>>(a); } \
-            else { if (vec) KERNEL<float, false, true><<<BLOCKS, 256, 0, s>>>(a); else KERNEL<float, false, false><<<BLOCKS, 256, 0, s>>>(a); } \
-        } \
-        BMU_LAUNCHED(); \
-    } while (0)
+#define BMU_VERIFY(KERNEL, C) \
+    (a.f16 ? (top2 ? (screen_vec(a) ? cudaLaunchKernelEx(&C, KERNEL<__half, true, true>, a) : cudaLaunchKernelEx(&C, KERNEL<__half, true, false>, a)) \
+                   : (screen_vec(a) ? cudaLaunchKernelEx(&C, KERNEL<__half, false, true>, a) : cudaLaunchKernelEx(&C, KERNEL<__half, false, false>, a))) \
+           : (top2 ? (screen_vec(a) ? cudaLaunchKernelEx(&C, KERNEL<float, true, true>, a) : cudaLaunchKernelEx(&C, KERNEL<float, true, false>, a)) \
+                   : (screen_vec(a) ? cudaLaunchKernelEx(&C, KERNEL<float, false, true>, a) : cudaLaunchKernelEx(&C, KERNEL<float, false, false>, a))))
 
 int launch_screen_collect(const VerifyArgs &a, bool top2, cudaStream_t s)
 {
-    BMU_VERIFY(screen_collect_kernel, (unsigned)((a.N + 63) / 64));
-    BMU_CUDA(cudaGetLastError());
+    ScreenLaunch l((unsigned)((a.N + 63) / 64), 256, s, false);
+    BMU_CUDA(BMU_VERIFY(screen_collect_kernel, l.c));
+    BMU_LAUNCHED();
     return BMU_OK;
 }
 
 int launch_screen_verify(const VerifyArgs &a, bool top2, cudaStream_t s)
 {
-    BMU_VERIFY(screen_verify_kernel, (unsigned)((a.N + 15) / 16));
-    BMU_CUDA(cudaGetLastError());
+    ScreenLaunch l((unsigned)((a.N + 15) / 16), 256, s, true);
+    BMU_CUDA(BMU_VERIFY(screen_verify_kernel, l.c));
+    BMU_LAUNCHED();
     return BMU_OK;
 }
 

@@ -140,6 +140,105 @@ def test_lists_that_fill_over_many_launches(bmu, kind, M):
     np.testing.assert_allclose(e2.cpu().numpy(), d2.cpu().numpy(), rtol=1e-6)
 
 
+@pytest.mark.parametrize("M", [1, 40, 300, 1000, 1003, 2304])
+@pytest.mark.parametrize("f16", [False, True])
+def test_documents_evaluated_whole(bmu, M, f16):
+    """Every unit within the window of every document (equal units), lists that end in every place of a batch
+    of 64 ids or 8 rows: best and second-best unit, whole and ragged rows and slabs."""
+    if f16 and M % 256:
+        pytest.skip("half precision takes whole slabs of 256 units")
+    D = 2000
+    r = np.random.default_rng(12)
+    rows = [np.sort(r.permutation(D)[:n]) for n in (0, 1, 7, 8, 9, 63, 64, 65, 71, 72, 128, 200, 1100)] * 3
+    rowptr = torch.zeros(len(rows) + 1, dtype=torch.int32)
+    rowptr[1:] = torch.cumsum(torch.tensor([len(x) for x in rows]), 0)
+    colidx = torch.from_numpy(np.concatenate(rows).astype(np.int32))
+    W = torch.rand((D, 1), generator=torch.Generator().manual_seed(2)).expand(D, M)
+    W = (W * (1 + 1e-3 * (torch.arange(M) // 100 % 2))[None, :]).half().float().contiguous()
+    Wd, rp, ci, o = W.cuda(), rowptr.cuda(), colidx.cuda(), opts_of(bmu, chunk_neurons=512)
+    args = (W.numpy(), rowptr.numpy(), colidx.numpy())
+    if f16:
+        b1, d1, b2, d2 = bmu.bmu_search_f16_ws(Wd.half(), rp, ci, opts=o, top2=True)
+    else:
+        check(bmu, W, rowptr, colidx, chunk_neurons=512)
+        b1, d1, b2, d2 = bmu.bmu_search_top2_ws(Wd, rp, ci, opts=o)
+    parity.compare(b1.cpu().numpy(), d1.cpu().numpy(), *args)
+    if M == 1:
+        assert int(b2.max()) == -1 and bool(torch.isinf(d2).all())
+    else:
+        e2 = oracle.bmu2(*args)[3]
+        np.testing.assert_allclose(d2.cpu().numpy(), e2, rtol=1e-5)
+        assert bool((b2 != b1).all())
+
+
+@pytest.mark.parametrize("how", ["weights", "norms"])
+def test_distances_that_are_not_finite(bmu, how):
+    """A unit at infinity is never chosen; where all are, the answer is the single-stage kernels' one."""
+    cfg = synth.CONFIGS["cfg1"]
+    rowptr, colidx = synth.make_corpus(cfg, n_docs=200)
+    W = synth.make_codebook(cfg.D, 768, 69, kind="scaled")
+    far = list(range(0, 768, 3))
+    if how == "weights":
+        W[5, far] = 3e38                              # its norm and the row's range overflow
+    Wd, rp, ci = W.cuda(), rowptr.cuda(), colidx.cuda()
+    norms = bmu.bmu_codebook_norms(Wd)
+    if how == "norms":
+        norms[far] = float("inf")
+    assert bool(torch.isinf(norms[far]).all()) and int(torch.isinf(norms).sum()) == len(far)
+    single = bmu.Opts()
+    single.kernel, single.two_stage = 3, 2
+    for n in (norms, torch.full_like(norms, float("inf"))):
+        ob, od = bmu.bmu_search_ws(Wd, rp, ci, norms=n, opts=opts_of(bmu))
+        rb, rd = bmu.bmu_search_ws(Wd, rp, ci, norms=n, opts=single)
+        assert torch.equal(ob, rb)
+        assert torch.equal(torch.isinf(od), torch.isinf(rd))
+        ok = ~torch.isinf(rd)
+        assert bool(((od - rd).abs() <= 1e-5 * rd.abs())[ok].all())
+
+
+def timed(bmu, W, rp, ci, two_stage, norms=None):
+    o = bmu.Opts()
+    o.two_stage = two_stage
+    need = bmu.bmu_search_workspace_bytes(W.shape[0], W.shape[1], rp.numel() - 1, ci.numel(), o)
+    ws = torch.empty(need + 256, dtype=torch.uint8, device="cuda")
+    ms = []
+    for _ in range(8):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        bmu.bmu_search_ws(W, rp, ci, opts=o, workspace=ws, norms=norms)
+        b.record()
+        torch.cuda.synchronize()
+        ms.append(a.elapsed_time(b))
+    return min(ms[2:])
+
+
+@pytest.mark.parametrize("what,most", [("equal units", 2.8), ("an outlier", 2.8), ("long lists", 1.5),
+                                       ("some long lists", 0.8)])
+def test_where_the_screen_cannot_rule_out_it_costs_little(bmu, what, most):
+    """The automatic choice against the single-stage one, where nothing (or for some documents nothing) can
+    be ruled out: at most the screening and, once more, all units.  Evaluated by scattered groups instead of
+    whole it was 5.4, 8.0, 3.0 and 2.9 times as long."""
+    D, M, dev = 16384, 4096, torch.device("cuda")
+    g = torch.Generator(device=dev).manual_seed(6)
+    n = 60_000 if what == "some long lists" else 20_000
+    lens = torch.full((n,), 80, dtype=torch.int64, device=dev)
+    if what == "long lists":
+        n, lens = 5_000, lens[:5_000] * 25
+    rp, ci = synth.draw_corpus(n, D, 1.1 if what != "long lists" else 0.2, lens, 6, dev)
+    if what == "some long lists":
+        extra = torch.cat([torch.randperm(D, generator=g, device=dev)[:3000].sort().values for _ in range(60)])
+        rp = torch.cat([rp, rp[-1] + 3000 * torch.arange(1, 61, dtype=torch.int32, device=dev)])
+        ci = torch.cat([ci, extra.to(torch.int32)])
+    if what == "equal units":
+        W = torch.rand((D, 1), generator=g, device=dev).expand(D, M).contiguous()
+    else:
+        W = synth.make_codebook(D, M, 3, dev)
+    if what == "an outlier":
+        W[D - 5, 77] = 1000.0
+    assert bmu.bmu_describe_search(D, M, rp.numel() - 1, ci.numel()).two_stage
+    assert timed(bmu, W, rp, ci, 0) <= most * timed(bmu, W, rp, ci, 2)
+
+
 @pytest.mark.parametrize("n,fewer", [(45_500, 45_000), (45_500, 9_000), (2_500, 1_500), (2_500, 300)])
 def test_a_workspace_for_more_documents_serves_fewer(bmu, n, fewer):
     """Best unit, second-best unit and half precision with the workspace of a larger search."""
