@@ -33,8 +33,8 @@ static const int SC_DOCS = 128;          // documents per block
 static const int SC_MAX_HEAD = 1536;     // X_head in tensor memory: one column per four features
 static const int SC_MAX_SLABS = 32;      // per launch: four bits each in a stripe's group mask
 static const int SC_K_MAX = 32;          // largest integer row scale of a head feature
-// -2 d_head, -2 d_tail, 1 / d_tail, d_head, q_max, max |norm|, 65535 / q_max, whether the images have
-// to be made, largest range of the head rows and of the others
+// -2 d_head, -2 d_tail, 1 / d_tail, unused, q_max, max |norm|, 65535 / q_max (the longest list that is
+// screened), whether the images have to be made, largest range of the head rows and of the others
 static const int SC_SCALARS = 16;
 // Candidates wait in a list per document until every unit has been screened: a launch's local
 // minimum says little before the document's own region of the map has been seen.

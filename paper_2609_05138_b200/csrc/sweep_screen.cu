@@ -234,7 +234,8 @@ sweep_screen_kernel(const ScreenArgs a)
         const uint4 *ids = a.tile_ids;
         [[maybe_unused]] size_t room = a.tile_rows_cap;
         if (tile < a.n_tiles) {
-            const uint32_t rows = __ldg(a.tile_len + tile) & 0xffffu;
+            // (longer lists than the sums hold are evaluated whole)
+            const uint32_t rows = min(__ldg(a.tile_len + tile) & 0xffffu, (uint32_t)__ldg(a.scalars + 6));
             quads = (rows + 3) / 4;
             const uint32_t off = BMU_IDX(__ldg(a.tile_off + tile), a.tile_rows_cap, a.status);
             ids += off; room -= off;
