@@ -476,7 +476,8 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
     a.tile_head = reinterpret_cast<const uint32_t *>(pw + l.plan.tilehead_off);
     int rc = launch_screen_prepare(W, f16, D, M, norms, rowptr, colidx, N, head, feat, rank, perm,
                                    reinterpret_cast<const uint32_t *>(pw + l.plan.docoff_off), a.tile_len, cb, cl,
-                                   scalars, earlier, reinterpret_cast<float *>(sb + l.screen.window),
+                                   scalars, earlier, reinterpret_cast<float *>(sb + l.screen.sample),
+                                   reinterpret_cast<float *>(sb + l.screen.window),
                                    l.screen.n_pad, status, s);
     if (rc) return rc;
     a.kpack = reinterpret_cast<const uint32_t *>(cb + cl.kpack);
@@ -503,6 +504,7 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
     v.out_bmu = out_bmu; v.out_dist = out_dist; v.out_bmu2 = out_bmu2; v.out_dist2 = out_dist2;
     v.dense = reinterpret_cast<uint32_t *>(sb + l.screen.cval);         // (after the last launch)
     v.dense_count = status + STATUS_DENSE;
+    v.scalars = scalars;
     a.amin = v.amin; a.amin2 = v.amin2;
     // the slabs are dealt to the launches in turn, so that every launch sees the whole map: after
     // the first one a document's smallest value is near its final one and little joins its list

@@ -36,6 +36,8 @@ static const int SC_K_MAX = 32;          // largest integer row scale of a head 
 // -2 d_head, -2 d_tail, 1 / d_tail, unused, q_max, max |norm|, 65535 / q_max (the longest list that is
 // screened), whether the images have to be made, largest range of the head rows and of the others
 static const int SC_SCALARS = 16;
+// ... and, as integers, how many of the sampled documents are to be evaluated whole, and how many were sampled
+static const int SC_VOTES = 10, SC_SAMPLED = 11, SC_SAMPLE = 16;
 // Candidates wait in a list per document until every unit has been screened: a launch's local
 // minimum says little before the document's own region of the map has been seen.
 static const int SC_LIST = 12;           // entries: smallest value, group mask, first group
@@ -43,7 +45,7 @@ static const uint32_t SC_DENSE = 1u << 30;           // in a document's count: t
 
 // Device arrays of one search: offsets into the workspace, relative to its screen part.
 struct ScreenLayout {
-    size_t scalars, rmin, rmax, table, kpack, khead, window, amin, amin2;
+    size_t scalars, rmin, rmax, table, kpack, khead, sample, window, amin, amin2;
     size_t cval, cval2, cmask, lcount, lval, lmask, lbase, img8, head_img, normp, total;
     int64_t n_pad;                       // documents rounded up to whole blocks
     int head_pad;                        // head rows rounded up to a stage (128)
@@ -99,12 +101,22 @@ struct VerifyArgs {
     uint32_t *lbase;
     u64 *state, *state2;                 // exact keys of what did not fit a list
     uint32_t *dense, *dense_count;       // planned documents to be evaluated whole
+    const float *scalars;
     int32_t *out_bmu, *out_bmu2;
     float *out_dist, *out_dist2;
     uint32_t *status;
     int64_t launch, launches;            // slab s of the launch is launch + s * launches of the map
     int32_t splits, first, f16;
 };
+
+#ifdef __CUDACC__
+// Most of the sampled documents are better evaluated whole: nothing is screened, all documents are.
+__device__ __forceinline__ bool screen_whole(const float *scalars)
+{
+    const uint32_t *s = reinterpret_cast<const uint32_t *>(scalars);
+    return 2u * __ldg(s + SC_VOTES) > __ldg(s + SC_SAMPLED);
+}
+#endif
 
 // Rows are whole 16-byte pieces
 inline bool screen_vec(const VerifyArgs &a)
@@ -139,7 +151,7 @@ int launch_screen_prepare(const void *W, int f16, int64_t D, int64_t M, const fl
                           const int32_t *rowptr, const int32_t *colidx, int64_t N, int head,
                           const uint16_t *feat, const uint16_t *rank, const int32_t *perm,
                           const uint32_t *key, const uint32_t *tile_len, char *cb, const ScreenLayout &cl,
-                          float *scalars, const float *earlier, float *window, int64_t n_pad,
+                          float *scalars, const float *earlier, float *sample, float *window, int64_t n_pad,
                           uint32_t *status, cudaStream_t s);
 // the 8-bit images and the norms of the n_slabs slabs of launch k (neurons beyond M: never chosen), into the slots from `slot` on; nothing if the scalars say that they stand, as may
 // be `expected`

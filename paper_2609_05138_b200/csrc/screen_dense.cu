@@ -2,12 +2,12 @@
 // chip.  The verify stage hands over those with more candidate groups than screen_dense_groups -- exact
 // or near ties all over the map, as after an epoch with a wide neighbourhood, weights the 8-bit image does
 // not resolve, lists too long for its sums -- and those without any candidate (distances that are not
-// finite).
+// finite).  Where most of a sample of the documents would come here, all do, and nothing is screened.
 //
-// A warp takes a document and a piece of the map, slabs of 256 units (128 where rows are not whole 16-byte
-// pieces): every lane owns eight of a slab and adds its part of each listed row of W, fp32 sums in the row's
-// order, ids through shared memory.  Pieces outside, documents inside, so that the warps in flight share a
-// few slabs of W in L2 and the rows of frequent features in L1.  Keys meet in the per-document state; the
+// A warp takes a document and a piece of 256 units (128 where rows are not whole 16-byte pieces): every
+// lane owns eight of them and adds its part of each listed row of W, fp32 sums in the row's order, ids
+// through shared memory.  Pieces outside, documents inside, so that all warps in flight share one piece or
+// two: rows of W in L2, those of frequent features in L1 (two or four pieces per warp, a quarter slower).  Keys meet in the per-document state; the
 // warp that arrives last at a document (a ticket each) writes its outputs.
 //
 // Bound by the L2 -> SM path, less what L1 holds: all of 50,000 documents of 80 ids on 4,096 units take 2.6
@@ -53,73 +53,72 @@ screen_dense_kernel(const VerifyArgs a)
     __shared__ uint4 s_ids[DENSE_WARPS][16];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t *mine = reinterpret_cast<uint32_t *>(s_ids[warp]);
+    const uint32_t stride = (uint32_t)a.M * (uint32_t)sizeof(WT);        // (M < 2^30)
     asm volatile("griddepcontrol.wait;" ::: "memory");       // for the verify stage, under whose end it is launched
     if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(a.status), 0)) return;
-    const int64_t docs = *a.dense_count, warps = (int64_t)gridDim.x * DENSE_WARPS;
+    const bool whole = screen_whole(a.scalars);              // all documents, in the planned order
+    const int64_t docs = whole ? a.N : (int64_t)*a.dense_count, warps = (int64_t)gridDim.x * DENSE_WARPS;
     if (docs == 0) return;
-    // pieces of up to four slabs while every warp still gets eight
-    const int64_t slabs = (a.M + 32 * V - 1) / (32 * V), share = docs * slabs / (warps * 8);
-    const int64_t per = share < 1 ? 1 : share > 4 ? 4 : share, pieces = (slabs + per - 1) / per;
+    const int64_t pieces = (a.M + 32 * V - 1) / (32 * V);
     for (int64_t item = (int64_t)blockIdx.x * DENSE_WARPS + warp; item < docs * pieces; item += warps) {
-        const int64_t p = a.dense[item % docs], j_lo = item / docs * per * (32 * V), j_hi = min(j_lo + per * (32 * V), a.M);
+        const int64_t at = item % docs, p = whole ? at : (int64_t)a.dense[at];
+        const int64_t j0 = item / docs * (32 * V);
         const int32_t orig = a.perm[p];
         const int beg = __ldg(a.rowptr + orig), end = __ldg(a.rowptr + orig + 1);
         Best<TOP2> best;
         best.init();
-        for (int64_t j0 = j_lo; j0 < j_hi; j0 += 32 * V) {
-            // where the lane's loads start; beyond the last unit they repeat it (and count for nothing)
-            const WT *col[NL];
+        // where the lane's loads start; beyond the last unit they repeat it (and count for nothing)
+        const WT *col[NL];
 #pragma unroll
-            for (int l = 0; l < NL; ++l)
-                col[l] = static_cast<const WT *>(a.W) + min(j0 + (32 * l + lane) * STEP, a.M - STEP);
-            u64 acc[(V + 1) / 2];
-            float one[V];
+        for (int l = 0; l < NL; ++l)
+            col[l] = static_cast<const WT *>(a.W) + min(j0 + (32 * l + lane) * STEP, a.M - STEP);
+        u64 acc[(V + 1) / 2];
+        float one[V];
 #pragma unroll
-            for (int v = 0; v < V; ++v) { acc[v / 2] = 0ull; one[v] = 0.f; }
-            // rows q .. of the ids at hand: ROWS of them if full, else those below c
-            auto rows = [&](int q, int c, auto full) {
-                uint4 f4[ROWS / 4];
+        for (int v = 0; v < V; ++v) { acc[v / 2] = 0ull; one[v] = 0.f; }
+        // rows q .. of the ids at hand: ROWS of them if full, else those below c
+        auto rows = [&](int q, int c, auto full) {
+            uint4 f4[ROWS / 4];
 #pragma unroll
-                for (int k = 0; k < ROWS / 4; ++k) f4[k] = s_ids[warp][q / 4 + k];
-                Load w[ROWS][NL];
+            for (int k = 0; k < ROWS / 4; ++k) f4[k] = s_ids[warp][q / 4 + k];
+            Load w[ROWS][NL];
 #pragma unroll
-                for (int u = 0; u < ROWS; ++u)
+            for (int u = 0; u < ROWS; ++u)
 #pragma unroll
-                    for (int l = 0; l < NL; ++l) {
-                        w[u][l] = Load();
-                        if (decltype(full)::value || q + u < c) {
-                            const uint4 t = f4[u / 4];
-                            const uint32_t f = u % 4 == 0 ? t.x : u % 4 == 1 ? t.y : u % 4 == 2 ? t.z : t.w;
-                            const WT *at = col[l] + (int64_t)f * a.M;
-                            if constexpr (VEC) w[u][l] = __ldg(reinterpret_cast<const ulonglong2 *>(at));
-                            else w[u][l] = dense_ld(at);
-                        }
+                for (int l = 0; l < NL; ++l) {
+                    w[u][l] = Load();
+                    if (decltype(full)::value || q + u < c) {
+                        const uint4 t = f4[u / 4];
+                        const uint32_t f = u % 4 == 0 ? t.x : u % 4 == 1 ? t.y : u % 4 == 2 ? t.z : t.w;
+                        const char *from = reinterpret_cast<const char *>(col[l]) + (u64)f * stride;
+                        if constexpr (VEC) w[u][l] = __ldg(reinterpret_cast<const ulonglong2 *>(from));
+                        else w[u][l] = dense_ld(reinterpret_cast<const WT *>(from));
                     }
+                }
 #pragma unroll
-                for (int u = 0; u < ROWS; ++u)
+            for (int u = 0; u < ROWS; ++u)
 #pragma unroll
-                    for (int l = 0; l < NL; ++l) {
-                        if constexpr (VEC) dense_add16(acc + l * STEP / 2, w[u][l], WT());
-                        else one[l] += w[u][l];
-                    }
-            };
-            for (int eb = beg; eb < end; eb += 64) {
-                const int c = min(64, end - eb);
-                __syncwarp();                                // the ids before these have been used
+                for (int l = 0; l < NL; ++l) {
+                    if constexpr (VEC) dense_add16(acc + l * STEP / 2, w[u][l], WT());
+                    else one[l] += w[u][l];
+                }
+        };
+        for (int eb = beg; eb < end; eb += 64) {
+            const int c = min(64, end - eb);
+            __syncwarp();                                // the ids before these have been used
 #pragma unroll
-                for (int k = 0; k < 2; ++k)
-                    mine[32 * k + lane] = 32 * k + lane < c ? BMU_IDX((uint32_t)__ldg(a.colidx + eb + 32 * k + lane), a.D, a.status) : 0u;
-                __syncwarp();
-                int q = 0;
-                for (; q + ROWS <= c; q += ROWS) rows(q, c, std::true_type());
-                if (q < c) rows(q, c, std::false_type());
-            }
+            for (int k = 0; k < 2; ++k)
+                mine[32 * k + lane] = 32 * k + lane < c ? BMU_IDX((uint32_t)__ldg(a.colidx + eb + 32 * k + lane), a.D, a.status) : 0u;
+            __syncwarp();
+            int q = 0;
+            for (; q + ROWS <= c; q += ROWS) rows(q, c, std::true_type());
+            if (q < c) rows(q, c, std::false_type());
+        }
 #pragma unroll
-            for (int v = 0; v < V; ++v) {
-                const int64_t j = j0 + (32 * (v / STEP) + lane) * STEP + v % STEP;
-                const float sum = !VEC ? one[v] : v % 2 ? hi_f(acc[v / 2]) : lo_f(acc[v / 2]);
-                if (j < a.M) best.push(fmaf(-2.f, sum, __ldg(a.norms + j)), (int)j);
-            }
+        for (int v = 0; v < V; ++v) {
+            const int64_t j = j0 + (32 * (v / STEP) + lane) * STEP + v % STEP;
+            const float sum = !VEC ? one[v] : v % 2 ? hi_f(acc[v / 2]) : lo_f(acc[v / 2]);
+            if (j < a.M) best.push(fmaf(-2.f, sum, __ldg(a.norms + j)), (int)j);
         }
         u64 k1, k2;
         best.warp_keys(k1, k2);

@@ -38,6 +38,7 @@ void screen_layout(int64_t D, int64_t M, int64_t N, int head, int64_t chunk, boo
     const size_t n4 = (size_t)l->n_pad * 4;
     const size_t stripes = (size_t)screen_split_blocks(blocks, slabs, sms) * SC_DOCS * 4;
     codebook_layout(D, l->chunk_slabs, 1, take, l);
+    l->sample = take((size_t)SC_SAMPLE * (size_t)((M + SC_GROUP - 1) / SC_GROUP) * 4);
     l->window = take(n4);
     l->amin = take(n4); l->amin2 = top2 ? take(n4) : l->amin;
     l->cval = take(stripes * sizeof(float2)); l->cmask = take(stripes * sizeof(uint4));
@@ -76,22 +77,91 @@ __device__ __forceinline__ void screen_ld16(const __half *p, float v[4])
     v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
 }
 
+// A few documents, evenly through the corpus, against all units in fp32: the smallest value of each 8-unit
+// group.  From these the windows' kernel sees how much of the map their windows hold.  A block takes a document
+// and 128 units, each of its warps an eighth of the list (one warp for all of it: 26 us longer than the rest of
+// the kernel where a list of 400 ids is met).  Its blocks run beside those that read the codebook anyway.
+__device__ __forceinline__ int64_t screen_sample_doc(int s, int sampled, int64_t N) { return (2 * s + 1) * N / (2 * sampled); }
+
+template <typename WT, bool VEC>
+__device__ __forceinline__ void screen_sample(const WT *__restrict__ W, int64_t D, int64_t M, const float *__restrict__ norms,
+                                              const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
+                                              int64_t N, int sampled, int64_t item, float *__restrict__ groups,
+                                              [[maybe_unused]] uint32_t *status)
+{
+    constexpr int R = VEC ? 8 : 2;                   // rows in flight
+    __shared__ float4 part[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t pieces = (M + 127) / 128;
+    const int sd = (int)(item / pieces);
+    const int64_t i = screen_sample_doc(sd, sampled, N), j = item % pieces * 128 + 4 * lane;
+    const int first = __ldg(rowptr + i), last = __ldg(rowptr + i + 1), share = (last - first + 7) / 8;
+    const int beg = min(first + warp * share, last), end = min(beg + share, last);
+    const WT *col = W + (VEC && j < M ? j : 0);
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int e0 = beg; e0 < end; e0 += 32) {
+        const int mine = e0 + lane < end ? __ldg(colidx + e0 + lane) : 0, c = min(32, end - e0);
+        for (int q = 0; q < c; q += R) {
+            float v[R][4];
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+                const uint32_t f = BMU_IDX((uint32_t)__shfl_sync(0xffffffffu, mine, q + u), D, status);
+#pragma unroll
+                for (int x = 0; x < 4; ++x) v[u][x] = 0.f;
+                if (q + u < c) {
+                    if (VEC) screen_ld16(col + (int64_t)f * M, v[u]);
+                    else {
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) v[u][x] = screen_ld(W + (int64_t)f * M + (j + x < M ? j + x : 0));
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < R; ++u)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) s[x] += v[u][x];
+        }
+    }
+    part[warp][lane] = make_float4(s[0], s[1], s[2], s[3]);
+    __syncthreads();
+    if (warp) return;
+#pragma unroll
+    for (int w = 1; w < 8; ++w) {
+        const float4 t = part[w][lane];
+        s[0] += t.x; s[1] += t.y; s[2] += t.z; s[3] += t.w;
+    }
+    float least = CUDART_INF_F;
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+        if (j + x < M) least = fminf(least, fmaf(-2.f, s[x], __ldg(norms + j + x)));
+    least = fminf(least, __shfl_xor_sync(0xffffffffu, least, 1));
+    if (!(lane & 1) && j < M) groups[(int64_t)sd * ((M + SC_GROUP - 1) / SC_GROUP) + j / SC_GROUP] = least;
+}
+
 // Smallest and largest weight of each row: one read of the codebook.  BW warps take a row.  Beside
 // them the largest range of the head rows (most[0 .. 7]) and of the others (most[8 .. 15]) and the
 // largest |norm| (most[16 .. 23]), as bit patterns of non-negative floats; each eight times, a block
 // adds to one of them (thousands of atomics on one word: 10 us for 4096 rows of 1024, 4.3 so).
+// The first blocks sample documents (above).
 template <typename WT, bool VEC, int BW>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, VEC ? 4 : 6)
 screen_range_kernel(const WT *__restrict__ W, int64_t D, int64_t M, const float *__restrict__ norms,
                     const uint16_t *__restrict__ rank, int32_t head, float *__restrict__ rmin,
-                    float *__restrict__ rmax, uint32_t *__restrict__ most)
+                    float *__restrict__ rmax, uint32_t *__restrict__ most, const int32_t *__restrict__ rowptr,
+                    const int32_t *__restrict__ colidx, int64_t N, int sampled, int sample_blocks,
+                    float *__restrict__ groups, uint32_t *status)
 {
+    if ((int)blockIdx.x < sample_blocks) {
+        screen_sample<WT, VEC>(W, D, M, norms, rowptr, colidx, N, sampled, blockIdx.x, groups, status);
+        return;
+    }
+    const unsigned block = blockIdx.x - sample_blocks, blocks = gridDim.x - sample_blocks;
     constexpr int ROWS = 8 / BW;
     __shared__ float s_lo[8], s_hi[8];
     __shared__ uint32_t s_most[3];
     if (threadIdx.x < 3) s_most[threadIdx.x] = 0u;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t f = (int64_t)blockIdx.x * ROWS + warp / BW;
+    const int64_t f = (int64_t)block * ROWS + warp / BW;
     const int part = (warp % BW) * 32 + lane;
     float lo = CUDART_INF_F, hi = -CUDART_INF_F;
     if (f < D) {
@@ -128,24 +198,24 @@ screen_range_kernel(const WT *__restrict__ W, int64_t D, int64_t M, const float 
     }
     if (lane == 0) { s_lo[warp] = lo; s_hi[warp] = hi; }
     __syncthreads();
-    if (threadIdx.x < ROWS && (int64_t)blockIdx.x * ROWS + threadIdx.x < D) {
+    if (threadIdx.x < ROWS && (int64_t)block * ROWS + threadIdx.x < D) {
         for (int w = 0; w < BW; ++w) {
             lo = w ? fminf(lo, s_lo[threadIdx.x * BW + w]) : s_lo[threadIdx.x * BW];
             hi = w ? fmaxf(hi, s_hi[threadIdx.x * BW + w]) : s_hi[threadIdx.x * BW];
         }
-        const int64_t row = (int64_t)blockIdx.x * ROWS + threadIdx.x;
+        const int64_t row = (int64_t)block * ROWS + threadIdx.x;
         rmin[row] = lo;
         rmax[row] = hi;
         atomicMax(&s_most[(rank ? (int)rank[row] : (int)row) < head ? 0 : 1], __float_as_uint(__fsub_ru(hi, lo)));
     }
     uint32_t nm = 0;
-    for (int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x; j < M; j += (int64_t)gridDim.x * 256)
+    for (int64_t j = (int64_t)block * 256 + threadIdx.x; j < M; j += (int64_t)blocks * 256)
         nm = max(nm, __float_as_uint(fabsf(__ldg(norms + j))));
     nm = __reduce_max_sync(0xffffffffu, nm);
     if (lane == 0 && nm > 0) atomicMax(&s_most[2], nm);
     __syncthreads();
     if (threadIdx.x < 3) {
-        uint32_t *to = most + 8 * threadIdx.x + (blockIdx.x & 7);
+        uint32_t *to = most + 8 * threadIdx.x + (block & 7);
         const uint32_t v = s_most[threadIdx.x];
         if (v > *reinterpret_cast<volatile uint32_t *>(to)) atomicMax(to, v);
     }
@@ -175,7 +245,7 @@ __global__ void __launch_bounds__(256)
 screen_table_kernel(const float *__restrict__ rmin, const float *__restrict__ rmax, int32_t D, int32_t head,
                     int32_t head_pad, const uint16_t *__restrict__ feat, const uint16_t *__restrict__ rank,
                     const uint32_t *__restrict__ tile_len, int64_t few, const uint32_t *__restrict__ most,
-                    const float *__restrict__ earlier, float *__restrict__ scalars, float4 *__restrict__ table,
+                    const float *__restrict__ earlier, int sampled, float *__restrict__ scalars, float4 *__restrict__ table,
                     unsigned char *__restrict__ kpack, float *__restrict__ khead)
 {
     uint32_t m3[3];
@@ -200,6 +270,8 @@ screen_table_kernel(const float *__restrict__ rmin, const float *__restrict__ rm
         scalars[2] = 1.f / dt; scalars[4] = (float)q_max;
         scalars[5] = norm; scalars[6] = (float)(65535 / q_max);
         scalars[7] = stand ? 0.f : 1.f; scalars[8] = rh; scalars[9] = rt;
+        scalars[SC_VOTES] = earlier ? earlier[SC_VOTES] : __uint_as_float(0u);
+        scalars[SC_SAMPLED] = earlier ? earlier[SC_SAMPLED] : __uint_as_float((uint32_t)sampled);
     }
     // errors: half a step, widened by 2^-10 for the roundings of the coding itself
     const float half = 0.5f * (1.f + 1.f / 1024.f);
@@ -230,20 +302,13 @@ screen_table_kernel(const float *__restrict__ rmin, const float *__restrict__ rm
 }
 
 // ---- windows: one warp per planned document -----------------------------------------------
-__global__ void __launch_bounds__(256)
-screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
-                     const int32_t *__restrict__ perm, const uint32_t *__restrict__ key, int64_t N, int64_t n_pad,
-                     const float4 *__restrict__ table, const float *__restrict__ scalars,
-                     float *__restrict__ window, [[maybe_unused]] int64_t D, uint32_t *__restrict__ status)
+// 2 B of what the rows of a document's ids bring
+__device__ __forceinline__ float screen_window_of(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
+                                                  int64_t i, const uint32_t *__restrict__ key,
+                                                  const float4 *__restrict__ table, const float *__restrict__ scalars,
+                                                  [[maybe_unused]] int64_t D, [[maybe_unused]] uint32_t *status)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (p >= n_pad) return;
-    if (p >= N || (*status & PLAN_STATUS_OVERFLOW)) {
-        if (lane == 0) window[p] = 0.f;
-        return;
-    }
-    const int32_t i = perm[p];
     const int beg = __ldg(rowptr + i), end = __ldg(rowptr + i + 1);
     float en = 0.f, eo = 0.f, aa = 0.f, in = 0.f;
     for (int e0 = beg; e0 < end; e0 += 128) {
@@ -266,23 +331,71 @@ screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restri
         aa += __shfl_xor_sync(0xffffffffu, aa, m);
         in += __shfl_xor_sync(0xffffffffu, in, m);
     }
-    if (lane == 0) {
-        // a list that repeats a head id is gathered whole
-        const float n = (float)(end - beg), gathered = (float)key[i];
-        const float E = in > 0.f && gathered == n ? eo : en;
-        float B = 2.f * E + 1.1920929e-7f * (n * aa + 4.f * scalars[5] + 8.f * aa);
-        B *= 1.f + 1.f / 4096.f + 2.f * n * 1.1920929e-7f;    // the roundings of these sums themselves
-        window[p] = (gathered > scalars[6] || !(B < 1e37f)) ? CUDART_INF_F : 2.f * B;
+    // a list that repeats a head id is gathered whole
+    const float n = (float)(end - beg), gathered = (float)key[i];
+    const float E = in > 0.f && gathered == n ? eo : en;
+    float B = 2.f * E + 1.1920929e-7f * (n * aa + 4.f * scalars[5] + 8.f * aa);
+    B *= 1.f + 1.f / 4096.f + 2.f * n * 1.1920929e-7f;    // the roundings of these sums themselves
+    return (gathered > scalars[6] || !(B < 1e37f)) ? CUDART_INF_F : 2.f * B;
+}
+
+// The first blocks, one per sampled document: how many of its groups lie within its window.
+__global__ void __launch_bounds__(256)
+screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
+                     const int32_t *__restrict__ perm, const uint32_t *__restrict__ key, int64_t N, int64_t n_pad,
+                     const float4 *__restrict__ table, float *scalars, float *__restrict__ window, int64_t D,
+                     int sampled, const float *__restrict__ groups, int64_t M, uint32_t *__restrict__ status)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if ((int)blockIdx.x < sampled) {
+        __shared__ float s_win, s_least[8];
+        __shared__ uint32_t s_in[8];
+        const int64_t n = (M + SC_GROUP - 1) / SC_GROUP;
+        const float *of = groups + blockIdx.x * n;
+        if (warp == 0) {
+            const float w = screen_window_of(rowptr, colidx, screen_sample_doc(blockIdx.x, sampled, N), key, table, scalars, D, status);
+            if (lane == 0) s_win = w;
+        }
+        float least = CUDART_INF_F;
+        for (int64_t g = threadIdx.x; g < n; g += 256) least = fminf(least, __ldg(of + g));
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) least = fminf(least, __shfl_xor_sync(0xffffffffu, least, m));
+        if (lane == 0) s_least[warp] = least;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < 8; ++w) least = fminf(least, s_least[w]);
+        const float limit = least + s_win;
+        uint32_t within = 0;
+        for (int64_t g = threadIdx.x; g < n; g += 256) within += __ldg(of + g) <= limit;
+        within = __reduce_add_sync(0xffffffffu, within);
+        if (lane == 0) s_in[warp] = within;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < 8; ++w) within += s_in[w];
+            if (within > screen_dense_groups(M) || s_win == CUDART_INF_F)
+                atomicAdd(reinterpret_cast<uint32_t *>(scalars) + SC_VOTES, 1u);
+        }
+        return;
     }
+    const int64_t p = ((int64_t)(blockIdx.x - sampled) * blockDim.x + threadIdx.x) >> 5;
+    if (p >= n_pad) return;
+    if (p >= N || (*status & PLAN_STATUS_OVERFLOW)) {
+        if (lane == 0) window[p] = 0.f;
+        return;
+    }
+    const float w = screen_window_of(rowptr, colidx, perm[p], key, table, scalars, D, status);
+    if (lane == 0) window[p] = w;
 }
 
 template <typename WT>
 static int launch_range(const WT *W, int64_t D, int64_t M, const float *norms, const uint16_t *rank, int head,
-                        float *rmin, float *rmax, uint32_t *most, cudaStream_t s)
+                        float *rmin, float *rmax, uint32_t *most, const int32_t *rowptr, const int32_t *colidx,
+                        int64_t N, int sampled, float *sample, uint32_t *status, cudaStream_t s)
 {
     const bool vec = M % 4 == 0 && (reinterpret_cast<uintptr_t>(W) & (4 * sizeof(WT) - 1)) == 0;
-    const unsigned blocks = M >= 8192 ? (unsigned)D : (unsigned)((D + 3) / 4);
-#define BMU_RANGE(V, B) { screen_range_kernel<WT, V, B><<<blocks, 256, 0, s>>>(W, D, M, norms, rank, head, rmin, rmax, most); BMU_LAUNCHED(); }
+    const int64_t sb = (M + 127) / 128 * sampled;
+    const unsigned blocks = (unsigned)sb + (M >= 8192 ? (unsigned)D : (unsigned)((D + 3) / 4));
+#define BMU_RANGE(V, B) { screen_range_kernel<WT, V, B><<<blocks, 256, 0, s>>>(W, D, M, norms, rank, head, rmin, rmax, most, rowptr, colidx, N, sampled, (int)sb, sample, status); BMU_LAUNCHED(); }
     if (M >= 8192) { if (vec) BMU_RANGE(true, 8) else BMU_RANGE(false, 8) }
     else { if (vec) BMU_RANGE(true, 2) else BMU_RANGE(false, 2) }
 #undef BMU_RANGE
@@ -294,25 +407,29 @@ int launch_screen_prepare(const void *W, int f16, int64_t D, int64_t M, const fl
                           const int32_t *rowptr, const int32_t *colidx, int64_t N, int head,
                           const uint16_t *feat, const uint16_t *rank, const int32_t *perm,
                           const uint32_t *key, const uint32_t *tile_len, char *cb, const ScreenLayout &cl,
-                          float *scalars, const float *earlier, float *window, int64_t n_pad,
+                          float *scalars, const float *earlier, float *sample, float *window, int64_t n_pad,
                           uint32_t *status, cudaStream_t s)
 {
+    // (an earlier search of the same codebook has decided for this one too)
+    const int sampled = earlier ? 0 : (int)(N < SC_SAMPLE ? N : SC_SAMPLE);
     float *rmin = reinterpret_cast<float *>(cb + cl.rmin), *rmax = reinterpret_cast<float *>(cb + cl.rmax);
     float4 *table = reinterpret_cast<float4 *>(cb + cl.table);
     uint32_t *most = status + STATUS_MAXIMA;
     if (!earlier) {
-        const int rc = f16 ? launch_range(static_cast<const __half *>(W), D, M, norms, rank, head, rmin, rmax, most, s)
-                           : launch_range(static_cast<const float *>(W), D, M, norms, rank, head, rmin, rmax, most, s);
+        const int rc = f16 ? launch_range(static_cast<const __half *>(W), D, M, norms, rank, head, rmin, rmax, most,
+                                          rowptr, colidx, N, sampled, sample, status, s)
+                           : launch_range(static_cast<const float *>(W), D, M, norms, rank, head, rmin, rmax, most,
+                                          rowptr, colidx, N, sampled, sample, status, s);
         if (rc) return rc;
     }
     const int64_t rows = D > cl.head_pad ? D : cl.head_pad;
     // up to a thousandth of the tiles, or four where they are few (32 documents of 1000 ids: 27 us for 4,096 units)
     const int64_t tiles = (N + 7) / 8, four = tiles / 64 < 4 ? tiles / 64 : 4, few = tiles / 1024 > four ? tiles / 1024 : four;
     { screen_table_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, s>>>(
-        rmin, rmax, (int32_t)D, head, cl.head_pad, feat, rank, tile_len, few, most, earlier, scalars, table,
+        rmin, rmax, (int32_t)D, head, cl.head_pad, feat, rank, tile_len, few, most, earlier, sampled, scalars, table,
         reinterpret_cast<unsigned char *>(cb + cl.kpack), reinterpret_cast<float *>(cb + cl.khead)); BMU_LAUNCHED(); }
-    { screen_window_kernel<<<(unsigned)((n_pad * 32 + 255) / 256), 256, 0, s>>>(
-        rowptr, colidx, perm, key, N, n_pad, table, scalars, window, D, status); BMU_LAUNCHED(); }
+    { screen_window_kernel<<<(unsigned)(sampled + (n_pad * 32 + 255) / 256), 256, 0, s>>>(
+        rowptr, colidx, perm, key, N, n_pad, table, scalars, window, D, sampled, sample, M, status); BMU_LAUNCHED(); }
     BMU_CUDA(cudaGetLastError());
     return BMU_OK;
 }
@@ -471,7 +588,7 @@ screen_image_kernel(const WT *__restrict__ W, int64_t D, int64_t M, int64_t k, i
                     const float *__restrict__ norms, unsigned char *__restrict__ img8,
                     unsigned char *__restrict__ head_img, float *__restrict__ normp)
 {
-    if (__ldg(scalars + 7) == 0.f) return;             // the images of an earlier search stand
+    if (__ldg(scalars + 7) == 0.f || screen_whole(scalars)) return;   // the images of an earlier search stand
     const int heads = head_pad / 32;
     auto one = [&](const int64_t slab) {
         const int64_t j_slab = (k + launches * slab) * SC_SLAB;

@@ -192,7 +192,7 @@ screen_collect_kernel(const VerifyArgs a)
     const int64_t p = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 8 + (lane >> 2);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // (the verify stage, after the last launch)
     // (one lane reads the status word for its warp: the lanes must stay together)
-    if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(a.status), 0)) return;
+    if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(a.status), 0) || screen_whole(a.scalars)) return;
     const bool there = p < a.N;
     const float win = there ? a.window[p] : 0.f;
     const uint32_t seg = 15u << (lane & ~3), most = screen_early_groups(a.M);
@@ -333,12 +333,12 @@ screen_verify_kernel(const VerifyArgs a)
     const int lane = threadIdx.x & 31, e = lane & 15;
     const int64_t p = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 2 + (lane >> 4);
     if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(a.status), 0)) return;
-    const bool there = p < a.N;
+    const bool there = p < a.N, whole = screen_whole(a.scalars);
     uint32_t count = 0, base = 0;
     uint4 todo = make_uint4(0u, 0u, 0u, 0u);
     int32_t orig = 0, beg = 0, end = 0;
     if (there) {
-        count = a.lcount[p];
+        count = whole ? SC_DENSE : a.lcount[p];
         orig = a.perm[p];
         beg = __ldg(a.rowptr + orig);
         end = __ldg(a.rowptr + orig + 1);
@@ -376,7 +376,7 @@ screen_verify_kernel(const VerifyArgs a)
             a.state[orig] = KEY_WORST;
             if (TOP2) a.state2[orig] = KEY_WORST;
             a.lcount[p] = 0u;                                // its ticket from here on
-            a.dense[atomicAdd(a.dense_count, 1u)] = (uint32_t)p;
+            if (!whole) a.dense[atomicAdd(a.dense_count, 1u)] = (uint32_t)p;
         }
         return;
     }

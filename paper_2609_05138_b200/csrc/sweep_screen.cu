@@ -118,10 +118,10 @@ sweep_screen_kernel(const ScreenArgs a)
         mm_bar_init(drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         *abort_flag = 0u;
-        *skip_flag = *reinterpret_cast<volatile uint32_t *>(a.status);
+        *skip_flag = *reinterpret_cast<volatile uint32_t *>(a.status) | (screen_whole(a.scalars) ? 1u : 0u);
     }
     __syncthreads();
-    if (*skip_flag) return;          // a block before this one gave up: let the grid drain
+    if (*skip_flag) return;          // a block before this one gave up: let the grid drain; or nothing is screened
 
     if (warp == NTW) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"

@@ -239,12 +239,51 @@ def test_where_the_screen_cannot_rule_out_it_costs_little(bmu, what, most):
     assert timed(bmu, W, rp, ci, 0) <= most * timed(bmu, W, rp, ci, 2)
 
 
-@pytest.mark.parametrize("n", [3000, 60_000])
-def test_a_long_list_costs_the_others_nothing(bmu, n):
+def smooth_map(bmu, rp, ci, D, edge):
+    """A map after one update from random units with the widest neighbourhood."""
+    M, dev = edge * edge, rp.device
+    unit = torch.randint(0, M, (rp.numel() - 1,), generator=torch.Generator(device=dev).manual_seed(3), device=dev,
+                         dtype=torch.int32)
+    num = torch.zeros((D, M), dtype=torch.int32, device=dev)
+    cnt = torch.zeros(M, dtype=torch.int32, device=dev)
+    W = torch.zeros((D, M), device=dev)
+    bmu.bmu_update_scatter(rp, ci, unit, num, cnt)
+    bmu.bmu_update_writeback(*bmu.bmu_update_blur(num, cnt, edge, edge, 8.0), W)
+    return W
+
+
+@pytest.mark.parametrize("f16", [False, True])
+def test_nothing_is_screened_where_most_documents_are_evaluated_whole(bmu, f16):
+    """Equal units on 128 x 128: little more than the single-stage search.  A smooth map whose units lie close
+    together: same units up to near ties; the plan, the batches of a call and half precision take the same way."""
+    D, edge, dev = 16384, 128, torch.device("cuda")
+    rp, ci = synth.draw_corpus(20_000, D, 1.1, torch.full((20_000,), 80, dtype=torch.int64, device=dev), 6, dev)
+    W = smooth_map(bmu, rp, ci, D, edge)
+    if f16:
+        Wh = W.half()
+        hb, hd = bmu.bmu_search_f16_ws(Wh, rp, ci)
+        ob, od = bmu.bmu_search_ws(Wh.float(), rp, ci)
+        assert torch.equal(hb, ob) and torch.equal(hd, od)
+        return
+    ob, od = bmu.bmu_search_ws(W, rp, ci)
+    some = list(range(0, 20_000, 400))
+    parity.compare(ob.cpu().numpy(), od.cpu().numpy(), W.cpu().numpy(), rp.cpu().numpy(), ci.cpu().numpy(), docs=some)
+    plan = bmu.Plan(rp, ci, D, edge * edge)
+    pb, pd = plan.search(W)
+    plan.close()
+    assert torch.equal(pb, ob) and torch.equal(pd, od)
+    host = (rp.cpu().pin_memory(), ci.cpu().pin_memory())
+    for hb, hd in bmu.bmu_search_batches_host(W, [host, host]):
+        assert torch.equal(hb, ob.cpu()) and torch.equal(hd, od.cpu())
+    W.copy_(W[:, :1].clone().expand(D, edge * edge))
+    assert timed(bmu, W, rp, ci, 0) <= 1.9 * timed(bmu, W, rp, ci, 2)
+
+
+def test_a_long_list_costs_the_others_nothing(bmu):
     """One list of 1000 ids among ordinary ones: neither the codes of all others nor the time of their tiles
-    follow it (0.64 and 0.49 ms more when they did; 0.35 and 0.24, the walk along the one list, as it is).
-    Same results, the long one among them."""
-    D, M, dev = 16384, 4096, torch.device("cuda")
+    follow it (1.67 -> 3.05 ms when they did); what is left is the walk along the one list.  Same results, the
+    long one among them."""
+    D, M, n, dev = 16384, 16384, 20_000, torch.device("cuda")
     g = torch.Generator(device=dev).manual_seed(6)
     rp, ci = synth.draw_corpus(n, D, 1.1, torch.full((n,), 80, dtype=torch.int64, device=dev), 6, dev)
     more = torch.randperm(D, generator=g, device=dev)[:1000].sort().values.to(torch.int32)
@@ -256,7 +295,8 @@ def test_a_long_list_costs_the_others_nothing(bmu, n):
     assert torch.equal(lb[:n], ob) and torch.equal(ld[:n], od)
     parity.compare(lb.cpu().numpy(), ld.cpu().numpy(), W.cpu().numpy(), rpl.cpu().numpy(), cil.cpu().numpy(),
                    docs=[0, 1, n])
-    assert timed(bmu, W, rpl, cil, 1) <= timed(bmu, W, rp, ci, 1) + 0.42
+    more, without = timed(bmu, W, rpl, cil, 1), timed(bmu, W, rp, ci, 1)
+    assert more <= without + 0.9, (more, without)
 
 
 @pytest.mark.parametrize("n,fewer", [(45_500, 45_000), (45_500, 9_000), (2_500, 1_500), (2_500, 300)])
