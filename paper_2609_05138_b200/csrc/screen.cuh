@@ -16,7 +16,7 @@
 // weight w of feature f is stored as q = round((w - c_f) / step_f), c_f the row's minimum, so
 // |w - (c_f + step_f q)| <= e_f; the sum of c_f over a document is the same for every neuron
 // and plays no part.  With E = sum of e_f over the document's ids, A = sum of the rows' largest
-// |w|, n the norms and |x| ids, the approximate distance differs from the exact real value of
+// |w|, n the finite norms and |x| ids, the approximate distance differs from the exact real value of
 // n_j - 2 s_ij (minus that constant) by at most 2 E + rounding, and the verify stage's fp32
 // value by at most 2^-23 |x| A + rounding; together B = 2 E + 2^-23 (|x| A + 4 max|n| + 8 A).
 // If j* wins the exact comparison then, for every j, approx(j*) <= approx(j) + 2 B: a neuron

@@ -210,7 +210,11 @@ screen_range_kernel(const WT *__restrict__ W, int64_t D, int64_t M, const float 
     }
     uint32_t nm = 0;
     for (int64_t j = (int64_t)block * 256 + threadIdx.x; j < M; j += (int64_t)blocks * 256)
-        nm = max(nm, __float_as_uint(fabsf(__ldg(norms + j))));
+    {
+        // (a unit at infinity is never within a finite window: it widens nobody's)
+        const uint32_t n = __float_as_uint(fabsf(__ldg(norms + j)));
+        if (n < 0x7f800000u) nm = max(nm, n);
+    }
     nm = __reduce_max_sync(0xffffffffu, nm);
     if (lane == 0 && nm > 0) atomicMax(&s_most[2], nm);
     __syncthreads();

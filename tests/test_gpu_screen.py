@@ -239,6 +239,22 @@ def test_where_the_screen_cannot_rule_out_it_costs_little(bmu, what, most):
     assert timed(bmu, W, rp, ci, 0) <= most * timed(bmu, W, rp, ci, 2)
 
 
+def test_units_at_infinity_do_not_widen_the_windows(bmu):
+    """Norms that rule units out (masked units, weights whose square overflows): screened like any other map,
+    where every document used to be evaluated whole (1.6 times the single-stage search; 0.5 without them)."""
+    D, M, dev = 16384, 4096, torch.device("cuda")
+    rp, ci = synth.draw_corpus(20_000, D, 1.1, torch.full((20_000,), 80, dtype=torch.int64, device=dev), 6, dev)
+    W = synth.make_codebook(D, M, 3, dev)
+    norms = bmu.bmu_codebook_norms(W)
+    norms[::5] = float("inf")
+    ob, od = bmu.bmu_search_ws(W, rp, ci, norms=norms)
+    keep = [j for j in range(M) if j % 5]
+    rb, rd = bmu.bmu_search_ws(W[:, keep].contiguous(), rp, ci)
+    assert torch.equal(ob, torch.tensor(keep, dtype=torch.int32, device=dev)[rb.long()])
+    assert bool(((od - rd).abs() <= 1e-5 * rd.abs()).all())
+    assert timed(bmu, W, rp, ci, 0, norms) <= 0.9 * timed(bmu, W, rp, ci, 2, norms)
+
+
 def smooth_map(bmu, rp, ci, D, edge):
     """A map after one update from random units with the widest neighbourhood."""
     M, dev = edge * edge, rp.device
