@@ -282,8 +282,9 @@ BMU_API int bmu_search_f16_ws(const void *W16, int64_t D, int64_t M, const float
  * One-shot form.  Same as bmu_search_ws with norms == NULL and default options,
  * but the scratch is a library-owned buffer per device that only ever grows
  * (cudaMalloc on first use or growth; freed by bmu_release_scratch or at
- * process exit).  Unless the documents are few (below 1024) it reads rowptr[N]
- * back to size the scratch, so the call synchronises the stream once before the
+ * process exit).  Unless the documents are few (N below 1024 and N * M below
+ * 2^25, or the stream being captured) it reads rowptr[N] back to size the scratch
+ * and to choose the kernel, so the call synchronises the stream once before the
  * kernels are queued.  Calls on
  * different streams of one device share the scratch and must not overlap.
  * The status word of the search (see bmu_search_ws) sits in that scratch:

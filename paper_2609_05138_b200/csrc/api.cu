@@ -180,10 +180,15 @@ static int plan_order(const bmu_opts &o, bool tensor_core_sweep)
 //             D = 4,096, 30,000 documents of 64 ids: 244, two-stage 160; 256 units: 122 and 148)
 //   two-stage 90 + 0.0022 D + 0.009 M + 1.6e-6 D M + 0.002 N + U / 3.3e7
 // e.g. D = 4,096, M = 1,024: 4,000 documents 90 / 161 / 144 us, 10,000: 215 / 208 / 174; D = 16,384,
-// M = 4,096: 1,000 documents 92 / 454 / 269, 10,000: 761 / 757 / 450.  Two lines beside the model: below
-// 1,024 documents it is always the first (a one-shot search then need not know the number of
-// listings), and from 600,000 listings on it never is.
-static const int64_t FEW_MAX_DOCS = 1024, FEW_MAX_LISTINGS = 600000;
+// M = 4,096: 1,000 documents 92 / 454 / 269, 10,000: 761 / 757 / 450.  Two lines beside the model: from
+// 1,024 documents and 600,000 listings on it is never the first, and below 1,024 documents never the second
+// (its warps would not fill the chip) unless two stages are ruled out and the sweep is large (2e10 updates).
+// There the first takes 60 + U / 6.1e6 (3.1e6) for more than a few hundred us, and two stages 0.2 us more
+// per id of a list, whose ends nothing hides; they are chosen where they promise a tenth.  First / two
+// stages in us, 1,000 documents: 80 ids, 127 x 127, D = 4,096 493 / 367, 400 ids 2091 / 580; 400 ids,
+// M = 65,536, D = 16,384 4344 / 3324, M = 16,384 1083 / 916; but 700 ids, M = 4,096 506 / 456 (left),
+// 500 of 400 ids on 75 x 75 407 / 440.
+static const int64_t FEW_MAX_DOCS = 1024, FEW_MAX_LISTINGS = 600000, ONE_SHOT_READS = (int64_t)1 << 25;
 
 static double few_us(int64_t M, double u) { return 15.0 + u / (M % 4 == 0 ? 4.5e6 : 1.9e6); }
 static double planned_us(int64_t M, double nnz, bool f16)
@@ -206,13 +211,18 @@ static bool screen_possible(const bmu_opts &o, int64_t D, int64_t M)
     return o.cluster != 2 && D >= 1 && D <= LANES_MAX_D && M >= 1 && screen_head_rows(o, D) <= SC_MAX_HEAD;
 }
 
+// (a one-shot search that has not read its number of listings back says 0: the first)
 static bool few_wanted(const bmu_opts &o, int64_t D, int64_t M, int64_t N, int64_t nnz)
 {
     if (o.kernel != 0 || o.two_stage == 1 || o.chunk_neurons || rows_opts(o)) return false;
-    if (N < FEW_MAX_DOCS) return true;
     const double u = (double)nnz * (double)M;
-    return nnz < FEW_MAX_LISTINGS &&
-           (o.two_stage == 2 || !screen_possible(o, D, M) || few_us(M, u) < two_stage_us(D, M, N, u));
+    const bool screened = o.two_stage != 2 && screen_possible(o, D, M);
+    if (N < FEW_MAX_DOCS) {
+        if (!screened) return u < 2e10 || D > LANES_MAX_D || M % 4 != 0 || M < 256;
+        const double list = (double)nnz / (double)(N > 0 ? N : 1);
+        return 60.0 + u / (M % 4 == 0 ? 6.1e6 : 3.1e6) < 1.1 * (two_stage_us(D, M, 0, u) + 0.2 * list);
+    }
+    return nnz < FEW_MAX_LISTINGS && (!screened || few_us(M, u) < two_stage_us(D, M, N, u));
 }
 
 static bool screen_wanted(const bmu_opts &o, int64_t D, int64_t M, int64_t N, int64_t nnz, bool f16 = false)
@@ -222,6 +232,7 @@ static bool screen_wanted(const bmu_opts &o, int64_t D, int64_t M, int64_t N, in
     if (o.kernel != 0 || (!f16 && few_wanted(o, D, M, N, nnz))) return false;
     const double u = (double)nnz * (double)M;
     if (rows_opts(o) || o.chunk_neurons) return u >= 2e10;
+    if (N < FEW_MAX_DOCS && !f16) return true;
     const bool planned_ok = f16 || (M % 4 == 0 && M >= 256);
     return !planned_ok || two_stage_us(D, M, N, u) < planned_us(M, (double)nnz, f16);
 }
@@ -262,12 +273,14 @@ static Layout layout_of(const bmu_opts &o, int64_t D, int64_t M, int64_t N, int6
 }
 
 // Could a search of no more documents and listings take the two-stage form?  Its model grows slower in the
-// listings than the others' and with the documents, theirs do not: most likely all listings in a single
-// document, or in the fewest that the line beside the model lets it have.
+// listings than the others': most likely with all of them.  Below 1,024 documents it gains with the
+// documents (shorter lists), above it loses; with a half-precision codebook it only loses.
 static bool screen_within(const bmu_opts &o, int64_t D, int64_t M, int64_t N, int64_t nnz, bool f16 = false)
 {
-    return N > 0 && (screen_wanted(o, D, M, 1, nnz, f16) ||
-                     (N >= FEW_MAX_DOCS && screen_wanted(o, D, M, FEW_MAX_DOCS, nnz, f16)));
+    if (N <= 0) return false;
+    if (f16) return screen_wanted(o, D, M, 1, nnz, true);
+    return screen_wanted(o, D, M, N < FEW_MAX_DOCS ? N : FEW_MAX_DOCS - 1, nnz) ||
+           (N >= FEW_MAX_DOCS && screen_wanted(o, D, M, FEW_MAX_DOCS, nnz));
 }
 
 // What the workspace queries answer: room for every way that a search of these or smaller sizes may take
@@ -1136,7 +1149,12 @@ int bmu_search(const float *W, int64_t D, int64_t M, const int32_t *rowptr,
     bmu_opts none;
     memset(&none, 0, sizeof(none));
     int32_t nnz = 0;
-    if (N >= FEW_MAX_DOCS || !colidx) {          // (few documents need no scratch by the listing)
+    // Few documents need no scratch by the listing.  Read back all the same where the few-documents kernel
+    // takes more than half a millisecond even for short lists and long ones would go another way (10 us;
+    // not while the stream is captured).
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (N < FEW_MAX_DOCS && N * M >= ONE_SHOT_READS) BMU_CUDA(cudaStreamIsCapturing(s, &capture));
+    if (N >= FEW_MAX_DOCS || !colidx || (N * M >= ONE_SHOT_READS && capture == cudaStreamCaptureStatusNone)) {
         BMU_CUDA(cudaMemcpyAsync(&nnz, rowptr + N, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
         BMU_CUDA(cudaStreamSynchronize(s));
     }

@@ -147,6 +147,23 @@ def test_describe_search_needs_no_gpu_and_names_the_kernel(lib):
     assert lib.bmu_describe_search(32, 1024, 10, 100, None, None) == 1
 
 
+@pytest.mark.parametrize("D,M,N,length,two_stage", [
+    (4096, 1024, 48, 64, 0), (16384, 16384, 256, 79, 0), (16384, 65536, 1000, 80, 0), (4096, 1024, 1000, 80, 0),
+    (4096, 127 * 127, 1000, 400, 1), (4096, 127 * 127, 1000, 80, 1), (16384, 65536, 1000, 400, 1),
+    (16384, 262144, 1000, 400, 1)])
+def test_few_documents_take_the_faster_way(lib, D, M, N, length, two_stage):
+    """The few-documents kernel where it is faster, not wherever the documents are few: long lists and large
+    maps are screened (or, with that ruled out, swept on the tensor cores)."""
+    from paper_2609_05138_b200 import Opts, SearchDesc
+    d, o = SearchDesc(), Opts()
+    assert lib.bmu_describe_search(D, M, N, N * length, None, ctypes.byref(d)) == 0
+    assert (d.kernel, d.two_stage > 0) == ((6, True) if two_stage else (1, False))
+    o.two_stage = 2
+    assert lib.bmu_describe_search(D, M, N, N * length, ctypes.byref(o), ctypes.byref(d)) == 0
+    large = N * length * M >= 2e10 and M % 4 == 0
+    assert (d.kernel, d.two_stage) == ((6 if large else 1), 0)
+
+
 def test_status_words_map_to_errors_without_a_gpu(lib):
     """The host entry points that read a search's status word back (bmu_search_host,
     bmu_search_batches_host, bmu_plan_create, bmu_last_status) turn it into an error through

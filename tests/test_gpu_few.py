@@ -63,3 +63,26 @@ def test_empty_repeated_and_unaligned(bmu):
         torch.cuda.synchronize()
         parity.compare(ob.cpu().numpy(), od.cpu().numpy(), W.numpy(), rowptr.numpy(), colidx.numpy(),
                        cancel_floor=True)
+
+
+@pytest.mark.parametrize("n_docs,M", [(48, 512), (700, 65_536)])
+def test_one_shot_reads_back_where_it_pays_and_can_be_captured(bmu, n_docs, M):
+    """The one-shot search agrees with the workspace form, whether it knows the number of listings (large
+    maps) or not, and is still captured in a graph."""
+    r = np.random.default_rng(3)
+    D = 400
+    rows = [np.sort(r.permutation(D)[:int(r.integers(1, 60))]) for _ in range(n_docs)]
+    rp = torch.zeros(n_docs + 1, dtype=torch.int32)
+    rp[1:] = torch.cumsum(torch.tensor([len(x) for x in rows]), 0)
+    rp, ci = rp.cuda(), torch.from_numpy(np.concatenate(rows).astype(np.int32)).cuda()
+    W = synth.make_codebook(D, M, 72, kind="scaled").cuda()
+    ob, od = bmu.bmu_search(W, rp, ci)
+    wb, wd = bmu.bmu_search_ws(W, rp, ci)
+    assert torch.equal(ob, wb) and torch.equal(od, wd)
+    graph = torch.cuda.CUDAGraph()
+    gb, gd = torch.empty_like(ob), torch.empty_like(od)
+    with torch.cuda.graph(graph):
+        bmu.bmu_search(W, rp, ci, gb, gd)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(gb, ob) and torch.equal(gd, od)
