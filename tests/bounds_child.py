@@ -71,6 +71,35 @@ def main():
                        colidx.numpy())
     res["clean"].append({"kernel": "6 f16", "M": 1024, "status": 0, "failed": r["failed"], "docs": r["docs"]})
 
+    # the two-stage search: whole and ragged rows, a second-best unit, half precision, documents evaluated
+    # whole (equal units, a long list), several launches; and the few-documents kernel
+    few_rp, few_ci = rp[:301].contiguous(), ci[:int(rp[300])].contiguous()
+    long_rp = torch.cat([rowptr, rowptr[-1:] + 1300])
+    long_ci = torch.cat([colidx, torch.arange(0, 3 * 1300, 3, dtype=torch.int32)])
+    res["two_stage"] = []
+    for name, M, kind, kw in (("aligned", 1024, "scaled", {}), ("ragged", 1003, "scaled", {"chunk_neurons": 256}),
+                              ("top2", 1028, "dupes", {"chunk_neurons": 256}), ("f16", 1024, "scaled", {}),
+                              ("equal", 1003, "const", {}), ("long", 1024, "scaled", {"head_rows": 64}),
+                              ("few", 1027, "scaled", {"two_stage": 0})):
+        W = synth.make_codebook(cfg.D, M, 8, kind=kind).half().float()
+        o = bmu.Opts()
+        o.two_stage = 1
+        for k, v in kw.items():
+            setattr(o, k, v)
+        r, c = (few_rp, few_ci) if name == "few" else (long_rp.cuda(), long_ci.cuda()) if name == "long" else (rp, ci)
+        if name == "f16":
+            need = int(bmu.load().bmu_search_f16_workspace_bytes(cfg.D, M, 1500, c.numel(), None))
+            ws = torch.zeros(max(need, 1 << 26), dtype=torch.uint8, device="cuda")
+            out = bmu.bmu_search_f16_ws(W.cuda().half(), r, c, opts=o, workspace=ws)
+            torch.cuda.synchronize()
+            st = status_word(ws)
+        else:
+            out, st = search(W.cuda(), r, c, o, top2=name == "top2")
+        got = compare(out[0].cpu().numpy(), out[1].cpu().numpy(), W.numpy(), r.cpu().numpy(), c.cpu().numpy())
+        res["two_stage"].append({"name": name, "status": st, "failed": got["failed"], "docs": got["docs"],
+                                 "detail": got.get("detail")})
+    W = synth.make_codebook(cfg.D, 1024, 7, kind="scaled")
+
     # an id beyond the vocabulary: the checked build records it and leaves the access out.  The
     # codebook sits at the start of a larger allocation, so nothing here can leave memory that
     # the test owns.
@@ -84,6 +113,11 @@ def main():
         o.kernel = kernel
         _, st = search(Wd, rp, bad.cuda(), o)
         res["flagged"].append({"kernel": kernel, "status": st})
+    for two_stage, (r, c) in ((1, (rp, bad.cuda())), (0, (few_rp, bad[:few_ci.numel()].cuda()))):
+        o = bmu.Opts()
+        o.two_stage = two_stage
+        _, st = search(Wd, r, c, o)
+        res["flagged"].append({"kernel": "two-stage" if two_stage else "few", "status": st})
     # the context is still usable and a clean search still passes
     o = bmu.Opts()
     o.kernel = 6

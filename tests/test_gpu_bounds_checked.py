@@ -38,6 +38,13 @@ def test_small_cases_run_clean_under_the_checked_build(report):
         assert case["status"] == 0 and case["failed"] == 0 and case["docs"] == 1500, case
 
 
+def test_the_two_stage_search_and_few_documents_run_clean(report):
+    assert len(report["two_stage"]) == 7
+    for case in report["two_stage"]:
+        docs = {"few": 300, "long": 1501}.get(case["name"], 1500)
+        assert case["status"] == 0 and case["failed"] == 0 and case["docs"] == docs, case
+
+
 def test_an_id_beyond_the_vocabulary_is_reported_not_performed(report):
     for case in report["flagged"]:
         assert case["status"] & 128, case

@@ -137,3 +137,32 @@ def test_random_cases_against_oracle(bmu, seed):
                                    cancel_floor=True, ref=ref16)
                     ran += 1
     assert ran >= 24                                   # the generic kernel alone guarantees twelve
+
+
+@pytest.mark.parametrize("seed", range(6))
+def test_random_two_stage_cases_against_oracle(bmu, seed):
+    """The same draws through the two-stage search: best and second-best unit, options, half precision."""
+    rng, own = random.Random(2000 + seed), random.Random(3000 + seed)
+    for case in range(10):
+        rowptr, colidx, W, what = draw_case(rng)
+        D, M = W.shape
+        if D > 65024:
+            continue
+        o = bmu.Opts()
+        o.two_stage = 1
+        o.chunk_neurons = own.choice([0, 0, 256, 512])
+        o.head_rows = own.choice([0, 0, 64, 512, 1024, 1536])
+        o.relabel, o.cluster = own.choice([0, 1, 2]), own.choice([0, 1, 3])
+        Wd, rpd, cid, rp, ci = W.cuda(), rowptr.cuda(), colidx.cuda(), rowptr.numpy(), colidx.numpy()
+        forms = [(W, lambda: bmu.bmu_search_top2_ws(Wd, rpd, cid, opts=o)), (W, lambda: bmu.bmu_search_ws(Wd, rpd, cid, opts=o))]
+        if M % 256 == 0 and bool(torch.isfinite(W.half()).all()):
+            forms.append((W.half().float(), lambda: bmu.bmu_search_f16_ws(Wd.half(), rpd, cid, opts=o, top2=True)))
+        for Wx, call in forms:
+            out = [x.cpu().numpy() for x in call()]
+            nrm = oracle.norms(Wx.numpy())
+            ref = (nrm,) + tuple(oracle.bmu(Wx.numpy(), rp, ci, nrm))
+            parity.compare(out[0], out[1], Wx.numpy(), rp, ci, cancel_floor=True, ref=ref)
+            if len(out) == 4 and M >= 2:
+                scale = np.maximum(np.abs(ref[3]), (np.diff(rp) + nrm.max() + np.abs(np.diff(rp) + nrm.max() - ref[3])) * 2.0 ** -21 / 1e-5)
+                assert np.all(np.abs(out[3] - ref[3]) <= 1e-5 * scale), what
+                assert np.all(out[2] != out[0])
