@@ -125,7 +125,9 @@ typedef struct bmu_opts {
                                8-bit image of the codebook screens all units, those it cannot
                                rule out are evaluated exactly in fp32 (same results: the screen
                                keeps every unit within a rigorous error bound of the smallest);
-                               2 never; 0 = with kernel 0 where it is the faster way (a
+                               2 never (up to twice as fast on maps whose units
+                               lie close together all over, as after a first epoch with
+                               a wide neighbourhood); 0 = with kernel 0 where it is the faster way (a
                                search below 2e10 updates that sets chunk_neurons, vec, warps or
                                docs_per_warp keeps the kernels these belong to) */
     int32_t reserved[2];    /* must be 0 */
@@ -264,7 +266,8 @@ BMU_API int bmu_search_top2_ws(const float *W, int64_t D, int64_t M, const float
  * to get the second-best unit as in bmu_search_top2_ws.  bmu_opts.kernel: 3 the
  * planned kernel, 6 the wide tensor-core sweep (needs D >=
  * head_rows; the weights being fp16 already, its head image has one part), 0
- * the tensor-core sweep for large sweeps, else the planned kernel; head_rows
+ * the two-stage search where it is faster (bmu_opts.two_stage), else the planned
+ * kernel; with two_stage 2 the wide sweep for large sweeps, whose head_rows
  * defaults to 576 here.  Workspace: bmu_search_f16_workspace_bytes(...) with the
  * same sizes and options (enough with or without the second-best outputs).
  */

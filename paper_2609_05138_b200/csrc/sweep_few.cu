@@ -9,7 +9,7 @@
 // search behind the norms is one clearing of the tickets and one launch.
 //
 // What bounds it: the L2 -> SM path once the pieces fill the SMs, the latency of one pass over a
-// row's ids before that.  256 documents on a 128 x 128 map: 2058 -> 116 us per call (22
+// row's ids before that.  256 documents on a 128 x 128 map: 2074 -> 118 us per call (22
 // launches of 16 blocks before); 48 documents on 32 x 32: 87 -> 19 us,
 // half of them the norms.
 #include "common.cuh"

@@ -23,7 +23,7 @@
 // gathered loads, 64 KB in flight per SM, which the registers of the tail warps bound; no unit is full
 // (L1 data path 66 %, integer ALU 64, L2 55, tensor pipe 36).  The gather alone takes 373 us, the
 // epilogue 85, and the head's MMAs (194 us alone) run underneath.  Six instead of the four instructions
-// per two words of sc_add took 511 us where these took 507, three and two multiply-adds 513.  Nor did
+// per two words of sc_add took 511 us where these took 507 at the time, three and two multiply-adds 513.  Nor did
 // deeper rings, 7-bit codes, pairs of blocks that share the head's stages (524) or touching the next
 // rows into L1 (525) help.  A head of 1024 with two accumulators is level with 1536 and one.
 //
