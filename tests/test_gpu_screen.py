@@ -196,30 +196,6 @@ def test_distances_that_are_not_finite(bmu, how):
         assert bool(((od - rd).abs() <= 1e-5 * rd.abs())[ok].all())
 
 
-@pytest.mark.parametrize("kind", ["scaled", "const"])
-def test_captured_in_a_graph(bmu, kind):
-    """Launches that begin under the end of the one before stay in order when they are captured and replayed,
-    with documents evaluated whole (const) and without, on new inputs in the same buffers."""
-    cfg = synth.CONFIGS["cfg1"]
-    rowptr, colidx = synth.make_corpus(cfg, n_docs=900)
-    W = synth.make_codebook(cfg.D, 1500, 73, kind=kind).cuda()
-    other = synth.make_codebook(cfg.D, 1500, 74, kind="signed").cuda()
-    rp, ci, o = rowptr.cuda(), colidx.cuda(), opts_of(bmu, chunk_neurons=512)
-    need = bmu.bmu_search_workspace_bytes(cfg.D, 1500, 900, ci.numel(), o)
-    ws = torch.empty(need + 256, dtype=torch.uint8, device="cuda")
-    want = [bmu.bmu_search_ws(x, rp, ci, opts=o) for x in (W, other)]
-    buf, ob = W.clone(), torch.empty(900, dtype=torch.int32, device="cuda")
-    od = torch.empty(900, device="cuda")
-    graph = torch.cuda.CUDAGraph()
-    with torch.cuda.graph(graph):
-        bmu.bmu_search_ws(buf, rp, ci, opts=o, workspace=ws, out_bmu=ob, out_dist=od)
-    for x, (wb, wd) in [(W, want[0]), (other, want[1]), (W, want[0])]:
-        buf.copy_(x)
-        graph.replay()
-        torch.cuda.synchronize()
-        assert torch.equal(ob, wb) and torch.equal(od, wd)
-
-
 def timed(bmu, W, rp, ci, two_stage, norms=None):
     o = bmu.Opts()
     o.two_stage = two_stage
