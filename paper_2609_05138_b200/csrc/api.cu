@@ -127,6 +127,7 @@ static Layout layout_for(int64_t D, int64_t M, int64_t N, int64_t nnz, int kerne
     Layout l;
     size_t off = 0;
     l.status_off = off; off = 256;
+    if (screen_chunk) off = align_up((size_t)STATUS_WORDS * 4, 256);
     l.count_off = off;                   // (the features' counters, cleared with the status word)
     if (screen_chunk) off = align_up(off + (size_t)D * sizeof(uint32_t), 256);
     l.tickets_off = l.slots_off = off;
@@ -491,15 +492,23 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
                                    reinterpret_cast<const uint32_t *>(pw + l.plan.docoff_off), a.tile_len, cb, cl,
                                    scalars, earlier, reinterpret_cast<float *>(sb + l.screen.sample),
                                    reinterpret_cast<float *>(sb + l.screen.window),
-                                   l.screen.n_pad, status, s);
+                                   reinterpret_cast<float2 *>(sb + l.screen.reach),
+                                   reinterpret_cast<uint32_t *>(sb + l.screen.amin),
+                                   reinterpret_cast<uint32_t *>(sb + l.screen.lcount), l.screen.n_pad, top2, status, s);
     if (rc) return rc;
+    const int64_t slabs = (M + SC_SLAB - 1) / SC_SLAB;
+    const int64_t launches = (slabs + l.screen.chunk_slabs - 1) / l.screen.chunk_slabs;
+    const bool order = M >= SC_ORDER_MIN && launches <= SC_MAX_LAUNCHES;
+    if (order && (rc = launch_screen_order(norms, D, M, N, launches, cb, cl, scalars, earlier, shared != nullptr, status,
+                                           reinterpret_cast<uint32_t *>(sb + l.screen.tickets), s)))
+        return rc;
     a.kpack = reinterpret_cast<const uint32_t *>(cb + cl.kpack);
     a.scalars = scalars;
     a.window = reinterpret_cast<const float *>(sb + l.screen.window);
     a.cval = reinterpret_cast<float2 *>(sb + l.screen.cval);
     a.cval2 = reinterpret_cast<float *>(sb + l.screen.cval2);
     a.cmask = reinterpret_cast<uint4 *>(sb + l.screen.cmask);
-    a.status = status;
+    a.status = status; a.ticket = status + STATUS_SWEEP_TICKET;
     a.D = D; a.n_tiles = (N + 7) / 8; a.n_pad = l.screen.n_pad; a.tile_rows_cap = l.plan.tile_rows_cap;
     a.head = head; a.head_pad = l.screen.head_pad;
     a.splits = l.screen.splits; a.blocks = (int32_t)(l.screen.n_pad / SC_DOCS);
@@ -515,6 +524,18 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
     v.lbase = reinterpret_cast<uint32_t *>(sb + l.screen.lbase);
     v.state = state; v.state2 = state2; v.status = status; v.splits = a.splits;
     v.out_bmu = out_bmu; v.out_dist = out_dist; v.out_bmu2 = out_bmu2; v.out_dist2 = out_dist2;
+    // ... and with slabs in the order of the norms, in the same room
+    OrderedArgs o;
+    v.reach = o.reach = reinterpret_cast<const float2 *>(sb + l.screen.reach);
+    v.bound = o.bound = reinterpret_cast<uint32_t *>(sb + l.screen.amin);
+    v.own_list = o.list = reinterpret_cast<uint4 *>(sb + l.screen.lval);
+    o.count = v.lcount;
+    o.items = reinterpret_cast<const uint2 *>(sb + l.screen.items);
+    v.units = reinterpret_cast<const int32_t *>(cb + cl.units);
+    ImageArgs g;
+    g.launches = launches; g.head = head; g.sets = a.blocks; g.expected = earlier != nullptr;
+    g.reach = o.reach; g.window = a.window; g.bound = o.bound;
+    g.items = reinterpret_cast<uint2 *>(sb + l.screen.items);
     v.dense = reinterpret_cast<uint32_t *>(sb + l.screen.cval);         // (after the last launch)
     v.dense_count = status + STATUS_DENSE;
     v.scalars = scalars;
@@ -522,10 +543,11 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
     // the slabs are dealt to the launches in turn, so that every launch sees the whole map: after
     // the first one a document's smallest value is near its final one and little joins its list
     // (two neighbouring slabs at a time: 134 us instead of 17 for collecting on a trained 75 x 75 map)
-    const int64_t slabs = (M + SC_SLAB - 1) / SC_SLAB;
-    const int64_t launches = (slabs + l.screen.chunk_slabs - 1) / l.screen.chunk_slabs;
+    // (in the order of the norms: to one after the other)
     v.launches = launches;
-    for (int64_t k = 0; k < launches; ++k) {
+    const int sms = device_sms();
+    int64_t slab0 = 0;
+    for (int64_t k = 0; k < launches; ++k, slab0 += a.n_slabs) {
         a.n_slabs = (int32_t)((slabs - k + launches - 1) / launches);
         a.first = v.first = k == 0;
         v.launch = k;
@@ -533,14 +555,17 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
         a.img8 = reinterpret_cast<const unsigned char *>(cb + cl.img8) + (size_t)slot * (D + 1) * SC_SLAB;
         a.head_img = reinterpret_cast<const unsigned char *>(cb + cl.head_img) + (size_t)slot * cl.head_pad * SC_SLAB;
         a.normp = reinterpret_cast<const float *>(cb + cl.normp) + slot * SC_SLAB;
-        if ((rc = launch_screen_quantize(W, f16, D, M, norms, k, launches, a.n_slabs, slot, head, feat, cb, cl,
-                                         scalars, earlier != nullptr, s)))
-            return rc;
-        if ((rc = launch_sweep_screen(a, top2, s))) return rc;
-        if ((rc = launch_screen_collect(v, top2, s))) return rc;
+        g.k = k; g.n_slabs = a.n_slabs; g.slab0 = slab0; g.slot = slot; g.first = k == 0;
+        o.tickets = g.tickets = reinterpret_cast<uint32_t *>(sb + l.screen.tickets) + k * (SC_PARTS + 1);
+        o.slab0 = slab0;
+        o.unit_norm = reinterpret_cast<const float *>(cb + cl.unit_norm) + slab0 * SC_SLAB;
+        if ((rc = launch_screen_quantize(W, f16, D, M, norms, g, feat, cb, cl, scalars, s))) return rc;
+        if ((rc = launch_sweep_screen(a, o, top2, false, sms, s))) return rc;
+        if (order && (rc = launch_sweep_screen(a, o, top2, true, sms, s))) return rc;
+        if ((rc = launch_screen_collect(v, top2, sms, s))) return rc;
     }
     if ((rc = launch_screen_verify(v, top2, s))) return rc;
-    return launch_screen_dense(v, top2, device_sms(), s);
+    return launch_screen_dense(v, top2, sms, s);
 }
 
 static int search_impl(const float *W, int64_t D, int64_t M, const float *norms,

@@ -21,6 +21,15 @@
 // value by at most 2^-23 |x| A + rounding; together B = 2 E + 2^-23 (|x| A + 4 max|n| + 8 A).
 // If j* wins the exact comparison then, for every j, approx(j*) <= approx(j) + 2 B: a neuron
 // further than 2 B above the smallest approximate distance cannot win, whatever the weights.
+//
+// Units by norm (screen_order.cu).  Relative to the same constant no unit comes below n_j - 2 R, R = sum of
+// (largest - smallest weight) over the rows of the document's ids, and some unit with a small norm gives an upper
+// bound of the document's smallest value before anything has been summed.  So a unit whose norm lies more than
+// 2 R + 2 B above what is still within the window cannot be in it.  Where the norms of the units spread further
+// than that -- a codebook as it is first filled: 16,384 iid U[0,1) weights have norms of 5461 +- 38, a document of 80
+// ids a 2 R of 160, of which the winner's own sum uses up half -- the slabs are made of units in the order of
+// their norms, every document stops at the first slab beyond its reach, and most of the map is never summed (all
+// but 12 % on 64 x 64, all but 4 % on 128 x 128).  Otherwise the slabs follow the map.
 #pragma once
 
 #include "common.cuh"
@@ -35,18 +44,33 @@ static const int SC_MAX_SLABS = 32;      // per launch: four bits each in a stri
 static const int SC_K_MAX = 32;          // largest integer row scale of a head feature
 // -2 d_head, -2 d_tail, 1 / d_tail, unused, q_max, max |norm|, 65535 / q_max (the longest list that is
 // screened), whether the images have to be made, largest range of the head rows and of the others
-static const int SC_SCALARS = 16;
-// ... and, as integers, how many of the sampled documents are to be evaluated whole, and how many were sampled
-static const int SC_VOTES = 10, SC_SAMPLED = 11, SC_SAMPLE = 16;
+// ... and, as integers, how many of the sampled documents are to be evaluated whole, and how many were sampled;
+// whether the slabs are in the order of the norms, how many of them any document needs, up to which norm units are
+// in order (documents that reach further are evaluated whole); the two units whose distances bound a document's
+// smallest value (the smallest norms at even and at odd indices); whether the images of the slabs in that order
+// stand from an earlier search, and how many units are in order
+static const int SC_VOTES = 10, SC_SAMPLED = 11, SC_ORDERED = 12, SC_NEEDED = 13, SC_TOP = 15,
+                 SC_REF = 16, SC_STAND = 18, SC_KEPT = 19, SC_SAMPLE = 16, SC_SCALARS = 32;
+// Below this many units slabs always follow the map: too few for an order to spare many
+static const int64_t SC_ORDER_MIN = 1024;
 // Candidates wait in a list per document until every unit has been screened: a launch's local
 // minimum says little before the document's own region of the map has been seen.
 static const int SC_LIST = 12;           // entries: smallest value, group mask, first group
+// ... where slabs are in the order of the norms, in the same room: smallest value, slab, which of the 32 units of a
+// lane, the lane
+static const int SC_OWN_LIST = 16;
+// A block of that sweep takes up to this many slabs of a launch for a set of documents; sets and parts wait in lists
+static const int SC_PART = 8, SC_PARTS = SC_MAX_SLABS / SC_PART;
+// Documents and units are counted by how far they reach, in this many steps
+static const int SC_BINS = 4096;
+static const int SC_MAX_LAUNCHES = 1024;                     // ... with slabs in the order of the norms
 static const uint32_t SC_DENSE = 1u << 30;           // in a document's count: to be evaluated whole
 
 // Device arrays of one search: offsets into the workspace, relative to its screen part.
 struct ScreenLayout {
     size_t scalars, rmin, rmax, table, kpack, khead, sample, window, amin, amin2;
     size_t cval, cval2, cmask, lcount, lval, lmask, lbase, img8, head_img, normp, total;
+    size_t units, unit_norm, unit_tmp, rank_of, picks, reach, items, tickets;        // of slabs in the order of the norms
     int64_t n_pad;                       // documents rounded up to whole blocks
     int head_pad;                        // head rows rounded up to a stage (128)
     int64_t chunk_slabs;                 // slabs of the largest launch
@@ -78,10 +102,22 @@ struct ScreenArgs {
                                          // smallest value, and the first slab its mask counts from
     float *cval2;                        // second smallest value of the document
     uint4 *cmask;                        // the stripe's 8-neuron groups within the window: bit 4 s + c
-    uint32_t *status;
+    uint32_t *status, *ticket;           // of the next item, zero
     int64_t D, n_tiles, n_pad;
     size_t tile_rows_cap;
     int32_t head, head_pad, n_slabs, splits, blocks, first;
+};
+
+// The same search with slabs in the order of the norms
+struct OrderedArgs {
+    const float2 *reach;                 // per planned document: the largest norm it may need, and 2 R + 2 B
+    uint32_t *bound;                     // of its smallest (second smallest) value, as float_to_ordered
+    const float *unit_norm;              // norms in ascending order, from the launch's first slab on
+    const uint2 *items;                  // [SC_PARTS][blocks]: set of documents, first slab | last << 16
+    uint32_t *tickets;                   // SC_PARTS lengths of these lists, and the next to be taken
+    uint4 *list;                         // [n_pad][SC_OWN_LIST]
+    uint32_t *count;
+    int64_t slab0;                       // the launch's first slab in that order
 };
 
 struct VerifyArgs {
@@ -99,6 +135,10 @@ struct VerifyArgs {
     float *lval;
     uint4 *lmask;
     uint32_t *lbase;
+    const uint4 *own_list;               // slabs in the order of the norms
+    const float2 *reach;
+    const uint32_t *bound;
+    const int32_t *units;
     u64 *state, *state2;                 // exact keys of what did not fit a list
     uint32_t *dense, *dense_count;       // planned documents to be evaluated whole
     const float *scalars;
@@ -116,6 +156,27 @@ __device__ __forceinline__ bool screen_whole(const float *scalars)
     const uint32_t *s = reinterpret_cast<const uint32_t *>(scalars);
     return 2u * __ldg(s + SC_VOTES) > __ldg(s + SC_SAMPLED);
 }
+__device__ __forceinline__ bool screen_ordered(const float *scalars)
+{
+    return __ldg(reinterpret_cast<const uint32_t *>(scalars) + SC_ORDERED) != 0u;
+}
+// Steps between the smallest norm and the largest
+struct ScreenSteps {
+    float lo, top, scale;
+    __device__ __forceinline__ ScreenSteps(float least, float most) : lo(least), top(most)
+    {
+        scale = top > lo ? (float)SC_BINS / (top - lo) : 0.f;
+    }
+    __device__ __forceinline__ ScreenSteps(const float *scalars, const float *norms)
+        : ScreenSteps(least_of(scalars, norms), scalars[5]) {}
+    static __device__ __forceinline__ float least_of(const float *scalars, const float *norms)
+    {
+        const int32_t a = __float_as_int(scalars[SC_REF]), b = __float_as_int(scalars[SC_REF + 1]);
+        const float inf = __int_as_float(0x7f800000);
+        return fminf(a < 0 ? inf : __ldg(norms + a), b < 0 ? inf : __ldg(norms + b));
+    }
+    __device__ __forceinline__ int of(float n) const { return max(0, min((int)((n - lo) * scale), SC_BINS - 1)); }
+};
 #endif
 
 // Rows are whole 16-byte pieces
@@ -151,14 +212,27 @@ int launch_screen_prepare(const void *W, int f16, int64_t D, int64_t M, const fl
                           const int32_t *rowptr, const int32_t *colidx, int64_t N, int head,
                           const uint16_t *feat, const uint16_t *rank, const int32_t *perm,
                           const uint32_t *key, const uint32_t *tile_len, char *cb, const ScreenLayout &cl,
-                          float *scalars, const float *earlier, float *sample, float *window, int64_t n_pad,
-                          uint32_t *status, cudaStream_t s);
-// the 8-bit images and the norms of the n_slabs slabs of launch k (neurons beyond M: never chosen), into the slots from `slot` on; nothing if the scalars say that they stand, as may
-// be `expected`
-int launch_screen_quantize(const void *W, int f16, int64_t D, int64_t M, const float *norms,
-                           int64_t k, int64_t launches, int64_t n_slabs, int64_t slot, int head,
-                           const uint16_t *feat, char *cb, const ScreenLayout &cl, const float *scalars,
-                           bool expected, cudaStream_t s);
+                          float *scalars, const float *earlier, float *sample, float *window, float2 *reach,
+                          uint32_t *bound, uint32_t *count, int64_t n_pad, bool top2, uint32_t *status, cudaStream_t s);
+// whether the slabs follow the norms, and the units in that order
+int launch_screen_order(const float *norms, int64_t D, int64_t M, int64_t N, int64_t launches, char *cb,
+                        const ScreenLayout &cl, float *scalars, const float *earlier, bool shared,
+                        const uint32_t *status, uint32_t *tickets, cudaStream_t s);
+// the 8-bit images and the norms of the n_slabs slabs of launch k (neurons beyond M: never chosen), into the slots
+// from `slot` on; nothing if the scalars say that they stand, as may be `expected`.  In the order of the norms also
+// the list of the sweep's items (sets: of 128 documents).
+struct ImageArgs {
+    int64_t k, launches, n_slabs, slab0, slot;
+    int head, sets, first;
+    bool expected;
+    const float2 *reach;
+    const float *window;
+    const uint32_t *bound;
+    uint2 *items;
+    uint32_t *tickets;
+};
+int launch_screen_quantize(const void *W, int f16, int64_t D, int64_t M, const float *norms, const ImageArgs &g,
+                           const uint16_t *feat, char *cb, const ScreenLayout &cl, const float *scalars, cudaStream_t s);
 // A launch that may begin under the end of the one before it on the stream, if that one's blocks allow it
 // (griddepcontrol.launch_dependents) and the kernel waits before it reads or writes (griddepcontrol.wait).
 struct ScreenLaunch {
@@ -173,9 +247,10 @@ struct ScreenLaunch {
     }
     ScreenLaunch(const ScreenLaunch &) = delete;
 };
-int launch_sweep_screen(const ScreenArgs &a, bool top2, cudaStream_t s);
+// one launch for either order of the slabs: the one that the scalars do not name returns at once
+int launch_sweep_screen(const ScreenArgs &a, const OrderedArgs &o, bool top2, bool ordered, int sms, cudaStream_t s);
 // after each launch: what it could not rule out, into the documents' lists
-int launch_screen_collect(const VerifyArgs &a, bool top2, cudaStream_t s);
+int launch_screen_collect(const VerifyArgs &a, bool top2, int sms, cudaStream_t s);
 // after the last: the lists evaluated exactly, and the outputs
 int launch_screen_verify(const VerifyArgs &a, bool top2, cudaStream_t s);
 // directly behind it: the documents it handed over (none, as a rule)

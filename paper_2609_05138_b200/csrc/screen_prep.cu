@@ -11,7 +11,7 @@ namespace bmu {
 static inline size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 
 template <typename Take>
-static void codebook_layout(int64_t D, int64_t slots, int sets, Take take, ScreenLayout *l)
+static void codebook_layout(int64_t D, int64_t M, int64_t slots, int sets, Take take, ScreenLayout *l)
 {
     const size_t d4 = (size_t)D * 4;
     l->scalars = take((size_t)sets * SC_SCALARS * 4);
@@ -21,6 +21,9 @@ static void codebook_layout(int64_t D, int64_t slots, int sets, Take take, Scree
     l->img8 = take((size_t)slots * (size_t)(D + 1) * SC_SLAB);
     l->head_img = take((size_t)slots * (size_t)l->head_pad * SC_SLAB);
     l->normp = take((size_t)slots * SC_SLAB * 4);
+    const size_t m4 = M >= SC_ORDER_MIN ? (size_t)((M + SC_SLAB - 1) / SC_SLAB * SC_SLAB) * 4 : 0;
+    l->units = take(m4); l->unit_norm = take(m4); l->unit_tmp = take(2 * m4);
+    l->rank_of = take(m4); l->picks = take(2 * m4);
 }
 
 void screen_layout(int64_t D, int64_t M, int64_t N, int head, int64_t chunk, bool top2, int sms,
@@ -37,14 +40,20 @@ void screen_layout(int64_t D, int64_t M, int64_t N, int head, int64_t chunk, boo
     l->splits = screen_splits(blocks, slabs, sms);
     const size_t n4 = (size_t)l->n_pad * 4;
     const size_t stripes = (size_t)screen_split_blocks(blocks, slabs, sms) * SC_DOCS * 4;
-    codebook_layout(D, l->chunk_slabs, 1, take, l);
+    codebook_layout(D, M, l->chunk_slabs, 1, take, l);
     l->sample = take((size_t)SC_SAMPLE * (size_t)((M + SC_GROUP - 1) / SC_GROUP) * 4);
     l->window = take(n4);
     l->amin = take(n4); l->amin2 = top2 ? take(n4) : l->amin;
     l->cval = take(stripes * sizeof(float2)); l->cmask = take(stripes * sizeof(uint4));
     l->cval2 = top2 ? take(stripes * sizeof(float)) : l->cval;
     l->lcount = take(n4);
+    // (one after the other: n_pad is a multiple of 128)
+    static_assert(SC_LIST * 24 >= SC_OWN_LIST * 16, "room for the lists of slabs in the order of the norms");
     l->lval = take(n4 * SC_LIST); l->lmask = take(n4 * SC_LIST * 4); l->lbase = take(n4 * SC_LIST);
+    const bool order = M >= SC_ORDER_MIN;
+    l->reach = take(order ? 2 * n4 : 0);
+    l->items = take(order ? (size_t)blocks * SC_PARTS * sizeof(uint2) : 0);
+    l->tickets = take(order && launches <= SC_MAX_LAUNCHES ? (size_t)launches * (SC_PARTS + 1) * 4 : 0);
     l->total = off;
 }
 
@@ -56,7 +65,7 @@ void screen_shared_layout(int64_t D, int64_t M, int head, int64_t chunk, ScreenL
     const int64_t all = (M + SC_SLAB - 1) / SC_SLAB;
     l->chunk_slabs = chunk / SC_SLAB < all ? chunk / SC_SLAB : all;
     const int64_t launches = (all + l->chunk_slabs - 1) / l->chunk_slabs;
-    codebook_layout(D, launches * l->chunk_slabs, 2, take, l);
+    codebook_layout(D, M, launches * l->chunk_slabs, 2, take, l);
     l->rank = take((size_t)D * 2); l->feat = take((size_t)D * 2);
     l->total = off;
 }
@@ -209,11 +218,20 @@ screen_range_kernel(const WT *__restrict__ W, int64_t D, int64_t M, const float 
         atomicMax(&s_most[(rank ? (int)rank[row] : (int)row) < head ? 0 : 1], __float_as_uint(__fsub_ru(hi, lo)));
     }
     uint32_t nm = 0;
+    u64 least = KEY_WORST;                                 // (a thread's units are all even or all odd)
     for (int64_t j = (int64_t)block * 256 + threadIdx.x; j < M; j += (int64_t)blocks * 256)
     {
         // (a unit at infinity is never within a finite window: it widens nobody's)
-        const uint32_t n = __float_as_uint(fabsf(__ldg(norms + j)));
-        if (n < 0x7f800000u) nm = max(nm, n);
+        const float v = __ldg(norms + j);
+        const uint32_t n = __float_as_uint(fabsf(v));
+        if (n < 0x7f800000u) { nm = max(nm, n); least = min(least, make_key(v, (int32_t)j)); }
+    }
+    if (M >= SC_ORDER_MIN && __any_sync(0xffffffffu, least != KEY_WORST)) {
+#pragma unroll
+        for (int m = 16; m > 1; m >>= 1) least = min(least, __shfl_xor_sync(0xffffffffu, least, m));
+        // (kept as complements: the words begin as zeros)
+        u64 *to = reinterpret_cast<u64 *>(status + STATUS_REFS) + 8 * (lane & 1) + (block & 7);
+        if (lane < 2 && ~least > *reinterpret_cast<volatile u64 *>(to)) atomicMax(to, ~least);
     }
     nm = __reduce_max_sync(0xffffffffu, nm);
     if (lane == 0 && nm > 0) atomicMax(&s_most[2], nm);
@@ -244,12 +262,18 @@ __device__ __forceinline__ uint32_t screen_longest(const uint32_t *tile_len, int
 // The gathered rows share one step d_tail = (largest range) / q_max; a head row has the step k d_head
 // with an integer k of its own (its entries of X_head are k instead of 1), so that rows of small range
 // keep their resolution.  table[f] = error in the head's image (or the gathered one's), error in the
-// gathered image, largest |w|, 1 if the row is in the head.
+// gathered image (the last bit of the first: whether the row is in the head); and as pairs of 16 bits, rounded to the
+// safe side, largest |w| and the range, and by how much the two reference units lie above the smallest weight.
+__device__ __forceinline__ uint32_t screen_up16(float x) { return (__float_as_uint(x) + 0xffffu) >> 16; }
+__device__ __forceinline__ float screen_lo16(uint32_t x) { return __uint_as_float(x << 16); }
+__device__ __forceinline__ float screen_hi16(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }
+
+template <typename WT>
 __global__ void __launch_bounds__(256)
-screen_table_kernel(const float *__restrict__ rmin, const float *__restrict__ rmax, int32_t D, int32_t head,
+screen_table_kernel(const WT *__restrict__ W, int64_t M, const uint32_t *__restrict__ status, const float *__restrict__ rmin, const float *__restrict__ rmax, int32_t D, int32_t head,
                     int32_t head_pad, const uint16_t *__restrict__ feat, const uint16_t *__restrict__ rank,
                     const uint32_t *__restrict__ tile_len, int64_t few, const uint32_t *__restrict__ most,
-                    const float *__restrict__ earlier, int sampled, float *__restrict__ scalars, float4 *__restrict__ table,
+                    const float *__restrict__ earlier, int sampled, float *__restrict__ scalars, uint4 *__restrict__ table,
                     unsigned char *__restrict__ kpack, float *__restrict__ khead)
 {
     uint32_t m3[3];
@@ -261,6 +285,16 @@ screen_table_kernel(const float *__restrict__ rmin, const float *__restrict__ rm
     }
     const float rh = earlier ? earlier[8] : __uint_as_float(m3[0]), rt = earlier ? earlier[9] : __uint_as_float(m3[1]);
     const float norm = earlier ? earlier[5] : __uint_as_float(m3[2]);
+    int32_t ref[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        u64 k = 0ull;
+        if (M >= SC_ORDER_MIN) {
+#pragma unroll
+            for (int x = 0; x < 8; ++x) k = max(k, __ldg(reinterpret_cast<const u64 *>(status + STATUS_REFS) + 8 * c + x));
+        }
+        ref[c] = earlier ? __float_as_int(earlier[SC_REF + c]) : k ? (int32_t)(uint32_t)~k : -1;
+    }
     const uint32_t longest = screen_longest(tile_len, few);
     int q_max = longest <= 65535u / SC_Q_TOP ? SC_Q_TOP : max(SC_Q_MIN, min(SC_Q_TOP, (int)(65535u / longest)));
     const bool stand = earlier && (int)earlier[4] <= q_max;      // images of fewer steps do as well
@@ -275,6 +309,8 @@ screen_table_kernel(const float *__restrict__ rmin, const float *__restrict__ rm
         scalars[5] = norm; scalars[6] = (float)(65535 / q_max);
         scalars[7] = stand ? 0.f : 1.f; scalars[8] = rh; scalars[9] = rt;
         scalars[SC_VOTES] = earlier ? earlier[SC_VOTES] : __uint_as_float(0u);
+        scalars[SC_ORDERED] = __uint_as_float(0u);           // (screen_order_kernel decides)
+        scalars[SC_REF] = __int_as_float(ref[0]); scalars[SC_REF + 1] = __int_as_float(ref[1]);
         scalars[SC_SAMPLED] = earlier ? earlier[SC_SAMPLED] : __uint_as_float((uint32_t)sampled);
     }
     // errors: half a step, widened by 2^-10 for the roundings of the coding itself
@@ -294,7 +330,13 @@ screen_table_kernel(const float *__restrict__ rmin, const float *__restrict__ rm
             e = half * k * dh;
             if (range > 255.f * k * dh) e += __fsub_ru(range, __fmul_rd(255.f * k, dh)) * (1.f + 1.f / 1024.f);
         }
-        table[i] = make_float4(e, tail, fmaxf(fabsf(rmin[i]), fabsf(rmax[i])), in ? 1.f : 0.f);
+        float above[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+            above[c] = ref[c] < 0 ? 0.f : __fsub_rd(screen_ld(W + (int64_t)i * M + ref[c]), rmin[i]);
+        table[i] = make_uint4(((__float_as_uint(e) + 1u) & ~1u) | (in ? 1u : 0u), __float_as_uint(tail),
+                              screen_up16(fmaxf(fabsf(rmin[i]), fabsf(rmax[i]))) | screen_up16(range) << 16,
+                              __float_as_uint(above[0]) >> 16 | (__float_as_uint(above[1]) & 0xffff0000u));
     }
     if (i < head_pad) {
         const bool in = i < head && i < D;
@@ -306,15 +348,21 @@ screen_table_kernel(const float *__restrict__ rmin, const float *__restrict__ rm
 }
 
 // ---- windows: one warp per planned document -----------------------------------------------
-// 2 B of what the rows of a document's ids bring
-__device__ __forceinline__ float screen_window_of(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
-                                                  int64_t i, const uint32_t *__restrict__ key,
-                                                  const float4 *__restrict__ table, const float *__restrict__ scalars,
-                                                  [[maybe_unused]] int64_t D, [[maybe_unused]] uint32_t *status)
+// 2 B of what the rows of a document's ids bring; and, by `order`, how far it reaches: a bound of its smallest
+// (TOP2: second smallest) approximate value from the reference units, which is their own value and B (and B once
+// more, so that the bound holds for what the verify stage computes), and 2 R + 2 B.
+struct ScreenWindow { float window, bound, reach; };
+
+__device__ __forceinline__ ScreenWindow screen_window_of(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
+                                                         int64_t i, const uint32_t *__restrict__ key,
+                                                         const uint4 *__restrict__ table, const float *scalars,
+                                                         const float *__restrict__ norms, bool order, bool top2,
+                                                         [[maybe_unused]] int64_t D, [[maybe_unused]] uint32_t *status)
 {
     const int lane = threadIdx.x & 31;
     const int beg = __ldg(rowptr + i), end = __ldg(rowptr + i + 1);
-    float en = 0.f, eo = 0.f, aa = 0.f, in = 0.f;
+    float en = 0.f, eo = 0.f, aa = 0.f, rr = 0.f, ra = 0.f, rb = 0.f;
+    uint32_t in = 0u;
     for (int e0 = beg; e0 < end; e0 += 128) {
         int f[4];
 #pragma unroll
@@ -322,32 +370,55 @@ __device__ __forceinline__ float screen_window_of(const int32_t *__restrict__ ro
             const int e = e0 + 32 * u + lane;
             f[u] = e < end ? (int)BMU_IDX((uint32_t)__ldg(colidx + e), D, status) : -1;
         }
-        float4 t[4];
+        uint4 t[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) t[u] = f[u] >= 0 ? __ldg(table + f[u]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int u = 0; u < 4; ++u) t[u] = f[u] >= 0 ? __ldg(table + f[u]) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) { en += t[u].x; eo += t[u].y; aa += t[u].z; in += t[u].w; }
+        for (int u = 0; u < 4; ++u) {
+            en += __uint_as_float(t[u].x); eo += __uint_as_float(t[u].y); aa += screen_lo16(t[u].z); in |= t[u].x;
+            if (order) { rr += screen_hi16(t[u].z); ra += screen_lo16(t[u].w); rb += screen_hi16(t[u].w); }
+        }
     }
+    in = __reduce_or_sync(0xffffffffu, in);
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1) {
         en += __shfl_xor_sync(0xffffffffu, en, m);
         eo += __shfl_xor_sync(0xffffffffu, eo, m);
         aa += __shfl_xor_sync(0xffffffffu, aa, m);
-        in += __shfl_xor_sync(0xffffffffu, in, m);
+        if (order) {
+            rr += __shfl_xor_sync(0xffffffffu, rr, m);
+            ra += __shfl_xor_sync(0xffffffffu, ra, m);
+            rb += __shfl_xor_sync(0xffffffffu, rb, m);
+        }
     }
     // a list that repeats a head id is gathered whole
     const float n = (float)(end - beg), gathered = (float)key[i];
-    const float E = in > 0.f && gathered == n ? eo : en;
+    const float E = (in & 1u) && gathered == n ? eo : en;
     float B = 2.f * E + 1.1920929e-7f * (n * aa + 4.f * scalars[5] + 8.f * aa);
-    B *= 1.f + 1.f / 4096.f + 2.f * n * 1.1920929e-7f;    // the roundings of these sums themselves
-    return (gathered > scalars[6] || !(B < 1e37f)) ? CUDART_INF_F : 2.f * B;
+    const float wide = 1.f + 1.f / 4096.f + 2.f * n * 1.1920929e-7f;    // the roundings of these sums themselves
+    B *= wide;
+    ScreenWindow w;
+    w.window = (gathered > scalars[6] || !(B < 1e37f)) ? CUDART_INF_F : 2.f * B;
+    w.bound = w.reach = CUDART_INF_F;
+    if (order) {
+        const int32_t a = __float_as_int(scalars[SC_REF]), b = __float_as_int(scalars[SC_REF + 1]);
+        float va = a < 0 ? CUDART_INF_F : __ldg(norms + a) - 2.f * (ra * (2.f - wide)) + 2.f * B;
+        float vb = b < 0 ? CUDART_INF_F : __ldg(norms + b) - 2.f * (rb * (2.f - wide)) + 2.f * B;
+        if (!(va < CUDART_INF_F)) va = CUDART_INF_F;               // (not a number either)
+        if (!(vb < CUDART_INF_F)) vb = CUDART_INF_F;
+        w.bound = top2 ? fmaxf(va, vb) : fminf(va, vb);
+        w.reach = 2.f * rr * wide + 2.f * B;
+    }
+    return w;
 }
 
 // The first blocks, one per sampled document: how many of its groups lie within its window.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 6)
 screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
                      const int32_t *__restrict__ perm, const uint32_t *__restrict__ key, int64_t N, int64_t n_pad,
-                     const float4 *__restrict__ table, float *scalars, float *__restrict__ window, int64_t D,
+                     const uint4 *__restrict__ table, float *scalars, const float *__restrict__ norms, int order, int top2,
+                     float *__restrict__ window, float2 *__restrict__ reach, uint32_t *__restrict__ bound,
+                     uint32_t *__restrict__ count, int64_t D,
                      int sampled, const float *__restrict__ groups, int64_t M, uint32_t *__restrict__ status)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -357,8 +428,9 @@ screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restri
         const int64_t n = (M + SC_GROUP - 1) / SC_GROUP;
         const float *of = groups + blockIdx.x * n;
         if (warp == 0) {
-            const float w = screen_window_of(rowptr, colidx, screen_sample_doc(blockIdx.x, sampled, N), key, table, scalars, D, status);
-            if (lane == 0) s_win = w;
+            const ScreenWindow w = screen_window_of(rowptr, colidx, screen_sample_doc(blockIdx.x, sampled, N), key, table,
+                                                    scalars, norms, false, top2, D, status);
+            if (lane == 0) s_win = w.window;
         }
         float least = CUDART_INF_F;
         for (int64_t g = threadIdx.x; g < n; g += 256) least = fminf(least, __ldg(of + g));
@@ -383,12 +455,20 @@ screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restri
     }
     const int64_t p = ((int64_t)(blockIdx.x - sampled) * blockDim.x + threadIdx.x) >> 5;
     if (p >= n_pad) return;
-    if (p >= N || (*status & PLAN_STATUS_OVERFLOW)) {
-        if (lane == 0) window[p] = 0.f;
-        return;
-    }
-    const float w = screen_window_of(rowptr, colidx, perm[p], key, table, scalars, D, status);
-    if (lane == 0) window[p] = w;
+    const bool there = p < N && !(*status & PLAN_STATUS_OVERFLOW);
+    ScreenWindow w = {0.f, -CUDART_INF_F, 0.f};
+    if (there) w = screen_window_of(rowptr, colidx, perm[p], key, table, scalars, norms, order, top2, D, status);
+    if (lane) return;
+    window[p] = w.window;
+    if (!order) return;
+    // (documents that are evaluated whole need no slab)
+    const bool none = !there || w.window == CUDART_INF_F;
+    const float t = none ? -CUDART_INF_F : w.bound + w.window + w.reach;
+    reach[p] = make_float2(t == t ? t : CUDART_INF_F, w.reach);
+    bound[p] = float_to_ordered(none ? -CUDART_INF_F : w.bound);
+    count[p] = 0u;
+    const ScreenSteps steps(scalars, norms);
+    if (!none && t < steps.top) atomicAdd(status + STATUS_REACH + steps.of(t), 1u);
 }
 
 template <typename WT>
@@ -411,13 +491,14 @@ int launch_screen_prepare(const void *W, int f16, int64_t D, int64_t M, const fl
                           const int32_t *rowptr, const int32_t *colidx, int64_t N, int head,
                           const uint16_t *feat, const uint16_t *rank, const int32_t *perm,
                           const uint32_t *key, const uint32_t *tile_len, char *cb, const ScreenLayout &cl,
-                          float *scalars, const float *earlier, float *sample, float *window, int64_t n_pad,
-                          uint32_t *status, cudaStream_t s)
+                          float *scalars, const float *earlier, float *sample, float *window, float2 *reach,
+                          uint32_t *bound, uint32_t *count, int64_t n_pad, bool top2, uint32_t *status, cudaStream_t s)
 {
+    const int order = M >= SC_ORDER_MIN;
     // (an earlier search of the same codebook has decided for this one too)
     const int sampled = earlier ? 0 : (int)(N < SC_SAMPLE ? N : SC_SAMPLE);
     float *rmin = reinterpret_cast<float *>(cb + cl.rmin), *rmax = reinterpret_cast<float *>(cb + cl.rmax);
-    float4 *table = reinterpret_cast<float4 *>(cb + cl.table);
+    uint4 *table = reinterpret_cast<uint4 *>(cb + cl.table);
     uint32_t *most = status + STATUS_MAXIMA;
     if (!earlier) {
         const int rc = f16 ? launch_range(static_cast<const __half *>(W), D, M, norms, rank, head, rmin, rmax, most,
@@ -429,11 +510,17 @@ int launch_screen_prepare(const void *W, int f16, int64_t D, int64_t M, const fl
     const int64_t rows = D > cl.head_pad ? D : cl.head_pad;
     // up to a thousandth of the tiles, or four where they are few (32 documents of 1000 ids: 27 us for 4,096 units)
     const int64_t tiles = (N + 7) / 8, four = tiles / 64 < 4 ? tiles / 64 : 4, few = tiles / 1024 > four ? tiles / 1024 : four;
-    { screen_table_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, s>>>(
-        rmin, rmax, (int32_t)D, head, cl.head_pad, feat, rank, tile_len, few, most, earlier, sampled, scalars, table,
-        reinterpret_cast<unsigned char *>(cb + cl.kpack), reinterpret_cast<float *>(cb + cl.khead)); BMU_LAUNCHED(); }
+    const auto tables = [&](auto w) {
+        screen_table_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, s>>>(
+            w, M, status, rmin, rmax, (int32_t)D, head, cl.head_pad, feat, rank, tile_len, few, most, earlier, sampled,
+            scalars, table, reinterpret_cast<unsigned char *>(cb + cl.kpack), reinterpret_cast<float *>(cb + cl.khead));
+        BMU_LAUNCHED();
+    };
+    if (f16) tables(static_cast<const __half *>(W));
+    else tables(static_cast<const float *>(W));
     { screen_window_kernel<<<(unsigned)(sampled + (n_pad * 32 + 255) / 256), 256, 0, s>>>(
-        rowptr, colidx, perm, key, N, n_pad, table, scalars, window, D, sampled, sample, M, status); BMU_LAUNCHED(); }
+        rowptr, colidx, perm, key, N, n_pad, table, scalars, norms, order, top2, window, reach, bound, count, D, sampled,
+        sample, M, status); BMU_LAUNCHED(); }
     BMU_CUDA(cudaGetLastError());
     return BMU_OK;
 }
@@ -581,17 +668,154 @@ __device__ __forceinline__ void screen_head_block(const WT *__restrict__ W, int6
     __syncthreads();                                       // (the caller may take another slab)
 }
 
+// ---- images of slabs in the order of the norms --------------------------------------------
+// A launch's units, in the order of the map (`picks`: unit, place in the order of the norms; no unit beyond the
+// last), so that neighbouring lanes read neighbouring weights of a row; the bytes meet in shared memory.  What is
+// read are the sectors that hold a unit: some of a row where few units are needed, all of it, once, where many are.
+// (A lane per place, its weight wherever it lies: 463 us for 32 slabs of 64 x 64, D = 16,384.)
+static const int ORD_ROWS = 4;                             // rows a block takes at a time
+static const int ORD_HEAD = 16;                            // head features a block takes at a time
+
+template <typename WT>
+__device__ __forceinline__ void ordered_rows(const WT *__restrict__ W, int64_t D, int64_t M, int64_t f0, int slots,
+                                             int place0, const int2 *__restrict__ picks, const float *__restrict__ rmin,
+                                             float inv, float q_max, unsigned char *__restrict__ img8)
+{
+    __shared__ __align__(16) unsigned char bytes[ORD_ROWS * SC_MAX_SLABS * SC_SLAB];
+    float c[ORD_ROWS];
+    const WT *row[ORD_ROWS];
+#pragma unroll
+    for (int u = 0; u < ORD_ROWS; ++u) {
+        const int64_t f = f0 + u < D ? f0 + u : D - 1;
+        row[u] = W + f * M;
+        c[u] = __ldg(rmin + f);
+    }
+    for (int i = threadIdx.x; i < slots; i += 256) {
+        const int2 t = __ldg(picks + i);
+        const int at = t.y - place0, jn = at & (SC_SLAB - 1);
+        // in the slab's 128 bytes of a row: as screen_image_block has it
+        unsigned char *to = bytes + (at - jn) * ORD_ROWS + (((jn >> 4) & 1) * 4 + (jn >> 5)) * 16 + ((jn >> 2) & 3) * 4 +
+                            ((jn & 1) << 1) + ((jn >> 1) & 1);
+        float v[ORD_ROWS];
+#pragma unroll
+        for (int u = 0; u < ORD_ROWS; ++u) v[u] = t.x >= 0 && f0 + u < D ? screen_ld(row[u] + t.x) : c[u];
+#pragma unroll
+        for (int u = 0; u < ORD_ROWS; ++u) to[u * SC_SLAB] = (unsigned char)screen_code(v[u], c[u], inv, q_max);
+    }
+    __syncthreads();
+    for (int v = threadIdx.x; v < slots * ORD_ROWS / 16; v += 256) {
+        const int slab = v / (ORD_ROWS * 8), u = v / 8 % ORD_ROWS, piece = v % 8;
+        if (f0 + u <= D)                                   // row D: zeros
+            *reinterpret_cast<uint4 *>(img8 + ((size_t)slab * (D + 1) + f0 + u) * SC_SLAB + piece * 16) =
+                reinterpret_cast<const uint4 *>(bytes)[v];
+    }
+    __syncthreads();
+}
+
+template <typename WT>
+__device__ __forceinline__ void ordered_head(const WT *__restrict__ W, int64_t D, int64_t M, int h0, int slots, int place0,
+                                             const int2 *__restrict__ picks, int32_t head, int32_t head_pad,
+                                             const uint16_t *__restrict__ feat, const float *__restrict__ rmin,
+                                             const float *__restrict__ khead, unsigned char *__restrict__ img)
+{
+    __shared__ float s_c[ORD_HEAD], s_k[ORD_HEAD];
+    __shared__ int64_t s_row[ORD_HEAD];
+    if (threadIdx.x < ORD_HEAD) {
+        const int h = h0 + threadIdx.x;
+        const bool in = h < head && h < D;
+        const int64_t f = in ? (feat ? (int64_t)__ldg(feat + h) : (int64_t)h) : -1;
+        s_row[threadIdx.x] = in ? f * M : -1;
+        s_c[threadIdx.x] = in ? __ldg(rmin + f) : 0.f;
+        s_k[threadIdx.x] = __ldg(khead + h);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < slots; i += 256) {
+        const int2 t = __ldg(picks + i);
+        const int at = t.y - place0, n = screen_col(at & (SC_SLAB - 1));
+        uint32_t q[4];
+#pragma unroll
+        for (int w = 0; w < 4; w += 2) {                   // eight rows in flight
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int64_t r = s_row[4 * w + u];
+                v[u] = t.x >= 0 && r >= 0 ? screen_ld(W + r + t.x) : s_c[4 * w + u];
+            }
+            uint32_t b[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) b[u] = screen_code(v[u], s_c[4 * w + u], s_k[4 * w + u], 255.f);
+            q[w] = screen_pack(b[0], b[1], b[2], b[3]);
+            q[w + 1] = screen_pack(b[4], b[5], b[6], b[7]);
+        }
+        unsigned char *dst = img + ((size_t)(at / SC_SLAB) * (head_pad / 128) + (h0 >> 7)) * MMA_STAGE_BYTES +
+                             (n >> 3) * 1024 + ((h0 & 127) >> 4) * 128 + (n & 7) * 16;
+        *reinterpret_cast<uint4 *>(dst) = make_uint4(q[0], q[1], q[2], q[3]);
+    }
+    __syncthreads();
+}
+
+// A warp per set of 128 documents: which of the launch's slabs any of them reaches, as items of up to SC_PART.
+__device__ __forceinline__ void ordered_items(const ImageArgs &g, int set, int slabs, const float *__restrict__ unit_norm,
+                                              const float *__restrict__ scalars)
+{
+    const int lane = threadIdx.x & 31;
+    const float top = __ldg(scalars + SC_TOP);
+    float far = -CUDART_INF_F;
+#pragma unroll
+    for (int u = 0; u < SC_DOCS / 32; ++u) {
+        const int64_t p = (int64_t)set * SC_DOCS + 32 * u + lane;
+        const float2 r = __ldg(g.reach + p);
+        if (r.x > top) continue;                           // evaluated whole
+        // (what the launches before have found)
+        const float t = g.first ? r.x : fminf(r.x, ordered_to_float(__ldcg(g.bound + p)) + __ldg(g.window + p) + r.y);
+        far = fmaxf(far, t);
+    }
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) far = fmaxf(far, __shfl_xor_sync(0xffffffffu, far, m));
+    const bool in = lane < slabs && __ldg(unit_norm + lane * SC_SLAB) <= far;
+    const int n = __popc(__ballot_sync(0xffffffffu, in));  // (ascending: the first ones)
+    if (lane < (n + SC_PART - 1) / SC_PART)
+        g.items[(size_t)lane * g.sets + atomicAdd(g.tickets + lane, 1u)] =
+            make_uint2((uint32_t)set, (uint32_t)(lane * SC_PART) | (uint32_t)min(n, (lane + 1) * SC_PART) << 16);
+}
+
 // Both images of a slab in one grid, the head's blocks in front.  LOOP: a block takes every gridDim.y-th
 // slab -- slower where there is work (a shared codebook's images usually stand), 9 -> 3 us where not.
 template <typename WT, bool VEC, bool LOOP>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, LOOP ? 3 : sizeof(WT) == 2 && VEC ? 4 : 6)
 screen_image_kernel(const WT *__restrict__ W, int64_t D, int64_t M, int64_t k, int64_t launches, int64_t n_slabs,
-                    int32_t head,
+                    const ImageArgs g, const int2 *__restrict__ picks, const float *__restrict__ unit_norm, int32_t head,
                     int32_t head_pad, const uint16_t *__restrict__ feat, const float *__restrict__ rmin,
                     const float *__restrict__ khead, const float *__restrict__ scalars,
                     const float *__restrict__ norms, unsigned char *__restrict__ img8,
                     unsigned char *__restrict__ head_img, float *__restrict__ normp)
 {
+    if (screen_ordered(scalars)) {
+        const uint32_t *sc = reinterpret_cast<const uint32_t *>(scalars);
+        const int slabs = (int)min(n_slabs, (int64_t)__ldg(sc + SC_NEEDED) - g.slab0);
+        if (slabs <= 0) return;
+        const int place0 = (int)g.slab0 * SC_SLAB, slots = slabs * SC_SLAB;
+        const bool stand = __ldg(sc + SC_STAND) != 0u;     // the images of an earlier search
+        const int lists = (g.sets + 7) / 8, rows = (int)((D + ORD_ROWS) / ORD_ROWS), heads = head_pad / ORD_HEAD;
+        const int all = stand ? lists : lists + heads + rows;
+        for (int item = blockIdx.y * gridDim.x + blockIdx.x; item < all; item += gridDim.x * gridDim.y) {
+            if (item < lists) {
+                const int set = item * 8 + (threadIdx.x >> 5);
+                if (set < g.sets) ordered_items(g, set, slabs, unit_norm + place0, scalars);
+            } else if (item < lists + heads) {
+                ordered_head(W, D, M, (item - lists) * ORD_HEAD, slots, place0, picks + place0, head, head_pad, feat, rmin, khead, head_img);
+                if (item == lists)
+                    for (int x = threadIdx.x; x < slots; x += 256) {
+                        const int jn = x & (SC_SLAB - 1);
+                        normp[x - jn + ((jn & 31) >> 2) * 16 + (jn >> 5) * 4 + (jn & 3)] = __ldg(unit_norm + place0 + x);
+                    }
+            } else {
+                ordered_rows(W, D, M, (int64_t)(item - lists - heads) * ORD_ROWS, slots, place0, picks + place0, rmin,
+                             __ldg(scalars + 2), __ldg(scalars + 4), img8);
+            }
+        }
+        return;
+    }
     if (__ldg(scalars + 7) == 0.f || screen_whole(scalars)) return;   // the images of an earlier search stand
     const int heads = head_pad / 32;
     auto one = [&](const int64_t slab) {
@@ -608,35 +832,33 @@ screen_image_kernel(const WT *__restrict__ W, int64_t D, int64_t M, int64_t k, i
 }
 
 template <typename WT>
-static int launch_images(const WT *W, int64_t D, int64_t M, const float *norms, int64_t k,
-                         int64_t launches, int64_t n_slabs, int64_t slot, int head, const uint16_t *feat, char *base,
-                         const ScreenLayout &l, const float *scalars, bool expected, cudaStream_t s)
+static int launch_images(const WT *W, int64_t D, int64_t M, const float *norms, const ImageArgs &g,
+                         const uint16_t *feat, char *base, const ScreenLayout &l, const float *scalars, cudaStream_t s)
 {
     const float *rmin = reinterpret_cast<const float *>(base + l.rmin);
     const float *khead = reinterpret_cast<const float *>(base + l.khead);
-    unsigned char *img8 = reinterpret_cast<unsigned char *>(base + l.img8) + (size_t)slot * (D + 1) * SC_SLAB;
-    unsigned char *head_img = reinterpret_cast<unsigned char *>(base + l.head_img) + (size_t)slot * l.head_pad * SC_SLAB;
-    float *normp = reinterpret_cast<float *>(base + l.normp) + slot * SC_SLAB;
+    const int2 *picks = reinterpret_cast<const int2 *>(base + l.picks);
+    const float *unit_norm = reinterpret_cast<const float *>(base + l.unit_norm);
+    unsigned char *img8 = reinterpret_cast<unsigned char *>(base + l.img8) + (size_t)g.slot * (D + 1) * SC_SLAB;
+    unsigned char *head_img = reinterpret_cast<unsigned char *>(base + l.head_img) + (size_t)g.slot * l.head_pad * SC_SLAB;
+    float *normp = reinterpret_cast<float *>(base + l.normp) + g.slot * SC_SLAB;
     const bool vec = M % (16 / sizeof(WT)) == 0 && (reinterpret_cast<uintptr_t>(W) & 15) == 0;
     const int rows = vec ? IMAGE_ROWS<WT, true> : IMAGE_ROWS<WT, false>;
     const dim3 grid((unsigned)(l.head_pad / 32 + (D + 1 + rows - 1) / rows),
-                    expected ? 1u : (unsigned)n_slabs);       // few blocks where there is likely nothing to do
-#define BMU_IMG(V, L) { screen_image_kernel<WT, V, L><<<grid, 256, 0, s>>>(W, D, M, k, launches, n_slabs, head, l.head_pad, feat, rmin, khead, scalars, norms, img8, head_img, normp); BMU_LAUNCHED(); }
-    if (expected) { if (vec) BMU_IMG(true, true) else BMU_IMG(false, true) }
+                    g.expected ? 1u : (unsigned)g.n_slabs);     // few blocks where there is likely nothing to do
+#define BMU_IMG(V, L) { screen_image_kernel<WT, V, L><<<grid, 256, 0, s>>>(W, D, M, g.k, g.launches, g.n_slabs, g, picks, unit_norm, g.head, l.head_pad, feat, rmin, khead, scalars, norms, img8, head_img, normp); BMU_LAUNCHED(); }
+    if (g.expected) { if (vec) BMU_IMG(true, true) else BMU_IMG(false, true) }
     else if (vec) BMU_IMG(true, false) else BMU_IMG(false, false)
 #undef BMU_IMG
     BMU_CUDA(cudaGetLastError());
     return BMU_OK;
 }
 
-int launch_screen_quantize(const void *W, int f16, int64_t D, int64_t M, const float *norms,
-                           int64_t k, int64_t launches, int64_t n_slabs, int64_t slot, int head,
-                           const uint16_t *feat, char *cb, const ScreenLayout &cl, const float *scalars,
-                           bool expected, cudaStream_t s)
+int launch_screen_quantize(const void *W, int f16, int64_t D, int64_t M, const float *norms, const ImageArgs &g,
+                           const uint16_t *feat, char *cb, const ScreenLayout &cl, const float *scalars, cudaStream_t s)
 {
-    if (f16)
-        return launch_images(static_cast<const __half *>(W), D, M, norms, k, launches, n_slabs, slot, head, feat, cb, cl, scalars, expected, s);
-    return launch_images(static_cast<const float *>(W), D, M, norms, k, launches, n_slabs, slot, head, feat, cb, cl, scalars, expected, s);
+    if (f16) return launch_images(static_cast<const __half *>(W), D, M, norms, g, feat, cb, cl, scalars, s);
+    return launch_images(static_cast<const float *>(W), D, M, norms, g, feat, cb, cl, scalars, s);
 }
 
 }  // namespace bmu

@@ -160,6 +160,36 @@ __device__ __forceinline__ void verify_groups(const VerifyArgs &a, const uint4 m
     }
 }
 
+// The whole warp evaluates the units of `bits`, numbers first .. first + 31 in the order of the norms: a lane per
+// listed row, a 32-byte sector each, four rows in flight.
+template <typename WT, bool TOP2>
+__device__ __forceinline__ void verify_units(const VerifyArgs &a, uint32_t bits, int64_t first, int beg, int end,
+                                             u64 &best, u64 &best2)
+{
+    const int lane = threadIdx.x & 31;
+    const WT *W = static_cast<const WT *>(a.W);
+    for (; bits; bits &= bits - 1) {
+        const int32_t j = __ldg(a.units + first + __ffs(bits) - 1);
+        if (j < 0) continue;                                 // (beyond the last unit; never within a window)
+        float s = 0.f;
+        for (int e0 = beg; e0 < end; e0 += 128) {
+            float w[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int e = e0 + 32 * u + lane;
+                w[u] = e < end ? verify_ld(W + (int64_t)BMU_IDX((uint32_t)__ldg(a.colidx + e), a.D, a.status) * a.M + j) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) s += w[u];
+        }
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+        const u64 k = make_key(fmaf(-2.f, s, __ldg(a.norms + j)), j);
+        if (TOP2) { if (lane == 0) Best<true>::merge(best, best2, k, KEY_WORST); }
+        else best = k < best ? k : best;
+    }
+}
+
 // the warp's best (and second-best) key, on every lane
 template <bool TOP2>
 __device__ __forceinline__ void verify_merge(u64 &best, u64 &best2)
@@ -183,19 +213,22 @@ __device__ __forceinline__ uint4 shfl4(const uint4 v, int src)
                       __shfl_sync(0xffffffffu, v.z, src), __shfl_sync(0xffffffffu, v.w, src));
 }
 
-// Eight documents per warp, a lane per stripe.
+// Eight documents per warp, a lane per stripe.  (Few blocks, for those times when there is nothing to do.)
 template <typename WT, bool TOP2, bool VEC>
 __global__ void __launch_bounds__(256, 4)
 screen_collect_kernel(const VerifyArgs a)
 {
     const int lane = threadIdx.x & 31, k = lane & 3;
-    const int64_t p = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 8 + (lane >> 2);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // (the verify stage, after the last launch)
     // (one lane reads the status word for its warp: the lanes must stay together)
-    if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(a.status), 0) || screen_whole(a.scalars)) return;
+    // (where slabs are in the order of the norms the sweep keeps the lists and the bounds itself)
+    if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(a.status), 0) || screen_whole(a.scalars) ||
+        screen_ordered(a.scalars)) return;
+    const uint32_t seg = 15u << (lane & ~3), most = screen_early_groups(a.M);
+    for (int64_t p8 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 8; p8 < a.N; p8 += (int64_t)gridDim.x * (blockDim.x / 4)) {
+    const int64_t p = p8 + (lane >> 2);
     const bool there = p < a.N;
     const float win = there ? a.window[p] : 0.f;
-    const uint32_t seg = 15u << (lane & ~3), most = screen_early_groups(a.M);
     // pass 1: the document's smallest (and second smallest) approximate value so far.  The stripes of
     // a split bring the same second smallest, over all their groups and the earlier launches;
     // whatever a merge of such pairs leaves out only makes it larger, which keeps more.
@@ -320,6 +353,7 @@ screen_collect_kernel(const VerifyArgs a)
         if (TOP2) a.amin2[p] = v2;
         if (touched) a.lcount[p] = (count & 0x80000000u) | (dense ? SC_DENSE : done << 4 | n);
     }
+    }
 }
 
 // Two documents per warp, sixteen lanes each: a lane takes one list entry.
@@ -327,13 +361,13 @@ template <typename WT, bool TOP2, bool VEC>
 __global__ void __launch_bounds__(256, 5)
 screen_verify_kernel(const VerifyArgs a)
 {
-    static_assert(SC_LIST <= 15, "a lane per entry, four bits of the count");
+    static_assert(SC_LIST <= 15 && SC_OWN_LIST <= 16, "a lane per entry, four bits of the count");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // screen_dense_kernel waits for the rest
     asm volatile("griddepcontrol.wait;" ::: "memory");                   // as this does for the last collection
     const int lane = threadIdx.x & 31, e = lane & 15;
     const int64_t p = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 2 + (lane >> 4);
     if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(a.status), 0)) return;
-    const bool there = p < a.N, whole = screen_whole(a.scalars);
+    const bool there = p < a.N, whole = screen_whole(a.scalars), ordered = screen_ordered(a.scalars);
     uint32_t count = 0, base = 0;
     uint4 todo = make_uint4(0u, 0u, 0u, 0u);
     int32_t orig = 0, beg = 0, end = 0;
@@ -342,13 +376,22 @@ screen_verify_kernel(const VerifyArgs a)
         orig = a.perm[p];
         beg = __ldg(a.rowptr + orig);
         end = __ldg(a.rowptr + orig + 1);
-        if ((uint32_t)e < (count & 15u)) {
+        if (ordered && !whole) {
+            const float win = a.window[p];
+            const uint32_t n = count;
+            count = win == CUDART_INF_F || n > (uint32_t)SC_OWN_LIST || a.reach[p].x > __ldg(a.scalars + SC_TOP) ? SC_DENSE : 0u;
+            if ((uint32_t)e < n && !count) {
+                const uint4 t = a.own_list[p * SC_OWN_LIST + e];
+                if (__uint_as_float(t.x) <= ordered_to_float(a.bound[p]) + win) todo.x = t.z;
+                base = t.y * SC_SLAB + t.w * 32u;
+            }
+        } else if ((uint32_t)e < (count & 15u)) {
             const float limit = (TOP2 ? a.amin2[p] : a.amin[p]) + a.window[p];
             if (a.lval[(size_t)p * SC_LIST + e] <= limit) todo = a.lmask[(size_t)p * SC_LIST + e];
             base = a.lbase[(size_t)p * SC_LIST + e];
         }
     }
-    // too many groups, or none (no distance of it is finite), or given up before
+    // too many groups (or units), or none (no distance of it is finite), or given up before
     uint32_t groups = popc4(todo);
 #pragma unroll
     for (int m = 8; m > 0; m >>= 1) groups += __shfl_xor_sync(0xffffffffu, groups, m);
@@ -362,11 +405,13 @@ screen_verify_kernel(const VerifyArgs a)
         if (!lanes) continue;
         const int b0 = __shfl_sync(0xffffffffu, beg, 16 * d), e0 = __shfl_sync(0xffffffffu, end, 16 * d);
         uint32_t ids[4];
-        if (VEC) VerifyVec<WT>::ids_of(a, b0, e0, ids);
+        if (VEC && !ordered) VerifyVec<WT>::ids_of(a, b0, e0, ids);
         u64 k1 = KEY_WORST, k2 = KEY_WORST;
         for (; lanes; lanes &= lanes - 1) {
             const int src = __ffs(lanes) - 1;
-            verify_groups<WT, TOP2, VEC>(a, shfl4(todo, src), __shfl_sync(0xffffffffu, base, src), b0, e0, ids, k1, k2);
+            if (ordered)
+                verify_units<WT, TOP2>(a, __shfl_sync(0xffffffffu, todo.x, src), __shfl_sync(0xffffffffu, base, src), b0, e0, k1, k2);
+            else verify_groups<WT, TOP2, VEC>(a, shfl4(todo, src), __shfl_sync(0xffffffffu, base, src), b0, e0, ids, k1, k2);
         }
         verify_merge<TOP2>(k1, k2);
         if (lane >> 4 == d) { best = k1; best2 = k2; }
@@ -402,9 +447,10 @@ screen_verify_kernel(const VerifyArgs a)
            : (top2 ? (screen_vec(a) ? cudaLaunchKernelEx(&C, KERNEL<float, true, true>, a) : cudaLaunchKernelEx(&C, KERNEL<float, true, false>, a)) \
                    : (screen_vec(a) ? cudaLaunchKernelEx(&C, KERNEL<float, false, true>, a) : cudaLaunchKernelEx(&C, KERNEL<float, false, false>, a))))
 
-int launch_screen_collect(const VerifyArgs &a, bool top2, cudaStream_t s)
+int launch_screen_collect(const VerifyArgs &a, bool top2, int sms, cudaStream_t s)
 {
-    ScreenLaunch l((unsigned)((a.N + 63) / 64), 256, s, false);
+    const int64_t blocks = (a.N + 63) / 64;
+    ScreenLaunch l((unsigned)(blocks < 4 * sms ? blocks : 4 * sms), 256, s, false);
     BMU_CUDA(BMU_VERIFY(screen_collect_kernel, l.c));
     BMU_LAUNCHED();
     return BMU_OK;

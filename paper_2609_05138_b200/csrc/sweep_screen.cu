@@ -31,11 +31,24 @@
 // ceiling with 4 bytes per update.  Whole searches before / after: 100,000 documents on a 512 x 512
 // map 206.7 / 69.5 ms, 200,000 on a trained 128 x 128 map 32.8 / 10.9 ms, 120,000 on 64 x 64 4.76 /
 // 1.71 ms, 60,000 against an fp16 256 x 256 map 22.7 / 11.3 ms.
+//
+// The blocks stay, one per SM, and take sets of 128 documents and stretches of slabs one after the other; barriers and
+// accumulators go on from item to item.
+//
+// ORDERED: slabs in the order of the norms (screen.cuh, screen_order.cu).  What differs:
+//   items      a set of documents reaches a few slabs of a launch, another set many: (set, up to SC_PART slabs),
+//              from the lists that screen_image_kernel has made, the first parts of all sets before the second ones.
+//   stopping   a warp leaves an item at the first slab that no document of its tile reaches any more.
+//   candidates the bound of a document's smallest value is good from the start and slabs with the smallest
+//              norms come first, so that little is ever within a window: what is, is looked up once more, unit by
+//              unit, and joins the document's one list.  Parts of the same set share list and bound by atomics.
 
 #include "screen.cuh"
 #include "mma_ptx.cuh"
 
 #include <math_constants.h>
+
+#include <type_traits>
 
 namespace bmu {
 
@@ -91,38 +104,34 @@ __device__ __forceinline__ u64 sc_dist2(u64 n2, uint32_t h0, uint32_t h1, uint32
     return sc_fma2(tf, st, sc_fma2(hf, sh, n2));
 }
 
-template <bool TOP2>
+// (all warps, from two places of the code)
+__device__ __forceinline__ void block_sync() { asm volatile("barrier.sync 0, %0;" ::"n"(SC_THREADS) : "memory"); }
+
+template <bool TOP2, bool ORDERED>
 __global__ void __launch_bounds__(SC_THREADS, 1)
-sweep_screen_kernel(const ScreenArgs a)
+sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
 {
     constexpr int NS = SC_NS, KS = SC_KS, NTW = SC_TAIL_WARPS;
     extern __shared__ __align__(128) unsigned char smem[];
     u64 *bars = reinterpret_cast<u64 *>(smem + NS * KS * MMA_STAGE_BYTES);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * NS + 5);
-    volatile uint32_t *abort_flag = tmem_slot + 1;
-    uint32_t *skip_flag = tmem_slot + 2;
+    volatile uint32_t *abort_flag = tmem_slot + 1, *item_slot = tmem_slot + 2;
     const uint32_t wfull0 = mm_smem(bars), wempty0 = mm_smem(bars + NS);
     const uint32_t tfull0 = mm_smem(bars + 2 * NS), tempty0 = tfull0 + 16, drain = tfull0 + 32;
     const int two = a.head_pad <= 1024, x_col = 512 - a.head_pad / 4;
+    if (screen_ordered(a.scalars) != ORDERED || screen_whole(a.scalars)) return;
+    if (ORDERED && o.slab0 >= (int64_t)__ldg(reinterpret_cast<const uint32_t *>(a.scalars) + SC_NEEDED)) return;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t group = blockIdx.x;
-    // this block's slabs of the launch
-    const int s_lo = (int)((int64_t)a.n_slabs * blockIdx.y / a.splits);
-    const int s_hi = (int)((int64_t)a.n_slabs * (blockIdx.y + 1) / a.splits);
     const int KB = a.head_pad / 128;
-
     if (threadIdx.x == 0) {
         for (int i = 0; i < NS; ++i) { mm_bar_init(wfull0 + 8 * i, 1); mm_bar_init(wempty0 + 8 * i, 1); }
         for (int i = 0; i < 2; ++i) { mm_bar_init(tfull0 + 8 * i, 1); mm_bar_init(tempty0 + 8 * i, NTW); }
         mm_bar_init(drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         *abort_flag = 0u;
-        *skip_flag = *reinterpret_cast<volatile uint32_t *>(a.status) | (screen_whole(a.scalars) ? 1u : 0u);
     }
     __syncthreads();
-    if (*skip_flag) return;          // a block before this one gave up: let the grid drain; or nothing is screened
-
     if (warp == NTW) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(mm_smem(tmem_slot)), "r"(512u) : "memory");
@@ -132,99 +141,139 @@ sweep_screen_kernel(const ScreenArgs a)
     __syncthreads();
     mm_fence_after();
     const uint32_t tmem = *tmem_slot;
-    if (warp < NTW) {
-        // X_head into tensor memory: lane 32q + l = document, a column = four features
-        const int q = warp & 3, words = a.head / 32;
-        const int64_t p = group * SC_DOCS + 32 * q + lane;
-        const bool there = p < a.n_tiles * 8;
-        for (int wd = warp >> 2; wd < a.head_pad / 32; wd += 4) {
-            const uint32_t m = there && wd < words ? __ldg(a.tile_head + (size_t)p * words + wd) : 0u;
-            const uint4 k0 = __ldg(reinterpret_cast<const uint4 *>(a.kpack) + 2 * wd);
-            const uint4 k1 = __ldg(reinterpret_cast<const uint4 *>(a.kpack) + 2 * wd + 1);
-            const uint32_t k[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
-            uint32_t v[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c)          // four mask bits -> four byte masks
-                v[c] = ((((m >> (4 * c)) & 15u) * 0x00204081u) & 0x01010101u) * 255u & k[c];
-            mm_tmem_st8(tmem + ((uint32_t)(q * 32) << 16) + x_col + wd * 8, v);
-        }
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    }
-    mm_fence_before();
-    __syncthreads();
-    mm_fence_after();
-
-    // The control warpgroup (producer, MMA issuer and two idle warps) hands registers to the four
-    // tail warpgroups, whose loads in flight are bounded by their registers.  The block is
-    // launched with 96 per thread (640 x 96 = 61440 = 128 x 32 + 512 x 112), so the increase
-    // never waits for registers that nobody releases (the launcher checks the build).
+    // Registers change hands as in sweep_screen.cu.  The loops over the items meet three times an item: the item is
+    // known; X_head is in place; X_head has been read, for every accumulator has been waited for.
+    int done = 0;                                         // slabs before this item: which accumulator, which phase
     if (warp >= NTW) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SC_CTRL_REGS));
-    if (warp == NTW) {
-        // ---------------- producer: the W stages of every slab, in order, through the ring
-        if (lane == 0) {
-            int slot = 0, issued = 0;
-            uint32_t phase = 1;                       // a fresh ring counts as empty
-            const unsigned char *src = a.head_img + (size_t)s_lo * KB * MMA_STAGE_BYTES;
-            for (int sl = s_lo; sl < s_hi && issued >= 0; ++sl)
-                for (int kb = 0; kb < KB; kb += KS) {
-                    if (!mm_wait(wempty0 + 8 * slot, phase, abort_flag, a.status, 1u)) { issued = ~issued; break; }
-                    const uint32_t bytes = (uint32_t)(min(KS, KB - kb) * (int)MMA_STAGE_BYTES);
-                    mm_bar_expect_tx(wfull0 + 8 * slot, bytes);
-                    mm_bulk_load(mm_smem(smem + (size_t)slot * KS * MMA_STAGE_BYTES), src, bytes, wfull0 + 8 * slot);
-                    src += bytes;
-                    ++issued;
-                    if (++slot == NS) { slot = 0; phase ^= 1; }
-                }
-            if (issued < 0) {        // gave up: let the copies in flight land before leaving
-                issued = ~issued;
-                for (int c = issued > NS ? issued - NS : 0; c < issued; ++c)
-                    for (uint32_t spin = 0; spin < MMA_WAIT_LIMIT; ++spin)
-                        if (mm_bar_try(wfull0 + 8 * (c % NS), (c / NS) & 1)) break;
+    int slot = 0, issued = 0;                             // ring of W stages: the producer's and the issuer's
+    uint32_t phase = warp == NTW ? 1u : 0u;               // (a fresh ring counts as empty)
+    bool ok = true;
+    for (;;) {
+        block_sync();
+        const int s_lo = (int)(item_slot[1] & 0xffffu), slabs = (int)(item_slot[1] >> 16) - s_lo;
+        if (item_slot[0] == ~0u) break;
+        mm_fence_before();
+        block_sync();
+        mm_fence_after();
+        if (warp == NTW) {
+            // ---------------- producer: the W stages of every slab, in order, through the ring
+            if (lane == 0 && ok) {
+                const unsigned char *src = a.head_img + (size_t)s_lo * KB * MMA_STAGE_BYTES;
+                for (int n = 0; n < slabs && ok; ++n)
+                    for (int kb = 0; kb < KB; kb += KS) {
+                        if (!mm_wait(wempty0 + 8 * slot, phase, abort_flag, a.status, 1u)) { ok = false; break; }
+                        const uint32_t bytes = (uint32_t)(min(KS, KB - kb) * (int)MMA_STAGE_BYTES);
+                        mm_bar_expect_tx(wfull0 + 8 * slot, bytes);
+                        mm_bulk_load(mm_smem(smem + (size_t)slot * KS * MMA_STAGE_BYTES), src, bytes, wfull0 + 8 * slot);
+                        src += bytes;
+                        ++issued;
+                        if (++slot == NS) { slot = 0; phase ^= 1; }
+                    }
             }
-        }
-        __syncwarp();
-    } else if (warp == NTW + 1) {
-        // ---------------- one elected thread issues every MMA: 32-bit sums, unsigned bytes, 128 x 128
-        const uint32_t idesc = (2u << 4) | (16u << 17) | (8u << 24);
-        const uint32_t ring = mm_smem(smem);
-        bool ok = true;
-        int slot = 0;
-        uint32_t phase = 0;
-        for (int n = 0; n < s_hi - s_lo && ok; ++n) {
-            const int buf = n & two;
-            if (n > two)
-                ok = __all_sync(0xffffffffu, mm_wait(tempty0 + 8 * buf, ((n >> two) - 1) & 1, abort_flag, a.status, 2u));
-            mm_fence_after();
-            for (int kb = 0; kb < KB && ok; kb += KS) {
-                ok = __all_sync(0xffffffffu, mm_wait(wfull0 + 8 * slot, phase, abort_flag, a.status, 4u));
-                if (!ok) break;
-                const uint32_t stage = ring + slot * (uint32_t)(KS * MMA_STAGE_BYTES);
+            __syncwarp();
+        } else if (warp == NTW + 1) {
+            // ---------------- one elected thread issues every MMA: 32-bit sums, unsigned bytes, 128 x 128
+            const uint32_t idesc = (2u << 4) | (16u << 17) | (8u << 24);
+            const uint32_t ring = mm_smem(smem);
+            for (int n = done; n < done + slabs && ok; ++n) {
+                const int buf = n & two;
+                if (n > two)
+                    ok = __all_sync(0xffffffffu, mm_wait(tempty0 + 8 * buf, ((n >> two) - 1) & 1, abort_flag, a.status, 2u));
+                mm_fence_after();
+                for (int kb = 0; kb < KB && ok; kb += KS) {
+                    ok = __all_sync(0xffffffffu, mm_wait(wfull0 + 8 * slot, phase, abort_flag, a.status, 4u));
+                    if (!ok) break;
+                    const uint32_t stage = ring + slot * (uint32_t)(KS * MMA_STAGE_BYTES);
 #pragma unroll
-                for (int x = 0; x < KS; ++x)
-                    if (kb + x < KB) {
+                    for (int x = 0; x < KS; ++x)
+                        if (kb + x < KB) {
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
+                            for (int u = 0; u < 4; ++u)
                                 mm_mma_i8_ts(tmem + buf * 128, tmem + x_col + (kb + x) * 32 + u * 8,
                                              mm_desc(stage + x * (uint32_t)MMA_STAGE_BYTES + u * 256, 128, 1024),
                                              idesc, (kb | x | u) != 0);
                         }
-                mm_commit_warp(wempty0 + 8 * slot);
-                if (++slot == NS) { slot = 0; phase ^= 1; }
+                    mm_commit_warp(wempty0 + 8 * slot);
+                    if (++slot == NS) { slot = 0; phase ^= 1; }
+                }
+                if (ok) mm_commit_warp(tfull0 + 8 * buf);
             }
-            if (ok) mm_commit_warp(tfull0 + 8 * buf);
         }
+        done += slabs;
+        mm_fence_before();
+        block_sync();
+        mm_fence_after();
+    }
+    if (warp == NTW && lane == 0 && !ok) {
+        // gave up: let the copies in flight land before leaving
+        for (int c = issued > NS ? issued - NS : 0; c < issued; ++c)
+            for (uint32_t spin = 0; spin < MMA_WAIT_LIMIT; ++spin)
+                if (mm_bar_try(wfull0 + 8 * (c % NS), (c / NS) & 1)) break;
+    }
+    if (warp == NTW + 1) {
         mm_commit_warp(drain);
         for (uint32_t spin = 0; spin < MMA_WAIT_LIMIT; ++spin)
             if (mm_bar_try(drain, 0)) break;
-        __syncwarp();
-    }   // (two warps only complete the control warpgroup)
+    }
+    __syncwarp();
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SC_TAIL_REGS));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SC_TAIL_REGS));
+    const int q = warp & 3, e = warp >> 2;
+    for (;;) {
+        // the next item (a block that gave up: let the grid drain)
+        if (threadIdx.x == 0) {
+            uint32_t set = ~0u, range = 0u, part = 0u;       // (no set: there are no more items)
+            if (*abort_flag || *reinterpret_cast<volatile uint32_t *>(a.status)) {
+            } else if (!ORDERED) {
+                // (as many tickets as items and one more for each block: then the counter is zero again)
+                const uint32_t items = (uint32_t)a.blocks * (uint32_t)a.splits, t = atomicInc(a.ticket, items + gridDim.x - 1u);
+                if (t < items) {
+                    set = t % (uint32_t)a.blocks;
+                    part = t / (uint32_t)a.blocks;
+                    range = (uint32_t)a.n_slabs * part / a.splits | (uint32_t)a.n_slabs * (part + 1) / a.splits << 16;
+                }
+            } else {
+                uint32_t t = atomicAdd(o.tickets + SC_PARTS, 1u);        // the lists one after the other
+                for (int c = 0; c < SC_PARTS; ++c) {
+                    const uint32_t n = __ldcg(o.tickets + c);
+                    if (t < n) {
+                        const uint2 item = __ldg(o.items + (size_t)c * a.blocks + t);
+                        set = item.x; range = item.y;
+                        break;
+                    }
+                    t -= n;
+                }
+            }
+            item_slot[0] = set; item_slot[1] = range; item_slot[2] = part;
+        }
+        block_sync();
+        if (item_slot[0] == ~0u) break;
+        const int64_t group = item_slot[0];
+        const int s_lo = (int)(item_slot[1] & 0xffffu), s_hi = (int)(item_slot[1] >> 16), slabs = s_hi - s_lo;
+        {
+            // X_head into tensor memory: lane 32q + l = document, a column = four features
+            const int words = a.head / 32;
+            const int64_t p = group * SC_DOCS + 32 * q + lane;
+            const bool there = p < a.n_tiles * 8;
+            for (int wd = e; wd < a.head_pad / 32; wd += 4) {
+                const uint32_t m = there && wd < words ? __ldg(a.tile_head + (size_t)p * words + wd) : 0u;
+                const uint4 k0 = __ldg(reinterpret_cast<const uint4 *>(a.kpack) + 2 * wd);
+                const uint4 k1 = __ldg(reinterpret_cast<const uint4 *>(a.kpack) + 2 * wd + 1);
+                const uint32_t k[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
+                uint32_t v[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c)          // four mask bits -> four byte masks
+                    v[c] = ((((m >> (4 * c)) & 15u) * 0x00204081u) & 0x01010101u) * 255u & k[c];
+                mm_tmem_st8(tmem + ((uint32_t)(q * 32) << 16) + x_col + wd * 8, v);
+            }
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        }
+        mm_fence_before();
+        block_sync();
+        mm_fence_after();
         // ---------------- tail: documents 32q + 8e .. + 7 of a block, one tile
-        const int q = warp & 3, e = warp >> 2;
         const int s = lane >> 3, hb = (lane >> 2) & 1, li = lane & 3;
-        // which half of an id word is this lane's own document (2s + hb), which its partner's
         const uint32_t sel_own = hb ? 0x4432u : 0x4410u, sel_other = hb ? 0x4410u : 0x4432u;
         const u64 sh = sc_pack(__ldg(a.scalars), __ldg(a.scalars)), st = sc_pack(__ldg(a.scalars + 1), __ldg(a.scalars + 1));
         const u64 minus_2p23 = sc_pack(-8388608.f, -8388608.f);
@@ -234,7 +283,6 @@ sweep_screen_kernel(const ScreenArgs a)
         const uint4 *ids = a.tile_ids;
         [[maybe_unused]] size_t room = a.tile_rows_cap;
         if (tile < a.n_tiles) {
-            // (longer lists than the sums hold are evaluated whole)
             const uint32_t rows = min(__ldg(a.tile_len + tile) & 0xffffu, (uint32_t)__ldg(a.scalars + 6));
             quads = (rows + 3) / 4;
             const uint32_t off = BMU_IDX(__ldg(a.tile_off + tile), a.tile_rows_cap, a.status);
@@ -243,23 +291,27 @@ sweep_screen_kernel(const ScreenArgs a)
         ids += s;
         const int64_t p = tile * 8 + (lane >> 2);                        // this lane's document
         const float win = __ldg(a.window + p);
-        float own = 3.0e38f, m1 = 3.0e38f, m2 = 3.0e38f;                 // the stripe's, the document's
-        if (!a.first) {
+        float m1 = 3.0e38f, m2 = 3.0e38f;                                // smallest (and second) value of the document
+        // ORDERED: how far it reaches (evaluated whole: not at all), and what bounds its smallest (second) value
+        [[maybe_unused]] float reach = -CUDART_INF_F, known = 0.f;
+        // otherwise the stripe's smallest value, and the mask: eight slabs a word, stored when full; what lies before
+        // slab `valid` does not count
+        [[maybe_unused]] float own = 3.0e38f;
+        [[maybe_unused]] uint32_t mask = 0u;
+        [[maybe_unused]] int valid = s_lo;
+        [[maybe_unused]] const size_t at = ((size_t)item_slot[2] * a.n_pad + p) * 4 + li;
+        if constexpr (ORDERED) {
+            const float2 r = __ldg(o.reach + p);
+            if (r.x <= __ldg(a.scalars + SC_TOP)) reach = r.y;
+            known = ordered_to_float(__ldcg(o.bound + p));
+            if (TOP2) m2 = known; else m1 = known;
+        } else if (!a.first) {
             m1 = __ldg(a.amin + p);
             if (TOP2) m2 = __ldg(a.amin2 + p);
         }
-        // the mask: eight slabs a word, stored when full; what lies before slab `valid` does not count
-        uint32_t mask = 0u;
-        int valid = s_lo;
-        const size_t at = ((size_t)blockIdx.y * a.n_pad + p) * 4 + li;
-        uint32_t *words_out = reinterpret_cast<uint32_t *>(a.cmask + at);
         const unsigned char *base = a.img8 + (size_t)s_lo * slab_bytes + (lane & 7) * 16;
         const float *np = a.normp + (size_t)s_lo * SC_SLAB + li * 4;
 
-        // The rows of all slabs form one stream: a quad of rows (four pieces of the own and four of
-        // the partner's document) is in flight all the time, each half of it replaced by the same
-        // half of the next quad as soon as it is added -- the first quad of the next slab at the
-        // end of one, so that its loads run under the epilogue.
         uint4 w[8], ix = make_uint4(0u, 0u, 0u, 0u);
         auto quad = [&](uint32_t h) { return __ldg(ids + BMU_IDX(4 * h, room - s, a.status)); };
         auto load = [&](const unsigned char *from, uint4 *d, uint32_t x0, uint32_t x1) {
@@ -277,14 +329,22 @@ sweep_screen_kernel(const ScreenArgs a)
             load(base, w + 4, i0.z, i0.w);
         }
         for (int sl = s_lo; sl < s_hi; ++sl, np += SC_SLAB) {
-            const int n = sl - s_lo;
+            const int n = done + sl - s_lo;
+            // no document of the tile reaches this slab, nor any behind it: the accumulators still change hands
+            if (ORDERED && !__any_sync(0xffffffffu, __ldg(o.unit_norm + sl * SC_SLAB) <= (TOP2 ? m2 : m1) + win + reach)) {
+                for (int r = n; r < done + slabs; ++r) {
+                    mm_wait(tfull0 + 8 * (r & two), (r >> two) & 1, abort_flag, a.status, 8u);
+                    __syncwarp();
+                    if (lane == 0) mm_bar_arrive(tempty0 + 8 * (r & two));
+                }
+                break;
+            }
             uint32_t acc[2][8];                       // own, other document
 #pragma unroll
             for (int t = 0; t < 2; ++t)
 #pragma unroll
                 for (int x = 0; x < 8; ++x) acc[t][x] = 0u;
             for (uint32_t h = 0; h < quads; ++h) {
-                // (the last quad of the last slab fetches rows that nobody adds)
                 if (h + 1 == quads && sl + 1 < s_hi) base += slab_bytes;
                 sc_add(acc[0], w[0], w[1]);
                 sc_add(acc[1], w[2], w[3]);
@@ -309,15 +369,13 @@ sweep_screen_kernel(const ScreenArgs a)
             mm_wait(tfull0 + 8 * (n & two), (n >> two) & 1, abort_flag, a.status, 8u);
             mm_fence_after();
             const uint32_t taddr = tmem + ((uint32_t)(q * 32 + (e >> 1) * 16) << 16) + (uint32_t)((n & two) * 128);
-            float mc[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {             // eight neurons of the lane's 32 at a time
+            auto dist8 = [&](int c, u64 x[4], auto last) {
                 uint32_t v[16];
                 mm_tmem_ld_16x256b_x4(taddr + c * 32, v);
                 const ulonglong2 n0 = __ldg(reinterpret_cast<const ulonglong2 *>(np + (2 * c) * 16));
                 const ulonglong2 n1 = __ldg(reinterpret_cast<const ulonglong2 *>(np + (2 * c + 1) * 16));
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (c == 3) {                         // the accumulator is free
+                if (decltype(last)::value && c == 3) {        // the accumulator is free
                     mm_fence_before();
                     __syncwarp();
                     if (lane == 0) mm_bar_arrive(tempty0 + 8 * (n & two));
@@ -330,16 +388,23 @@ sweep_screen_kernel(const ScreenArgs a)
                 }
                 const uint32_t *t = c < 2 ? lo : hi;
                 const int w0 = 2 * (c & 1);
-                const u64 x0 = sc_dist2(n0.x, hs[0], hs[1], t[w0], sh, st, minus_2p23);
-                const u64 x1 = sc_dist2(n0.y, hs[2], hs[3], t[4 + w0], sh, st, minus_2p23);
-                const u64 x2 = sc_dist2(n1.x, hs[4], hs[5], t[w0 + 1], sh, st, minus_2p23);
-                const u64 x3 = sc_dist2(n1.y, hs[6], hs[7], t[5 + w0], sh, st, minus_2p23);
-                mc[c] = fminf(fminf(fminf(lo_f(x0), hi_f(x0)), fminf(lo_f(x1), hi_f(x1))),
-                              fminf(fminf(lo_f(x2), hi_f(x2)), fminf(lo_f(x3), hi_f(x3))));
+                x[0] = sc_dist2(n0.x, hs[0], hs[1], t[w0], sh, st, minus_2p23);
+                x[1] = sc_dist2(n0.y, hs[2], hs[3], t[4 + w0], sh, st, minus_2p23);
+                x[2] = sc_dist2(n1.x, hs[4], hs[5], t[w0 + 1], sh, st, minus_2p23);
+                x[3] = sc_dist2(n1.y, hs[6], hs[7], t[5 + w0], sh, st, minus_2p23);
+            };
+            // the distances of eight neurons of the lane's 32 at a time, in pairs
+            float mc[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                u64 x[4];
+                dist8(c, x, std::integral_constant<bool, !ORDERED>());
+                mc[c] = fminf(fminf(fminf(lo_f(x[0]), hi_f(x[0])), fminf(lo_f(x[1]), hi_f(x[1]))),
+                              fminf(fminf(lo_f(x[2]), hi_f(x[2])), fminf(lo_f(x[3]), hi_f(x[3]))));
             }
             // the document's smallest (and second smallest) value over its four lanes
             const float m = fminf(fminf(mc[0], mc[1]), fminf(mc[2], mc[3]));
-            own = fminf(own, m);
+            if (!ORDERED) own = fminf(own, m);
             float g1 = m, g2 = CUDART_INF_F;
 #pragma unroll
             for (int x = 1; x < 4; x <<= 1) {
@@ -350,24 +415,55 @@ sweep_screen_kernel(const ScreenArgs a)
                 }
                 g1 = fminf(g1, o1);
             }
-            const float before = m1;
+            [[maybe_unused]] const float before = m1;
             if (TOP2) m2 = fminf(fminf(m2, g2), fmaxf(m1, g1));
             m1 = fminf(m1, g1);
             const float limit = (TOP2 ? m2 : m1) + win;
-            if (before > limit) { mask = 0u; valid = sl; own = m; }      // nothing before this slab can win
-            if (m <= limit)
-                mask |= ((mc[0] <= limit ? 1u : 0u) | (mc[1] <= limit ? 2u : 0u) | (mc[2] <= limit ? 4u : 0u) |
-                         (mc[3] <= limit ? 8u : 0u)) << (4 * (sl & 7));
-            if ((sl & 7) == 7 || sl + 1 == s_hi) {
-                words_out[sl >> 3] = mask;
-                mask = 0u;
+            if constexpr (!ORDERED) {
+                if (before > limit) { mask = 0u; valid = sl; own = m; }      // nothing before this slab can win
+                if (m <= limit)
+                    mask |= ((mc[0] <= limit ? 1u : 0u) | (mc[1] <= limit ? 2u : 0u) | (mc[2] <= limit ? 4u : 0u) |
+                             (mc[3] <= limit ? 8u : 0u)) << (4 * (sl & 7));
+                if ((sl & 7) == 7 || sl + 1 == s_hi) {
+                    reinterpret_cast<uint32_t *>(a.cmask + at)[sl >> 3] = mask;
+                    mask = 0u;
+                }
+                continue;
             }
+            // some unit of the warp's is within a window: which ones, from the sums once more
+            if (__any_sync(0xffffffffu, m <= limit)) {
+                uint32_t bits = 0u;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    u64 x[4];
+                    dist8(c, x, std::false_type());
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        bits |= ((lo_f(x[i]) <= limit ? 1u : 0u) | (hi_f(x[i]) <= limit ? 2u : 0u)) << (8 * c + 2 * i);
+                }
+                if (bits) {
+                    const uint32_t n_at = atomicAdd(o.count + p, 1u);
+                    if (n_at < (uint32_t)SC_OWN_LIST)
+                        o.list[p * SC_OWN_LIST + n_at] = make_uint4(__float_as_uint(m), (uint32_t)(o.slab0 + sl), bits, (uint32_t)li);
+                }
+            }
+            mm_fence_before();                        // the accumulator is free
+            __syncwarp();
+            if (lane == 0) mm_bar_arrive(tempty0 + 8 * (n & two));
         }
-        a.cval[at] = make_float2(own, __int_as_float(valid | (s_hi << 8)));
-        if (TOP2) a.cval2[at] = m2;
-        __syncwarp();
+        if constexpr (ORDERED) {
+            const float found = TOP2 ? m2 : m1;
+            if (li == 0 && found < known) atomicMin(o.bound + p, float_to_ordered(found));
+        } else {
+            a.cval[at] = make_float2(own, __int_as_float(valid | (s_hi << 8)));
+            if (TOP2) a.cval2[at] = m2;
+        }
+        done += slabs;
+        mm_fence_before();
+        block_sync();
+        mm_fence_after();
     }
-
+    }
     mm_fence_before();
     __syncthreads();
     mm_fence_after();
@@ -403,35 +499,38 @@ int screen_splits(int64_t blocks, int64_t n_slabs, int sms)
     return best;
 }
 
-int launch_sweep_screen(const ScreenArgs &a, bool top2, cudaStream_t s)
+template <bool TOP2, bool ORDERED>
+static int launch_sweep(const ScreenArgs &a, const OrderedArgs &o, int sms, cudaStream_t s)
+{
+    static bool configured[64];
+    int dev = 0;
+    BMU_CUDA(cudaGetDevice(&dev));
+    if (dev >= 0 && dev < 64 && !configured[dev]) {
+        // refuse a build whose launch registers do not cover the hand-over inside the kernel
+        cudaFuncAttributes f;
+        BMU_CUDA(cudaFuncGetAttributes(&f, sweep_screen_kernel<TOP2, ORDERED>));
+        if (SC_THREADS * f.numRegs < 128 * SC_CTRL_REGS + 32 * SC_TAIL_WARPS * SC_TAIL_REGS) {
+            set_error("screening sweep: built with %d registers per thread, too few for the hand-over", f.numRegs);
+            return BMU_ERR_UNSUPPORTED;
+        }
+        BMU_CUDA(cudaFuncSetAttribute(sweep_screen_kernel<TOP2, ORDERED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SC_SMEM));
+        configured[dev] = true;
+    }
+    const int64_t items = (int64_t)a.blocks * (ORDERED ? SC_PARTS : a.splits);
+    { sweep_screen_kernel<TOP2, ORDERED><<<(unsigned)(items < sms ? items : sms), SC_THREADS, SC_SMEM, s>>>(a, o); BMU_LAUNCHED(); }
+    BMU_CUDA(cudaGetLastError());
+    return BMU_OK;
+}
+
+int launch_sweep_screen(const ScreenArgs &a, const OrderedArgs &o, bool top2, bool ordered, int sms, cudaStream_t s)
 {
     if (a.n_slabs <= 0 || a.blocks <= 0) return BMU_OK;
     if (a.n_slabs > SC_MAX_SLABS || a.head_pad > SC_MAX_HEAD) {
         set_error("screening sweep: at most %d slabs per launch and %d head rows", SC_MAX_SLABS, SC_MAX_HEAD);
         return BMU_ERR_INVALID_ARG;
     }
-    static bool configured[64];
-    int dev = 0;
-    BMU_CUDA(cudaGetDevice(&dev));
-    if (dev >= 0 && dev < 64 && !configured[dev]) {
-        // refuse a build whose launch registers do not cover the hand-over inside the kernel
-        cudaFuncAttributes fa, fb;
-        BMU_CUDA(cudaFuncGetAttributes(&fa, sweep_screen_kernel<false>));
-        BMU_CUDA(cudaFuncGetAttributes(&fb, sweep_screen_kernel<true>));
-        const int regs = fa.numRegs < fb.numRegs ? fa.numRegs : fb.numRegs;
-        if (SC_THREADS * regs < 128 * SC_CTRL_REGS + 32 * SC_TAIL_WARPS * SC_TAIL_REGS) {
-            set_error("screening sweep: built with %d registers per thread, too few for the hand-over", regs);
-            return BMU_ERR_UNSUPPORTED;
-        }
-        BMU_CUDA(cudaFuncSetAttribute(sweep_screen_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SC_SMEM));
-        BMU_CUDA(cudaFuncSetAttribute(sweep_screen_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SC_SMEM));
-        configured[dev] = true;
-    }
-    const dim3 grid((unsigned)a.blocks, (unsigned)a.splits);
-    if (top2) { sweep_screen_kernel<true><<<grid, SC_THREADS, SC_SMEM, s>>>(a); BMU_LAUNCHED(); }
-    else { sweep_screen_kernel<false><<<grid, SC_THREADS, SC_SMEM, s>>>(a); BMU_LAUNCHED(); }
-    BMU_CUDA(cudaGetLastError());
-    return BMU_OK;
+    if (ordered) return top2 ? launch_sweep<true, true>(a, o, sms, s) : launch_sweep<false, true>(a, o, sms, s);
+    return top2 ? launch_sweep<true, false>(a, o, sms, s) : launch_sweep<false, false>(a, o, sms, s);
 }
 
 }  // namespace bmu

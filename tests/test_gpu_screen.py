@@ -358,3 +358,96 @@ def test_batches_share_the_images_of_the_codebook(bmu):
         assert rp.numel() < 1000 or bmu.bmu_describe_search(D, M, rp.numel() - 1, ci.numel()).two_stage
         rb, rd = bmu.bmu_search(W, rp.cuda(), ci.cuda())
         assert torch.equal(rb.cpu(), ob) and torch.equal(rd.cpu(), od)
+
+
+def lists(lens, D, seed):
+    r = np.random.default_rng(seed)
+    rows = [np.sort(r.permutation(D)[:n]) for n in lens]
+    rowptr = torch.zeros(len(rows) + 1, dtype=torch.int32)
+    rowptr[1:] = torch.cumsum(torch.tensor([len(x) for x in rows]), 0)
+    return rowptr, torch.from_numpy(np.concatenate(rows).astype(np.int32))
+
+
+@pytest.mark.parametrize("M,chunk", [(1024, 0), (1027, 256), (2304, 1024), (5000, 512)])
+@pytest.mark.parametrize("n_docs", [1, 129, 700])
+def test_slabs_in_the_order_of_the_norms(bmu, M, chunk, n_docs):
+    """Norms that spread further than a document reaches: short lists on an iid U[0,1) codebook.  Some lists are
+    empty, some reach half of the map, one all of it; best and second-best unit, half precision, a plan."""
+    D = 4096
+    r = np.random.default_rng(M + n_docs)
+    lens = r.integers(0, 24, n_docs)
+    lens[::50] = 60
+    if n_docs > 300:
+        lens[300] = 900
+    rowptr, colidx = lists(lens, D, M)
+    W = torch.rand((D, M), generator=torch.Generator().manual_seed(M)).half().float()
+    ob, od = check(bmu, W, rowptr, colidx, chunk_neurons=chunk)
+    Wd, rp, ci, o = W.cuda(), rowptr.cuda(), colidx.cuda(), opts_of(bmu, chunk_neurons=chunk)
+    b1, d1, b2, d2 = bmu.bmu_search_top2_ws(Wd, rp, ci, opts=o)
+    assert torch.equal(b1, ob)
+    np.testing.assert_allclose(d2.cpu().numpy(), oracle.bmu2(W.numpy(), rowptr.numpy(), colidx.numpy())[3], rtol=1e-6)
+    assert bool((b2 != b1).all())
+    plan = bmu.Plan(rp, ci, D, M, o) if M % 4 == 0 else None
+    if plan:
+        pb, pd = plan.search(Wd)
+        plan.close()
+        assert torch.equal(pb, ob) and torch.equal(pd, od)
+    if M % 256 == 0:
+        hb, hd = bmu.bmu_search_f16_ws(Wd.half(), rp, ci, opts=o)[:2]
+        assert torch.equal(hb, ob) and torch.equal(hd, od)
+
+
+@pytest.mark.parametrize("copies", [2, 40, 1500])
+def test_equal_units_in_the_order_of_the_norms(bmu, copies):
+    """The unit of the smallest norm many times over the map: the lowest index wins, the next one is second; 1,500
+    of them are more than a document's list holds."""
+    D, M = 4096, 4096
+    rowptr, colidx = lists(np.random.default_rng(3).integers(0, 24, 300), D, 4)
+    W = torch.rand((D, M), generator=torch.Generator().manual_seed(5))
+    W[:, 7] = 0.98 * W[:, int((W ** 2).sum(0).argmin())]
+    where = 7 + (4000 // copies) * torch.arange(copies)
+    W[:, where] = W[:, 7:8]
+    check(bmu, W, rowptr, colidx)
+    b1, d1, b2, d2 = bmu.bmu_search_top2_ws(W.cuda(), rowptr.cuda(), colidx.cuda(), opts=opts_of(bmu))
+    assert bool((b1 == 7).all()) and bool((b2 == int(where[1])).all())
+    assert torch.equal(d1, d2)
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan")])
+def test_norms_that_have_no_place_in_an_order(bmu, value):
+    """A unit at plus infinity or without a number as its norm never wins; at minus infinity it always does."""
+    D, M = 4096, 2048
+    rowptr, colidx = lists(np.random.default_rng(6).integers(1, 24, 200), D, 7)
+    W = torch.rand((D, M), generator=torch.Generator().manual_seed(8))
+    Wd, rp, ci = W.cuda(), rowptr.cuda(), colidx.cuda()
+    norms = bmu.bmu_codebook_norms(Wd)
+    far = int(norms.argmin())
+    norms[far] = value
+    ob, od = bmu.bmu_search_ws(Wd, rp, ci, norms=norms, opts=opts_of(bmu))
+    if value < 0:
+        assert bool((ob == far).all()) and bool(torch.isinf(od).all())
+    else:
+        keep = [j for j in range(M) if j != far]
+        rb, rd = bmu.bmu_search_ws(Wd[:, keep].contiguous(), rp, ci, opts=opts_of(bmu))
+        assert torch.equal(ob, rb + (rb >= far).int())
+        assert bool(((od - rd).abs() <= 1e-5 * rd.abs()).all())
+
+
+def test_batches_that_reach_further_than_the_first(bmu):
+    """Batches share order and images: one whose lists reach further than the first one's, one of long lists only,
+    which needs the slabs in the order of the map, and a short one again."""
+    D, M = 4096, 4096
+    W = torch.rand((D, M), generator=torch.Generator().manual_seed(9)).cuda()
+    r = np.random.default_rng(10)
+    batches = [lists(lens, D, 11 + i) for i, lens in enumerate((r.integers(0, 16, 3000), r.integers(10, 50, 3000),
+                                                                 r.integers(200, 500, 2000), r.integers(0, 16, 3000)))]
+    outs = [(torch.empty(rp.numel() - 1, dtype=torch.int32).pin_memory(),
+             torch.empty(rp.numel() - 1, dtype=torch.float32).pin_memory()) for rp, _ in batches]
+    bmu.bmu_search_batches_host(W, [(rp.pin_memory(), ci.pin_memory()) for rp, ci in batches], outs)
+    single = bmu.Opts()
+    single.two_stage = 2
+    for (rp, ci), (ob, od) in zip(batches, outs):
+        rb, rd = bmu.bmu_search_ws(W, rp.cuda(), ci.cuda(), opts=single)
+        parity.compare(ob.numpy(), od.numpy(), W.cpu().numpy(), rp.numpy(), ci.numpy(), docs=np.arange(0, 2000, 97))
+        assert float((ob == rb.cpu()).float().mean()) > 0.999
+        assert bool(((od - rd.cpu()).abs() <= 1e-5 * rd.cpu().abs()).all())
