@@ -34,7 +34,7 @@ static const int64_t MAX_I32 = 0x7fffffff;
 
 // ---- workspace layout -----------------------------------------------------
 struct Layout {
-    size_t status_off, count_off, tickets_off, slots_off, norms_off, state_off, state2_off, head_off, repack_off, screen_off, plan_off, total;
+    size_t status_off, count_off, sets_off, tickets_off, slots_off, norms_off, state_off, state2_off, head_off, repack_off, screen_off, plan_off, total;
     PlanLayout plan;
     ScreenLayout screen;
 };
@@ -130,6 +130,8 @@ static Layout layout_for(int64_t D, int64_t M, int64_t N, int64_t nnz, int kerne
     if (screen_chunk) off = align_up((size_t)STATUS_WORDS * 4, 256);
     l.count_off = off;                   // (the features' counters, cleared with the status word)
     if (screen_chunk) off = align_up(off + (size_t)D * sizeof(uint32_t), 256);
+    l.sets_off = off;                    // (how far each set of documents reaches, cleared too)
+    if (screen_chunk) off = align_up(off + (size_t)((N + SC_DOCS - 1) / SC_DOCS) * sizeof(uint32_t), 256);
     l.tickets_off = l.slots_off = off;
     if (few) {                           // (the tickets behind the status word: cleared with it)
         off = align_up(off + (size_t)N * sizeof(uint32_t), 256);
@@ -483,6 +485,7 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
         if (shared->used) earlier = scalars + (shared->used - 1) % 2 * SC_SCALARS;
         scalars += shared->used++ % 2 * SC_SCALARS;
     }
+    uint32_t *set_reach = reinterpret_cast<uint32_t *>(base + l.sets_off);
     ScreenArgs a;
     a.tile_len = reinterpret_cast<const uint32_t *>(pw + l.plan.tilelen_off);
     a.tile_off = reinterpret_cast<const uint32_t *>(pw + l.plan.tileoff_off);
@@ -494,13 +497,17 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
                                    reinterpret_cast<float *>(sb + l.screen.window),
                                    reinterpret_cast<float2 *>(sb + l.screen.reach),
                                    reinterpret_cast<uint32_t *>(sb + l.screen.amin),
-                                   reinterpret_cast<uint32_t *>(sb + l.screen.lcount), l.screen.n_pad, top2, status, s);
+                                   reinterpret_cast<uint32_t *>(sb + l.screen.lcount), set_reach, l.screen.n_pad, top2,
+                                   status, s);
     if (rc) return rc;
     const int64_t slabs = (M + SC_SLAB - 1) / SC_SLAB;
     const int64_t launches = (slabs + l.screen.chunk_slabs - 1) / l.screen.chunk_slabs;
-    const bool order = M >= SC_ORDER_MIN && launches <= SC_MAX_LAUNCHES;
-    if (order && (rc = launch_screen_order(norms, D, M, N, launches, cb, cl, scalars, earlier, shared != nullptr, status,
-                                           reinterpret_cast<uint32_t *>(sb + l.screen.tickets), s)))
+    uint32_t *tickets = reinterpret_cast<uint32_t *>(sb + l.screen.tickets);
+    uint32_t *nat_list = reinterpret_cast<uint32_t *>(sb + l.screen.nat_list);
+    const int sets = (int)(l.screen.n_pad / SC_DOCS);
+    const int64_t ord_launches = M >= SC_ORDER_MIN ? cl.ord_launches : 0;
+    if (ord_launches && (rc = launch_screen_order(norms, D, M, N, launches, cb, cl, scalars, earlier, status, set_reach, sets,
+                                                  tickets, nat_list, s)))
         return rc;
     a.kpack = reinterpret_cast<const uint32_t *>(cb + cl.kpack);
     a.scalars = scalars;
@@ -511,7 +518,7 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
     a.status = status; a.ticket = status + STATUS_SWEEP_TICKET;
     a.D = D; a.n_tiles = (N + 7) / 8; a.n_pad = l.screen.n_pad; a.tile_rows_cap = l.plan.tile_rows_cap;
     a.head = head; a.head_pad = l.screen.head_pad;
-    a.splits = l.screen.splits; a.blocks = (int32_t)(l.screen.n_pad / SC_DOCS);
+    a.splits = l.screen.splits; a.most_splits = l.screen.most_splits; a.blocks = sets; a.nat_list = nat_list;
     VerifyArgs v;
     v.W = W; v.f16 = f16; v.D = D; v.M = M; v.N = N; v.n_pad = a.n_pad; v.norms = norms;
     v.rowptr = rowptr; v.colidx = colidx; v.perm = perm; v.window = a.window;
@@ -519,22 +526,21 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
     v.amin = reinterpret_cast<float *>(sb + l.screen.amin);
     v.amin2 = reinterpret_cast<float *>(sb + l.screen.amin2);
     v.lcount = reinterpret_cast<uint32_t *>(sb + l.screen.lcount);
-    v.lval = reinterpret_cast<float *>(sb + l.screen.lval);
-    v.lmask = reinterpret_cast<uint4 *>(sb + l.screen.lmask);
-    v.lbase = reinterpret_cast<uint32_t *>(sb + l.screen.lbase);
-    v.state = state; v.state2 = state2; v.status = status; v.splits = a.splits;
+    v.lists = sb + l.screen.lists;
+    v.state = state; v.state2 = state2; v.status = status; v.splits = a.splits; v.most_splits = a.most_splits;
     v.out_bmu = out_bmu; v.out_dist = out_dist; v.out_bmu2 = out_bmu2; v.out_dist2 = out_dist2;
     // ... and with slabs in the order of the norms, in the same room
     OrderedArgs o;
-    v.reach = o.reach = reinterpret_cast<const float2 *>(sb + l.screen.reach);
+    o.reach = reinterpret_cast<const float2 *>(sb + l.screen.reach);
+    v.set_reach = set_reach; v.reach = o.reach;
     v.bound = o.bound = reinterpret_cast<uint32_t *>(sb + l.screen.amin);
-    v.own_list = o.list = reinterpret_cast<uint4 *>(sb + l.screen.lval);
+    o.lists = v.lists;
     o.count = v.lcount;
     o.items = reinterpret_cast<const uint2 *>(sb + l.screen.items);
     v.units = reinterpret_cast<const int32_t *>(cb + cl.units);
-    ImageArgs g;
-    g.launches = launches; g.head = head; g.sets = a.blocks; g.expected = earlier != nullptr;
-    g.reach = o.reach; g.window = a.window; g.bound = o.bound;
+    OrderedImages g;
+    g.head = head; g.sets = sets;
+    g.set_reach = set_reach; g.reach = o.reach; g.window = a.window; g.bound = o.bound;
     g.items = reinterpret_cast<uint2 *>(sb + l.screen.items);
     v.dense = reinterpret_cast<uint32_t *>(sb + l.screen.cval);         // (after the last launch)
     v.dense_count = status + STATUS_DENSE;
@@ -543,11 +549,9 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
     // the slabs are dealt to the launches in turn, so that every launch sees the whole map: after
     // the first one a document's smallest value is near its final one and little joins its list
     // (two neighbouring slabs at a time: 134 us instead of 17 for collecting on a trained 75 x 75 map)
-    // (in the order of the norms: to one after the other)
     v.launches = launches;
     const int sms = device_sms();
-    int64_t slab0 = 0;
-    for (int64_t k = 0; k < launches; ++k, slab0 += a.n_slabs) {
+    for (int64_t k = 0; k < launches; ++k) {
         a.n_slabs = (int32_t)((slabs - k + launches - 1) / launches);
         a.first = v.first = k == 0;
         v.launch = k;
@@ -555,16 +559,28 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
         a.img8 = reinterpret_cast<const unsigned char *>(cb + cl.img8) + (size_t)slot * (D + 1) * SC_SLAB;
         a.head_img = reinterpret_cast<const unsigned char *>(cb + cl.head_img) + (size_t)slot * cl.head_pad * SC_SLAB;
         a.normp = reinterpret_cast<const float *>(cb + cl.normp) + slot * SC_SLAB;
-        g.k = k; g.n_slabs = a.n_slabs; g.slab0 = slab0; g.slot = slot; g.first = k == 0;
-        o.tickets = g.tickets = reinterpret_cast<uint32_t *>(sb + l.screen.tickets) + k * (SC_PARTS + 1);
-        o.slab0 = slab0;
-        o.unit_norm = reinterpret_cast<const float *>(cb + cl.unit_norm) + slab0 * SC_SLAB;
-        if ((rc = launch_screen_quantize(W, f16, D, M, norms, g, feat, cb, cl, scalars, s))) return rc;
+        if ((rc = launch_screen_quantize(W, f16, D, M, norms, k, launches, a.n_slabs, slot, head, feat, cb, cl,
+                                         scalars, earlier != nullptr, s)))
+            return rc;
         if ((rc = launch_sweep_screen(a, o, top2, false, sms, s))) return rc;
-        if (order && (rc = launch_sweep_screen(a, o, top2, true, sms, s))) return rc;
-        if ((rc = launch_screen_collect(v, top2, sms, s))) return rc;
+        if ((rc = launch_screen_collect(v, top2, s))) return rc;
+    }
+    // ... and those in the order of the norms, to one launch after the other
+    int64_t slab0 = 0;
+    for (int64_t k = 0; k < ord_launches; ++k, slab0 += a.n_slabs) {
+        a.n_slabs = (int32_t)((slabs - k + launches - 1) / launches);
+        const int64_t slot = shared ? k * cl.chunk_slabs : 0;
+        a.img8 = reinterpret_cast<const unsigned char *>(cb + cl.ord8) + (size_t)slot * (D + 1) * SC_SLAB;
+        a.head_img = reinterpret_cast<const unsigned char *>(cb + cl.ord_head) + (size_t)slot * cl.head_pad * SC_SLAB;
+        a.normp = reinterpret_cast<const float *>(cb + cl.ord_normp) + slot * SC_SLAB;
+        g.n_slabs = a.n_slabs; g.slab0 = o.slab0 = slab0; g.slot = slot; g.first = k == 0;
+        o.tickets = g.tickets = tickets + k * (SC_PARTS + 1);
+        o.unit_norm = reinterpret_cast<const float *>(cb + cl.unit_norm) + slab0 * SC_SLAB;
+        if ((rc = launch_screen_ordered_images(W, f16, D, M, g, feat, cb, cl, scalars, sms, s))) return rc;
+        if ((rc = launch_sweep_screen(a, o, top2, true, sms, s))) return rc;
     }
     if ((rc = launch_screen_verify(v, top2, s))) return rc;
+    if (ord_launches && (rc = launch_screen_verify_units(v, top2, sms, s))) return rc;
     return launch_screen_dense(v, top2, sms, s);
 }
 

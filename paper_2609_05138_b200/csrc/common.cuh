@@ -197,10 +197,10 @@ static const int TILE_HEAD_ROWS = 32;    // ids below this are swept densely, on
 static const int HEAD_ROWS_MAX = 2048;   // widest dense head (the tensor-core sweep's)
 // words behind the status word, zero when a search begins: the longest list, the tiles' cursor and the
 // ticket of the two-stage tiling pass; its documents to be evaluated whole; the sweep's ticket; the codebook's
-// maxima, eight copies each (screen_range_kernel).  From STATUS_REFS on only a two-stage search has room: the smallest norms at
-// even and at odd units, eight 64-bit words each; documents by how far they reach
-static const int STATUS_PLAN_MOST = 35, STATUS_TILE_CURSOR = 36, STATUS_KEY_TICKET = 37, STATUS_DENSE = 38, STATUS_SWEEP_TICKET = 39,
-                 STATUS_MAXIMA = 40, STATUS_REFS = 64, STATUS_REACH = 128, STATUS_WORDS = 128 + 4096;
+// maxima, eight copies each (screen_range_kernel).  From STATUS_REFS on only a two-stage search has room: the smallest norms
+// at even and at odd units, eight 64-bit words each; documents by how far they reach (SC_BINS)
+static const int STATUS_PLAN_MOST = 35, STATUS_TILE_CURSOR = 36, STATUS_KEY_TICKET = 37, STATUS_DENSE = 38,
+                 STATUS_SWEEP_TICKET = 39, STATUS_MAXIMA = 40, STATUS_REFS = 64, STATUS_REACH = 128, STATUS_WORDS = 128 + 4096;
 // status-word bit set when a scanned offset of the tiling pass exceeds its reserved room
 static const uint32_t PLAN_STATUS_OVERFLOW = 64u;
 int launch_plan_tiles(const int32_t *rowptr, int64_t N, int interleave, int head, int relabel,

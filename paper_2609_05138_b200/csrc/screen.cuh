@@ -29,7 +29,8 @@
 // than that -- a codebook as it is first filled: 16,384 iid U[0,1) weights have norms of 5461 +- 38, a document of 80
 // ids a 2 R of 160, of which the winner's own sum uses up half -- the slabs are made of units in the order of
 // their norms, every document stops at the first slab beyond its reach, and most of the map is never summed (all
-// but 12 % on 64 x 64, all but 4 % on 128 x 128).  Otherwise the slabs follow the map.
+// but 12 % on 64 x 64, all but 4 % on 128 x 128).  Otherwise the slabs follow the map.  Both may be swept, one for
+// the sets of 128 documents that reach a little, the other for those that reach far.
 #pragma once
 
 #include "common.cuh"
@@ -42,15 +43,19 @@ static const int SC_DOCS = 128;          // documents per block
 static const int SC_MAX_HEAD = 1536;     // X_head in tensor memory: one column per four features
 static const int SC_MAX_SLABS = 32;      // per launch: four bits each in a stripe's group mask
 static const int SC_K_MAX = 32;          // largest integer row scale of a head feature
-// -2 d_head, -2 d_tail, 1 / d_tail, unused, q_max, max |norm|, 65535 / q_max (the longest list that is
+// -2 d_head, -2 d_tail, 1 / d_tail, whether the codes are an earlier search's, q_max, max |norm|, 65535 / q_max (the longest list that is
 // screened), whether the images have to be made, largest range of the head rows and of the others
 // ... and, as integers, how many of the sampled documents are to be evaluated whole, and how many were sampled;
-// whether the slabs are in the order of the norms, how many of them any document needs, up to which norm units are
-// in order (documents that reach further are evaluated whole); the two units whose distances bound a document's
+// whether slabs are swept in the order of the norms, how many of them have an image, up to which norm units are in
+// order, and how far a set of documents may reach to be swept so; the two units whose distances bound a document's
 // smallest value (the smallest norms at even and at odd indices); whether the images of the slabs in that order
-// stand from an earlier search, and how many units are in order
-static const int SC_VOTES = 10, SC_SAMPLED = 11, SC_ORDERED = 12, SC_NEEDED = 13, SC_TOP = 15,
-                 SC_REF = 16, SC_STAND = 18, SC_KEPT = 19, SC_SAMPLE = 16, SC_SCALARS = 32;
+// stand from an earlier search, and how many units are in order; the two units' norms; how many sets of documents
+// are swept in the order of the map (SC_ALL: each of them), and whether the images in that order are or will be made;
+// how far a document may reach not to be evaluated whole
+static const int SC_VOTES = 10, SC_SAMPLED = 11, SC_ORDERED = 12, SC_NEEDED = 13, SC_SORTED = 14, SC_TOP = 15,
+                 SC_REF = 16, SC_STAND = 18, SC_KEPT = 19, SC_REFN = 20, SC_NAT = 22, SC_NATMADE = 23, SC_DOC_TOP = 24, SC_SAMPLE = 16,
+                 SC_SCALARS = 32;
+static const uint32_t SC_ALL = ~0u;
 // Below this many units slabs always follow the map: too few for an order to spare many
 static const int64_t SC_ORDER_MIN = 1024;
 // Candidates wait in a list per document until every unit has been screened: a launch's local
@@ -59,6 +64,8 @@ static const int SC_LIST = 12;           // entries: smallest value, group mask,
 // ... where slabs are in the order of the norms, in the same room: smallest value, slab, which of the 32 units of a
 // lane, the lane
 static const int SC_OWN_LIST = 16;
+static const size_t SC_LIST_BYTES = (size_t)SC_LIST * 24;                 // masks, values, groups
+static_assert(SC_OWN_LIST * 16 <= SC_LIST * 24 && SC_LIST * 24 % 16 == 0, "one list per document");
 // A block of that sweep takes up to this many slabs of a launch for a set of documents; sets and parts wait in lists
 static const int SC_PART = 8, SC_PARTS = SC_MAX_SLABS / SC_PART;
 // Documents and units are counted by how far they reach, in this many steps
@@ -69,12 +76,14 @@ static const uint32_t SC_DENSE = 1u << 30;           // in a document's count: t
 // Device arrays of one search: offsets into the workspace, relative to its screen part.
 struct ScreenLayout {
     size_t scalars, rmin, rmax, table, kpack, khead, sample, window, amin, amin2;
-    size_t cval, cval2, cmask, lcount, lval, lmask, lbase, img8, head_img, normp, total;
-    size_t units, unit_norm, unit_tmp, rank_of, picks, reach, items, tickets;        // of slabs in the order of the norms
+    size_t cval, cval2, cmask, lcount, lists, img8, head_img, normp, total;
+    // of slabs in the order of the norms
+    size_t units, unit_norm, unit_tmp, rank_of, picks, ord8, ord_head, ord_normp, reach, items, tickets, nat_list;
+    int64_t ord_launches;                // how many launches may sweep them
     int64_t n_pad;                       // documents rounded up to whole blocks
     int head_pad;                        // head rows rounded up to a stage (128)
     int64_t chunk_slabs;                 // slabs of the largest launch
-    int splits;                          // blocks that share a launch's slabs
+    int splits, most_splits;             // blocks that share a launch's slabs for a set of documents; room for so many
     size_t rank, feat;                   // only in a ScreenShared
 };
 
@@ -103,9 +112,10 @@ struct ScreenArgs {
     float *cval2;                        // second smallest value of the document
     uint4 *cmask;                        // the stripe's 8-neuron groups within the window: bit 4 s + c
     uint32_t *status, *ticket;           // of the next item, zero
+    const uint32_t *nat_list;            // sets of documents, if not all
     int64_t D, n_tiles, n_pad;
     size_t tile_rows_cap;
-    int32_t head, head_pad, n_slabs, splits, blocks, first;
+    int32_t head, head_pad, n_slabs, splits, most_splits, blocks, first;
 };
 
 // The same search with slabs in the order of the norms
@@ -115,7 +125,7 @@ struct OrderedArgs {
     const float *unit_norm;              // norms in ascending order, from the launch's first slab on
     const uint2 *items;                  // [SC_PARTS][blocks]: set of documents, first slab | last << 16
     uint32_t *tickets;                   // SC_PARTS lengths of these lists, and the next to be taken
-    uint4 *list;                         // [n_pad][SC_OWN_LIST]
+    char *lists;                         // a document's SC_OWN_LIST entries, SC_LIST_BYTES apart
     uint32_t *count;
     int64_t slab0;                       // the launch's first slab in that order
 };
@@ -132,10 +142,8 @@ struct VerifyArgs {
     float *amin, *amin2;                 // smallest (second) approximate value so far
     uint32_t *lcount;                    // bits 0 .. 3: entries of the list; 4 .. 29: groups evaluated already;
                                          // 30: to be evaluated whole; 31: state[] holds exact keys
-    float *lval;
-    uint4 *lmask;
-    uint32_t *lbase;
-    const uint4 *own_list;               // slabs in the order of the norms
+    char *lists;
+    const uint32_t *set_reach;           // how far each set of documents reaches, as float_to_ordered
     const float2 *reach;
     const uint32_t *bound;
     const int32_t *units;
@@ -146,7 +154,7 @@ struct VerifyArgs {
     float *out_dist, *out_dist2;
     uint32_t *status;
     int64_t launch, launches;            // slab s of the launch is launch + s * launches of the map
-    int32_t splits, first, f16;
+    int32_t splits, most_splits, first, f16;
 };
 
 #ifdef __CUDACC__
@@ -156,9 +164,23 @@ __device__ __forceinline__ bool screen_whole(const float *scalars)
     const uint32_t *s = reinterpret_cast<const uint32_t *>(scalars);
     return 2u * __ldg(s + SC_VOTES) > __ldg(s + SC_SAMPLED);
 }
-__device__ __forceinline__ bool screen_ordered(const float *scalars)
+__device__ __forceinline__ bool screen_ordered(const float *scalars)         // some sets are
 {
     return __ldg(reinterpret_cast<const uint32_t *>(scalars) + SC_ORDERED) != 0u;
+}
+__device__ __forceinline__ uint32_t screen_natural(const float *scalars)      // how many sets are not
+{
+    return __ldg(reinterpret_cast<const uint32_t *>(scalars) + SC_NAT);
+}
+// ... and how many parts a launch's slabs are cut into for each: more than `splits` where they are few
+__device__ __forceinline__ int screen_parts(const float *scalars, int splits, int most)
+{
+    const uint32_t n = screen_natural(scalars);
+    return n == SC_ALL || n == 0u ? splits : (int)min((uint32_t)most, max((uint32_t)splits, 512u / n));
+}
+__device__ __forceinline__ bool screen_by_norm(const float *scalars, const uint32_t *set_reach, int64_t p)
+{
+    return screen_ordered(scalars) && ordered_to_float(__ldg(set_reach + p / SC_DOCS)) <= __ldg(scalars + SC_TOP);
 }
 // Steps between the smallest norm and the largest
 struct ScreenSteps {
@@ -167,14 +189,8 @@ struct ScreenSteps {
     {
         scale = top > lo ? (float)SC_BINS / (top - lo) : 0.f;
     }
-    __device__ __forceinline__ ScreenSteps(const float *scalars, const float *norms)
-        : ScreenSteps(least_of(scalars, norms), scalars[5]) {}
-    static __device__ __forceinline__ float least_of(const float *scalars, const float *norms)
-    {
-        const int32_t a = __float_as_int(scalars[SC_REF]), b = __float_as_int(scalars[SC_REF + 1]);
-        const float inf = __int_as_float(0x7f800000);
-        return fminf(a < 0 ? inf : __ldg(norms + a), b < 0 ? inf : __ldg(norms + b));
-    }
+    __device__ __forceinline__ ScreenSteps(const float *scalars)
+        : ScreenSteps(fminf(scalars[SC_REFN], scalars[SC_REFN + 1]), scalars[5]) {}
     __device__ __forceinline__ int of(float n) const { return max(0, min((int)((n - lo) * scale), SC_BINS - 1)); }
 };
 #endif
@@ -213,36 +229,42 @@ int launch_screen_prepare(const void *W, int f16, int64_t D, int64_t M, const fl
                           const uint16_t *feat, const uint16_t *rank, const int32_t *perm,
                           const uint32_t *key, const uint32_t *tile_len, char *cb, const ScreenLayout &cl,
                           float *scalars, const float *earlier, float *sample, float *window, float2 *reach,
-                          uint32_t *bound, uint32_t *count, int64_t n_pad, bool top2, uint32_t *status, cudaStream_t s);
-// whether the slabs follow the norms, and the units in that order
+                          uint32_t *bound, uint32_t *count, uint32_t *set_reach, int64_t n_pad, bool top2,
+                          uint32_t *status, cudaStream_t s);
+// which sets of documents are swept in the order of the norms, and the units in that order
 int launch_screen_order(const float *norms, int64_t D, int64_t M, int64_t N, int64_t launches, char *cb,
-                        const ScreenLayout &cl, float *scalars, const float *earlier, bool shared,
-                        const uint32_t *status, uint32_t *tickets, cudaStream_t s);
+                        const ScreenLayout &cl, float *scalars, const float *earlier, const uint32_t *status,
+                        const uint32_t *set_reach, int sets, uint32_t *tickets, uint32_t *nat_list, cudaStream_t s);
 // the 8-bit images and the norms of the n_slabs slabs of launch k (neurons beyond M: never chosen), into the slots
-// from `slot` on; nothing if the scalars say that they stand, as may be `expected`.  In the order of the norms also
-// the list of the sweep's items (sets: of 128 documents).
-struct ImageArgs {
-    int64_t k, launches, n_slabs, slab0, slot;
-    int head, sets, first;
-    bool expected;
+// from `slot` on; nothing if the scalars say that they stand, as may be `expected`
+int launch_screen_quantize(const void *W, int f16, int64_t D, int64_t M, const float *norms,
+                           int64_t k, int64_t launches, int64_t n_slabs, int64_t slot, int head,
+                           const uint16_t *feat, char *cb, const ScreenLayout &cl, const float *scalars,
+                           bool expected, cudaStream_t s);
+// ... of slabs in the order of the norms, slab0 and the following, and the lists of the sweep's items
+struct OrderedImages {
+    int64_t slab0, slot;
+    int n_slabs, head, sets, first;
+    const uint32_t *set_reach, *bound;
     const float2 *reach;
     const float *window;
-    const uint32_t *bound;
     uint2 *items;
     uint32_t *tickets;
 };
-int launch_screen_quantize(const void *W, int f16, int64_t D, int64_t M, const float *norms, const ImageArgs &g,
-                           const uint16_t *feat, char *cb, const ScreenLayout &cl, const float *scalars, cudaStream_t s);
+int launch_screen_ordered_images(const void *W, int f16, int64_t D, int64_t M, const OrderedImages &g,
+                                 const uint16_t *feat, char *cb, const ScreenLayout &cl, const float *scalars, int sms,
+                                 cudaStream_t s);
 // A launch that may begin under the end of the one before it on the stream, if that one's blocks allow it
-// (griddepcontrol.launch_dependents) and the kernel waits before it reads or writes (griddepcontrol.wait).
+// (griddepcontrol.launch_dependents).  Every kernel launched so waits for it first of all (griddepcontrol.wait), also
+// where it has nothing to do: whoever waits for the end of one kernel has then waited for all before it.
 struct ScreenLaunch {
     cudaLaunchAttribute attr;
     cudaLaunchConfig_t c;
-    ScreenLaunch(unsigned blocks, unsigned threads, cudaStream_t s, bool early) : c()
+    ScreenLaunch(dim3 blocks, unsigned threads, cudaStream_t s, bool early, size_t smem = 0) : c()
     {
         attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr.val.programmaticStreamSerializationAllowed = 1;
-        c.gridDim = dim3(blocks); c.blockDim = dim3(threads);
+        c.gridDim = blocks; c.blockDim = dim3(threads); c.dynamicSmemBytes = smem;
         c.stream = s; c.attrs = &attr; c.numAttrs = early ? 1 : 0;
     }
     ScreenLaunch(const ScreenLaunch &) = delete;
@@ -250,10 +272,12 @@ struct ScreenLaunch {
 // one launch for either order of the slabs: the one that the scalars do not name returns at once
 int launch_sweep_screen(const ScreenArgs &a, const OrderedArgs &o, bool top2, bool ordered, int sms, cudaStream_t s);
 // after each launch: what it could not rule out, into the documents' lists
-int launch_screen_collect(const VerifyArgs &a, bool top2, int sms, cudaStream_t s);
+int launch_screen_collect(const VerifyArgs &a, bool top2, cudaStream_t s);
 // after the last: the lists evaluated exactly, and the outputs
 int launch_screen_verify(const VerifyArgs &a, bool top2, cudaStream_t s);
-// directly behind it: the documents it handed over (none, as a rule)
+// the same for slabs in the order of the norms
+int launch_screen_verify_units(const VerifyArgs &a, bool top2, int sms, cudaStream_t s);
+// directly behind them: the documents they handed over (none, as a rule)
 int launch_screen_dense(const VerifyArgs &a, bool top2, int sms, cudaStream_t s);
 
 }  // namespace bmu

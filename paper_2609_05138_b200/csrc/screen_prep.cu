@@ -5,13 +5,14 @@
 
 #include <cuda_fp16.h>
 #include <math_constants.h>
+#include <type_traits>
 
 namespace bmu {
 
 static inline size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 
 template <typename Take>
-static void codebook_layout(int64_t D, int64_t M, int64_t slots, int sets, Take take, ScreenLayout *l)
+static void codebook_layout(int64_t D, int64_t M, int64_t slots, int64_t ord_slots, int sets, Take take, ScreenLayout *l)
 {
     const size_t d4 = (size_t)D * 4;
     l->scalars = take((size_t)sets * SC_SCALARS * 4);
@@ -24,6 +25,13 @@ static void codebook_layout(int64_t D, int64_t M, int64_t slots, int sets, Take 
     const size_t m4 = M >= SC_ORDER_MIN ? (size_t)((M + SC_SLAB - 1) / SC_SLAB * SC_SLAB) * 4 : 0;
     l->units = take(m4); l->unit_norm = take(m4); l->unit_tmp = take(2 * m4);
     l->rank_of = take(m4); l->picks = take(2 * m4);
+    // (a search on its own sweeps one order after the other)
+    l->ord8 = l->img8; l->ord_head = l->head_img; l->ord_normp = l->normp;
+    if (ord_slots && m4) {
+        l->ord8 = take((size_t)ord_slots * (size_t)(D + 1) * SC_SLAB);
+        l->ord_head = take((size_t)ord_slots * (size_t)l->head_pad * SC_SLAB);
+        l->ord_normp = take((size_t)ord_slots * SC_SLAB * 4);
+    }
 }
 
 void screen_layout(int64_t D, int64_t M, int64_t N, int head, int64_t chunk, bool top2, int sms,
@@ -39,21 +47,26 @@ void screen_layout(int64_t D, int64_t M, int64_t N, int head, int64_t chunk, boo
     const int64_t blocks = l->n_pad / SC_DOCS, slabs = (all + launches - 1) / launches;
     l->splits = screen_splits(blocks, slabs, sms);
     const size_t n4 = (size_t)l->n_pad * 4;
-    const size_t stripes = (size_t)screen_split_blocks(blocks, slabs, sms) * SC_DOCS * 4;
-    codebook_layout(D, M, l->chunk_slabs, 1, take, l);
+    const int64_t room = screen_split_blocks(blocks, slabs, sms);
+    const size_t stripes = (size_t)room * SC_DOCS * 4;
+    l->most_splits = (int)(room / blocks < slabs ? room / blocks : slabs);
+    if (l->most_splits > 16) l->most_splits = 16;
+    if (l->most_splits < l->splits) l->most_splits = l->splits;
+    codebook_layout(D, M, l->chunk_slabs, 0, 1, take, l);
+    // a quarter of the launches' slabs: far beyond that the order of the map is the better one
+    l->ord_launches = launches <= SC_MAX_LAUNCHES ? (launches + 3) / 4 : 0;
     l->sample = take((size_t)SC_SAMPLE * (size_t)((M + SC_GROUP - 1) / SC_GROUP) * 4);
     l->window = take(n4);
     l->amin = take(n4); l->amin2 = top2 ? take(n4) : l->amin;
     l->cval = take(stripes * sizeof(float2)); l->cmask = take(stripes * sizeof(uint4));
     l->cval2 = top2 ? take(stripes * sizeof(float)) : l->cval;
     l->lcount = take(n4);
-    // (one after the other: n_pad is a multiple of 128)
-    static_assert(SC_LIST * 24 >= SC_OWN_LIST * 16, "room for the lists of slabs in the order of the norms");
-    l->lval = take(n4 * SC_LIST); l->lmask = take(n4 * SC_LIST * 4); l->lbase = take(n4 * SC_LIST);
+    l->lists = take((size_t)l->n_pad * SC_LIST_BYTES);
     const bool order = M >= SC_ORDER_MIN;
     l->reach = take(order ? 2 * n4 : 0);
     l->items = take(order ? (size_t)blocks * SC_PARTS * sizeof(uint2) : 0);
     l->tickets = take(order && launches <= SC_MAX_LAUNCHES ? (size_t)launches * (SC_PARTS + 1) * 4 : 0);
+    l->nat_list = take(order ? (size_t)blocks * 4 : 0);
     l->total = off;
 }
 
@@ -65,7 +78,8 @@ void screen_shared_layout(int64_t D, int64_t M, int head, int64_t chunk, ScreenL
     const int64_t all = (M + SC_SLAB - 1) / SC_SLAB;
     l->chunk_slabs = chunk / SC_SLAB < all ? chunk / SC_SLAB : all;
     const int64_t launches = (all + l->chunk_slabs - 1) / l->chunk_slabs;
-    codebook_layout(D, M, launches * l->chunk_slabs, 2, take, l);
+    l->ord_launches = launches <= SC_MAX_LAUNCHES ? (launches + 3) / 4 : 0;
+    codebook_layout(D, M, launches * l->chunk_slabs, l->ord_launches * l->chunk_slabs, 2, take, l);
     l->rank = take((size_t)D * 2); l->feat = take((size_t)D * 2);
     l->total = off;
 }
@@ -270,12 +284,14 @@ __device__ __forceinline__ float screen_hi16(uint32_t x) { return __uint_as_floa
 
 template <typename WT>
 __global__ void __launch_bounds__(256)
-screen_table_kernel(const WT *__restrict__ W, int64_t M, const uint32_t *__restrict__ status, const float *__restrict__ rmin, const float *__restrict__ rmax, int32_t D, int32_t head,
+screen_table_kernel(const WT *__restrict__ W, int64_t M, const float *__restrict__ norms, const uint32_t *__restrict__ status, const float *__restrict__ rmin, const float *__restrict__ rmax, int32_t D, int32_t head,
                     int32_t head_pad, const uint16_t *__restrict__ feat, const uint16_t *__restrict__ rank,
                     const uint32_t *__restrict__ tile_len, int64_t few, const uint32_t *__restrict__ most,
                     const float *__restrict__ earlier, int sampled, float *__restrict__ scalars, uint4 *__restrict__ table,
                     unsigned char *__restrict__ kpack, float *__restrict__ khead)
 {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     uint32_t m3[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -305,12 +321,18 @@ screen_table_kernel(const WT *__restrict__ W, int64_t M, const uint32_t *__restr
     const int i = blockIdx.x * 256 + threadIdx.x;
     if (i == 0) {
         scalars[0] = -2.f * dh; scalars[1] = -2.f * dt;
-        scalars[2] = 1.f / dt; scalars[4] = (float)q_max;
+        scalars[2] = 1.f / dt; scalars[3] = stand ? 1.f : 0.f; scalars[4] = (float)q_max;
         scalars[5] = norm; scalars[6] = (float)(65535 / q_max);
-        scalars[7] = stand ? 0.f : 1.f; scalars[8] = rh; scalars[9] = rt;
+        scalars[7] = stand && __float_as_uint(earlier[SC_NATMADE]) ? 0.f : 1.f; scalars[8] = rh; scalars[9] = rt;
         scalars[SC_VOTES] = earlier ? earlier[SC_VOTES] : __uint_as_float(0u);
-        scalars[SC_ORDERED] = __uint_as_float(0u);           // (screen_order_kernel decides)
-        scalars[SC_REF] = __int_as_float(ref[0]); scalars[SC_REF + 1] = __int_as_float(ref[1]);
+        // (screen_order_kernel decides otherwise)
+        scalars[SC_ORDERED] = __uint_as_float(0u);
+        scalars[SC_NAT] = __uint_as_float(SC_ALL); scalars[SC_NATMADE] = __uint_as_float(1u);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            scalars[SC_REF + c] = __int_as_float(ref[c]);
+            scalars[SC_REFN + c] = ref[c] < 0 ? CUDART_INF_F : __ldg(norms + ref[c]);
+        }
         scalars[SC_SAMPLED] = earlier ? earlier[SC_SAMPLED] : __uint_as_float((uint32_t)sampled);
     }
     // errors: half a step, widened by 2^-10 for the roundings of the coding itself
@@ -356,7 +378,7 @@ struct ScreenWindow { float window, bound, reach; };
 __device__ __forceinline__ ScreenWindow screen_window_of(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
                                                          int64_t i, const uint32_t *__restrict__ key,
                                                          const uint4 *__restrict__ table, const float *scalars,
-                                                         const float *__restrict__ norms, bool order, bool top2,
+                                                         bool order, bool top2,
                                                          [[maybe_unused]] int64_t D, [[maybe_unused]] uint32_t *status)
 {
     const int lane = threadIdx.x & 31;
@@ -401,9 +423,8 @@ __device__ __forceinline__ ScreenWindow screen_window_of(const int32_t *__restri
     w.window = (gathered > scalars[6] || !(B < 1e37f)) ? CUDART_INF_F : 2.f * B;
     w.bound = w.reach = CUDART_INF_F;
     if (order) {
-        const int32_t a = __float_as_int(scalars[SC_REF]), b = __float_as_int(scalars[SC_REF + 1]);
-        float va = a < 0 ? CUDART_INF_F : __ldg(norms + a) - 2.f * (ra * (2.f - wide)) + 2.f * B;
-        float vb = b < 0 ? CUDART_INF_F : __ldg(norms + b) - 2.f * (rb * (2.f - wide)) + 2.f * B;
+        float va = scalars[SC_REFN] - 2.f * (ra * (2.f - wide)) + 2.f * B;
+        float vb = scalars[SC_REFN + 1] - 2.f * (rb * (2.f - wide)) + 2.f * B;
         if (!(va < CUDART_INF_F)) va = CUDART_INF_F;               // (not a number either)
         if (!(vb < CUDART_INF_F)) vb = CUDART_INF_F;
         w.bound = top2 ? fmaxf(va, vb) : fminf(va, vb);
@@ -416,11 +437,13 @@ __device__ __forceinline__ ScreenWindow screen_window_of(const int32_t *__restri
 __global__ void __launch_bounds__(256, 6)
 screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
                      const int32_t *__restrict__ perm, const uint32_t *__restrict__ key, int64_t N, int64_t n_pad,
-                     const uint4 *__restrict__ table, float *scalars, const float *__restrict__ norms, int order, int top2,
+                     const uint4 *__restrict__ table, float *scalars, int order, int top2,
                      float *__restrict__ window, float2 *__restrict__ reach, uint32_t *__restrict__ bound,
-                     uint32_t *__restrict__ count, int64_t D,
+                     uint32_t *__restrict__ count, uint32_t *__restrict__ set_reach, int64_t D,
                      int sampled, const float *__restrict__ groups, int64_t M, uint32_t *__restrict__ status)
 {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if ((int)blockIdx.x < sampled) {
         __shared__ float s_win, s_least[8];
@@ -429,7 +452,7 @@ screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restri
         const float *of = groups + blockIdx.x * n;
         if (warp == 0) {
             const ScreenWindow w = screen_window_of(rowptr, colidx, screen_sample_doc(blockIdx.x, sampled, N), key, table,
-                                                    scalars, norms, false, top2, D, status);
+                                                    scalars, false, top2, D, status);
             if (lane == 0) s_win = w.window;
         }
         float least = CUDART_INF_F;
@@ -453,22 +476,30 @@ screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restri
         }
         return;
     }
+    // (n_pad is a multiple of the eight documents of a block, and so is a set of them)
+    __shared__ uint32_t s_far[8];
     const int64_t p = ((int64_t)(blockIdx.x - sampled) * blockDim.x + threadIdx.x) >> 5;
-    if (p >= n_pad) return;
     const bool there = p < N && !(*status & PLAN_STATUS_OVERFLOW);
     ScreenWindow w = {0.f, -CUDART_INF_F, 0.f};
-    if (there) w = screen_window_of(rowptr, colidx, perm[p], key, table, scalars, norms, order, top2, D, status);
-    if (lane) return;
-    window[p] = w.window;
+    if (there) w = screen_window_of(rowptr, colidx, perm[p], key, table, scalars, order, top2, D, status);
+    if (lane == 0) window[p] = w.window;
     if (!order) return;
-    // (documents that are evaluated whole need no slab)
-    const bool none = !there || w.window == CUDART_INF_F;
-    const float t = none ? -CUDART_INF_F : w.bound + w.window + w.reach;
-    reach[p] = make_float2(t == t ? t : CUDART_INF_F, w.reach);
-    bound[p] = float_to_ordered(none ? -CUDART_INF_F : w.bound);
-    count[p] = 0u;
-    const ScreenSteps steps(scalars, norms);
-    if (!none && t < steps.top) atomicAdd(status + STATUS_REACH + steps.of(t), 1u);
+    if (lane == 0) {
+        // (documents that are evaluated whole need no slab)
+        const bool none = !there || w.window == CUDART_INF_F;
+        const float t = none ? -CUDART_INF_F : w.bound + w.window + w.reach;
+        reach[p] = make_float2(t == t ? t : CUDART_INF_F, w.reach);
+        bound[p] = float_to_ordered(none ? -CUDART_INF_F : w.bound);
+        count[p] = 0u;
+        s_far[warp] = none ? 0u : float_to_ordered(t == t ? t : CUDART_INF_F);
+        const ScreenSteps steps(scalars);
+        if (!none && t < steps.top) atomicAdd(status + STATUS_REACH + steps.of(t), 1u);
+    }
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        const uint32_t far = __reduce_max_sync(0xffu, s_far[threadIdx.x]);
+        if (threadIdx.x == 0 && far) atomicMax(set_reach + p / SC_DOCS, far);
+    }
 }
 
 template <typename WT>
@@ -492,7 +523,8 @@ int launch_screen_prepare(const void *W, int f16, int64_t D, int64_t M, const fl
                           const uint16_t *feat, const uint16_t *rank, const int32_t *perm,
                           const uint32_t *key, const uint32_t *tile_len, char *cb, const ScreenLayout &cl,
                           float *scalars, const float *earlier, float *sample, float *window, float2 *reach,
-                          uint32_t *bound, uint32_t *count, int64_t n_pad, bool top2, uint32_t *status, cudaStream_t s)
+                          uint32_t *bound, uint32_t *count, uint32_t *set_reach, int64_t n_pad, bool top2,
+                          uint32_t *status, cudaStream_t s)
 {
     const int order = M >= SC_ORDER_MIN;
     // (an earlier search of the same codebook has decided for this one too)
@@ -511,17 +543,21 @@ int launch_screen_prepare(const void *W, int f16, int64_t D, int64_t M, const fl
     // up to a thousandth of the tiles, or four where they are few (32 documents of 1000 ids: 27 us for 4,096 units)
     const int64_t tiles = (N + 7) / 8, four = tiles / 64 < 4 ? tiles / 64 : 4, few = tiles / 1024 > four ? tiles / 1024 : four;
     const auto tables = [&](auto w) {
-        screen_table_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, s>>>(
-            w, M, status, rmin, rmax, (int32_t)D, head, cl.head_pad, feat, rank, tile_len, few, most, earlier, sampled,
-            scalars, table, reinterpret_cast<unsigned char *>(cb + cl.kpack), reinterpret_cast<float *>(cb + cl.khead));
+        ScreenLaunch l((unsigned)((rows + 255) / 256), 256, s, true);
+        const cudaError_t e = cudaLaunchKernelEx(
+            &l.c, screen_table_kernel<std::remove_const_t<std::remove_pointer_t<decltype(w)>>>, w, M, norms, (const uint32_t *)status,
+            (const float *)rmin, (const float *)rmax, (int32_t)D, head, cl.head_pad, feat, rank, tile_len, few,
+            (const uint32_t *)most, earlier, sampled, scalars, table, reinterpret_cast<unsigned char *>(cb + cl.kpack),
+            reinterpret_cast<float *>(cb + cl.khead));
         BMU_LAUNCHED();
+        return e;
     };
-    if (f16) tables(static_cast<const __half *>(W));
-    else tables(static_cast<const float *>(W));
-    { screen_window_kernel<<<(unsigned)(sampled + (n_pad * 32 + 255) / 256), 256, 0, s>>>(
-        rowptr, colidx, perm, key, N, n_pad, table, scalars, norms, order, top2, window, reach, bound, count, D, sampled,
-        sample, M, status); BMU_LAUNCHED(); }
-    BMU_CUDA(cudaGetLastError());
+    BMU_CUDA(f16 ? tables(static_cast<const __half *>(W)) : tables(static_cast<const float *>(W)));
+    ScreenLaunch l((unsigned)(sampled + (n_pad * 32 + 255) / 256), 256, s, true);
+    BMU_CUDA(cudaLaunchKernelEx(&l.c, screen_window_kernel, rowptr, colidx, perm, key, N, n_pad, (const uint4 *)table, scalars,
+                                order, (int)top2, window, reach, bound, count, set_reach, D, sampled, (const float *)sample,
+                                M, status));
+    BMU_LAUNCHED();
     return BMU_OK;
 }
 
@@ -755,20 +791,20 @@ __device__ __forceinline__ void ordered_head(const WT *__restrict__ W, int64_t D
 }
 
 // A warp per set of 128 documents: which of the launch's slabs any of them reaches, as items of up to SC_PART.
-__device__ __forceinline__ void ordered_items(const ImageArgs &g, int set, int slabs, const float *__restrict__ unit_norm,
+__device__ __forceinline__ void ordered_items(const OrderedImages &g, int set, int slabs, const float *__restrict__ unit_norm,
                                               const float *__restrict__ scalars)
 {
     const int lane = threadIdx.x & 31;
-    const float top = __ldg(scalars + SC_TOP);
+    if (!(ordered_to_float(__ldg(g.set_reach + set)) <= __ldg(scalars + SC_TOP))) return;    // in the order of the map
+    const float top = __ldg(scalars + SC_DOC_TOP);
     float far = -CUDART_INF_F;
 #pragma unroll
     for (int u = 0; u < SC_DOCS / 32; ++u) {
         const int64_t p = (int64_t)set * SC_DOCS + 32 * u + lane;
         const float2 r = __ldg(g.reach + p);
         if (r.x > top) continue;                           // evaluated whole
-        // (what the launches before have found)
-        const float t = g.first ? r.x : fminf(r.x, ordered_to_float(__ldcg(g.bound + p)) + __ldg(g.window + p) + r.y);
-        far = fmaxf(far, t);
+        // (less what the launches before have found)
+        far = fmaxf(far, g.first ? r.x : fminf(r.x, ordered_to_float(__ldcg(g.bound + p)) + __ldg(g.window + p) + r.y));
     }
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1) far = fmaxf(far, __shfl_xor_sync(0xffffffffu, far, m));
@@ -779,44 +815,77 @@ __device__ __forceinline__ void ordered_items(const ImageArgs &g, int set, int s
             make_uint2((uint32_t)set, (uint32_t)(lane * SC_PART) | (uint32_t)min(n, (lane + 1) * SC_PART) << 16);
 }
 
+template <typename WT>
+__global__ void __launch_bounds__(256, 6)
+screen_ordered_image_kernel(const WT *__restrict__ W, int64_t D, int64_t M, const OrderedImages g,
+                            const int2 *__restrict__ picks, const float *__restrict__ unit_norm, int32_t head_pad,
+                            const uint16_t *__restrict__ feat, const float *__restrict__ rmin,
+                            const float *__restrict__ khead, const float *__restrict__ scalars,
+                            unsigned char *__restrict__ img8, unsigned char *__restrict__ head_img, float *__restrict__ normp)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!screen_ordered(scalars) || screen_whole(scalars)) return;
+    const uint32_t *sc = reinterpret_cast<const uint32_t *>(scalars);
+    const int slabs = (int)min((int64_t)g.n_slabs, (int64_t)__ldg(sc + SC_NEEDED) - g.slab0);
+    if (slabs <= 0) return;
+    const int place0 = (int)g.slab0 * SC_SLAB, slots = slabs * SC_SLAB;
+    const bool stand = __ldg(sc + SC_STAND) != 0u;         // the images of an earlier search
+    const int lists = (g.sets + 7) / 8, rows = (int)((D + ORD_ROWS) / ORD_ROWS), heads = head_pad / ORD_HEAD;
+    const int all = stand ? lists : lists + heads + rows;
+    for (int item = blockIdx.x; item < all; item += gridDim.x) {
+        if (item < lists) {
+            const int set = item * 8 + (threadIdx.x >> 5);
+            if (set < g.sets) ordered_items(g, set, slabs, unit_norm + place0, scalars);
+        } else if (item < lists + heads) {
+            ordered_head(W, D, M, (item - lists) * ORD_HEAD, slots, place0, picks + place0, g.head, head_pad, feat, rmin, khead, head_img);
+            if (item == lists)
+                for (int x = threadIdx.x; x < slots; x += 256) {
+                    const int jn = x & (SC_SLAB - 1);
+                    normp[x - jn + ((jn & 31) >> 2) * 16 + (jn >> 5) * 4 + (jn & 3)] = __ldg(unit_norm + place0 + x);
+                }
+        } else {
+            ordered_rows(W, D, M, (int64_t)(item - lists - heads) * ORD_ROWS, slots, place0, picks + place0, rmin,
+                         __ldg(scalars + 2), __ldg(scalars + 4), img8);
+        }
+    }
+}
+
+int launch_screen_ordered_images(const void *W, int f16, int64_t D, int64_t M, const OrderedImages &g,
+                                 const uint16_t *feat, char *cb, const ScreenLayout &l, const float *scalars, int sms,
+                                 cudaStream_t s)
+{
+    const auto go = [&](auto w) {
+        ScreenLaunch p((unsigned)(6 * sms), 256, s, true);
+        const cudaError_t e = cudaLaunchKernelEx(
+            &p.c, screen_ordered_image_kernel<std::remove_const_t<std::remove_pointer_t<decltype(w)>>>, w, D, M, g,
+            reinterpret_cast<const int2 *>(cb + l.picks), reinterpret_cast<const float *>(cb + l.unit_norm),
+            (int32_t)l.head_pad, feat, reinterpret_cast<const float *>(cb + l.rmin), reinterpret_cast<const float *>(cb + l.khead),
+            scalars, reinterpret_cast<unsigned char *>(cb + l.ord8) + (size_t)g.slot * (D + 1) * SC_SLAB,
+            reinterpret_cast<unsigned char *>(cb + l.ord_head) + (size_t)g.slot * l.head_pad * SC_SLAB,
+            reinterpret_cast<float *>(cb + l.ord_normp) + g.slot * SC_SLAB);
+        BMU_LAUNCHED();
+        return e;
+    };
+    BMU_CUDA(f16 ? go(static_cast<const __half *>(W)) : go(static_cast<const float *>(W)));
+    return BMU_OK;
+}
+
 // Both images of a slab in one grid, the head's blocks in front.  LOOP: a block takes every gridDim.y-th
 // slab -- slower where there is work (a shared codebook's images usually stand), 9 -> 3 us where not.
 template <typename WT, bool VEC, bool LOOP>
-__global__ void __launch_bounds__(256, LOOP ? 3 : sizeof(WT) == 2 && VEC ? 4 : 6)
+__global__ void __launch_bounds__(256)
 screen_image_kernel(const WT *__restrict__ W, int64_t D, int64_t M, int64_t k, int64_t launches, int64_t n_slabs,
-                    const ImageArgs g, const int2 *__restrict__ picks, const float *__restrict__ unit_norm, int32_t head,
+                    int32_t head,
                     int32_t head_pad, const uint16_t *__restrict__ feat, const float *__restrict__ rmin,
                     const float *__restrict__ khead, const float *__restrict__ scalars,
                     const float *__restrict__ norms, unsigned char *__restrict__ img8,
                     unsigned char *__restrict__ head_img, float *__restrict__ normp)
 {
-    if (screen_ordered(scalars)) {
-        const uint32_t *sc = reinterpret_cast<const uint32_t *>(scalars);
-        const int slabs = (int)min(n_slabs, (int64_t)__ldg(sc + SC_NEEDED) - g.slab0);
-        if (slabs <= 0) return;
-        const int place0 = (int)g.slab0 * SC_SLAB, slots = slabs * SC_SLAB;
-        const bool stand = __ldg(sc + SC_STAND) != 0u;     // the images of an earlier search
-        const int lists = (g.sets + 7) / 8, rows = (int)((D + ORD_ROWS) / ORD_ROWS), heads = head_pad / ORD_HEAD;
-        const int all = stand ? lists : lists + heads + rows;
-        for (int item = blockIdx.y * gridDim.x + blockIdx.x; item < all; item += gridDim.x * gridDim.y) {
-            if (item < lists) {
-                const int set = item * 8 + (threadIdx.x >> 5);
-                if (set < g.sets) ordered_items(g, set, slabs, unit_norm + place0, scalars);
-            } else if (item < lists + heads) {
-                ordered_head(W, D, M, (item - lists) * ORD_HEAD, slots, place0, picks + place0, head, head_pad, feat, rmin, khead, head_img);
-                if (item == lists)
-                    for (int x = threadIdx.x; x < slots; x += 256) {
-                        const int jn = x & (SC_SLAB - 1);
-                        normp[x - jn + ((jn & 31) >> 2) * 16 + (jn >> 5) * 4 + (jn & 3)] = __ldg(unit_norm + place0 + x);
-                    }
-            } else {
-                ordered_rows(W, D, M, (int64_t)(item - lists - heads) * ORD_ROWS, slots, place0, picks + place0, rmin,
-                             __ldg(scalars + 2), __ldg(scalars + 4), img8);
-            }
-        }
-        return;
-    }
-    if (__ldg(scalars + 7) == 0.f || screen_whole(scalars)) return;   // the images of an earlier search stand
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // the images of an earlier search stand; or nothing is swept in this order
+    if (__ldg(scalars + 7) == 0.f || screen_whole(scalars) || screen_natural(scalars) == 0u) return;
     const int heads = head_pad / 32;
     auto one = [&](const int64_t slab) {
         const int64_t j_slab = (k + launches * slab) * SC_SLAB;
@@ -832,33 +901,35 @@ screen_image_kernel(const WT *__restrict__ W, int64_t D, int64_t M, int64_t k, i
 }
 
 template <typename WT>
-static int launch_images(const WT *W, int64_t D, int64_t M, const float *norms, const ImageArgs &g,
-                         const uint16_t *feat, char *base, const ScreenLayout &l, const float *scalars, cudaStream_t s)
+static int launch_images(const WT *W, int64_t D, int64_t M, const float *norms, int64_t k,
+                         int64_t launches, int64_t n_slabs, int64_t slot, int head, const uint16_t *feat, char *base,
+                         const ScreenLayout &l, const float *scalars, bool expected, cudaStream_t s)
 {
     const float *rmin = reinterpret_cast<const float *>(base + l.rmin);
     const float *khead = reinterpret_cast<const float *>(base + l.khead);
-    const int2 *picks = reinterpret_cast<const int2 *>(base + l.picks);
-    const float *unit_norm = reinterpret_cast<const float *>(base + l.unit_norm);
-    unsigned char *img8 = reinterpret_cast<unsigned char *>(base + l.img8) + (size_t)g.slot * (D + 1) * SC_SLAB;
-    unsigned char *head_img = reinterpret_cast<unsigned char *>(base + l.head_img) + (size_t)g.slot * l.head_pad * SC_SLAB;
-    float *normp = reinterpret_cast<float *>(base + l.normp) + g.slot * SC_SLAB;
+    unsigned char *img8 = reinterpret_cast<unsigned char *>(base + l.img8) + (size_t)slot * (D + 1) * SC_SLAB;
+    unsigned char *head_img = reinterpret_cast<unsigned char *>(base + l.head_img) + (size_t)slot * l.head_pad * SC_SLAB;
+    float *normp = reinterpret_cast<float *>(base + l.normp) + slot * SC_SLAB;
     const bool vec = M % (16 / sizeof(WT)) == 0 && (reinterpret_cast<uintptr_t>(W) & 15) == 0;
     const int rows = vec ? IMAGE_ROWS<WT, true> : IMAGE_ROWS<WT, false>;
     const dim3 grid((unsigned)(l.head_pad / 32 + (D + 1 + rows - 1) / rows),
-                    g.expected ? 1u : (unsigned)g.n_slabs);     // few blocks where there is likely nothing to do
-#define BMU_IMG(V, L) { screen_image_kernel<WT, V, L><<<grid, 256, 0, s>>>(W, D, M, g.k, g.launches, g.n_slabs, g, picks, unit_norm, g.head, l.head_pad, feat, rmin, khead, scalars, norms, img8, head_img, normp); BMU_LAUNCHED(); }
-    if (g.expected) { if (vec) BMU_IMG(true, true) else BMU_IMG(false, true) }
+                    expected ? 1u : (unsigned)n_slabs);       // few blocks where there is likely nothing to do
+    ScreenLaunch p(grid, 256, s, true);
+#define BMU_IMG(V, L) { BMU_CUDA(cudaLaunchKernelEx(&p.c, screen_image_kernel<WT, V, L>, W, D, M, k, launches, n_slabs, (int32_t)head, (int32_t)l.head_pad, feat, rmin, khead, scalars, norms, img8, head_img, normp)); BMU_LAUNCHED(); }
+    if (expected) { if (vec) BMU_IMG(true, true) else BMU_IMG(false, true) }
     else if (vec) BMU_IMG(true, false) else BMU_IMG(false, false)
 #undef BMU_IMG
-    BMU_CUDA(cudaGetLastError());
     return BMU_OK;
 }
 
-int launch_screen_quantize(const void *W, int f16, int64_t D, int64_t M, const float *norms, const ImageArgs &g,
-                           const uint16_t *feat, char *cb, const ScreenLayout &cl, const float *scalars, cudaStream_t s)
+int launch_screen_quantize(const void *W, int f16, int64_t D, int64_t M, const float *norms,
+                           int64_t k, int64_t launches, int64_t n_slabs, int64_t slot, int head,
+                           const uint16_t *feat, char *cb, const ScreenLayout &cl, const float *scalars,
+                           bool expected, cudaStream_t s)
 {
-    if (f16) return launch_images(static_cast<const __half *>(W), D, M, norms, g, feat, cb, cl, scalars, s);
-    return launch_images(static_cast<const float *>(W), D, M, norms, g, feat, cb, cl, scalars, s);
+    if (f16)
+        return launch_images(static_cast<const __half *>(W), D, M, norms, k, launches, n_slabs, slot, head, feat, cb, cl, scalars, expected, s);
+    return launch_images(static_cast<const float *>(W), D, M, norms, k, launches, n_slabs, slot, head, feat, cb, cl, scalars, expected, s);
 }
 
 }  // namespace bmu

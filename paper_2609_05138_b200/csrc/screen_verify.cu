@@ -160,36 +160,6 @@ __device__ __forceinline__ void verify_groups(const VerifyArgs &a, const uint4 m
     }
 }
 
-// The whole warp evaluates the units of `bits`, numbers first .. first + 31 in the order of the norms: a lane per
-// listed row, a 32-byte sector each, four rows in flight.
-template <typename WT, bool TOP2>
-__device__ __forceinline__ void verify_units(const VerifyArgs &a, uint32_t bits, int64_t first, int beg, int end,
-                                             u64 &best, u64 &best2)
-{
-    const int lane = threadIdx.x & 31;
-    const WT *W = static_cast<const WT *>(a.W);
-    for (; bits; bits &= bits - 1) {
-        const int32_t j = __ldg(a.units + first + __ffs(bits) - 1);
-        if (j < 0) continue;                                 // (beyond the last unit; never within a window)
-        float s = 0.f;
-        for (int e0 = beg; e0 < end; e0 += 128) {
-            float w[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int e = e0 + 32 * u + lane;
-                w[u] = e < end ? verify_ld(W + (int64_t)BMU_IDX((uint32_t)__ldg(a.colidx + e), a.D, a.status) * a.M + j) : 0.f;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) s += w[u];
-        }
-#pragma unroll
-        for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
-        const u64 k = make_key(fmaf(-2.f, s, __ldg(a.norms + j)), j);
-        if (TOP2) { if (lane == 0) Best<true>::merge(best, best2, k, KEY_WORST); }
-        else best = k < best ? k : best;
-    }
-}
-
 // the warp's best (and second-best) key, on every lane
 template <bool TOP2>
 __device__ __forceinline__ void verify_merge(u64 &best, u64 &best2)
@@ -213,20 +183,22 @@ __device__ __forceinline__ uint4 shfl4(const uint4 v, int src)
                       __shfl_sync(0xffffffffu, v.z, src), __shfl_sync(0xffffffffu, v.w, src));
 }
 
-// Eight documents per warp, a lane per stripe.  (Few blocks, for those times when there is nothing to do.)
+// Eight documents per warp, a lane per stripe.
 template <typename WT, bool TOP2, bool VEC>
 __global__ void __launch_bounds__(256, 4)
 screen_collect_kernel(const VerifyArgs a)
 {
     const int lane = threadIdx.x & 31, k = lane & 3;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // (the verify stage, after the last launch)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     // (one lane reads the status word for its warp: the lanes must stay together)
-    // (where slabs are in the order of the norms the sweep keeps the lists and the bounds itself)
     if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(a.status), 0) || screen_whole(a.scalars) ||
-        screen_ordered(a.scalars)) return;
+        screen_natural(a.scalars) == 0u) return;
+    // (in the order of the norms the sweep keeps the lists and the bounds itself; eight documents are of one set)
+    const int64_t p = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 8 + (lane >> 2);
+    if (screen_by_norm(a.scalars, a.set_reach, p)) return;
     const uint32_t seg = 15u << (lane & ~3), most = screen_early_groups(a.M);
-    for (int64_t p8 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 8; p8 < a.N; p8 += (int64_t)gridDim.x * (blockDim.x / 4)) {
-    const int64_t p = p8 + (lane >> 2);
+    const int splits = screen_parts(a.scalars, a.splits, a.most_splits);
     const bool there = p < a.N;
     const float win = there ? a.window[p] : 0.f;
     // pass 1: the document's smallest (and second smallest) approximate value so far.  The stripes of
@@ -237,7 +209,7 @@ screen_collect_kernel(const VerifyArgs a)
         v1 = a.amin[p];
         if (TOP2) v2 = a.amin2[p];
     }
-    for (int c = 0; c < a.splits; ++c) {
+    for (int c = 0; c < splits; ++c) {
         const size_t at = ((size_t)c * a.n_pad + p) * 4 + k;
         float o1 = there ? a.cval[at].x : CUDART_INF_F, o2 = CUDART_INF_F;
         if (TOP2 && there) o2 = a.cval2[at];
@@ -253,11 +225,11 @@ screen_collect_kernel(const VerifyArgs a)
     const float limit = (TOP2 ? v2 : v1) + win;
     uint32_t count = there && !a.first ? a.lcount[p] : 0u, n = count & 15u, done = count >> 4 & 0x3ffffffu;
     bool touched = a.first, dense = (count & SC_DENSE) != 0u || win == CUDART_INF_F;
-    float *lv = a.lval + (size_t)p * SC_LIST;
-    uint4 *lm = a.lmask + (size_t)p * SC_LIST;
-    uint32_t *lb = a.lbase + (size_t)p * SC_LIST;
+    uint4 *lm = reinterpret_cast<uint4 *>(a.lists + (size_t)p * SC_LIST_BYTES);
+    float *lv = reinterpret_cast<float *>(lm + SC_LIST);
+    uint32_t *lb = reinterpret_cast<uint32_t *>(lv + SC_LIST);
     // pass 2: what is within the window joins the list
-    for (int c = 0; c < a.splits; ++c) {
+    for (int c = 0; c < splits; ++c) {
         const size_t at = ((size_t)c * a.n_pad + p) * 4 + k;
         const float2 cv = there ? a.cval[at] : make_float2(CUDART_INF_F, 0.f);
         const float own = cv.x;
@@ -353,7 +325,6 @@ screen_collect_kernel(const VerifyArgs a)
         if (TOP2) a.amin2[p] = v2;
         if (touched) a.lcount[p] = (count & 0x80000000u) | (dense ? SC_DENSE : done << 4 | n);
     }
-    }
 }
 
 // Two documents per warp, sixteen lanes each: a lane takes one list entry.
@@ -361,13 +332,14 @@ template <typename WT, bool TOP2, bool VEC>
 __global__ void __launch_bounds__(256, 5)
 screen_verify_kernel(const VerifyArgs a)
 {
-    static_assert(SC_LIST <= 15 && SC_OWN_LIST <= 16, "a lane per entry, four bits of the count");
+    static_assert(SC_LIST <= 15, "a lane per entry, four bits of the count");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // screen_dense_kernel waits for the rest
     asm volatile("griddepcontrol.wait;" ::: "memory");                   // as this does for the last collection
     const int lane = threadIdx.x & 31, e = lane & 15;
     const int64_t p = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 2 + (lane >> 4);
     if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(a.status), 0)) return;
-    const bool there = p < a.N, whole = screen_whole(a.scalars), ordered = screen_ordered(a.scalars);
+    const bool there = p < a.N, whole = screen_whole(a.scalars);
+    if (!whole && screen_by_norm(a.scalars, a.set_reach, p)) return;     // (sixteen documents are of one set)
     uint32_t count = 0, base = 0;
     uint4 todo = make_uint4(0u, 0u, 0u, 0u);
     int32_t orig = 0, beg = 0, end = 0;
@@ -376,22 +348,15 @@ screen_verify_kernel(const VerifyArgs a)
         orig = a.perm[p];
         beg = __ldg(a.rowptr + orig);
         end = __ldg(a.rowptr + orig + 1);
-        if (ordered && !whole) {
-            const float win = a.window[p];
-            const uint32_t n = count;
-            count = win == CUDART_INF_F || n > (uint32_t)SC_OWN_LIST || a.reach[p].x > __ldg(a.scalars + SC_TOP) ? SC_DENSE : 0u;
-            if ((uint32_t)e < n && !count) {
-                const uint4 t = a.own_list[p * SC_OWN_LIST + e];
-                if (__uint_as_float(t.x) <= ordered_to_float(a.bound[p]) + win) todo.x = t.z;
-                base = t.y * SC_SLAB + t.w * 32u;
-            }
-        } else if ((uint32_t)e < (count & 15u)) {
+        if ((uint32_t)e < (count & 15u)) {
             const float limit = (TOP2 ? a.amin2[p] : a.amin[p]) + a.window[p];
-            if (a.lval[(size_t)p * SC_LIST + e] <= limit) todo = a.lmask[(size_t)p * SC_LIST + e];
-            base = a.lbase[(size_t)p * SC_LIST + e];
+            const uint4 *lm = reinterpret_cast<const uint4 *>(a.lists + (size_t)p * SC_LIST_BYTES);
+            const float *lv = reinterpret_cast<const float *>(lm + SC_LIST);
+            if (lv[e] <= limit) todo = lm[e];
+            base = reinterpret_cast<const uint32_t *>(lv + SC_LIST)[e];
         }
     }
-    // too many groups (or units), or none (no distance of it is finite), or given up before
+    // too many groups, or none (no distance of it is finite), or given up before
     uint32_t groups = popc4(todo);
 #pragma unroll
     for (int m = 8; m > 0; m >>= 1) groups += __shfl_xor_sync(0xffffffffu, groups, m);
@@ -405,13 +370,11 @@ screen_verify_kernel(const VerifyArgs a)
         if (!lanes) continue;
         const int b0 = __shfl_sync(0xffffffffu, beg, 16 * d), e0 = __shfl_sync(0xffffffffu, end, 16 * d);
         uint32_t ids[4];
-        if (VEC && !ordered) VerifyVec<WT>::ids_of(a, b0, e0, ids);
+        if (VEC) VerifyVec<WT>::ids_of(a, b0, e0, ids);
         u64 k1 = KEY_WORST, k2 = KEY_WORST;
         for (; lanes; lanes &= lanes - 1) {
             const int src = __ffs(lanes) - 1;
-            if (ordered)
-                verify_units<WT, TOP2>(a, __shfl_sync(0xffffffffu, todo.x, src), __shfl_sync(0xffffffffu, base, src), b0, e0, k1, k2);
-            else verify_groups<WT, TOP2, VEC>(a, shfl4(todo, src), __shfl_sync(0xffffffffu, base, src), b0, e0, ids, k1, k2);
+            verify_groups<WT, TOP2, VEC>(a, shfl4(todo, src), __shfl_sync(0xffffffffu, base, src), b0, e0, ids, k1, k2);
         }
         verify_merge<TOP2>(k1, k2);
         if (lane >> 4 == d) { best = k1; best2 = k2; }
@@ -441,16 +404,95 @@ screen_verify_kernel(const VerifyArgs a)
     }
 }
 
+// The documents whose slabs were in the order of the norms, one per warp, a lane per list entry.  The units of an
+// entry are evaluated several at a time: as many lanes for each as rows are summed side by side above, and their
+// sums added in the same order, so that a unit has the same distance, bit for bit, whichever way it came here.  A
+// 32-byte sector per row.
+template <typename WT, bool TOP2, bool VEC>
+__global__ void __launch_bounds__(256, 5)
+screen_verify_units_kernel(const VerifyArgs a)
+{
+    constexpr int L = VEC ? VerifyVec<WT>::RS : 4, AT_ONCE = 32 / L, U = VEC ? 4 : 16;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int lane = threadIdx.x & 31, row = lane % L;
+    if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(a.status), 0) || screen_whole(a.scalars) ||
+        !screen_ordered(a.scalars)) return;
+    const WT *W = static_cast<const WT *>(a.W);
+    for (int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < a.N; p += (int64_t)gridDim.x * (blockDim.x / 32)) {
+        if (!screen_by_norm(a.scalars, a.set_reach, p)) continue;
+        const float win = a.window[p];
+        const uint32_t n = a.lcount[p];
+        const int32_t orig = a.perm[p];
+        const int beg = __ldg(a.rowptr + orig), end = __ldg(a.rowptr + orig + 1);
+        uint4 t = make_uint4(0u, 0u, 0u, 0u);
+        if (lane < SC_OWN_LIST && (uint32_t)lane < n) t = reinterpret_cast<const uint4 *>(a.lists + p * SC_LIST_BYTES)[lane];
+        if (!(__uint_as_float(t.x) <= ordered_to_float(a.bound[p]) + win)) t.z = 0u;
+        // too many units, or none (no distance of it is finite), or a list that was too short for them
+        const uint32_t units = __reduce_add_sync(0xffffffffu, __popc(t.z));
+        if (n > (uint32_t)SC_OWN_LIST || units == 0u || __ldg(a.reach + p).x > __ldg(a.scalars + SC_DOC_TOP) || units > screen_dense_groups(a.M) || win == CUDART_INF_F) {
+            if (lane == 0) {
+                a.state[orig] = KEY_WORST;
+                if (TOP2) a.state2[orig] = KEY_WORST;
+                a.lcount[p] = 0u;                            // its ticket from here on
+                a.dense[atomicAdd(a.dense_count, 1u)] = (uint32_t)p;
+            }
+            continue;
+        }
+        u64 best = KEY_WORST, best2 = KEY_WORST;
+        for (uint32_t entries = __ballot_sync(0xffffffffu, t.z != 0u); entries; entries &= entries - 1) {
+            const int src = __ffs(entries) - 1;
+            const int64_t first = (int64_t)__shfl_sync(0xffffffffu, t.y, src) * SC_SLAB + __shfl_sync(0xffffffffu, t.w, src) * 32;
+            uint32_t bits = __shfl_sync(0xffffffffu, t.z, src);
+            while (bits) {
+                int32_t j = -1;
+#pragma unroll
+                for (int i = 0; i < AT_ONCE; ++i) {
+                    if (!bits) break;
+                    if (i == lane / L) j = __ldg(a.units + first + __ffs(bits) - 1);     // (-1 beyond the last unit)
+                    bits &= bits - 1;
+                }
+                float s = 0.f;
+                for (int e0 = beg; e0 < end; e0 += L * U) {
+                    float w[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int e = e0 + u * L + row;
+                        w[u] = j >= 0 && e < end ? verify_ld(W + (int64_t)BMU_IDX((uint32_t)__ldg(a.colidx + e), a.D, a.status) * a.M + j) : 0.f;
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) s += w[u];
+                }
+#pragma unroll
+                for (int m = L / 2; m >= 1; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, VEC ? m : L / 2 / m);
+                const u64 k = row == 0 && j >= 0 ? make_key(fmaf(-2.f, s, __ldg(a.norms + j)), j) : KEY_WORST;
+                if (TOP2) Best<true>::merge(best, best2, k, KEY_WORST);
+                else best = k < best ? k : best;
+            }
+        }
+        verify_merge<TOP2>(best, best2);
+        if (lane == 0) {
+            const float nx = (float)(end - beg);
+            a.out_bmu[orig] = (int32_t)(uint32_t)best;
+            a.out_dist[orig] = nx + ordered_to_float((uint32_t)(best >> 32));
+            if (TOP2) {
+                const bool none = best2 == KEY_WORST;
+                a.out_bmu2[orig] = none ? -1 : (int32_t)(uint32_t)best2;
+                a.out_dist2[orig] = none ? CUDART_INF_F : nx + ordered_to_float((uint32_t)(best2 >> 32));
+            }
+        }
+    }
+}
+
 #define BMU_VERIFY(KERNEL, C) \
     (a.f16 ? (top2 ? (screen_vec(a) ? cudaLaunchKernelEx(&C, KERNEL<__half, true, true>, a) : cudaLaunchKernelEx(&C, KERNEL<__half, true, false>, a)) \
                    : (screen_vec(a) ? cudaLaunchKernelEx(&C, KERNEL<__half, false, true>, a) : cudaLaunchKernelEx(&C, KERNEL<__half, false, false>, a))) \
            : (top2 ? (screen_vec(a) ? cudaLaunchKernelEx(&C, KERNEL<float, true, true>, a) : cudaLaunchKernelEx(&C, KERNEL<float, true, false>, a)) \
                    : (screen_vec(a) ? cudaLaunchKernelEx(&C, KERNEL<float, false, true>, a) : cudaLaunchKernelEx(&C, KERNEL<float, false, false>, a))))
 
-int launch_screen_collect(const VerifyArgs &a, bool top2, int sms, cudaStream_t s)
+int launch_screen_collect(const VerifyArgs &a, bool top2, cudaStream_t s)
 {
-    const int64_t blocks = (a.N + 63) / 64;
-    ScreenLaunch l((unsigned)(blocks < 4 * sms ? blocks : 4 * sms), 256, s, false);
+    ScreenLaunch l((unsigned)((a.N + 63) / 64), 256, s, true);
     BMU_CUDA(BMU_VERIFY(screen_collect_kernel, l.c));
     BMU_LAUNCHED();
     return BMU_OK;
@@ -460,6 +502,15 @@ int launch_screen_verify(const VerifyArgs &a, bool top2, cudaStream_t s)
 {
     ScreenLaunch l((unsigned)((a.N + 15) / 16), 256, s, true);
     BMU_CUDA(BMU_VERIFY(screen_verify_kernel, l.c));
+    BMU_LAUNCHED();
+    return BMU_OK;
+}
+
+int launch_screen_verify_units(const VerifyArgs &a, bool top2, int sms, cudaStream_t s)
+{
+    const int64_t blocks = (a.N + 7) / 8;
+    ScreenLaunch l((unsigned)(blocks < 5 * sms ? blocks : 5 * sms), 256, s, true);
+    BMU_CUDA(BMU_VERIFY(screen_verify_units_kernel, l.c));
     BMU_LAUNCHED();
     return BMU_OK;
 }

@@ -119,7 +119,10 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
     const uint32_t wfull0 = mm_smem(bars), wempty0 = mm_smem(bars + NS);
     const uint32_t tfull0 = mm_smem(bars + 2 * NS), tempty0 = tfull0 + 16, drain = tfull0 + 32;
     const int two = a.head_pad <= 1024, x_col = 512 - a.head_pad / 4;
-    if (screen_ordered(a.scalars) != ORDERED || screen_whole(a.scalars)) return;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const uint32_t natural = screen_natural(a.scalars);
+    if (screen_whole(a.scalars) || (ORDERED ? !screen_ordered(a.scalars) : natural == 0u)) return;
     if (ORDERED && o.slab0 >= (int64_t)__ldg(reinterpret_cast<const uint32_t *>(a.scalars) + SC_NEEDED)) return;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -220,22 +223,28 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
     } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SC_TAIL_REGS));
     const int q = warp & 3, e = warp >> 2;
+    // (thread 0: the block's own item first; the ticket of the next one is on its way while an item is swept)
+    [[maybe_unused]] const uint32_t splits = (uint32_t)screen_parts(a.scalars, a.splits, a.most_splits);
+    [[maybe_unused]] const uint32_t items = (natural == SC_ALL ? (uint32_t)a.blocks : natural) * splits;
+    uint32_t ticket = blockIdx.x;
     for (;;) {
         // the next item (a block that gave up: let the grid drain)
         if (threadIdx.x == 0) {
             uint32_t set = ~0u, range = 0u, part = 0u;       // (no set: there are no more items)
+            uint32_t t = ticket;
             if (*abort_flag || *reinterpret_cast<volatile uint32_t *>(a.status)) {
             } else if (!ORDERED) {
-                // (as many tickets as items and one more for each block: then the counter is zero again)
-                const uint32_t items = (uint32_t)a.blocks * (uint32_t)a.splits, t = atomicInc(a.ticket, items + gridDim.x - 1u);
                 if (t < items) {
-                    set = t % (uint32_t)a.blocks;
-                    part = t / (uint32_t)a.blocks;
-                    range = (uint32_t)a.n_slabs * part / a.splits | (uint32_t)a.n_slabs * (part + 1) / a.splits << 16;
+                    const uint32_t sets = items / splits;
+                    set = t % sets;
+                    part = t / sets;
+                    if (natural != SC_ALL) set = __ldg(a.nat_list + set);
+                    range = (uint32_t)a.n_slabs * part / splits | (uint32_t)a.n_slabs * (part + 1) / splits << 16;
+                    // (as many tickets as items are taken, if any: then the counter is zero again)
+                    ticket = items > gridDim.x ? gridDim.x + atomicInc(a.ticket, items - 1u) : items;
                 }
             } else {
-                uint32_t t = atomicAdd(o.tickets + SC_PARTS, 1u);        // the lists one after the other
-                for (int c = 0; c < SC_PARTS; ++c) {
+                for (int c = 0; c < SC_PARTS; ++c) {         // the lists one after the other
                     const uint32_t n = __ldcg(o.tickets + c);
                     if (t < n) {
                         const uint2 item = __ldg(o.items + (size_t)c * a.blocks + t);
@@ -244,6 +253,7 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
                     }
                     t -= n;
                 }
+                if (set != ~0u) ticket = gridDim.x + atomicAdd(o.tickets + SC_PARTS, 1u);
             }
             item_slot[0] = set; item_slot[1] = range; item_slot[2] = part;
         }
@@ -302,7 +312,7 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
         [[maybe_unused]] const size_t at = ((size_t)item_slot[2] * a.n_pad + p) * 4 + li;
         if constexpr (ORDERED) {
             const float2 r = __ldg(o.reach + p);
-            if (r.x <= __ldg(a.scalars + SC_TOP)) reach = r.y;
+            if (r.x <= __ldg(a.scalars + SC_DOC_TOP)) reach = r.y;
             known = ordered_to_float(__ldcg(o.bound + p));
             if (TOP2) m2 = known; else m1 = known;
         } else if (!a.first) {
@@ -444,7 +454,7 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
                 if (bits) {
                     const uint32_t n_at = atomicAdd(o.count + p, 1u);
                     if (n_at < (uint32_t)SC_OWN_LIST)
-                        o.list[p * SC_OWN_LIST + n_at] = make_uint4(__float_as_uint(m), (uint32_t)(o.slab0 + sl), bits, (uint32_t)li);
+                        reinterpret_cast<uint4 *>(o.lists + p * SC_LIST_BYTES)[n_at] = make_uint4(__float_as_uint(m), (uint32_t)(o.slab0 + sl), bits, (uint32_t)li);
                 }
             }
             mm_fence_before();                        // the accumulator is free
@@ -516,9 +526,10 @@ static int launch_sweep(const ScreenArgs &a, const OrderedArgs &o, int sms, cuda
         BMU_CUDA(cudaFuncSetAttribute(sweep_screen_kernel<TOP2, ORDERED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SC_SMEM));
         configured[dev] = true;
     }
-    const int64_t items = (int64_t)a.blocks * (ORDERED ? SC_PARTS : a.splits);
-    { sweep_screen_kernel<TOP2, ORDERED><<<(unsigned)(items < sms ? items : sms), SC_THREADS, SC_SMEM, s>>>(a, o); BMU_LAUNCHED(); }
-    BMU_CUDA(cudaGetLastError());
+    const int64_t items = (int64_t)a.blocks * (ORDERED ? SC_PARTS : a.most_splits);
+    ScreenLaunch l((unsigned)(items < sms ? items : sms), SC_THREADS, s, true, SC_SMEM);
+    BMU_CUDA(cudaLaunchKernelEx(&l.c, sweep_screen_kernel<TOP2, ORDERED>, a, o));
+    BMU_LAUNCHED();
     return BMU_OK;
 }
 
