@@ -422,6 +422,134 @@ static int launch_blur_fast(const uint32_t *num, const uint32_t *cnt, int64_t D,
 }
 
 
+// ---- ... and of 16 to 512 units ------------------------------------------------------------
+// A thread owns four neighbouring columns of one plane and walks down its rows.  Column pass in registers: a
+// row is added, packed (fma.rn.f32x2), to the 2R + 1 sums it belongs to, which rotate through the unrolled
+// loop; the sum that is complete goes to shared memory.  Row pass: two complete rows at a time, a thread reads
+// the R columns on either side of its own four.  Rows come by asynchronous copies of sixteen bytes, AHEAD rows
+// ahead, each into a place that only its own thread reads; one barrier per two rows, between two buffers.
+// A block carries as many planes as fit its threads, and all rows of them, or an equal part of them with R more
+// on either side where planes are too few to fill the chip.
+//
+// Bound by HBM up to radius 5 (128 x 128 x 16,384, 2.15 GB: 369 us at radius 2, 374 at 5, 6 TB/s), then by the
+// multiplier, 2 (2R + 1) taps per output (429 at radius 6, 562 at 8).  The tiled kernel above, which exchanges every
+// tile through shared memory twice and is bound by that, took 457, 558, 594 and 677 us.
+template <int R> struct BlurStrip {
+    static constexpr int T = 2 * R + 1, PAD = (R + 3) / 4 * 4;
+    static constexpr int AHEAD = 8;
+    static constexpr int BLOCKS = R <= 2 ? 8 : R <= 4 ? 5 : 4;       // of 128 threads per SM
+};
+
+__device__ __forceinline__ void blur_copy16(uint32_t dst, const void *src, bool there)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(there ? 16 : 0) : "memory");
+}
+
+template <int R>
+__global__ void __launch_bounds__(128, BlurStrip<R>::BLOCKS)
+update_blur_strip_kernel(const uint32_t *__restrict__ num, const uint32_t *__restrict__ cnt, int64_t D,
+                         int32_t edge_x, int32_t edge_y, int32_t planes, int32_t part, const __grid_constant__ BlurTaps taps,
+                         float *__restrict__ num_blur, float *__restrict__ cnt_blur)
+{
+    using S = BlurStrip<R>;
+    constexpr int T = S::T, PAD = S::PAD, AHEAD = S::AHEAD;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    uint4 *ring = reinterpret_cast<uint4 *>(smraw);                          // [AHEAD][blockDim.x]
+    const int pitch = edge_x + 2 * PAD;                                      // floats per plane and row
+    float *rows = reinterpret_cast<float *>(ring + AHEAD * blockDim.x);      // [2][2][planes][pitch]
+    const int lanes = edge_x / 4, mine = (int)threadIdx.x / lanes, x4 = (int)threadIdx.x - mine * lanes;
+    const int64_t M = (int64_t)edge_x * edge_y, plane = (int64_t)blockIdx.x * planes + mine;
+    const bool act = mine < planes && plane <= D;
+    const uint32_t *src = act ? (plane < D ? num + plane * M : cnt) + 4 * x4 : cnt;
+    float *dst = (act && plane < D ? num_blur + plane * M : cnt_blur) + 4 * x4;
+    const int y0 = (int)blockIdx.y * part, y1 = min(edge_y, y0 + part), steps = y1 - y0 + 2 * R;
+    for (int i = threadIdx.x; i < 4 * planes * pitch; i += blockDim.x) rows[i] = 0.f;      // (the columns outside the map)
+    u64 ts[R + 1];
+#pragma unroll
+    for (int k = 0; k <= R; ++k) ts[k] = pack2(taps.g[k].x, taps.g[k].y);
+    const uint32_t slot = (uint32_t)__cvta_generic_to_shared(ring + threadIdx.x);
+    auto fetch = [&](int r) {                                                // row y0 - R + r of the plane
+        const int y = y0 - R + r;
+        const bool in = act && r < steps && y >= 0 && y < edge_y;
+        blur_copy16(slot + (uint32_t)((r % AHEAD) * blockDim.x * 16), src + (int64_t)(in ? y : 0) * edge_x, in);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int r = 0; r < AHEAD - 1; ++r) fetch(r);
+    const int row_floats = planes * pitch, at = (act ? mine : 0) * pitch + PAD + 4 * x4;
+    u64 acc[T][2];
+#pragma unroll
+    for (int k = 0; k < T; ++k) acc[k][0] = acc[k][1] = 0ull;
+    __syncthreads();
+    for (int base = 0; base < steps; base += 2 * T) {
+#pragma unroll
+        for (int k = 0; k < 2 * T; ++k) {
+            const int r = base + k;
+            if (r >= steps + (steps & 1)) break;                             // (an odd last row has a partner that is not there)
+            asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD - 2) : "memory");
+            const uint4 v = ring[(r % AHEAD) * blockDim.x + threadIdx.x];
+            fetch(r + AHEAD - 1);
+            const u64 a = pack2((float)v.x, (float)v.y), b = pack2((float)v.z, (float)v.w);
+#pragma unroll
+            for (int d = 0; d < T; ++d) {                                    // output row r - d, tap |R - d|
+                u64 *s = acc[(k + 2 * T - d) % T];
+                const u64 g = ts[d < R ? R - d : d - R];
+                if (d == 0) { s[0] = s[1] = 0ull; }
+                fma2(s[0], g, a);
+                fma2(s[1], g, b);
+            }
+            float *out = rows + ((r >> 1) & 1) * 2 * row_floats;
+            if (act) {
+                const u64 *s = acc[(k + 1) % T];
+                *reinterpret_cast<float4 *>(out + (k & 1) * row_floats + at) = make_float4(lo_f(s[0]), hi_f(s[0]), lo_f(s[1]), hi_f(s[1]));
+            }
+            if (k & 1) {
+                __syncthreads();
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int y = y0 + r - 1 + h - 2 * R;
+                    if (y < y0 || y >= y1) continue;
+                    const float *c = out + h * row_floats + at - PAD;
+                    float w[4 + 2 * PAD], o[4];
+#pragma unroll
+                    for (int i = 0; i < 4 + 2 * PAD; i += 4) {
+                        const float4 t = *reinterpret_cast<const float4 *>(c + i);
+                        w[i] = t.x; w[i + 1] = t.y; w[i + 2] = t.z; w[i + 3] = t.w;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        o[i] = 0.f;
+#pragma unroll
+                        for (int d = -R; d <= R; ++d) o[i] = fmaf(lo_f(ts[d < 0 ? -d : d]), w[PAD + i + d], o[i]);
+                    }
+                    if (act) __stcs(reinterpret_cast<float4 *>(dst + (int64_t)y * edge_x), make_float4(o[0], o[1], o[2], o[3]));
+                }
+            }
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+template <int R>
+static int launch_blur_strip(const uint32_t *num, const uint32_t *cnt, int64_t D, int32_t edge_x,
+                             int32_t edge_y, const BlurTaps &t, float *num_blur, float *cnt_blur, int sms,
+                             cudaStream_t s)
+{
+    using S = BlurStrip<R>;
+    const int lanes = edge_x / 4, planes = 128 / lanes, threads = (planes * lanes + 31) / 32 * 32;
+    const size_t smem = (size_t)S::AHEAD * threads * 16 + (size_t)4 * planes * (edge_x + 2 * S::PAD) * 4;
+    const int64_t blocks = (D + planes) / planes;
+    // parts of the rows: four waves of blocks, but no more halo rows than a quarter of the others
+    int parts = (int)((4ll * S::BLOCKS * sms + blocks - 1) / blocks);
+    const int most = edge_y / (8 * R) > 1 ? edge_y / (8 * R) : 1;
+    if (parts > most) parts = most;
+    const int part = (edge_y + parts - 1) / parts;
+    const dim3 grid((unsigned)blocks, (unsigned)((edge_y + part - 1) / part));
+    { update_blur_strip_kernel<R><<<grid, threads, smem, s>>>(num, cnt, D, edge_x, edge_y, planes, part, t, num_blur, cnt_blur); BMU_LAUNCHED(); }
+    BMU_CUDA(cudaGetLastError());
+    return BMU_OK;
+}
+
 // b / c, rounded to nearest.  Most sums of a rare feature are 0, which the division hands to its slow
 // path (475 us instead of 335 on such planes): divide something else there.
 __device__ __forceinline__ float writeback_div(float b, float c)
@@ -590,12 +718,29 @@ int launch_update_blur(const uint32_t *num, const uint32_t *cnt, int64_t D, int3
     a.num = num; a.cnt = cnt; a.num_blur = num_blur; a.cnt_blur = cnt_blur;
     a.D = D; a.edge_x = edge_x; a.edge_y = edge_y;
     a.vec = edge_x % 4 == 0 && ((reinterpret_cast<uintptr_t>(num) | reinterpret_cast<uintptr_t>(cnt)) & 15) == 0;
-    // Two kernels.  Maps of whole 16-byte rows at radii up to 8 whose 64 x 64 tiles are at least three
-    // quarters map: the tiled one (128 x 128 x 16,384, radius 2 / 6: 451 / 589 us, the other 616 / 723).
-    // Everything else: the one of whole-map tiles (90 x 70 x 10,007, radius 6 / 20: 230 / 400 us; before it
-    // a kernel with the radius in a loop took 543 / 1721; 32 x 32 x 4,096, radius 6: 33 us, tiled 41).
+    // Maps of whole 16-byte rows of 16 to 512 units at radii up to 8: the kernel that walks down the columns, faster
+    // than the others wherever it was measured there (4,096 x 32 x 32, radius 6: 24 us, 36; 6,000 x 100 x 90: 115, 211;
+    // 2,000 x 512 x 512: 855, 1,165; narrower rows leave its staging too little room, wider ones more than its 128
+    // threads).  Wider maps whose 64 x 64 tiles are at least three quarters map: the tiled one (128 x 128 x 16,384,
+    // radius 2 / 6: 451 / 589 us, that of whole-map tiles 616 / 723).  Everything else: the one of whole-map tiles
+    // (90 x 70 x 10,007, radius 6 / 20: 230 / 400 us; before it a kernel with the radius in a loop took 543 / 1721).
     const int64_t tiled_area = (int64_t)((edge_x + 63) / 64) * ((edge_y + 63) / 64) * 4096;
     const bool outs = ((reinterpret_cast<uintptr_t>(num_blur) | reinterpret_cast<uintptr_t>(cnt_blur)) & 15) == 0;
+    int dev = 0, sms = 148;
+    BMU_CUDA(cudaGetDevice(&dev));
+    BMU_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (a.vec && outs && R >= 1 && R <= 8 && edge_x >= 16 && edge_x <= 512) {
+        switch (R) {
+        case 1: return launch_blur_strip<1>(num, cnt, D, edge_x, edge_y, t, num_blur, cnt_blur, sms, s);
+        case 2: return launch_blur_strip<2>(num, cnt, D, edge_x, edge_y, t, num_blur, cnt_blur, sms, s);
+        case 3: return launch_blur_strip<3>(num, cnt, D, edge_x, edge_y, t, num_blur, cnt_blur, sms, s);
+        case 4: return launch_blur_strip<4>(num, cnt, D, edge_x, edge_y, t, num_blur, cnt_blur, sms, s);
+        case 5: return launch_blur_strip<5>(num, cnt, D, edge_x, edge_y, t, num_blur, cnt_blur, sms, s);
+        case 6: return launch_blur_strip<6>(num, cnt, D, edge_x, edge_y, t, num_blur, cnt_blur, sms, s);
+        case 7: return launch_blur_strip<7>(num, cnt, D, edge_x, edge_y, t, num_blur, cnt_blur, sms, s);
+        default: return launch_blur_strip<8>(num, cnt, D, edge_x, edge_y, t, num_blur, cnt_blur, sms, s);
+        }
+    }
     if (a.vec && outs && R >= 1 && R <= 8 && 3 * tiled_area <= 4 * (int64_t)edge_x * edge_y) {
         switch (R) {
         case 1: return launch_blur_fast<1>(num, cnt, D, edge_x, edge_y, t, num_blur, cnt_blur, s);

@@ -102,6 +102,23 @@ def test_blur_at_the_edges_of_its_tiles(bmu, ex, ey, sigma):
         np.testing.assert_allclose(cb.cpu().numpy(), oracle.blur(cnt.numpy(), ex, ey, sigma), rtol=6e-6, atol=1e-4)
 
 
+@pytest.mark.parametrize("ex,ey,D", [(16, 1, 140), (20, 7, 70), (44, 33, 25), (128, 127, 2), (132, 40, 3), (260, 25, 2),
+                                     (512, 30, 2), (516, 66, 1), (12, 40, 9)])
+@pytest.mark.parametrize("radius", [1, 2, 3, 4, 5, 6, 7, 8])
+def test_blur_of_columns_in_registers(bmu, ex, ey, D, radius):
+    """Rows of whole 16-byte pieces: odd and even numbers of rows, more planes than a block holds and fewer, rows in
+    parts, the widths at either end of the kernel's range; every radius is an instance of its own."""
+    M, sigma = ex * ey, radius / 3 - 1e-4
+    g = torch.Generator().manual_seed(ex + ey + radius)
+    num = torch.randint(0, 2_000_000, (D, M), generator=g, dtype=torch.int32)
+    cnt = torch.randint(0, 50, (M,), generator=g, dtype=torch.int32)
+    nb, cb = bmu.bmu_update_blur(num.cuda(), cnt.cuda(), ex, ey, sigma)
+    for got, ref in ((nb.cpu().numpy(), oracle.blur(num.numpy(), ex, ey, sigma)),
+                     (cb.cpu().numpy()[None], oracle.blur(cnt.numpy()[None], ex, ey, sigma).reshape(1, -1))):
+        got, ref = got.reshape(ref.shape[0], -1), ref.reshape(ref.shape[0], -1)
+        assert np.all(np.abs(got - ref) <= 2e-6 * ref.max(axis=1, keepdims=True))
+
+
 def test_blur_refuses_a_neighbourhood_it_cannot_hold(bmu):
     num = torch.zeros((1, 64), dtype=torch.int32, device="cuda")
     cnt = torch.zeros(64, dtype=torch.int32, device="cuda")
