@@ -33,15 +33,20 @@
 // 1.71 ms, 60,000 against an fp16 256 x 256 map 22.7 / 11.3 ms.
 //
 // The blocks stay, one per SM, and take sets of 128 documents and stretches of slabs one after the other; barriers and
-// accumulators go on from item to item.
+// accumulators go on from item to item: 200,000 documents on a trained 128 x 128 map 9.81 -> 9.62 ms, 30,011 on 75 x 75
+// 686 -> 663 us.
 //
 // ORDERED: slabs in the order of the norms (screen.cuh, screen_order.cu).  What differs:
 //   items      a set of documents reaches a few slabs of a launch, another set many: (set, up to SC_PART slabs),
-//              from the lists that screen_image_kernel has made, the first parts of all sets before the second ones.
+//              from the lists that screen_ordered_image_kernel makes, the first parts of all sets before the second ones.
 //   stopping   a warp leaves an item at the first slab that no document of its tile reaches any more.
 //   candidates the bound of a document's smallest value is good from the start and slabs with the smallest
 //              norms come first, so that little is ever within a window: what is, is looked up once more, unit by
 //              unit, and joins the document's one list.  Parts of the same set share list and bound by atomics.
+//   head first once a slab has brought the warp no candidate, the next ones are looked at with the head's sums and the
+//              most that the gathered rows could add; where that rules a slab out its rows are not gathered (for
+//              120,000 documents on 64 x 64 the search 970 -> 885 us).
+// The same documents take 1,255 us with all slabs in the order of the map; 100,000 on 512 x 512 57,000 and 1,500.
 
 #include "screen.cuh"
 #include "mma_ptx.cuh"
@@ -61,7 +66,7 @@ static const int SC_TAIL_REGS = 112, SC_CTRL_REGS = 32;      // registers after 
 static const int SC_KS = 4, SC_NS = 2;
 // Tensor memory: the accumulators from column 0 -- two that alternate between slabs if X_head
 // leaves room (up to 1024 features), else one --, X_head in the last head_pad / 4 columns.
-static const size_t SC_SMEM = SC_NS * SC_KS * MMA_STAGE_BYTES + (2 * SC_NS + 5) * 8 + 24;
+static const size_t SC_SMEM = SC_NS * SC_KS * MMA_STAGE_BYTES + (2 * SC_NS + 5) * 8 + 32;
 
 // Adds the sixteen bytes of two rows to a lane's sums.  acc[w] holds the sum of words w modulo 2^32,
 // acc[4 + w] the 16-bit sums of their bytes 1 and 3; sc_even takes those out of the former.
@@ -223,25 +228,35 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
     } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SC_TAIL_REGS));
     const int q = warp & 3, e = warp >> 2;
-    // (thread 0: the block's own item first; the ticket of the next one is on its way while an item is swept)
-    [[maybe_unused]] const uint32_t splits = (uint32_t)screen_parts(a.scalars, a.splits, a.most_splits);
-    [[maybe_unused]] const uint32_t items = (natural == SC_ALL ? (uint32_t)a.blocks : natural) * splits;
-    uint32_t ticket = blockIdx.x;
+    // Thread 0: the block's own item first; the ticket of the next one is on its way under an item's last slab (not
+    // from the item's beginning: whoever waits for a long one must not hold another).  As many tickets as items are
+    // taken, if any: then the counter is zero again.
+    auto sets_of = [&]() { const uint32_t n = screen_natural(a.scalars); return n == SC_ALL ? (uint32_t)a.blocks : n; };
+    auto take = [&]() {
+        if (threadIdx.x) return;
+        uint32_t t;
+        if (ORDERED) {
+            t = atomicAdd(o.tickets + SC_PARTS, 1u);
+        } else {
+            const uint32_t items = sets_of() * (uint32_t)screen_parts(a.scalars, a.splits, a.most_splits);
+            t = items > gridDim.x ? atomicInc(a.ticket, items - 1u) : items;
+        }
+        item_slot[3] = gridDim.x + t;
+    };
+    if (threadIdx.x == 0) item_slot[3] = blockIdx.x;
     for (;;) {
         // the next item (a block that gave up: let the grid drain)
         if (threadIdx.x == 0) {
             uint32_t set = ~0u, range = 0u, part = 0u;       // (no set: there are no more items)
-            uint32_t t = ticket;
+            uint32_t t = item_slot[3];
             if (*abort_flag || *reinterpret_cast<volatile uint32_t *>(a.status)) {
             } else if (!ORDERED) {
-                if (t < items) {
-                    const uint32_t sets = items / splits;
+                const uint32_t sets = sets_of(), splits = (uint32_t)screen_parts(a.scalars, a.splits, a.most_splits);
+                if (t < sets * splits) {
                     set = t % sets;
                     part = t / sets;
-                    if (natural != SC_ALL) set = __ldg(a.nat_list + set);
+                    if (screen_natural(a.scalars) != SC_ALL) set = __ldg(a.nat_list + set);
                     range = (uint32_t)a.n_slabs * part / splits | (uint32_t)a.n_slabs * (part + 1) / splits << 16;
-                    // (as many tickets as items are taken, if any: then the counter is zero again)
-                    ticket = items > gridDim.x ? gridDim.x + atomicInc(a.ticket, items - 1u) : items;
                 }
             } else {
                 for (int c = 0; c < SC_PARTS; ++c) {         // the lists one after the other
@@ -253,18 +268,17 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
                     }
                     t -= n;
                 }
-                if (set != ~0u) ticket = gridDim.x + atomicAdd(o.tickets + SC_PARTS, 1u);
             }
             item_slot[0] = set; item_slot[1] = range; item_slot[2] = part;
         }
         block_sync();
         if (item_slot[0] == ~0u) break;
-        const int64_t group = item_slot[0];
+        const int group = (int)item_slot[0];
         const int s_lo = (int)(item_slot[1] & 0xffffu), s_hi = (int)(item_slot[1] >> 16), slabs = s_hi - s_lo;
         {
             // X_head into tensor memory: lane 32q + l = document, a column = four features
             const int words = a.head / 32;
-            const int64_t p = group * SC_DOCS + 32 * q + lane;
+            const int64_t p = (int64_t)group * SC_DOCS + 32 * q + lane;
             const bool there = p < a.n_tiles * 8;
             for (int wd = e; wd < a.head_pad / 32; wd += 4) {
                 const uint32_t m = there && wd < words ? __ldg(a.tile_head + (size_t)p * words + wd) : 0u;
@@ -288,7 +302,7 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
         const u64 sh = sc_pack(__ldg(a.scalars), __ldg(a.scalars)), st = sc_pack(__ldg(a.scalars + 1), __ldg(a.scalars + 1));
         const u64 minus_2p23 = sc_pack(-8388608.f, -8388608.f);
         const size_t slab_bytes = (size_t)(a.D + 1) * SC_SLAB;
-        const int64_t tile = group * (SC_DOCS / 8) + 4 * q + e;
+        const int tile = group * (SC_DOCS / 8) + 4 * q + e;
         uint32_t quads = 0;                                              // groups of four rows
         const uint4 *ids = a.tile_ids;
         [[maybe_unused]] size_t room = a.tile_rows_cap;
@@ -299,7 +313,7 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
             ids += off; room -= off;
         }
         ids += s;
-        const int64_t p = tile * 8 + (lane >> 2);                        // this lane's document
+        const uint32_t p = (uint32_t)tile * 8 + (lane >> 2);             // this lane's document
         const float win = __ldg(a.window + p);
         float m1 = 3.0e38f, m2 = 3.0e38f;                                // smallest (and second) value of the document
         // ORDERED: how far it reaches (evaluated whole: not at all), and what bounds its smallest (second) value
@@ -309,7 +323,7 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
         [[maybe_unused]] float own = 3.0e38f;
         [[maybe_unused]] uint32_t mask = 0u;
         [[maybe_unused]] int valid = s_lo;
-        [[maybe_unused]] const size_t at = ((size_t)item_slot[2] * a.n_pad + p) * 4 + li;
+        auto stripe = [&]() { return ((size_t)item_slot[2] * a.n_pad + p) * 4 + li; };
         if constexpr (ORDERED) {
             const float2 r = __ldg(o.reach + p);
             if (r.x <= __ldg(a.scalars + SC_DOC_TOP)) reach = r.y;
@@ -332,14 +346,20 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
             d[0] = piece(x0, sel_own);   d[1] = piece(x1, sel_own);
             d[2] = piece(x0, sel_other); d[3] = piece(x1, sel_other);
         };
-        if (quads) {
+        auto begin = [&]() {                                             // the first quad of the slab at `base`
             const uint4 i0 = quad(0);
             ix = quad(quads > 1 ? 1 : 0);
             load(base, w, i0.x, i0.y);
             load(base, w + 4, i0.z, i0.w);
-        }
+        };
+        // ORDERED: whether the head alone is looked at first, and whether a slab's first quad is on its way
+        [[maybe_unused]] bool head_first = ORDERED && o.slab0 + s_lo > 0, begun = !head_first;
+        [[maybe_unused]] const u64 tail_most = sc_pack((float)(4u * quads) * __ldg(a.scalars + 4), (float)(4u * quads) * __ldg(a.scalars + 4));
+        if (quads && begun) begin();
+        bool taken = false;
         for (int sl = s_lo; sl < s_hi; ++sl, np += SC_SLAB) {
             const int n = done + sl - s_lo;
+            if (sl + 1 == s_hi) { take(); taken = true; }
             // no document of the tile reaches this slab, nor any behind it: the accumulators still change hands
             if (ORDERED && !__any_sync(0xffffffffu, __ldg(o.unit_norm + sl * SC_SLAB) <= (TOP2 ? m2 : m1) + win + reach)) {
                 for (int r = n; r < done + slabs; ++r) {
@@ -348,6 +368,54 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
                     if (lane == 0) mm_bar_arrive(tempty0 + 8 * (r & two));
                 }
                 break;
+            }
+            const uint32_t taddr = tmem + ((uint32_t)(q * 32 + (e >> 1) * 16) << 16) + (uint32_t)((n & two) * 128);
+            // integer head sums of eight neurons of the lane's 32 (the load covers two tiles of documents), and their norms
+            [[maybe_unused]] auto head8 = [&](int c, uint32_t hs[8], u64 nm[4]) {
+                uint32_t v[16];
+                mm_tmem_ld_16x256b_x4(taddr + c * 32, v);
+                const ulonglong2 n0 = __ldg(reinterpret_cast<const ulonglong2 *>(np + (2 * c) * 16));
+                const ulonglong2 n1 = __ldg(reinterpret_cast<const ulonglong2 *>(np + (2 * c + 1) * 16));
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    hs[2 * k] = (e & 1) ? v[4 * k + 2] : v[4 * k];
+                    hs[2 * k + 1] = (e & 1) ? v[4 * k + 3] : v[4 * k + 1];
+                }
+                nm[0] = n0.x; nm[1] = n0.y; nm[2] = n1.x; nm[3] = n1.y;
+            };
+            if constexpr (ORDERED) {
+                if (head_first) {
+                    // what the gathered rows can add at most: if that rules the slab out, they are not gathered
+                    mm_wait(tfull0 + 8 * (n & two), (n >> two) & 1, abort_flag, a.status, 8u);
+                    mm_fence_after();
+                    float least = CUDART_INF_F;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        uint32_t hs[8];
+                        u64 nm[4];
+                        head8(c, hs, nm);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const u64 x = sc_fma2(sc_pack(__uint2float_rn(hs[2 * k]), __uint2float_rn(hs[2 * k + 1])), sh, nm[k]);
+                            least = fminf(least, fminf(lo_f(x), hi_f(x)));
+                        }
+                    }
+                    // (the same operation as sc_dist2's last, with the largest sum there can be: never above what that gives)
+                    least = lo_f(sc_fma2(tail_most, st, sc_pack(least, least)));
+                    if (!__any_sync(0xffffffffu, least <= (TOP2 ? m2 : m1) + win)) {
+                        mm_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mm_bar_arrive(tempty0 + 8 * (n & two));
+                        begun = false;
+                        continue;
+                    }
+                }
+                if (!begun) {
+                    base = a.img8 + (size_t)sl * slab_bytes + (lane & 7) * 16;
+                    if (quads) begin();
+                    begun = true;
+                }
             }
             uint32_t acc[2][8];                       // own, other document
 #pragma unroll
@@ -378,39 +446,54 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
             }
             mm_wait(tfull0 + 8 * (n & two), (n >> two) & 1, abort_flag, a.status, 8u);
             mm_fence_after();
-            const uint32_t taddr = tmem + ((uint32_t)(q * 32 + (e >> 1) * 16) << 16) + (uint32_t)((n & two) * 128);
-            auto dist8 = [&](int c, u64 x[4], auto last) {
-                uint32_t v[16];
-                mm_tmem_ld_16x256b_x4(taddr + c * 32, v);
-                const ulonglong2 n0 = __ldg(reinterpret_cast<const ulonglong2 *>(np + (2 * c) * 16));
-                const ulonglong2 n1 = __ldg(reinterpret_cast<const ulonglong2 *>(np + (2 * c + 1) * 16));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (decltype(last)::value && c == 3) {        // the accumulator is free
-                    mm_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mm_bar_arrive(tempty0 + 8 * (n & two));
-                }
-                uint32_t hs[8];                       // (the load covers two tiles of documents)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    hs[2 * k] = (e & 1) ? v[4 * k + 2] : v[4 * k];
-                    hs[2 * k + 1] = (e & 1) ? v[4 * k + 3] : v[4 * k + 1];
-                }
+            [[maybe_unused]] auto dist8 = [&](int c, u64 x[4]) {
+                uint32_t hs[8];
+                u64 nm[4];
+                head8(c, hs, nm);
                 const uint32_t *t = c < 2 ? lo : hi;
                 const int w0 = 2 * (c & 1);
-                x[0] = sc_dist2(n0.x, hs[0], hs[1], t[w0], sh, st, minus_2p23);
-                x[1] = sc_dist2(n0.y, hs[2], hs[3], t[4 + w0], sh, st, minus_2p23);
-                x[2] = sc_dist2(n1.x, hs[4], hs[5], t[w0 + 1], sh, st, minus_2p23);
-                x[3] = sc_dist2(n1.y, hs[6], hs[7], t[5 + w0], sh, st, minus_2p23);
+                x[0] = sc_dist2(nm[0], hs[0], hs[1], t[w0], sh, st, minus_2p23);
+                x[1] = sc_dist2(nm[1], hs[2], hs[3], t[4 + w0], sh, st, minus_2p23);
+                x[2] = sc_dist2(nm[2], hs[4], hs[5], t[w0 + 1], sh, st, minus_2p23);
+                x[3] = sc_dist2(nm[3], hs[6], hs[7], t[5 + w0], sh, st, minus_2p23);
             };
-            // the distances of eight neurons of the lane's 32 at a time, in pairs
             float mc[4];
+            if constexpr (ORDERED) {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                u64 x[4];
-                dist8(c, x, std::integral_constant<bool, !ORDERED>());
-                mc[c] = fminf(fminf(fminf(lo_f(x[0]), hi_f(x[0])), fminf(lo_f(x[1]), hi_f(x[1]))),
-                              fminf(fminf(lo_f(x[2]), hi_f(x[2])), fminf(lo_f(x[3]), hi_f(x[3]))));
+                for (int c = 0; c < 4; ++c) {
+                    u64 x[4];
+                    dist8(c, x);
+                    mc[c] = fminf(fminf(fminf(lo_f(x[0]), hi_f(x[0])), fminf(lo_f(x[1]), hi_f(x[1]))),
+                                  fminf(fminf(lo_f(x[2]), hi_f(x[2])), fminf(lo_f(x[3]), hi_f(x[3]))));
+                }
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {             // eight neurons of the lane's 32 at a time
+                    uint32_t v[16];
+                    mm_tmem_ld_16x256b_x4(taddr + c * 32, v);
+                    const ulonglong2 n0 = __ldg(reinterpret_cast<const ulonglong2 *>(np + (2 * c) * 16));
+                    const ulonglong2 n1 = __ldg(reinterpret_cast<const ulonglong2 *>(np + (2 * c + 1) * 16));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (c == 3) {                         // the accumulator is free
+                        mm_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mm_bar_arrive(tempty0 + 8 * (n & two));
+                    }
+                    uint32_t hs[8];                       // (the load covers two tiles of documents)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        hs[2 * k] = (e & 1) ? v[4 * k + 2] : v[4 * k];
+                        hs[2 * k + 1] = (e & 1) ? v[4 * k + 3] : v[4 * k + 1];
+                    }
+                    const uint32_t *t = c < 2 ? lo : hi;
+                    const int w0 = 2 * (c & 1);
+                    const u64 x0 = sc_dist2(n0.x, hs[0], hs[1], t[w0], sh, st, minus_2p23);
+                    const u64 x1 = sc_dist2(n0.y, hs[2], hs[3], t[4 + w0], sh, st, minus_2p23);
+                    const u64 x2 = sc_dist2(n1.x, hs[4], hs[5], t[w0 + 1], sh, st, minus_2p23);
+                    const u64 x3 = sc_dist2(n1.y, hs[6], hs[7], t[5 + w0], sh, st, minus_2p23);
+                    mc[c] = fminf(fminf(fminf(lo_f(x0), hi_f(x0)), fminf(lo_f(x1), hi_f(x1))),
+                                  fminf(fminf(lo_f(x2), hi_f(x2)), fminf(lo_f(x3), hi_f(x3))));
+                }
             }
             // the document's smallest (and second smallest) value over its four lanes
             const float m = fminf(fminf(mc[0], mc[1]), fminf(mc[2], mc[3]));
@@ -435,18 +518,19 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
                     mask |= ((mc[0] <= limit ? 1u : 0u) | (mc[1] <= limit ? 2u : 0u) | (mc[2] <= limit ? 4u : 0u) |
                              (mc[3] <= limit ? 8u : 0u)) << (4 * (sl & 7));
                 if ((sl & 7) == 7 || sl + 1 == s_hi) {
-                    reinterpret_cast<uint32_t *>(a.cmask + at)[sl >> 3] = mask;
+                    reinterpret_cast<uint32_t *>(a.cmask + stripe())[sl >> 3] = mask;
                     mask = 0u;
                 }
                 continue;
             }
             // some unit of the warp's is within a window: which ones, from the sums once more
-            if (__any_sync(0xffffffffu, m <= limit)) {
+            head_first = !__any_sync(0xffffffffu, m <= limit);
+            if (!head_first) {
                 uint32_t bits = 0u;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     u64 x[4];
-                    dist8(c, x, std::false_type());
+                    dist8(c, x);
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
                         bits |= ((lo_f(x[i]) <= limit ? 1u : 0u) | (hi_f(x[i]) <= limit ? 2u : 0u)) << (8 * c + 2 * i);
@@ -454,7 +538,7 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
                 if (bits) {
                     const uint32_t n_at = atomicAdd(o.count + p, 1u);
                     if (n_at < (uint32_t)SC_OWN_LIST)
-                        reinterpret_cast<uint4 *>(o.lists + p * SC_LIST_BYTES)[n_at] = make_uint4(__float_as_uint(m), (uint32_t)(o.slab0 + sl), bits, (uint32_t)li);
+                        reinterpret_cast<uint4 *>(o.lists + (size_t)p * SC_LIST_BYTES)[n_at] = make_uint4(__float_as_uint(m), (uint32_t)(o.slab0 + sl), bits, (uint32_t)li);
                 }
             }
             mm_fence_before();                        // the accumulator is free
@@ -465,9 +549,10 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
             const float found = TOP2 ? m2 : m1;
             if (li == 0 && found < known) atomicMin(o.bound + p, float_to_ordered(found));
         } else {
-            a.cval[at] = make_float2(own, __int_as_float(valid | (s_hi << 8)));
-            if (TOP2) a.cval2[at] = m2;
+            a.cval[stripe()] = make_float2(own, __int_as_float(valid | (s_hi << 8)));
+            if (TOP2) a.cval2[stripe()] = m2;
         }
+        if (!taken) take();
         done += slabs;
         mm_fence_before();
         block_sync();
