@@ -49,8 +49,9 @@ void screen_layout(int64_t D, int64_t M, int64_t N, int head, int64_t chunk, boo
     const size_t n4 = (size_t)l->n_pad * 4;
     const int64_t room = screen_split_blocks(blocks, slabs, sms);
     const size_t stripes = (size_t)room * SC_DOCS * 4;
-    l->most_splits = (int)(room / blocks < slabs ? room / blocks : slabs);
-    if (l->most_splits > 16) l->most_splits = 16;
+    // (what they take together is within `room`, as screen_splits has it)
+    const int64_t most = blocks > 0 ? room / blocks : 1, cap = slabs < 16 ? slabs : 16;
+    l->most_splits = (int)(most < cap ? most : cap);
     if (l->most_splits < l->splits) l->most_splits = l->splits;
     codebook_layout(D, M, l->chunk_slabs, 0, 1, take, l);
     // a quarter of the launches' slabs: far beyond that the order of the map is the better one
