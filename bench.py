@@ -409,6 +409,10 @@ def measure_config(bmu, cfg, args, dev, rank, world, roofs, peaks, steps, warmup
         "fractions": {k: v[0] / v[1] for k, v in alg.items()},
         **extra,
     }
+    if desc.two_stage:
+        # units that a norm rules out are counted all the same
+        roofline["counts"] = ("every (document, unit) pair; the two-stage search sums only those that the units' norms "
+                              "leave, a few per cent on this codebook: fractions are of the work of summing all")
     frag = {
         "value": value, "ms_per_step": ms_per_step,
         "updates_per_s": float(total_nnz) * cfg.M * world / (ms_per_step * 1e-3),
