@@ -157,6 +157,13 @@ struct VerifyArgs {
     int32_t splits, most_splits, first, f16;
 };
 
+// In which order the fp32 weights of a unit are added wherever it is evaluated: N partial sums, the i-th over ids i,
+// i + N, ... of the list, then i and i + N / 2 of them, and so on (rows that are not whole 16-byte pieces, VEC false:
+// 0 and 1, 2 and 3, then those two).  As many as rows are loaded side by side in the verify stage.
+template <typename WT, bool VEC> struct ScreenSums {
+    static constexpr int N = !VEC ? 4 : sizeof(WT) == 4 ? 16 : 32;
+};
+
 #ifdef __CUDACC__
 // Most of the sampled documents are better evaluated whole: nothing is screened, all documents are.
 __device__ __forceinline__ bool screen_whole(const float *scalars)

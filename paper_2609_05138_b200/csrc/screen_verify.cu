@@ -53,6 +53,7 @@ template <typename WT>
 struct VerifyVec {
     static constexpr int V = 16 / (int)sizeof(WT), LPR = SC_GROUP / V, RS = 32 / LPR;
     static constexpr int REST = V == 4 ? 6 : 3;              // lane bits left over
+    static_assert(RS == ScreenSums<WT, true>::N, "a partial sum per row lane");
     using Vec = typename std::conditional<V == 4, float4, uint4>::type;
 
     static __device__ __forceinline__ void ids_of(const VerifyArgs &a, int e, int end, uint32_t ids[4])
@@ -412,7 +413,7 @@ template <typename WT, bool TOP2, bool VEC>
 __global__ void __launch_bounds__(256, 5)
 screen_verify_units_kernel(const VerifyArgs a)
 {
-    constexpr int L = VEC ? VerifyVec<WT>::RS : 4, AT_ONCE = 32 / L, U = VEC ? 4 : 16;
+    constexpr int L = ScreenSums<WT, VEC>::N, AT_ONCE = 32 / L, U = VEC ? 4 : 16;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int lane = threadIdx.x & 31, row = lane % L;

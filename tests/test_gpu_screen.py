@@ -451,3 +451,62 @@ def test_batches_that_reach_further_than_the_first(bmu):
         parity.compare(ob.numpy(), od.numpy(), W.cpu().numpy(), rp.numpy(), ci.numpy(), docs=np.arange(0, 2000, 97))
         assert float((ob == rb.cpu()).float().mean()) > 0.999
         assert bool(((od - rd.cpu()).abs() <= 1e-5 * rd.cpu().abs()).all())
+
+
+def added_as_documented(W, norms, rowptr, colidx, whole_rows):
+    """Distances with a unit's weights in partial sums over every 16th id (32nd: fp16; 4th: rows that are not whole
+    16-byte pieces), added in pairs, all in fp32.  (The 64-bit sum under a rounding to 32 is the fused one.)"""
+    parts = 4 if not whole_rows else 32 if W.dtype == np.float16 else 16
+    bmu, dist = [], []
+    for i in range(len(rowptr) - 1):
+        ids = colidx[rowptr[i]:rowptr[i + 1]]
+        s = np.zeros((parts, W.shape[1]), dtype=np.float32)
+        for e, f in enumerate(ids):
+            s[e % parts] += W[f].astype(np.float32)
+        while len(s) > 1:
+            s = s[:len(s) // 2] + s[len(s) // 2:] if whole_rows else s[0::2] + s[1::2]
+        d = (norms.astype(np.float64) - 2.0 * s[0].astype(np.float64)).astype(np.float32)
+        bmu.append(int(d.argmin()))
+        dist.append(np.float32(len(ids)) + d.min())
+    return np.array(bmu, dtype=np.int32), np.array(dist, dtype=np.float32)
+
+
+@pytest.mark.parametrize("M,f16", [(1280, False), (1003, False), (1280, True)])
+def test_a_distance_is_the_same_whichever_way_it_was_evaluated(bmu, M, f16):
+    """The same documents by themselves, where candidates are verified, and among twice as many long lists, where
+    all documents are evaluated whole: the same bits, and those of the order of additions that is documented."""
+    D = 3000
+    r = np.random.default_rng(21)
+    lens = [0, 1, 3, 4, 5, 7, 15, 16, 17, 31, 32, 33, 47, 48, 63, 64, 65, 80, 81, 127, 128, 129, 200, 300]
+    some, many = lists(lens, D, 22), lists(lens + [int(n) for n in r.integers(1100, 1400, 2 * len(lens) + 8)], D, 22)
+    W = torch.rand((D, M), generator=torch.Generator().manual_seed(23)) * torch.rand((D, 1), generator=torch.Generator().manual_seed(24))
+    W = W.cuda().half() if f16 else W.cuda()
+    norms = (bmu.bmu_codebook_norms_f16 if f16 else bmu.bmu_codebook_norms)(W)
+    search = bmu.bmu_search_f16_ws if f16 else bmu.bmu_search_ws
+    n = len(lens)
+    want = added_as_documented(W.cpu().numpy(), norms.cpu().numpy(), some[0].numpy(), some[1].numpy(), M % 4 == 0)
+    for rowptr, colidx in (some, many):
+        assert torch.equal(colidx[:some[1].numel()], some[1])
+        ob, od = search(W, rowptr.cuda(), colidx.cuda(), norms=norms, opts=opts_of(bmu, head_rows=64))[:2]
+        np.testing.assert_array_equal(ob[:n].cpu().numpy(), want[0])
+        np.testing.assert_array_equal(od[:n].cpu().numpy(), want[1])
+
+
+def test_a_document_is_answered_alike_in_any_company(bmu):
+    """Documents on both sides of the reach up to which slabs are swept in the order of the norms: the whole corpus,
+    parts of it (which draw the line elsewhere), other chunks, a plan, and the same call again."""
+    D, M, n, dev = 16384, 4096, 120_000, torch.device("cuda")
+    lens = synth.draw_nnz("poisson", 80.0, n, torch.Generator(device=dev).manual_seed(4), dev)
+    rp, ci = synth.draw_corpus(n, D, 1.0, lens, 4, dev)
+    W = synth.make_codebook(D, M, 5, dev)
+    ob, od = bmu.bmu_search_ws(W, rp, ci)
+    same = [bmu.bmu_search_ws(W, rp, ci) for _ in range(3)]
+    same += [bmu.bmu_search_ws(W, rp, ci, opts=opts_of(bmu, chunk_neurons=c)) for c in (512, 1024)]
+    plan = bmu.Plan(rp, ci, D, M)
+    same.append(plan.search(W))
+    parts = [bmu.bmu_search_ws(W, (rp[a:b + 1] - rp[a]).contiguous(), ci[int(rp[a]):int(rp[b])].contiguous(), opts=opts_of(bmu))
+             for a, b in ((0, 30_000), (30_000, 37_000), (37_000, n))]
+    same.append([torch.cat([x[i] for x in parts]) for i in (0, 1)])
+    for k, (sb, sd) in enumerate(same):
+        assert torch.equal(sb, ob) and torch.equal(sd, od), (k, int((sb != ob).sum()), int((sd != od).sum()))
+    plan.close()
