@@ -8,19 +8,22 @@
 // every sixteenth id, added in pairs), so that a unit has the same distance, bit for bit, whichever way it came
 // here: which documents come depends on the others in the call, and on when a bound was lowered.
 //
-// A warp takes a document and a piece of 512 units, 64 of them at a time (128 where rows are not whole 16-byte
-// pieces).  Two halves of the warp take every other id (fp16: four quarters every fourth), a lane carries the
-// partial sums of its ids for the four (eight) units of a 16-byte load; the next row of a partial sum is asked for
-// as soon as the one before has been added, also across the 64s, ids through shared memory.  Pieces outside, documents
-// inside, so that all warps in flight share one piece or two: rows of W in L2, those of frequent features in L1.
-// Keys meet in the per-document state; the warp that arrives last at a document (a ticket each) writes its outputs.
+// A warp takes a document and a piece of 384 units (fp16: 1,024), 128 of them at a time, in two passes: the partial
+// sums of the even places of the list, then those of the odd ones.  A lane carries the partial sums of four (fp16: eight,
+// where half of the warp takes every other id of a pass) units, 32 (64) registers, and asks for the next row of each as
+// soon as the one before has been added, also across passes and stretches; ids through shared memory.  Pieces outside,
+// documents inside, so that all warps in flight share one piece or two: rows of W in L2, those of frequent features
+// in L1.  Keys meet in the per-document state; the warp that arrives last at a document (a ticket each) writes its
+// outputs.
 //
-// Bound by the latency of its loads: 64 KB in flight per SM, which the sums' registers bound.  All of 50,000
-// documents of 80 ids on 4,096 units take 3.3 ms, 20,000 on 16,384 units 5.4, 50,000 on 4,096 units of fp16 3.4,
-// 20,000 on 4,099 units 1.9.  (One sum per unit over all ids, eight units to a lane, twice the warps: 3.0, 5.8, 2.8
-// and 2.2, with distances of its own.)  The sixteen sums one after the other, those that wait for their pair in
-// registers or shared memory: 3.8, 6.4, 4.6, 2.6.  Pieces of 64, 128, 256 and 1,024 units: 4.8, 4.0, 3.6 and 3.8 for
-// the first; twelve warps in two blocks 4.5.
+// Bound by the latency of its loads, 64 KB in flight per SM, which the sums' registers bound, and by L1 hits.  All of
+// 50,000 documents of 80 ids on 4,096 units take 3.1 ms, 20,000 on 16,384 units 5.3, 50,000 on 4,096 units of fp16 3.1,
+// 20,000 on 4,099 units 1.9.  (One sum per unit over all ids, eight units to a lane, twice the warps: 3.0, 5.6, 2.8
+// and 2.2, with distances of its own.)  Pieces of 256, 512 and 768 units: 3.3 / 5.4, 3.0 / 6.4, 3.3 / 6.6 for the first two.
+// One pass over 64 units, half of the warp for each half of the list: 3.3, 5.4, 3.4; the sixteen sums one after the
+// other, those that wait for their pair in registers or shared memory: 3.8, 6.4, 4.6, 2.6; rows asked for sixteen at a time
+// and then added: 3.6, 5.9, 4.0; touching a piece's rows ahead in L2: 3.4, 5.5, 3.5, and 5 % more for 100,000 documents
+// on 512 x 512.
 #include "screen.cuh"
 
 #include <cuda_fp16.h>
@@ -51,35 +54,34 @@ __device__ __forceinline__ void dense_add(u64 *acc, const u64 w[2])
 __device__ __forceinline__ float dense_ld(const float *p) { return __ldg(p); }
 __device__ __forceinline__ float dense_ld(const __half *p) { return __half2float(__ldg(p)); }
 
-// A list's partial sums are shared out to GROUPS groups of lanes, SUMS to a lane; a lane owns V units of a stretch of
-// UNITS, VEC: with one load per row.
+// A list's partial sums are shared out to PASSES over a stretch of UNITS and, in each, GROUPS groups of lanes: SUMS to a
+// lane, which owns V units of the stretch, VEC: with one load per row.
 template <typename WT, bool VEC> struct Dense {
     using Sums = ScreenSums<WT, VEC>;
-    static constexpr int V = VEC ? 16 / (int)sizeof(WT) : 4, GROUPS = !VEC ? 1 : V == 4 ? 2 : 4;
-    static constexpr int LANES = 32 / GROUPS, UNITS = LANES * V, SUMS = Sums::N / GROUPS;
-    static constexpr int WARPS = VEC ? 16 : 24;              // of the one block per SM
+    static constexpr int V = VEC ? 16 / (int)sizeof(WT) : 4, PASSES = VEC ? 2 : 1, GROUPS = VEC && V == 8 ? 2 : 1;
+    static constexpr int LANES = 32 / GROUPS, UNITS = LANES * V, SHARES = PASSES * GROUPS, SUMS = Sums::N / SHARES;
+    static constexpr int WARPS = VEC ? 16 : 24, PIECE = V == 8 ? 1024 : 384;     // of the one block per SM; units of an item
 };
-static const int DENSE_PIECE = 512, DENSE_IDS = 128;
+static const int DENSE_IDS = 128;
 
 template <typename WT, bool TOP2, bool VEC>
 __global__ void __launch_bounds__(Dense<WT, VEC>::WARPS * 32, 1)
 screen_dense_kernel(const VerifyArgs a)
 {
     using X = Dense<WT, VEC>;
-    constexpr int P = X::Sums::N, C = X::SUMS, V = X::V, H = V / 2, GROUPS = X::GROUPS;
-    __shared__ uint4 s_ids[X::WARPS][DENSE_IDS / 4];         // the ids of a group of lanes one after the other
+    constexpr int P = X::Sums::N, C = X::SUMS, V = X::V, H = V / 2, SHARES = X::SHARES, OWN = V / X::GROUPS;
+    __shared__ uint4 s_ids[X::WARPS][DENSE_IDS / 4];         // the ids of a share one after the other
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = lane / X::LANES;
     uint32_t *mine = reinterpret_cast<uint32_t *>(s_ids[warp]);
-    const uint4 *ids = s_ids[warp] + group * (DENSE_IDS / GROUPS / 4);
     const uint32_t stride = (uint32_t)a.M * (uint32_t)sizeof(WT);        // (M < 2^30)
     asm volatile("griddepcontrol.wait;" ::: "memory");       // for the verify stage, under whose end it is launched
     if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(a.status), 0)) return;
     const bool whole = screen_whole(a.scalars);              // all documents, in the planned order
     const int64_t docs = whole ? a.N : (int64_t)*a.dense_count, warps = (int64_t)gridDim.x * X::WARPS;
     if (docs == 0) return;
-    const int64_t pieces = (a.M + DENSE_PIECE - 1) / DENSE_PIECE;
+    const int64_t pieces = (a.M + X::PIECE - 1) / X::PIECE;
     int64_t at = (int64_t)blockIdx.x * X::WARPS + warp, j0 = 0;      // the item: a document and the first unit of a piece
-    auto in_turn = [&]() { for (; at >= docs; at -= docs) j0 += DENSE_PIECE; return j0 < a.M; };
+    auto in_turn = [&]() { for (; at >= docs; at -= docs) j0 += X::PIECE; return j0 < a.M; };
     bool more = in_turn();
     int64_t p_next = 0;
     int32_t orig_next = 0;
@@ -99,107 +101,112 @@ screen_dense_kernel(const VerifyArgs a)
         int64_t j = jp + (VEC ? lane % X::LANES * V : lane);
         const WT *col = column(j);
         u64 w[C][VEC ? 2 : H];
-        bool ahead = false;                                  // the first rows of this stretch are on their way
-        for (int x = 0; x < DENSE_PIECE && jp + x < a.M; x += X::UNITS, j += X::UNITS) {
-            const bool last = x + X::UNITS >= DENSE_PIECE || jp + x + X::UNITS >= a.M;
+        bool ahead = false;                                  // the first rows of a pass are on their way
+        for (int x = 0; x < X::PIECE && jp + x < a.M; x += X::UNITS, j += X::UNITS) {
+            const bool last = x + X::UNITS >= X::PIECE || jp + x + X::UNITS >= a.M;
             const WT *next = column(j + X::UNITS);
-            u64 acc[C][H];
+            float sum[OWN];
+            int64_t own = j;
 #pragma unroll
-            for (int c = 0; c < C; ++c)
+            for (int pass = 0; pass < X::PASSES; ++pass) {
+                u64 acc[C][H];
 #pragma unroll
-                for (int v = 0; v < H; ++v) acc[c][v] = 0ull;
-            // the weights of P ids from place q on, one for every partial sum: all of them, or those below `most`;
-            // each is asked for as soon as the one before it has been added
-            auto rows = [&](const WT *from, int64_t at, int q, int most, auto full, auto add) {
-                uint4 f4[C / 4];
+                for (int c = 0; c < C; ++c)
 #pragma unroll
-                for (int c = 0; c < C / 4; ++c) f4[c] = ids[q / GROUPS / 4 + c];
+                    for (int v = 0; v < H; ++v) acc[c][v] = 0ull;
+                // the weights of the next C ids of each share of pass `of`, from place q on: all of them, or those below
+                // `most`; each is asked for as soon as the one before it has been added
+                auto rows = [&](const WT *from, int64_t at, int of, int q, int most, auto full, auto add) {
+                    const uint4 *ids = s_ids[warp] + ((group * X::PASSES + of) * (DENSE_IDS / SHARES) + q) / 4;
+                    uint4 f4[C / 4];
 #pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    if (decltype(add)::value) dense_add<WT, VEC>(acc[c], w[c]);
-                    const uint4 t = f4[c / 4];
-                    const uint32_t f = c % 4 == 0 ? t.x : c % 4 == 1 ? t.y : c % 4 == 2 ? t.z : t.w;
-                    const bool there = decltype(full)::value || q + c * GROUPS + group < most;
-                    const WT *row = reinterpret_cast<const WT *>(reinterpret_cast<const char *>(from) + (u64)f * stride);
-                    if constexpr (VEC) {
-                        ulonglong2 t2 = make_ulonglong2(0ull, 0ull);
-                        if (there) t2 = __ldg(reinterpret_cast<const ulonglong2 *>(row));
-                        w[c][0] = t2.x; w[c][1] = t2.y;
-                    } else {
+                    for (int c = 0; c < C / 4; ++c) f4[c] = ids[c];
 #pragma unroll
-                        for (int v = 0; v < H; ++v) {
-                            const float lo = there ? dense_ld(row + min(at + 64 * v, a.M - 1)) : 0.f;
-                            const float hi = there ? dense_ld(row + min(at + 64 * v + 32, a.M - 1)) : 0.f;
-                            w[c][v] = (u64)__float_as_uint(hi) << 32 | __float_as_uint(lo);
+                    for (int c = 0; c < C; ++c) {
+                        if (decltype(add)::value) dense_add<WT, VEC>(acc[c], w[c]);
+                        const uint4 t = f4[c / 4];
+                        const uint32_t f = c % 4 == 0 ? t.x : c % 4 == 1 ? t.y : c % 4 == 2 ? t.z : t.w;
+                        const bool there = decltype(full)::value || (q + c) * SHARES + group * X::PASSES + of < most;
+                        const WT *row = reinterpret_cast<const WT *>(reinterpret_cast<const char *>(from) + (u64)f * stride);
+                        if constexpr (VEC) {
+                            ulonglong2 t2 = make_ulonglong2(0ull, 0ull);
+                            if (there) t2 = __ldg(reinterpret_cast<const ulonglong2 *>(row));
+                            w[c][0] = t2.x; w[c][1] = t2.y;
+                        } else {
+#pragma unroll
+                            for (int v = 0; v < H; ++v) {
+                                const float lo = there ? dense_ld(row + min(at + 64 * v, a.M - 1)) : 0.f;
+                                const float hi = there ? dense_ld(row + min(at + 64 * v + 32, a.M - 1)) : 0.f;
+                                w[c][v] = (u64)__float_as_uint(hi) << 32 | __float_as_uint(lo);
+                            }
                         }
                     }
-                }
-            };
-            auto step = [&](const WT *from, int64_t at, int q, int most, auto add) {
-                if (q + P <= most) rows(from, at, q, most, std::true_type(), add);
-                else rows(from, at, q, most, std::false_type(), add);
-            };
-            for (int eb = 0; eb < n; eb += DENSE_IDS) {
-                const int most = min(DENSE_IDS, n - eb);
-                if (x == 0 || n > DENSE_IDS) {
-                    __syncwarp();                            // the ids before these have been used
+                };
+                auto step = [&](const WT *from, int64_t at, int of, int q, int most, auto add) {
+                    if (q * SHARES + P <= most) rows(from, at, of, q, most, std::true_type(), add);
+                    else rows(from, at, of, q, most, std::false_type(), add);
+                };
+                for (int eb = 0; eb < n; eb += DENSE_IDS) {
+                    const int most = min(DENSE_IDS, n - eb);
+                    if ((x == 0 && pass == 0) || n > DENSE_IDS) {
+                        __syncwarp();                        // the ids before these have been used
 #pragma unroll
-                    for (int k = 0; k < DENSE_IDS / 32; ++k) {
-                        const int e = 32 * k + lane;
-                        mine[e % GROUPS * (DENSE_IDS / GROUPS) + e / GROUPS] =
-                            e < most ? BMU_IDX((uint32_t)__ldg(a.colidx + beg + eb + e), a.D, a.status) : 0u;
+                        for (int k = 0; k < DENSE_IDS / 32; ++k) {
+                            const int e = 32 * k + lane;
+                            mine[e % SHARES * (DENSE_IDS / SHARES) + e / SHARES] =
+                                e < most ? BMU_IDX((uint32_t)__ldg(a.colidx + beg + eb + e), a.D, a.status) : 0u;
+                        }
+                        __syncwarp();
                     }
-                    __syncwarp();
+                    if (!ahead) step(col, j, pass, 0, most, std::false_type());
+                    for (int q = C; q * SHARES + pass < most; q += C) step(col, j, pass, q, most, std::true_type());
+                    ahead = n <= DENSE_IDS && !(last && pass + 1 == X::PASSES);
+                    if (ahead && pass + 1 < X::PASSES) {
+                        step(col, j, pass + 1, 0, most, std::true_type());
+                    } else if (ahead) {
+                        step(next, j + X::UNITS, 0, 0, most, std::true_type());
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < C; ++c) dense_add<WT, VEC>(acc[c], w[c]);
+                    }
                 }
-                if (!ahead) step(col, j, 0, most, std::false_type());
-                for (int q = P; q < most; q += P) step(col, j, q, most, std::true_type());
-                ahead = n <= DENSE_IDS && !last;
-                if (ahead) {
-                    step(next, j + X::UNITS, 0, most, std::true_type());
+                // the lane's partial sums, in the order of the verify stage
+                if constexpr (VEC) {
+#pragma unroll
+                    for (int c = C / 2; c >= 1; c /= 2)
+#pragma unroll
+                        for (int i = 0; i < c; ++i)
+#pragma unroll
+                            for (int v = 0; v < H; ++v) add2(acc[i][v], acc[i + c][v]);
                 } else {
 #pragma unroll
-                    for (int c = 0; c < C; ++c) dense_add<WT, VEC>(acc[c], w[c]);
+                    for (int c = 1; c < C; c *= 2)
+#pragma unroll
+                        for (int i = 0; i < C; i += 2 * c)
+#pragma unroll
+                            for (int v = 0; v < H; ++v) add2(acc[i][v], acc[i + c][v]);
                 }
+                float s[V];
+#pragma unroll
+                for (int v = 0; v < V; ++v) s[v] = v % 2 ? hi_f(acc[0][v / 2]) : lo_f(acc[0][v / 2]);
+                // ... the groups', of every pair of lanes one keeps the first half of the units, and the passes'
+                if (X::GROUPS == 2) {
+                    const bool up = group != 0;
+#pragma unroll
+                    for (int i = 0; i < V / 2; ++i) {
+                        const float give = up ? s[i] : s[i + V / 2], keep = up ? s[i + V / 2] : s[i];
+                        s[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+                    }
+                    own = j + (up ? V / 2 : 0);
+                }
+#pragma unroll
+                for (int i = 0; i < OWN; ++i) sum[i] = pass ? sum[i] + s[i] : s[i];
             }
             col = next;
-            // the lane's partial sums, in the order of the verify stage
-            if constexpr (VEC) {
 #pragma unroll
-                for (int c = C / 2; c >= 1; c /= 2)
-#pragma unroll
-                    for (int i = 0; i < c; ++i)
-#pragma unroll
-                        for (int v = 0; v < H; ++v) add2(acc[i][v], acc[i + c][v]);
-            } else {
-#pragma unroll
-                for (int c = 1; c < C; c *= 2)
-#pragma unroll
-                    for (int i = 0; i < C; i += 2 * c)
-#pragma unroll
-                        for (int v = 0; v < H; ++v) add2(acc[i][v], acc[i + c][v]);
-            }
-            float s[V];
-#pragma unroll
-            for (int v = 0; v < V; ++v) s[v] = v % 2 ? hi_f(acc[0][v / 2]) : lo_f(acc[0][v / 2]);
-            // ... and the groups': of every pair of lanes, one keeps the first half of the units
-            int64_t at_j = j;
-            int k = V;
-#pragma unroll
-            for (int m = 16; m >= X::LANES; m /= 2) {
-                k /= 2;
-                const bool up = (lane & m) != 0;
-#pragma unroll
-                for (int i = 0; i < V / 2; ++i) {
-                    if (i >= k) continue;
-                    const float give = up ? s[i] : s[i + k], keep = up ? s[i + k] : s[i];
-                    s[i] = keep + __shfl_xor_sync(0xffffffffu, give, m);
-                }
-                if (up) at_j += k;
-            }
-#pragma unroll
-            for (int i = 0; i < V / GROUPS; ++i) {
-                const int64_t ji = at_j + (VEC ? i : 32 * i);
-                if (ji < a.M) best.push(fmaf(-2.f, s[i], __ldg(a.norms + ji)), (int)ji);
+            for (int i = 0; i < OWN; ++i) {
+                const int64_t ji = own + (VEC ? i : 32 * i);
+                if (ji < a.M) best.push(fmaf(-2.f, sum[i], __ldg(a.norms + ji)), (int)ji);
             }
         }
         u64 k1, k2;
