@@ -169,15 +169,15 @@ template <typename WT, bool VEC> struct ScreenSums {
 __device__ __forceinline__ bool screen_whole(const float *scalars)
 {
     const uint32_t *s = reinterpret_cast<const uint32_t *>(scalars);
-    return 2u * __ldg(s + SC_VOTES) > __ldg(s + SC_SAMPLED);
+    return 2u * s[SC_VOTES] > s[SC_SAMPLED];
 }
 __device__ __forceinline__ bool screen_ordered(const float *scalars)         // some sets are
 {
-    return __ldg(reinterpret_cast<const uint32_t *>(scalars) + SC_ORDERED) != 0u;
+    return reinterpret_cast<const uint32_t *>(scalars)[SC_ORDERED] != 0u;
 }
 __device__ __forceinline__ uint32_t screen_natural(const float *scalars)      // how many sets are not
 {
-    return __ldg(reinterpret_cast<const uint32_t *>(scalars) + SC_NAT);
+    return reinterpret_cast<const uint32_t *>(scalars)[SC_NAT];
 }
 // ... and how many parts a launch's slabs are cut into for each: more than `splits` where they are few
 __device__ __forceinline__ int screen_parts(const float *scalars, int splits, int most)
@@ -187,7 +187,7 @@ __device__ __forceinline__ int screen_parts(const float *scalars, int splits, in
 }
 __device__ __forceinline__ bool screen_by_norm(const float *scalars, const uint32_t *set_reach, int64_t p)
 {
-    return screen_ordered(scalars) && ordered_to_float(__ldg(set_reach + p / SC_DOCS)) <= __ldg(scalars + SC_TOP);
+    return screen_ordered(scalars) && ordered_to_float(set_reach[p / SC_DOCS]) <= scalars[SC_TOP];
 }
 // Steps between the smallest norm and the largest
 struct ScreenSteps {
@@ -264,6 +264,9 @@ int launch_screen_ordered_images(const void *W, int f16, int64_t D, int64_t M, c
 // A launch that may begin under the end of the one before it on the stream, if that one's blocks allow it
 // (griddepcontrol.launch_dependents).  Every kernel launched so waits for it first of all (griddepcontrol.wait), also
 // where it has nothing to do: whoever waits for the end of one kernel has then waited for all before it.
+// What a kernel of the chain reads from another of it, screen_range_kernel among them, it reads by ordinary loads: it
+// may live before that has been written, and read-only loads (__ldg, const __restrict__) promise that nobody writes while
+// it does.  The caller's arrays and those of the tiling pass are complete before the chain begins.
 struct ScreenLaunch {
     cudaLaunchAttribute attr;
     cudaLaunchConfig_t c;

@@ -59,8 +59,7 @@ __device__ __forceinline__ void order_units(const float *__restrict__ norms, int
 
 __global__ void __launch_bounds__(ORDER_THREADS)
 screen_order_kernel(const float *__restrict__ norms, int64_t D, int64_t M, int64_t N, int64_t launches, int32_t cap, float *scalars,
-                    const float *__restrict__ earlier, const uint32_t *__restrict__ status,
-                    const uint32_t *__restrict__ set_reach, int sets,
+                    const float *earlier, const uint32_t *status, const uint32_t *set_reach, int sets,
                     int32_t *__restrict__ units, float *__restrict__ unit_norm, u64 *__restrict__ tmp,
                     int32_t *__restrict__ rank_of, int2 *__restrict__ picks, uint32_t *__restrict__ tickets,
                     uint32_t *__restrict__ nat_list)
@@ -83,7 +82,7 @@ screen_order_kernel(const float *__restrict__ norms, int64_t D, int64_t M, int64
         else if (n < steps.lo) s_most = 0xffffffffu;         // a unit at minus infinity
     });
     for (int i = threadIdx.x; i < sets; i += ORDER_THREADS) {
-        const uint32_t v = __ldg(set_reach + i);
+        const uint32_t v = set_reach[i];
         if (v == 0u) continue;                               // none of its documents needs a slab
         const float t = ordered_to_float(v);
         atomicAdd(t < steps.top ? s_sets + steps.of(t) : &s_far, 1u);
@@ -108,7 +107,7 @@ screen_order_kernel(const float *__restrict__ norms, int64_t D, int64_t M, int64
     if (threadIdx.x == ORDER_THREADS - 1) s_within = within + mine;
     __syncthreads();
     const uint32_t total = s_within + s_far;
-    const uint4 docs = __ldg(reinterpret_cast<const uint4 *>(status + STATUS_REACH) + threadIdx.x);
+    const uint4 docs = reinterpret_cast<const uint4 *>(status + STATUS_REACH)[threadIdx.x];
     const uint32_t n4[4] = {docs.x, docs.y, docs.z, docs.w};
     uint32_t docs_in = order_scan(docs.x + docs.y + docs.z + docs.w, s_warp);
     const float near = fminf(1.f, 0.016f * (float)M * (float)launches / (float)(all * SC_SLAB));
@@ -195,7 +194,7 @@ screen_order_kernel(const float *__restrict__ norms, int64_t D, int64_t M, int64
     // the sets that reach further, in their order
     uint32_t n_nat = 0;
     for (int i0 = 0; i0 < sets; i0 += ORDER_THREADS) {
-        const uint32_t v = i0 + (int)threadIdx.x < sets ? __ldg(set_reach + i0 + threadIdx.x) : 0u;
+        const uint32_t v = i0 + (int)threadIdx.x < sets ? set_reach[i0 + threadIdx.x] : 0u;
         const bool far = v != 0u && !whole && !(ordered_to_float(v) <= top);
         const uint32_t at = order_scan(far, s_warp);
         if (far) nat_list[n_nat + at] = i0 + threadIdx.x;

@@ -285,10 +285,10 @@ __device__ __forceinline__ float screen_hi16(uint32_t x) { return __uint_as_floa
 
 template <typename WT>
 __global__ void __launch_bounds__(256)
-screen_table_kernel(const WT *__restrict__ W, int64_t M, const float *__restrict__ norms, const uint32_t *__restrict__ status, const float *__restrict__ rmin, const float *__restrict__ rmax, int32_t D, int32_t head,
+screen_table_kernel(const WT *__restrict__ W, int64_t M, const float *__restrict__ norms, const uint32_t *status, const float *rmin, const float *rmax, int32_t D, int32_t head,
                     int32_t head_pad, const uint16_t *__restrict__ feat, const uint16_t *__restrict__ rank,
-                    const uint32_t *__restrict__ tile_len, int64_t few, const uint32_t *__restrict__ most,
-                    const float *__restrict__ earlier, int sampled, float *__restrict__ scalars, uint4 *__restrict__ table,
+                    const uint32_t *__restrict__ tile_len, int64_t few, const uint32_t *most,
+                    const float *earlier, int sampled, float *__restrict__ scalars, uint4 *__restrict__ table,
                     unsigned char *__restrict__ kpack, float *__restrict__ khead)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -298,7 +298,7 @@ screen_table_kernel(const WT *__restrict__ W, int64_t M, const float *__restrict
     for (int c = 0; c < 3; ++c) {
         m3[c] = 0u;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) m3[c] = max(m3[c], __ldg(most + 8 * c + k));
+        for (int k = 0; k < 8; ++k) m3[c] = max(m3[c], most[8 * c + k]);
     }
     const float rh = earlier ? earlier[8] : __uint_as_float(m3[0]), rt = earlier ? earlier[9] : __uint_as_float(m3[1]);
     const float norm = earlier ? earlier[5] : __uint_as_float(m3[2]);
@@ -308,7 +308,7 @@ screen_table_kernel(const WT *__restrict__ W, int64_t M, const float *__restrict
         u64 k = 0ull;
         if (M >= SC_ORDER_MIN) {
 #pragma unroll
-            for (int x = 0; x < 8; ++x) k = max(k, __ldg(reinterpret_cast<const u64 *>(status + STATUS_REFS) + 8 * c + x));
+            for (int x = 0; x < 8; ++x) k = max(k, reinterpret_cast<const u64 *>(status + STATUS_REFS)[8 * c + x]);
         }
         ref[c] = earlier ? __float_as_int(earlier[SC_REF + c]) : k ? (int32_t)(uint32_t)~k : -1;
     }
@@ -378,7 +378,7 @@ struct ScreenWindow { float window, bound, reach; };
 
 __device__ __forceinline__ ScreenWindow screen_window_of(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
                                                          int64_t i, const uint32_t *__restrict__ key,
-                                                         const uint4 *__restrict__ table, const float *scalars,
+                                                         const uint4 *table, const float *scalars,
                                                          bool order, bool top2,
                                                          [[maybe_unused]] int64_t D, [[maybe_unused]] uint32_t *status)
 {
@@ -395,7 +395,7 @@ __device__ __forceinline__ ScreenWindow screen_window_of(const int32_t *__restri
         }
         uint4 t[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) t[u] = f[u] >= 0 ? __ldg(table + f[u]) : make_uint4(0u, 0u, 0u, 0u);
+        for (int u = 0; u < 4; ++u) t[u] = f[u] >= 0 ? table[f[u]] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             en += __uint_as_float(t[u].x); eo += __uint_as_float(t[u].y); aa += screen_lo16(t[u].z); in |= t[u].x;
@@ -438,10 +438,10 @@ __device__ __forceinline__ ScreenWindow screen_window_of(const int32_t *__restri
 __global__ void __launch_bounds__(256, 6)
 screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
                      const int32_t *__restrict__ perm, const uint32_t *__restrict__ key, int64_t N, int64_t n_pad,
-                     const uint4 *__restrict__ table, float *scalars, int order, int top2,
+                     const uint4 *table, float *scalars, int order, int top2,
                      float *__restrict__ window, float2 *__restrict__ reach, uint32_t *__restrict__ bound,
                      uint32_t *__restrict__ count, uint32_t *__restrict__ set_reach, int64_t D,
-                     int sampled, const float *__restrict__ groups, int64_t M, uint32_t *__restrict__ status)
+                     int sampled, const float *groups, int64_t M, uint32_t *__restrict__ status)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -457,7 +457,7 @@ screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restri
             if (lane == 0) s_win = w.window;
         }
         float least = CUDART_INF_F;
-        for (int64_t g = threadIdx.x; g < n; g += 256) least = fminf(least, __ldg(of + g));
+        for (int64_t g = threadIdx.x; g < n; g += 256) least = fminf(least, of[g]);
 #pragma unroll
         for (int m = 16; m > 0; m >>= 1) least = fminf(least, __shfl_xor_sync(0xffffffffu, least, m));
         if (lane == 0) s_least[warp] = least;
@@ -466,7 +466,7 @@ screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restri
         for (int w = 0; w < 8; ++w) least = fminf(least, s_least[w]);
         const float limit = least + s_win;
         uint32_t within = 0;
-        for (int64_t g = threadIdx.x; g < n; g += 256) within += __ldg(of + g) <= limit;
+        for (int64_t g = threadIdx.x; g < n; g += 256) within += of[g] <= limit;
         within = __reduce_add_sync(0xffffffffu, within);
         if (lane == 0) s_in[warp] = within;
         __syncthreads();
@@ -544,7 +544,7 @@ int launch_screen_prepare(const void *W, int f16, int64_t D, int64_t M, const fl
     // up to a thousandth of the tiles, or four where they are few (32 documents of 1000 ids: 27 us for 4,096 units)
     const int64_t tiles = (N + 7) / 8, four = tiles / 64 < 4 ? tiles / 64 : 4, few = tiles / 1024 > four ? tiles / 1024 : four;
     const auto tables = [&](auto w) {
-        ScreenLaunch l((unsigned)((rows + 255) / 256), 256, s, true);
+        ScreenLaunch l((unsigned)((rows + 255) / 256), 256, s, !earlier);         // (behind the tiling pass: ordinary)
         const cudaError_t e = cudaLaunchKernelEx(
             &l.c, screen_table_kernel<std::remove_const_t<std::remove_pointer_t<decltype(w)>>>, w, M, norms, (const uint32_t *)status,
             (const float *)rmin, (const float *)rmax, (int32_t)D, head, cl.head_pad, feat, rank, tile_len, few,
@@ -601,15 +601,15 @@ __device__ __forceinline__ void screen_ld_vec(const __half *p, float v[8])
 
 template <typename WT, bool VEC>
 __device__ __forceinline__ void screen_image_block(const WT *__restrict__ W, int64_t D, int64_t M, int64_t slab,
-                                                   int64_t j_slab, int block, const float *__restrict__ rmin,
-                                                   const float *__restrict__ scalars, const float *__restrict__ norms,
+                                                   int64_t j_slab, int block, const float *rmin,
+                                                   const float *scalars, const float *__restrict__ norms,
                                                    unsigned char *__restrict__ img8, float *__restrict__ normp)
 {
     constexpr int V = IMAGE_V<WT, VEC>, LPR = SC_SLAB / V, RPI = 32 / LPR;     // lanes per row, rows per instruction
     constexpr int R = 4;                                   // instructions per warp, loads issued together
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, l4 = (lane % LPR) * (V / 4);
     const int64_t j = j_slab + 4 * l4;
-    const float inv = __ldg(scalars + 2), q_max = __ldg(scalars + 4);
+    const float inv = scalars[2], q_max = scalars[4];
     const int i = l4 >> 3, hb = (l4 >> 2) & 1, wd = l4 & 3;
     unsigned char *out = img8 + (size_t)slab * (D + 1) * SC_SLAB + (hb * 4 + i) * 16 + wd * 4;
     const int64_t f0 = ((int64_t)block * 8 + warp) * R * RPI + lane / LPR;
@@ -617,7 +617,7 @@ __device__ __forceinline__ void screen_image_block(const WT *__restrict__ W, int
 #pragma unroll
     for (int u = 0; u < R; ++u) {
         const int64_t f = f0 + u * RPI;
-        c[u] = f < D ? __ldg(rmin + f) : 0.f;
+        c[u] = f < D ? rmin[f] : 0.f;
 #pragma unroll
         for (int e = 0; e < V; ++e) v[u][e] = c[u];
         if (f < D) {
@@ -656,8 +656,8 @@ __device__ __forceinline__ void screen_image_block(const WT *__restrict__ W, int
 template <typename WT, bool VEC>
 __device__ __forceinline__ void screen_head_block(const WT *__restrict__ W, int64_t D, int64_t M, int64_t slab,
                                                   int64_t j_slab, int block, int32_t head, int32_t head_pad,
-                                                  const uint16_t *__restrict__ feat, const float *__restrict__ rmin,
-                                                  const float *__restrict__ khead, unsigned char *__restrict__ img)
+                                                  const uint16_t *__restrict__ feat, const float *rmin,
+                                                  const float *khead, unsigned char *__restrict__ img)
 {
     constexpr int P = 9;                                   // words per neuron: eight, odd pitch
     __shared__ uint32_t tile[SC_SLAB * P];
@@ -667,13 +667,13 @@ __device__ __forceinline__ void screen_head_block(const WT *__restrict__ W, int6
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const int h = block * 32 + 4 * warp + u;
-        k[u] = __ldg(khead + h);
+        k[u] = khead[h];
         c[u] = 0.f;
 #pragma unroll
         for (int e = 0; e < 4; ++e) v[u][e] = 0.f;
         if (h < head && h < D) {
             const int64_t f = feat ? (int64_t)__ldg(feat + h) : (int64_t)h;
-            c[u] = __ldg(rmin + f);
+            c[u] = rmin[f];
             if (VEC) { if (j < M) screen_ld16(W + f * M + j, v[u]); }
             else {
 #pragma unroll
@@ -715,7 +715,7 @@ static const int ORD_HEAD = 16;                            // head features a bl
 
 template <typename WT>
 __device__ __forceinline__ void ordered_rows(const WT *__restrict__ W, int64_t D, int64_t M, int64_t f0, int slots,
-                                             int place0, const int2 *__restrict__ picks, const float *__restrict__ rmin,
+                                             int place0, const int2 *picks, const float *rmin,
                                              float inv, float q_max, unsigned char *__restrict__ img8)
 {
     __shared__ __align__(16) unsigned char bytes[ORD_ROWS * SC_MAX_SLABS * SC_SLAB];
@@ -725,10 +725,10 @@ __device__ __forceinline__ void ordered_rows(const WT *__restrict__ W, int64_t D
     for (int u = 0; u < ORD_ROWS; ++u) {
         const int64_t f = f0 + u < D ? f0 + u : D - 1;
         row[u] = W + f * M;
-        c[u] = __ldg(rmin + f);
+        c[u] = rmin[f];
     }
     for (int i = threadIdx.x; i < slots; i += 256) {
-        const int2 t = __ldg(picks + i);
+        const int2 t = picks[i];
         const int at = t.y - place0, jn = at & (SC_SLAB - 1);
         // in the slab's 128 bytes of a row: as screen_image_block has it
         unsigned char *to = bytes + (at - jn) * ORD_ROWS + (((jn >> 4) & 1) * 4 + (jn >> 5)) * 16 + ((jn >> 2) & 3) * 4 +
@@ -751,9 +751,9 @@ __device__ __forceinline__ void ordered_rows(const WT *__restrict__ W, int64_t D
 
 template <typename WT>
 __device__ __forceinline__ void ordered_head(const WT *__restrict__ W, int64_t D, int64_t M, int h0, int slots, int place0,
-                                             const int2 *__restrict__ picks, int32_t head, int32_t head_pad,
-                                             const uint16_t *__restrict__ feat, const float *__restrict__ rmin,
-                                             const float *__restrict__ khead, unsigned char *__restrict__ img)
+                                             const int2 *picks, int32_t head, int32_t head_pad,
+                                             const uint16_t *__restrict__ feat, const float *rmin,
+                                             const float *khead, unsigned char *__restrict__ img)
 {
     __shared__ float s_c[ORD_HEAD], s_k[ORD_HEAD];
     __shared__ int64_t s_row[ORD_HEAD];
@@ -762,12 +762,13 @@ __device__ __forceinline__ void ordered_head(const WT *__restrict__ W, int64_t D
         const bool in = h < head && h < D;
         const int64_t f = in ? (feat ? (int64_t)__ldg(feat + h) : (int64_t)h) : -1;
         s_row[threadIdx.x] = in ? f * M : -1;
-        s_c[threadIdx.x] = in ? __ldg(rmin + f) : 0.f;
-        s_k[threadIdx.x] = __ldg(khead + h);
+        s_c[threadIdx.x] = in ? rmin[f] : 0.f;
+        s_k[threadIdx.x] = khead[h];
     }
     __syncthreads();
     for (int i = threadIdx.x; i < slots; i += 256) {
-        const int2 t = __ldg(picks + i);
+        asm volatile("" ::: "memory");                     // (or the sixteen rows' addresses are kept and spill)
+        const int2 t = picks[i];
         const int at = t.y - place0, n = screen_col(at & (SC_SLAB - 1));
         uint32_t q[4];
 #pragma unroll
@@ -792,24 +793,24 @@ __device__ __forceinline__ void ordered_head(const WT *__restrict__ W, int64_t D
 }
 
 // A warp per set of 128 documents: which of the launch's slabs any of them reaches, as items of up to SC_PART.
-__device__ __forceinline__ void ordered_items(const OrderedImages &g, int set, int slabs, const float *__restrict__ unit_norm,
-                                              const float *__restrict__ scalars)
+__device__ __forceinline__ void ordered_items(const OrderedImages &g, int set, int slabs, const float *unit_norm,
+                                              const float *scalars)
 {
     const int lane = threadIdx.x & 31;
-    if (!(ordered_to_float(__ldg(g.set_reach + set)) <= __ldg(scalars + SC_TOP))) return;    // in the order of the map
-    const float top = __ldg(scalars + SC_DOC_TOP);
+    if (!(ordered_to_float(g.set_reach[set]) <= scalars[SC_TOP])) return;    // in the order of the map
+    const float top = scalars[SC_DOC_TOP];
     float far = -CUDART_INF_F;
 #pragma unroll
     for (int u = 0; u < SC_DOCS / 32; ++u) {
         const int64_t p = (int64_t)set * SC_DOCS + 32 * u + lane;
-        const float2 r = __ldg(g.reach + p);
+        const float2 r = g.reach[p];
         if (r.x > top) continue;                           // evaluated whole
         // (less what the launches before have found)
-        far = fmaxf(far, g.first ? r.x : fminf(r.x, ordered_to_float(__ldcg(g.bound + p)) + __ldg(g.window + p) + r.y));
+        far = fmaxf(far, g.first ? r.x : fminf(r.x, ordered_to_float(__ldcg(g.bound + p)) + g.window[p] + r.y));
     }
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1) far = fmaxf(far, __shfl_xor_sync(0xffffffffu, far, m));
-    const bool in = lane < slabs && __ldg(unit_norm + lane * SC_SLAB) <= far;
+    const bool in = lane < slabs && unit_norm[lane * SC_SLAB] <= far;
     const int n = __popc(__ballot_sync(0xffffffffu, in));  // (ascending: the first ones)
     if (lane < (n + SC_PART - 1) / SC_PART)
         g.items[(size_t)lane * g.sets + atomicAdd(g.tickets + lane, 1u)] =
@@ -819,19 +820,19 @@ __device__ __forceinline__ void ordered_items(const OrderedImages &g, int set, i
 template <typename WT>
 __global__ void __launch_bounds__(256, 6)
 screen_ordered_image_kernel(const WT *__restrict__ W, int64_t D, int64_t M, const OrderedImages g,
-                            const int2 *__restrict__ picks, const float *__restrict__ unit_norm, int32_t head_pad,
-                            const uint16_t *__restrict__ feat, const float *__restrict__ rmin,
-                            const float *__restrict__ khead, const float *__restrict__ scalars,
+                            const int2 *picks, const float *unit_norm, int32_t head_pad,
+                            const uint16_t *__restrict__ feat, const float *rmin,
+                            const float *khead, const float *scalars,
                             unsigned char *__restrict__ img8, unsigned char *__restrict__ head_img, float *__restrict__ normp)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!screen_ordered(scalars) || screen_whole(scalars)) return;
     const uint32_t *sc = reinterpret_cast<const uint32_t *>(scalars);
-    const int slabs = (int)min((int64_t)g.n_slabs, (int64_t)__ldg(sc + SC_NEEDED) - g.slab0);
+    const int slabs = (int)min((int64_t)g.n_slabs, (int64_t)sc[SC_NEEDED] - g.slab0);
     if (slabs <= 0) return;
     const int place0 = (int)g.slab0 * SC_SLAB, slots = slabs * SC_SLAB;
-    const bool stand = __ldg(sc + SC_STAND) != 0u;         // the images of an earlier search
+    const bool stand = sc[SC_STAND] != 0u;         // the images of an earlier search
     const int lists = (g.sets + 7) / 8, rows = (int)((D + ORD_ROWS) / ORD_ROWS), heads = head_pad / ORD_HEAD;
     const int all = stand ? lists : lists + heads + rows;
     for (int item = blockIdx.x; item < all; item += gridDim.x) {
@@ -843,11 +844,11 @@ screen_ordered_image_kernel(const WT *__restrict__ W, int64_t D, int64_t M, cons
             if (item == lists)
                 for (int x = threadIdx.x; x < slots; x += 256) {
                     const int jn = x & (SC_SLAB - 1);
-                    normp[x - jn + ((jn & 31) >> 2) * 16 + (jn >> 5) * 4 + (jn & 3)] = __ldg(unit_norm + place0 + x);
+                    normp[x - jn + ((jn & 31) >> 2) * 16 + (jn >> 5) * 4 + (jn & 3)] = unit_norm[place0 + x];
                 }
         } else {
             ordered_rows(W, D, M, (int64_t)(item - lists - heads) * ORD_ROWS, slots, place0, picks + place0, rmin,
-                         __ldg(scalars + 2), __ldg(scalars + 4), img8);
+                         scalars[2], scalars[4], img8);
         }
     }
 }
@@ -878,15 +879,15 @@ template <typename WT, bool VEC, bool LOOP>
 __global__ void __launch_bounds__(256)
 screen_image_kernel(const WT *__restrict__ W, int64_t D, int64_t M, int64_t k, int64_t launches, int64_t n_slabs,
                     int32_t head,
-                    int32_t head_pad, const uint16_t *__restrict__ feat, const float *__restrict__ rmin,
-                    const float *__restrict__ khead, const float *__restrict__ scalars,
+                    int32_t head_pad, const uint16_t *__restrict__ feat, const float *rmin,
+                    const float *khead, const float *scalars,
                     const float *__restrict__ norms, unsigned char *__restrict__ img8,
                     unsigned char *__restrict__ head_img, float *__restrict__ normp)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // the images of an earlier search stand; or nothing is swept in this order
-    if (__ldg(scalars + 7) == 0.f || screen_whole(scalars) || screen_natural(scalars) == 0u) return;
+    if (scalars[7] == 0.f || screen_whole(scalars) || screen_natural(scalars) == 0u) return;
     const int heads = head_pad / 32;
     auto one = [&](const int64_t slab) {
         const int64_t j_slab = (k + launches * slab) * SC_SLAB;

@@ -431,7 +431,7 @@ screen_verify_units_kernel(const VerifyArgs a)
         if (!(__uint_as_float(t.x) <= ordered_to_float(a.bound[p]) + win)) t.z = 0u;
         // too many units, or none (no distance of it is finite), or a list that was too short for them
         const uint32_t units = __reduce_add_sync(0xffffffffu, __popc(t.z));
-        if (n > (uint32_t)SC_OWN_LIST || units == 0u || __ldg(a.reach + p).x > __ldg(a.scalars + SC_DOC_TOP) || units > screen_dense_groups(a.M) || win == CUDART_INF_F) {
+        if (n > (uint32_t)SC_OWN_LIST || units == 0u || a.reach[p].x > a.scalars[SC_DOC_TOP] || units > screen_dense_groups(a.M) || win == CUDART_INF_F) {
             if (lane == 0) {
                 a.state[orig] = KEY_WORST;
                 if (TOP2) a.state2[orig] = KEY_WORST;
@@ -450,7 +450,7 @@ screen_verify_units_kernel(const VerifyArgs a)
 #pragma unroll
                 for (int i = 0; i < AT_ONCE; ++i) {
                     if (!bits) break;
-                    if (i == lane / L) j = __ldg(a.units + first + __ffs(bits) - 1);     // (-1 beyond the last unit)
+                    if (i == lane / L) j = a.units[first + __ffs(bits) - 1];     // (-1 beyond the last unit)
                     bits &= bits - 1;
                 }
                 float s = 0.f;

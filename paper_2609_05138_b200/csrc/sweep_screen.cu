@@ -128,7 +128,7 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint32_t natural = screen_natural(a.scalars);
     if (screen_whole(a.scalars) || (ORDERED ? !screen_ordered(a.scalars) : natural == 0u)) return;
-    if (ORDERED && o.slab0 >= (int64_t)__ldg(reinterpret_cast<const uint32_t *>(a.scalars) + SC_NEEDED)) return;
+    if (ORDERED && o.slab0 >= (int64_t)reinterpret_cast<const uint32_t *>(a.scalars)[SC_NEEDED]) return;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int KB = a.head_pad / 128;
@@ -255,14 +255,14 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
                 if (t < sets * splits) {
                     set = t % sets;
                     part = t / sets;
-                    if (screen_natural(a.scalars) != SC_ALL) set = __ldg(a.nat_list + set);
+                    if (screen_natural(a.scalars) != SC_ALL) set = a.nat_list[set];
                     range = (uint32_t)a.n_slabs * part / splits | (uint32_t)a.n_slabs * (part + 1) / splits << 16;
                 }
             } else {
                 for (int c = 0; c < SC_PARTS; ++c) {         // the lists one after the other
                     const uint32_t n = __ldcg(o.tickets + c);
                     if (t < n) {
-                        const uint2 item = __ldg(o.items + (size_t)c * a.blocks + t);
+                        const uint2 item = o.items[(size_t)c * a.blocks + t];
                         set = item.x; range = item.y;
                         break;
                     }
@@ -282,8 +282,8 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
             const bool there = p < a.n_tiles * 8;
             for (int wd = e; wd < a.head_pad / 32; wd += 4) {
                 const uint32_t m = there && wd < words ? __ldg(a.tile_head + (size_t)p * words + wd) : 0u;
-                const uint4 k0 = __ldg(reinterpret_cast<const uint4 *>(a.kpack) + 2 * wd);
-                const uint4 k1 = __ldg(reinterpret_cast<const uint4 *>(a.kpack) + 2 * wd + 1);
+                const uint4 k0 = reinterpret_cast<const uint4 *>(a.kpack)[2 * wd];
+                const uint4 k1 = reinterpret_cast<const uint4 *>(a.kpack)[2 * wd + 1];
                 const uint32_t k[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
                 uint32_t v[8];
 #pragma unroll
@@ -299,7 +299,7 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
         // ---------------- tail: documents 32q + 8e .. + 7 of a block, one tile
         const int s = lane >> 3, hb = (lane >> 2) & 1, li = lane & 3;
         const uint32_t sel_own = hb ? 0x4432u : 0x4410u, sel_other = hb ? 0x4410u : 0x4432u;
-        const u64 sh = sc_pack(__ldg(a.scalars), __ldg(a.scalars)), st = sc_pack(__ldg(a.scalars + 1), __ldg(a.scalars + 1));
+        const u64 sh = sc_pack(a.scalars[0], a.scalars[0]), st = sc_pack(a.scalars[1], a.scalars[1]);
         const u64 minus_2p23 = sc_pack(-8388608.f, -8388608.f);
         const size_t slab_bytes = (size_t)(a.D + 1) * SC_SLAB;
         const int tile = group * (SC_DOCS / 8) + 4 * q + e;
@@ -307,14 +307,14 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
         const uint4 *ids = a.tile_ids;
         [[maybe_unused]] size_t room = a.tile_rows_cap;
         if (tile < a.n_tiles) {
-            const uint32_t rows = min(__ldg(a.tile_len + tile) & 0xffffu, (uint32_t)__ldg(a.scalars + 6));
+            const uint32_t rows = min(__ldg(a.tile_len + tile) & 0xffffu, (uint32_t)a.scalars[6]);
             quads = (rows + 3) / 4;
             const uint32_t off = BMU_IDX(__ldg(a.tile_off + tile), a.tile_rows_cap, a.status);
             ids += off; room -= off;
         }
         ids += s;
         const uint32_t p = (uint32_t)tile * 8 + (lane >> 2);             // this lane's document
-        const float win = __ldg(a.window + p);
+        const float win = a.window[p];
         float m1 = 3.0e38f, m2 = 3.0e38f;                                // smallest (and second) value of the document
         // ORDERED: how far it reaches (evaluated whole: not at all), and what bounds its smallest (second) value
         [[maybe_unused]] float reach = -CUDART_INF_F, known = 0.f;
@@ -325,13 +325,13 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
         [[maybe_unused]] int valid = s_lo;
         auto stripe = [&]() { return ((size_t)item_slot[2] * a.n_pad + p) * 4 + li; };
         if constexpr (ORDERED) {
-            const float2 r = __ldg(o.reach + p);
-            if (r.x <= __ldg(a.scalars + SC_DOC_TOP)) reach = r.y;
+            const float2 r = o.reach[p];
+            if (r.x <= a.scalars[SC_DOC_TOP]) reach = r.y;
             known = ordered_to_float(__ldcg(o.bound + p));
             if (TOP2) m2 = known; else m1 = known;
         } else if (!a.first) {
-            m1 = __ldg(a.amin + p);
-            if (TOP2) m2 = __ldg(a.amin2 + p);
+            m1 = a.amin[p];
+            if (TOP2) m2 = a.amin2[p];
         }
         const unsigned char *base = a.img8 + (size_t)s_lo * slab_bytes + (lane & 7) * 16;
         const float *np = a.normp + (size_t)s_lo * SC_SLAB + li * 4;
@@ -341,7 +341,7 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
         auto load = [&](const unsigned char *from, uint4 *d, uint32_t x0, uint32_t x1) {
             auto piece = [&](uint32_t word, uint32_t sel) {
                 const uint32_t f = __byte_perm(word, 0, sel);
-                return __ldg(reinterpret_cast<const uint4 *>(from + (size_t)(BMU_IDX(f, a.D + 1, a.status) * (uint32_t)SC_SLAB)));
+                return *reinterpret_cast<const uint4 *>(from + (size_t)(BMU_IDX(f, a.D + 1, a.status) * (uint32_t)SC_SLAB));
             };
             d[0] = piece(x0, sel_own);   d[1] = piece(x1, sel_own);
             d[2] = piece(x0, sel_other); d[3] = piece(x1, sel_other);
@@ -354,14 +354,14 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
         };
         // ORDERED: whether the head alone is looked at first, and whether a slab's first quad is on its way
         [[maybe_unused]] bool head_first = ORDERED && o.slab0 + s_lo > 0, begun = !head_first;
-        [[maybe_unused]] const u64 tail_most = sc_pack((float)(4u * quads) * __ldg(a.scalars + 4), (float)(4u * quads) * __ldg(a.scalars + 4));
+        [[maybe_unused]] const u64 tail_most = sc_pack((float)(4u * quads) * a.scalars[4], (float)(4u * quads) * a.scalars[4]);
         if (quads && begun) begin();
         bool taken = false;
         for (int sl = s_lo; sl < s_hi; ++sl, np += SC_SLAB) {
             const int n = done + sl - s_lo;
             if (sl + 1 == s_hi) { take(); taken = true; }
             // no document of the tile reaches this slab, nor any behind it: the accumulators still change hands
-            if (ORDERED && !__any_sync(0xffffffffu, __ldg(o.unit_norm + sl * SC_SLAB) <= (TOP2 ? m2 : m1) + win + reach)) {
+            if (ORDERED && !__any_sync(0xffffffffu, o.unit_norm[sl * SC_SLAB] <= (TOP2 ? m2 : m1) + win + reach)) {
                 for (int r = n; r < done + slabs; ++r) {
                     mm_wait(tfull0 + 8 * (r & two), (r >> two) & 1, abort_flag, a.status, 8u);
                     __syncwarp();
@@ -374,8 +374,8 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
             [[maybe_unused]] auto head8 = [&](int c, uint32_t hs[8], u64 nm[4]) {
                 uint32_t v[16];
                 mm_tmem_ld_16x256b_x4(taddr + c * 32, v);
-                const ulonglong2 n0 = __ldg(reinterpret_cast<const ulonglong2 *>(np + (2 * c) * 16));
-                const ulonglong2 n1 = __ldg(reinterpret_cast<const ulonglong2 *>(np + (2 * c + 1) * 16));
+                const ulonglong2 n0 = *reinterpret_cast<const ulonglong2 *>(np + (2 * c) * 16);
+                const ulonglong2 n1 = *reinterpret_cast<const ulonglong2 *>(np + (2 * c + 1) * 16);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
@@ -471,8 +471,8 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
                 for (int c = 0; c < 4; ++c) {             // eight neurons of the lane's 32 at a time
                     uint32_t v[16];
                     mm_tmem_ld_16x256b_x4(taddr + c * 32, v);
-                    const ulonglong2 n0 = __ldg(reinterpret_cast<const ulonglong2 *>(np + (2 * c) * 16));
-                    const ulonglong2 n1 = __ldg(reinterpret_cast<const ulonglong2 *>(np + (2 * c + 1) * 16));
+                    const ulonglong2 n0 = *reinterpret_cast<const ulonglong2 *>(np + (2 * c) * 16);
+                    const ulonglong2 n1 = *reinterpret_cast<const ulonglong2 *>(np + (2 * c + 1) * 16);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                     if (c == 3) {                         // the accumulator is free
                         mm_fence_before();
