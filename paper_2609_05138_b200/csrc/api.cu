@@ -1247,9 +1247,10 @@ int bmu_search_host(const float *W, int64_t D, int64_t M, const int32_t *rowptr_
     return BMU_OK;
 }
 
-// The batches of one call share the 8-bit images of the codebook up to this size (a quarter of its own);
-// the scratch keeps them until bmu_release_scratch.  150,000 documents in three batches to 128 x 128 units:
-// 9.10 ms with ranges, head and images made for each batch, 8.2 shared.
+// The batches of one call share the 8-bit images of the codebook up to this size (a quarter of its own, and
+// the head's); those of slabs in the order of the norms come on top: as many where the map takes one launch, half where it takes
+// two, a quarter from four on, as at this limit.  The scratch keeps them until bmu_release_scratch.  150,000 documents
+// in three batches to 128 x 128 units: 9.10 ms with ranges, head and images made for each batch, 8.2 shared.
 static const size_t SHARED_IMAGE_MAX = (size_t)2 << 30;
 
 // ---- streamed batches from host memory (config 5: a corpus fed in batches) ----
@@ -1316,7 +1317,7 @@ int bmu_search_batches_host(const float *W, int64_t D, int64_t M, int32_t n_batc
     ScreenShared shared;
     memset(&shared, 0, sizeof(shared));
     if (sharing > 1) screen_shared_layout(D, M, screen_head_rows(none, D), screen_chunk(none, D), &shared.lay);
-    if (shared.lay.total > SHARED_IMAGE_MAX) sharing = 0;
+    if (shared.lay.map_total > SHARED_IMAGE_MAX) sharing = 0;
     const size_t shared_bytes = sharing > 1 ? align_up(shared.lay.total, 256) : 0;
     const size_t rp_off = align_up(ws_need, 256);
     const size_t ci_off = align_up(rp_off + (size_t)(max_n + 1) * 4, 256);

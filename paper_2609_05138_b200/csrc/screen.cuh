@@ -84,7 +84,7 @@ struct ScreenLayout {
     int head_pad;                        // head rows rounded up to a stage (128)
     int64_t chunk_slabs;                 // slabs of the largest launch
     int splits, most_splits;             // blocks that share a launch's slabs for a set of documents; room for so many
-    size_t rank, feat;                   // only in a ScreenShared
+    size_t rank, feat, map_total;        // only in a ScreenShared; without the images in the order of the norms
 };
 
 // What the searches of one call share that read the same codebook: the head they agree on, the row

@@ -83,6 +83,7 @@ void screen_shared_layout(int64_t D, int64_t M, int head, int64_t chunk, ScreenL
     codebook_layout(D, M, launches * l->chunk_slabs, l->ord_launches * l->chunk_slabs, 2, take, l);
     l->rank = take((size_t)D * 2); l->feat = take((size_t)D * 2);
     l->total = off;
+    l->map_total = off - (l->ord8 == l->img8 ? 0 : l->rank - l->ord8);
 }
 
 // ---- ranges of the rows -------------------------------------------------------------------

@@ -360,6 +360,29 @@ def test_batches_share_the_images_of_the_codebook(bmu):
         assert torch.equal(rb.cpu(), ob) and torch.equal(rd.cpu(), od)
 
 
+def test_a_large_codebook_shares_its_images(bmu):
+    """640,000 units of 1,536 features: 1.97 GB of images in the order of the map, which batches share, and as many as
+    a quarter of them again in the order of the norms, which must not keep the former from being shared."""
+    D, M, n, dev = 1536, 640_000, 1100, torch.device("cuda")
+    rp, ci = synth.draw_corpus(n, D, 1.0, torch.full((n,), 80, dtype=torch.int64, device=dev), 3, dev)
+    W = torch.rand((D, M), generator=torch.Generator(device=dev).manual_seed(4), device=dev)
+    assert bmu.bmu_describe_search(D, M, n, ci.numel()).two_stage
+    batch = (rp.cpu().pin_memory(), ci.cpu().pin_memory())
+
+    def launches(call):
+        before = bmu.bmu_kernel_launches()
+        out = call()
+        return bmu.bmu_kernel_launches() - before, out
+
+    norms, _ = launches(lambda: bmu.bmu_codebook_norms(W))
+    one, (first,) = launches(lambda: bmu.bmu_search_batches_host(W, [batch]))
+    two, both = launches(lambda: bmu.bmu_search_batches_host(W, [batch, batch]))
+    assert two < 2 * one - norms                     # no ranges and no choice of the head for the second batch
+    for ob, od in both:
+        assert torch.equal(ob, first[0]) and torch.equal(od, first[1])
+    bmu.bmu_release_scratch()
+
+
 def lists(lens, D, seed):
     r = np.random.default_rng(seed)
     rows = [np.sort(r.permutation(D)[:n]) for n in lens]
