@@ -8,7 +8,7 @@
 // every sixteenth id, added in pairs), so that a unit has the same distance, bit for bit, whichever way it came
 // here: which documents come depends on the others in the call, and on when a bound was lowered.
 //
-// A warp takes a document and a piece of 384 units (fp16: 1,024), 128 of them at a time, in two passes: the partial
+// A warp takes a document and a piece of up to 384 units (fp16: 1,024), 128 of them at a time, in two passes: the partial
 // sums of the even places of the list, then those of the odd ones.  A lane carries the partial sums of four (fp16: eight,
 // where half of the warp takes every other id of a pass) units, 32 (64) registers, and asks for the next row of each as
 // soon as the one before has been added, also across passes and stretches; ids through shared memory.  Pieces outside,
@@ -60,7 +60,7 @@ template <typename WT, bool VEC> struct Dense {
     using Sums = ScreenSums<WT, VEC>;
     static constexpr int V = VEC ? 16 / (int)sizeof(WT) : 4, PASSES = VEC ? 2 : 1, GROUPS = VEC && V == 8 ? 2 : 1;
     static constexpr int LANES = 32 / GROUPS, UNITS = LANES * V, SHARES = PASSES * GROUPS, SUMS = Sums::N / SHARES;
-    static constexpr int WARPS = VEC ? 16 : 24, PIECE = V == 8 ? 1024 : 384;     // of the one block per SM; units of an item
+    static constexpr int WARPS = VEC ? 16 : 24, MOST = V == 8 ? 8 : 3;      // of the one block per SM; stretches of an item
 };
 static const int DENSE_IDS = 128;
 
@@ -79,10 +79,14 @@ screen_dense_kernel(const VerifyArgs a)
     const bool whole = screen_whole(a.scalars);              // all documents, in the planned order
     const int64_t docs = whole ? a.N : (int64_t)*a.dense_count, warps = (int64_t)gridDim.x * X::WARPS;
     if (docs == 0) return;
-    const int64_t pieces = (a.M + X::PIECE - 1) / X::PIECE;
-    int64_t at = (int64_t)blockIdx.x * X::WARPS + warp, j0 = 0;      // the item: a document and the first unit of a piece
-    auto in_turn = [&]() { for (; at >= docs; at -= docs) j0 += X::PIECE; return j0 < a.M; };
-    bool more = in_turn();
+    // (few documents: pieces of fewer stretches, so that every warp has one or two)
+    const int64_t stretches = docs * ((a.M + X::UNITS - 1) / X::UNITS) / (2 * warps);
+    const int piece = X::UNITS * (int)max((int64_t)1, min((int64_t)X::MOST, stretches));
+    const int64_t pieces = (a.M + piece - 1) / piece;
+    // the item: a document and the first unit of a piece; and so many of either to the next one
+    const int64_t first = (int64_t)blockIdx.x * X::WARPS + warp, step_at = warps % docs, step_j = warps / docs * piece;
+    int64_t at = first % docs, j0 = first / docs * piece;
+    bool more = j0 < a.M;
     int64_t p_next = 0;
     int32_t orig_next = 0;
     auto ask = [&]() { if (more) { p_next = whole ? at : (int64_t)a.dense[at]; orig_next = a.perm[p_next]; } };
@@ -91,8 +95,10 @@ screen_dense_kernel(const VerifyArgs a)
         const int64_t p = p_next, jp = j0;
         const int32_t orig = orig_next;
         const int beg = __ldg(a.rowptr + orig), n = __ldg(a.rowptr + orig + 1) - beg;
-        at += warps;
-        more = in_turn();
+        at += step_at;
+        j0 += step_j;
+        if (at >= docs) { at -= docs; j0 += piece; }
+        more = j0 < a.M;
         ask();
         Best<TOP2> best;
         best.init();
@@ -102,8 +108,8 @@ screen_dense_kernel(const VerifyArgs a)
         const WT *col = column(j);
         u64 w[C][VEC ? 2 : H];
         bool ahead = false;                                  // the first rows of a pass are on their way
-        for (int x = 0; x < X::PIECE && jp + x < a.M; x += X::UNITS, j += X::UNITS) {
-            const bool last = x + X::UNITS >= X::PIECE || jp + x + X::UNITS >= a.M;
+        for (int x = 0; x < piece && jp + x < a.M; x += X::UNITS, j += X::UNITS) {
+            const bool last = x + X::UNITS >= piece || jp + x + X::UNITS >= a.M;
             const WT *next = column(j + X::UNITS);
             float sum[OWN];
             int64_t own = j;

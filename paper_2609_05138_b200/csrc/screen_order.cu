@@ -21,8 +21,10 @@ static const uint32_t ORDER_STEP_MAX = 256;          // units in one fine step, 
 // 0.85, 17 and 5.5 ps a weight.)
 static const float ORDER_SLAB = 40.f, ORDER_SLAB_BY_NORM = 46.f, ORDER_SET = 30.f;
 static const float ORDER_BESIDE = 30000.f;
-// ... and 10^-3 ns for a unit and a document that is evaluated whole
-static const float ORDER_WHOLE = 15.f;
+// ... and 10^-3 ns for a unit and a document that is evaluated whole.  Such documents are few here and come with the
+// codebook's latency from DRAM: 60,000 documents on fp16 256 x 256 2,962 us so, 3,008 at 15 and 3,043 at 34, 120,000 on
+// 64 x 64 840, 860 and 830, 100,000 on 512 x 512 12.84, 12.88 and 13.05 ms.
+static const float ORDER_WHOLE = 26.f;
 static const float ORDER_IMAGE = 0.9f, ORDER_IMAGE_ALONE = 12.f, ORDER_IMAGE_NEAR = 5.5f;
 
 __device__ __forceinline__ uint32_t order_scan(uint32_t v, uint32_t *s_warp)      // exclusive, over the block
