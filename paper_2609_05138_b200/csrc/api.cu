@@ -505,7 +505,7 @@ static int screen_search(const void *W, int f16, int64_t D, int64_t M, const flo
     uint32_t *tickets = reinterpret_cast<uint32_t *>(sb + l.screen.tickets);
     uint32_t *nat_list = reinterpret_cast<uint32_t *>(sb + l.screen.nat_list);
     const int sets = (int)(l.screen.n_pad / SC_DOCS);
-    const int64_t ord_launches = M >= SC_ORDER_MIN ? cl.ord_launches : 0;
+    const int64_t ord_launches = screen_order_possible(D, M, N) ? cl.ord_launches : 0;
     if (ord_launches && (rc = launch_screen_order(norms, D, M, N, launches, cb, cl, scalars, earlier, status, set_reach, sets,
                                                   tickets, nat_list, s)))
         return rc;

@@ -238,6 +238,8 @@ int launch_screen_prepare(const void *W, int f16, int64_t D, int64_t M, const fl
                           float *scalars, const float *earlier, float *sample, float *window, float2 *reach,
                           uint32_t *bound, uint32_t *count, uint32_t *set_reach, int64_t n_pad, bool top2,
                           uint32_t *status, cudaStream_t s);
+// whether that can be decided in favour of the order of the norms at all, or nothing of it is launched
+bool screen_order_possible(int64_t D, int64_t M, int64_t N);
 // which sets of documents are swept in the order of the norms, and the units in that order
 int launch_screen_order(const float *norms, int64_t D, int64_t M, int64_t N, int64_t launches, char *cb,
                         const ScreenLayout &cl, float *scalars, const float *earlier, const uint32_t *status,

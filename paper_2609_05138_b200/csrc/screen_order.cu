@@ -215,6 +215,14 @@ screen_order_kernel(const float *__restrict__ norms, int64_t D, int64_t M, int64
     }
 }
 
+// All of the map swept in its own order takes no more than the other costs beside it: the kernel would say so for every
+// codebook (4,000 documents on 1,024 units, D = 4,096: 105 us with its launches, 95 without them).
+bool screen_order_possible(int64_t D, int64_t M, int64_t N)
+{
+    const double sets = (double)((N + SC_DOCS - 1) / SC_DOCS), slabs = (double)((M + SC_SLAB - 1) / SC_SLAB);
+    return M >= SC_ORDER_MIN && 1e-3 * ORDER_IMAGE * (double)D * (double)M + ORDER_SLAB * sets * slabs > 0.999 * ORDER_BESIDE;
+}
+
 int launch_screen_order(const float *norms, int64_t D, int64_t M, int64_t N, int64_t launches, char *cb,
                         const ScreenLayout &cl, float *scalars, const float *earlier, const uint32_t *status,
                         const uint32_t *set_reach, int sets, uint32_t *tickets, uint32_t *nat_list, cudaStream_t s)

@@ -371,27 +371,29 @@ screen_table_kernel(const WT *__restrict__ W, int64_t M, const float *__restrict
     }
 }
 
-// ---- windows: one warp per planned document -----------------------------------------------
+// ---- windows: half a warp per planned document --------------------------------------------
 // 2 B of what the rows of a document's ids bring; and, by `order`, how far it reaches: a bound of its smallest
 // (TOP2: second smallest) approximate value from the reference units, which is their own value and B (and B once
 // more, so that the bound holds for what the verify stage computes), and 2 R + 2 B.
 struct ScreenWindow { float window, bound, reach; };
 
+// ... by LANES lanes, the rest of the warp the same for another document; `there`: or there is none
+template <int LANES>
 __device__ __forceinline__ ScreenWindow screen_window_of(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
                                                          int64_t i, const uint32_t *__restrict__ key,
                                                          const uint4 *table, const float *scalars,
-                                                         bool order, bool top2,
+                                                         bool there, bool order, bool top2,
                                                          [[maybe_unused]] int64_t D, [[maybe_unused]] uint32_t *status)
 {
-    const int lane = threadIdx.x & 31;
-    const int beg = __ldg(rowptr + i), end = __ldg(rowptr + i + 1);
+    const int lane = threadIdx.x & (LANES - 1);
+    const int beg = there ? __ldg(rowptr + i) : 0, end = there ? __ldg(rowptr + i + 1) : 0;
     float en = 0.f, eo = 0.f, aa = 0.f, rr = 0.f, ra = 0.f, rb = 0.f;
     uint32_t in = 0u;
-    for (int e0 = beg; e0 < end; e0 += 128) {
+    for (int e0 = beg; e0 < end; e0 += 4 * LANES) {
         int f[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int e = e0 + 32 * u + lane;
+            const int e = e0 + LANES * u + lane;
             f[u] = e < end ? (int)BMU_IDX((uint32_t)__ldg(colidx + e), D, status) : -1;
         }
         uint4 t[4];
@@ -403,9 +405,10 @@ __device__ __forceinline__ ScreenWindow screen_window_of(const int32_t *__restri
             if (order) { rr += screen_hi16(t[u].z); ra += screen_lo16(t[u].w); rb += screen_hi16(t[u].w); }
         }
     }
-    in = __reduce_or_sync(0xffffffffu, in);
+    __syncwarp();
+    in = __ballot_sync(0xffffffffu, in & 1u) & (LANES == 32 ? 0xffffffffu : threadIdx.x & 16 ? 0xffff0000u : 0xffffu);
 #pragma unroll
-    for (int m = 16; m > 0; m >>= 1) {
+    for (int m = LANES / 2; m > 0; m >>= 1) {
         en += __shfl_xor_sync(0xffffffffu, en, m);
         eo += __shfl_xor_sync(0xffffffffu, eo, m);
         aa += __shfl_xor_sync(0xffffffffu, aa, m);
@@ -416,8 +419,8 @@ __device__ __forceinline__ ScreenWindow screen_window_of(const int32_t *__restri
         }
     }
     // a list that repeats a head id is gathered whole
-    const float n = (float)(end - beg), gathered = (float)key[i];
-    const float E = (in & 1u) && gathered == n ? eo : en;
+    const float n = (float)(end - beg), gathered = there ? (float)key[i] : 0.f;
+    const float E = in && gathered == n ? eo : en;
     float B = 2.f * E + 1.1920929e-7f * (n * aa + 4.f * scalars[5] + 8.f * aa);
     const float wide = 1.f + 1.f / 4096.f + 2.f * n * 1.1920929e-7f;    // the roundings of these sums themselves
     B *= wide;
@@ -436,6 +439,8 @@ __device__ __forceinline__ ScreenWindow screen_window_of(const int32_t *__restri
 }
 
 // The first blocks, one per sampled document: how many of its groups lie within its window.
+// Bound by issue as much as by the latency of three dependent loads: with a warp per document, whose reductions and last
+// steps then serve one, 120,000 documents of 80 ids took 57 us instead of 39 (41 without the reaches).
 __global__ void __launch_bounds__(256, 6)
 screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx,
                      const int32_t *__restrict__ perm, const uint32_t *__restrict__ key, int64_t N, int64_t n_pad,
@@ -453,8 +458,8 @@ screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restri
         const int64_t n = (M + SC_GROUP - 1) / SC_GROUP;
         const float *of = groups + blockIdx.x * n;
         if (warp == 0) {
-            const ScreenWindow w = screen_window_of(rowptr, colidx, screen_sample_doc(blockIdx.x, sampled, N), key, table,
-                                                    scalars, false, top2, D, status);
+            const ScreenWindow w = screen_window_of<32>(rowptr, colidx, screen_sample_doc(blockIdx.x, sampled, N), key, table,
+                                                        scalars, true, false, top2, D, status);
             if (lane == 0) s_win = w.window;
         }
         float least = CUDART_INF_F;
@@ -478,28 +483,28 @@ screen_window_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restri
         }
         return;
     }
-    // (n_pad is a multiple of the eight documents of a block, and so is a set of them)
-    __shared__ uint32_t s_far[8];
-    const int64_t p = ((int64_t)(blockIdx.x - sampled) * blockDim.x + threadIdx.x) >> 5;
+    // (n_pad is a multiple of the sixteen documents of a block, and so is a set of them)
+    __shared__ uint32_t s_far[16];
+    const int64_t p = ((int64_t)(blockIdx.x - sampled) * blockDim.x + threadIdx.x) >> 4;
     const bool there = p < N && !(*status & PLAN_STATUS_OVERFLOW);
-    ScreenWindow w = {0.f, -CUDART_INF_F, 0.f};
-    if (there) w = screen_window_of(rowptr, colidx, perm[p], key, table, scalars, order, top2, D, status);
-    if (lane == 0) window[p] = w.window;
+    ScreenWindow w = screen_window_of<16>(rowptr, colidx, there ? perm[p] : 0, key, table, scalars, there, order, top2, D, status);
+    if (!there) w.window = 0.f;
+    if ((lane & 15) == 0) window[p] = w.window;
     if (!order) return;
-    if (lane == 0) {
+    if ((lane & 15) == 0) {
         // (documents that are evaluated whole need no slab)
         const bool none = !there || w.window == CUDART_INF_F;
         const float t = none ? -CUDART_INF_F : w.bound + w.window + w.reach;
         reach[p] = make_float2(t == t ? t : CUDART_INF_F, w.reach);
         bound[p] = float_to_ordered(none ? -CUDART_INF_F : w.bound);
         count[p] = 0u;
-        s_far[warp] = none ? 0u : float_to_ordered(t == t ? t : CUDART_INF_F);
+        s_far[threadIdx.x >> 4] = none ? 0u : float_to_ordered(t == t ? t : CUDART_INF_F);
         const ScreenSteps steps(scalars);
         if (!none && t < steps.top) atomicAdd(status + STATUS_REACH + steps.of(t), 1u);
     }
     __syncthreads();
-    if (threadIdx.x < 8) {
-        const uint32_t far = __reduce_max_sync(0xffu, s_far[threadIdx.x]);
+    if (threadIdx.x < 16) {
+        const uint32_t far = __reduce_max_sync(0xffffu, s_far[threadIdx.x]);
         if (threadIdx.x == 0 && far) atomicMax(set_reach + p / SC_DOCS, far);
     }
 }
@@ -528,7 +533,7 @@ int launch_screen_prepare(const void *W, int f16, int64_t D, int64_t M, const fl
                           uint32_t *bound, uint32_t *count, uint32_t *set_reach, int64_t n_pad, bool top2,
                           uint32_t *status, cudaStream_t s)
 {
-    const int order = M >= SC_ORDER_MIN;
+    const int order = screen_order_possible(D, M, N);
     // (an earlier search of the same codebook has decided for this one too)
     const int sampled = earlier ? 0 : (int)(N < SC_SAMPLE ? N : SC_SAMPLE);
     float *rmin = reinterpret_cast<float *>(cb + cl.rmin), *rmax = reinterpret_cast<float *>(cb + cl.rmax);
@@ -555,7 +560,7 @@ int launch_screen_prepare(const void *W, int f16, int64_t D, int64_t M, const fl
         return e;
     };
     BMU_CUDA(f16 ? tables(static_cast<const __half *>(W)) : tables(static_cast<const float *>(W)));
-    ScreenLaunch l((unsigned)(sampled + (n_pad * 32 + 255) / 256), 256, s, true);
+    ScreenLaunch l((unsigned)(sampled + n_pad / 16), 256, s, true);
     BMU_CUDA(cudaLaunchKernelEx(&l.c, screen_window_kernel, rowptr, colidx, perm, key, N, n_pad, (const uint4 *)table, scalars,
                                 order, (int)top2, window, reach, bound, count, set_reach, D, sampled, (const float *)sample,
                                 M, status));

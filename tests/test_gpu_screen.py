@@ -360,6 +360,22 @@ def test_batches_share_the_images_of_the_codebook(bmu):
         assert torch.equal(rb.cpu(), ob) and torch.equal(rd.cpu(), od)
 
 
+@pytest.mark.parametrize("n,more", [(1, 0), (4000, 0), (60_000, 4)])
+def test_nothing_is_launched_for_an_order_that_cannot_pay(bmu, n, more):
+    """A map of 1,024 units, from which on norms are looked at, against one of 1,023: the order kernel, the images, the
+    sweep and the verification of slabs by norm only where the whole sweep takes longer than these cost."""
+    D, dev = 4096, torch.device("cuda")
+    rp, ci = synth.draw_corpus(n, D, 1.0, torch.full((n,), 64, dtype=torch.int64, device=dev), 3, dev)
+    launches = []
+    for M in (1023, 1024):
+        W = torch.rand((D, M), generator=torch.Generator(device=dev).manual_seed(4), device=dev)
+        norms = bmu.bmu_codebook_norms(W)
+        before = bmu.bmu_kernel_launches()
+        bmu.bmu_search_ws(W, rp, ci, norms=norms, opts=opts_of(bmu))
+        launches.append(bmu.bmu_kernel_launches() - before)
+    assert launches[1] - launches[0] == more, launches
+
+
 def test_a_large_codebook_shares_its_images(bmu):
     """640,000 units of 1,536 features: 1.97 GB of images in the order of the map, which batches share, and as many as
     a quarter of them again in the order of the norms, which must not keep the former from being shared."""
