@@ -66,7 +66,7 @@ static const int SC_TAIL_REGS = 112, SC_CTRL_REGS = 32;      // registers after 
 static const int SC_KS = 4, SC_NS = 2;
 // Tensor memory: the accumulators from column 0 -- two that alternate between slabs if X_head
 // leaves room (up to 1024 features), else one --, X_head in the last head_pad / 4 columns.
-static const size_t SC_SMEM = SC_NS * SC_KS * MMA_STAGE_BYTES + (2 * SC_NS + 5) * 8 + 32;
+static const size_t SC_SMEM = SC_NS * SC_KS * MMA_STAGE_BYTES + (2 * SC_NS + 5) * 8 + 8 + 2 * 16;
 
 // Adds the sixteen bytes of two rows to a lane's sums.  acc[w] holds the sum of words w modulo 2^32,
 // acc[4 + w] the 16-bit sums of their bytes 1 and 3; sc_even takes those out of the former.
@@ -120,7 +120,7 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
     extern __shared__ __align__(128) unsigned char smem[];
     u64 *bars = reinterpret_cast<u64 *>(smem + NS * KS * MMA_STAGE_BYTES);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * NS + 5);
-    volatile uint32_t *abort_flag = tmem_slot + 1, *item_slot = tmem_slot + 2;
+    volatile uint32_t *abort_flag = tmem_slot + 1, *item_slot = tmem_slot + 2;       // (two items, four words each)
     const uint32_t wfull0 = mm_smem(bars), wempty0 = mm_smem(bars + NS);
     const uint32_t tfull0 = mm_smem(bars + 2 * NS), tempty0 = tfull0 + 16, drain = tfull0 + 32;
     const int two = a.head_pad <= 1024, x_col = 512 - a.head_pad / 4;
@@ -149,18 +149,51 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
     __syncthreads();
     mm_fence_after();
     const uint32_t tmem = *tmem_slot;
-    // Registers change hands as in sweep_screen.cu.  The loops over the items meet three times an item: the item is
-    // known; X_head is in place; X_head has been read, for every accumulator has been waited for.
-    int done = 0;                                         // slabs before this item: which accumulator, which phase
+    // The control warpgroup hands registers to the four tail warpgroups, whose loads in flight are bounded by theirs: the
+    // block is launched with 96 per thread (640 x 96 = 61440 = 128 x 32 + 512 x 112), so the increase never waits for
+    // registers that nobody releases (the launcher checks the build).
+    // The loops over the items meet twice an item: X_head is in place; X_head has been read, for every accumulator has
+    // been waited for, and the next item is known.
+    int done = 0, turn = 0;                               // slabs before this item: which accumulator, which phase; items
     if (warp >= NTW) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SC_CTRL_REGS));
     int slot = 0, issued = 0;                             // ring of W stages: the producer's and the issuer's
     uint32_t phase = warp == NTW ? 1u : 0u;               // (a fresh ring counts as empty)
     bool ok = true;
-    for (;;) {
-        block_sync();
-        const int s_lo = (int)(item_slot[1] & 0xffffu), slabs = (int)(item_slot[1] >> 16) - s_lo;
-        if (item_slot[0] == ~0u) break;
+    // Item t into the place of the `to`-th one: set of documents (none: there are no more; a block that gave up: let the
+    // grid drain), slabs, part.
+    auto decode = [&](uint32_t t, int to) {
+        uint32_t set = ~0u, range = 0u, part = 0u;
+        if (*abort_flag || *reinterpret_cast<volatile uint32_t *>(a.status)) {
+        } else if (!ORDERED) {
+            const uint32_t n = screen_natural(a.scalars), sets = n == SC_ALL ? (uint32_t)a.blocks : n;
+            const uint32_t splits = (uint32_t)screen_parts(a.scalars, a.splits, a.most_splits);
+            if (t < sets * splits) {
+                set = t % sets;
+                part = t / sets;
+                if (n != SC_ALL) set = a.nat_list[set];
+                range = (uint32_t)a.n_slabs * part / splits | (uint32_t)a.n_slabs * (part + 1) / splits << 16;
+            }
+        } else {
+            for (int c = 0; c < SC_PARTS; ++c) {          // the lists one after the other
+                const uint32_t n = __ldcg(o.tickets + c);
+                if (t < n) {
+                    const uint2 item = o.items[(size_t)c * a.blocks + t];
+                    set = item.x; range = item.y;
+                    break;
+                }
+                t -= n;
+            }
+        }
+        volatile uint32_t *d = item_slot + 4 * (to & 1);
+        d[0] = set; d[1] = range; d[2] = part;
+    };
+    if (warp == NTW + 1 && lane == 0) decode(blockIdx.x, 0);
+    block_sync();
+    for (;; ++turn) {
+        const uint32_t range = item_slot[4 * (turn & 1) + 1];
+        const int s_lo = (int)(range & 0xffffu), slabs = (int)(range >> 16) - s_lo;
+        if (item_slot[4 * (turn & 1)] == ~0u) break;
         mm_fence_before();
         block_sync();
         mm_fence_after();
@@ -207,7 +240,25 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
                 }
                 if (ok) mm_commit_warp(tfull0 + 8 * buf);
             }
+            // The next item, now that the last slab is all that is left to gather (two slabs with two accumulators; not at
+            // the item's beginning: whoever waits for a long one must not hold another).  By this warp, which has nothing
+            // else to do: a tail warp that drew it waited for the counter in front of its last slab, and all others for the
+            // item to be looked up (120,000 documents on 64 x 64, D = 4,096, 1,251 -> 1,223 us; 200,000 on a trained 128 x
+            // 128 map, planned, 10.65 -> 10.60 ms).  As many tickets as items are taken, if any: then the counter is
+            // zero again.
+            if (lane == 0) {
+                uint32_t t;
+                if (ORDERED) {
+                    t = atomicAdd(o.tickets + SC_PARTS, 1u);
+                } else {
+                    const uint32_t sets = screen_natural(a.scalars);
+                    const uint32_t items = (sets == SC_ALL ? (uint32_t)a.blocks : sets) * (uint32_t)screen_parts(a.scalars, a.splits, a.most_splits);
+                    t = items > gridDim.x ? atomicInc(a.ticket, items - 1u) : items;
+                }
+                decode(gridDim.x + t, turn + 1);
+            }
         }
+        __syncwarp();
         done += slabs;
         mm_fence_before();
         block_sync();
@@ -228,53 +279,13 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
     } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SC_TAIL_REGS));
     const int q = warp & 3, e = warp >> 2;
-    // Thread 0: the block's own item first; the ticket of the next one is on its way under an item's last slab (not
-    // from the item's beginning: whoever waits for a long one must not hold another).  As many tickets as items are
-    // taken, if any: then the counter is zero again.
-    auto sets_of = [&]() { const uint32_t n = screen_natural(a.scalars); return n == SC_ALL ? (uint32_t)a.blocks : n; };
-    auto take = [&]() {
-        if (threadIdx.x) return;
-        uint32_t t;
-        if (ORDERED) {
-            t = atomicAdd(o.tickets + SC_PARTS, 1u);
-        } else {
-            const uint32_t items = sets_of() * (uint32_t)screen_parts(a.scalars, a.splits, a.most_splits);
-            t = items > gridDim.x ? atomicInc(a.ticket, items - 1u) : items;
-        }
-        item_slot[3] = gridDim.x + t;
-    };
-    if (threadIdx.x == 0) item_slot[3] = blockIdx.x;
-    for (;;) {
-        // the next item (a block that gave up: let the grid drain)
-        if (threadIdx.x == 0) {
-            uint32_t set = ~0u, range = 0u, part = 0u;       // (no set: there are no more items)
-            uint32_t t = item_slot[3];
-            if (*abort_flag || *reinterpret_cast<volatile uint32_t *>(a.status)) {
-            } else if (!ORDERED) {
-                const uint32_t sets = sets_of(), splits = (uint32_t)screen_parts(a.scalars, a.splits, a.most_splits);
-                if (t < sets * splits) {
-                    set = t % sets;
-                    part = t / sets;
-                    if (screen_natural(a.scalars) != SC_ALL) set = a.nat_list[set];
-                    range = (uint32_t)a.n_slabs * part / splits | (uint32_t)a.n_slabs * (part + 1) / splits << 16;
-                }
-            } else {
-                for (int c = 0; c < SC_PARTS; ++c) {         // the lists one after the other
-                    const uint32_t n = __ldcg(o.tickets + c);
-                    if (t < n) {
-                        const uint2 item = o.items[(size_t)c * a.blocks + t];
-                        set = item.x; range = item.y;
-                        break;
-                    }
-                    t -= n;
-                }
-            }
-            item_slot[0] = set; item_slot[1] = range; item_slot[2] = part;
-        }
-        block_sync();
-        if (item_slot[0] == ~0u) break;
-        const int group = (int)item_slot[0];
-        const int s_lo = (int)(item_slot[1] & 0xffffu), s_hi = (int)(item_slot[1] >> 16), slabs = s_hi - s_lo;
+    block_sync();
+    for (;; ++turn) {
+        const volatile uint32_t *item = item_slot + 4 * (turn & 1);
+        if (item[0] == ~0u) break;
+        const int group = (int)item[0];
+        const int s_lo = (int)(item[1] & 0xffffu), s_hi = (int)(item[1] >> 16);
+        const int shift = done - s_lo;                    // from a slab of the launch to its number among the block's
         {
             // X_head into tensor memory: lane 32q + l = document, a column = four features
             const int words = a.head / 32;
@@ -323,7 +334,7 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
         [[maybe_unused]] float own = 3.0e38f;
         [[maybe_unused]] uint32_t mask = 0u;
         [[maybe_unused]] int valid = s_lo;
-        auto stripe = [&]() { return ((size_t)item_slot[2] * a.n_pad + p) * 4 + li; };
+        auto stripe = [&]() { return ((size_t)item[2] * a.n_pad + p) * 4 + li; };
         if constexpr (ORDERED) {
             const float2 r = o.reach[p];
             if (r.x <= a.scalars[SC_DOC_TOP]) reach = r.y;
@@ -356,13 +367,11 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
         [[maybe_unused]] bool head_first = ORDERED && o.slab0 + s_lo > 0, begun = !head_first;
         [[maybe_unused]] const u64 tail_most = sc_pack((float)(4u * quads) * a.scalars[4], (float)(4u * quads) * a.scalars[4]);
         if (quads && begun) begin();
-        bool taken = false;
         for (int sl = s_lo; sl < s_hi; ++sl, np += SC_SLAB) {
-            const int n = done + sl - s_lo;
-            if (sl + 1 == s_hi) { take(); taken = true; }
+            const int n = sl + shift;
             // no document of the tile reaches this slab, nor any behind it: the accumulators still change hands
             if (ORDERED && !__any_sync(0xffffffffu, o.unit_norm[sl * SC_SLAB] <= (TOP2 ? m2 : m1) + win + reach)) {
-                for (int r = n; r < done + slabs; ++r) {
+                for (int r = n; r < shift + s_hi; ++r) {
                     mm_wait(tfull0 + 8 * (r & two), (r >> two) & 1, abort_flag, a.status, 8u);
                     __syncwarp();
                     if (lane == 0) mm_bar_arrive(tempty0 + 8 * (r & two));
@@ -552,8 +561,7 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
             a.cval[stripe()] = make_float2(own, __int_as_float(valid | (s_hi << 8)));
             if (TOP2) a.cval2[stripe()] = m2;
         }
-        if (!taken) take();
-        done += slabs;
+        done = shift + s_hi;
         mm_fence_before();
         block_sync();
         mm_fence_after();
