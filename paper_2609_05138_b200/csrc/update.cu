@@ -721,9 +721,10 @@ int launch_update_blur(const uint32_t *num, const uint32_t *cnt, int64_t D, int3
     // Maps of whole 16-byte rows of 16 to 512 units at radii up to 8: the kernel that walks down the columns, faster
     // than the others wherever it was measured there (4,096 x 32 x 32, radius 6: 24 us, 36; 6,000 x 100 x 90: 115, 211;
     // 2,000 x 512 x 512: 855, 1,165; narrower rows leave its staging too little room, wider ones more than its 128
-    // threads).  Wider maps whose 64 x 64 tiles are at least three quarters map: the tiled one (128 x 128 x 16,384,
-    // radius 2 / 6: 451 / 589 us, that of whole-map tiles 616 / 723).  Everything else: the one of whole-map tiles
-    // (90 x 70 x 10,007, radius 6 / 20: 230 / 400 us; before it a kernel with the radius in a loop took 543 / 1721).
+    // threads).  Wider maps whose 64 x 64 tiles are at least three quarters map: the tiled one (500 x 2,048 x 512, radius
+    // 2 / 6: 911 / 1,166 us, that of whole-map tiles 1,469 / 1,766; 2,000 x 576 x 64 142 / 175, 191 / 220; 1,000 x 1,000 x
+    // 120 228 / 296, 290 / 387).  Everything else: the one of whole-map tiles (90 x 70 x 10,007, radius 6 / 20: 230 / 400
+    // us; before it a kernel with the radius in a loop took 543 / 1721).
     const int64_t tiled_area = (int64_t)((edge_x + 63) / 64) * ((edge_y + 63) / 64) * 4096;
     const bool outs = ((reinterpret_cast<uintptr_t>(num_blur) | reinterpret_cast<uintptr_t>(cnt_blur)) & 15) == 0;
     int dev = 0, sms = 148;

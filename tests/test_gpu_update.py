@@ -119,6 +119,22 @@ def test_blur_of_columns_in_registers(bmu, ex, ey, D, radius):
         assert np.all(np.abs(got - ref) <= 2e-6 * ref.max(axis=1, keepdims=True))
 
 
+@pytest.mark.parametrize("ex,ey,D", [(576, 64, 2), (640, 250, 1), (1000, 120, 1), (1024, 65, 2)])
+@pytest.mark.parametrize("radius", [1, 2, 3, 4, 5, 6, 7, 8])
+def test_blur_of_tiles_on_wide_maps(bmu, ex, ey, D, radius):
+    """Rows of more than 512 units, which the kernel above leaves to the one of 64 x 64 tiles where these are at least
+    three quarters map (1024 x 65: not; the one of whole-map tiles); every radius is an instance of its own."""
+    M, sigma = ex * ey, radius / 3 - 1e-4
+    g = torch.Generator().manual_seed(ex + ey + radius)
+    num = torch.randint(0, 2_000_000, (D, M), generator=g, dtype=torch.int32)
+    cnt = torch.randint(0, 50, (M,), generator=g, dtype=torch.int32)
+    nb, cb = bmu.bmu_update_blur(num.cuda(), cnt.cuda(), ex, ey, sigma)
+    for got, ref in ((nb.cpu().numpy(), oracle.blur(num.numpy(), ex, ey, sigma)),
+                     (cb.cpu().numpy()[None], oracle.blur(cnt.numpy()[None], ex, ey, sigma).reshape(1, -1))):
+        got, ref = got.reshape(ref.shape[0], -1), ref.reshape(ref.shape[0], -1)
+        assert np.all(np.abs(got - ref) <= 2e-6 * ref.max(axis=1, keepdims=True))
+
+
 def test_blur_refuses_a_neighbourhood_it_cannot_hold(bmu):
     num = torch.zeros((1, 64), dtype=torch.int32, device="cuda")
     cnt = torch.zeros(64, dtype=torch.int32, device="cuda")
