@@ -1,6 +1,7 @@
 """Child process of tests/test_gpu_bounds_checked.py: runs with BMU_LIBRARY pointing at the
 bounds-checked build of the library (every id- and offset-derived address checked, violations
 recorded in the status word instead of performed) and prints one JSON line."""
+import ctypes
 import json
 import sys
 
@@ -9,6 +10,7 @@ import torch
 
 from inputs import synth
 from tests import parity
+from tests.test_gpu_screen import order_of, short_lists
 import paper_2609_05138_b200 as bmu
 
 
@@ -98,6 +100,30 @@ def main():
         got = compare(out[0].cpu().numpy(), out[1].cpu().numpy(), W.numpy(), r.cpu().numpy(), c.cpu().numpy())
         res["two_stage"].append({"name": name, "status": st, "failed": got["failed"], "docs": got["docs"],
                                  "detail": got.get("detail")})
+    # ... and with slabs in the order of the norms: whole and ragged rows, several launches, a second-best unit, half
+    # precision; sets swept in the order of the map beside it, and documents evaluated whole
+    res["by_norm"] = []
+    for name, M, kw, every in (("aligned", 1024, {}, 50), ("ragged", 1027, {}, 0), ("top2", 1027, {}, 50),
+                               ("launches", 3330, {"chunk_neurons": 640}, 0), ("f16", 1024, {}, 50)):
+        r, c = (x.cuda() for x in short_lists(36_000, cfg.D, 9, every=every, extra=((300, 700),)))
+        W = torch.rand((cfg.D, M), generator=torch.Generator().manual_seed(M)).half().float()
+        norms = bmu.bmu_codebook_norms(W.cuda())
+        o = bmu.Opts()
+        o.two_stage = 1
+        for k, v in kw.items():
+            setattr(o, k, v)
+        need = max(int(getattr(bmu.load(), "bmu_search_%sworkspace_bytes" % q)(cfg.D, M, 36_000, c.numel(), ctypes.byref(o)))
+                   for q in ("top2_", "f16_"))
+        ws = torch.zeros(need + 256, dtype=torch.uint8, device="cuda")
+        if name == "f16":
+            out = bmu.bmu_search_f16_ws(W.cuda().half(), r, c, norms=norms, opts=o, workspace=ws)
+        else:
+            call = bmu.bmu_search_top2_ws if name == "top2" else bmu.bmu_search_ws
+            out = call(W.cuda(), r, c, norms=norms, opts=o, workspace=ws)
+        torch.cuda.synchronize()
+        got = compare(out[0].cpu().numpy(), out[1].cpu().numpy(), W.numpy(), r.cpu().numpy(), c.cpu().numpy())
+        res["by_norm"].append({"name": name, "status": status_word(ws), "failed": got["failed"], "docs": got["docs"],
+                               "detail": got.get("detail"), "order": order_of(ws, norms)})
     W = synth.make_codebook(cfg.D, 1024, 7, kind="scaled")
 
     # an id beyond the vocabulary: the checked build records it and leaves the access out.  The

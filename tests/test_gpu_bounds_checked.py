@@ -45,6 +45,12 @@ def test_the_two_stage_search_and_few_documents_run_clean(report):
         assert case["status"] == 0 and case["failed"] == 0 and case["docs"] == docs, case
 
 
+def test_slabs_in_the_order_of_the_norms_run_clean(report):
+    assert len(report["by_norm"]) == 5
+    for case in report["by_norm"]:
+        assert case["status"] == 0 and case["failed"] == 0 and case["docs"] == 36_000 and case["order"], case
+
+
 def test_an_id_beyond_the_vocabulary_is_reported_not_performed(report):
     for case in report["flagged"]:
         assert case["status"] & 128, case

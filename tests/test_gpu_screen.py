@@ -3,6 +3,8 @@ all units, what it cannot rule out is evaluated exactly in fp32) against the ora
 of its tiles: documents per tile and block, units per group, slab and launch, heads that fill part
 of a stage, lists that are empty, long, unsorted or repeat ids, and codebooks where nothing can be
 ruled out."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -411,7 +413,8 @@ def lists(lens, D, seed):
 @pytest.mark.parametrize("n_docs", [1, 129, 700])
 def test_slabs_in_the_order_of_the_norms(bmu, M, chunk, n_docs):
     """Norms that spread further than a document reaches: short lists on an iid U[0,1) codebook.  Some lists are
-    empty, some reach half of the map, one all of it; best and second-best unit, half precision, a plan."""
+    empty, some reach half of the map, one all of it; best and second-best unit, half precision, a plan.  So few that
+    the order of the norms cannot pay and none is made: the same lists by the thousand further down."""
     D = 4096
     r = np.random.default_rng(M + n_docs)
     lens = r.integers(0, 24, n_docs)
@@ -438,8 +441,8 @@ def test_slabs_in_the_order_of_the_norms(bmu, M, chunk, n_docs):
 
 @pytest.mark.parametrize("copies", [2, 40, 1500])
 def test_equal_units_in_the_order_of_the_norms(bmu, copies):
-    """The unit of the smallest norm many times over the map: the lowest index wins, the next one is second; 1,500
-    of them are more than a document's list holds."""
+    """The unit of the smallest norm many times over the map: the lowest index wins, the next one is second (300
+    documents: in the order of the map; where norms are in order, further down)."""
     D, M = 4096, 4096
     rowptr, colidx = lists(np.random.default_rng(3).integers(0, 24, 300), D, 4)
     W = torch.rand((D, M), generator=torch.Generator().manual_seed(5))
@@ -454,7 +457,8 @@ def test_equal_units_in_the_order_of_the_norms(bmu, copies):
 
 @pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan")])
 def test_norms_that_have_no_place_in_an_order(bmu, value):
-    """A unit at plus infinity or without a number as its norm never wins; at minus infinity it always does."""
+    """A unit at plus infinity or without a number as its norm never wins; at minus infinity it always does (200
+    documents: in the order of the map; where norms are in order, further down)."""
     D, M = 4096, 2048
     rowptr, colidx = lists(np.random.default_rng(6).integers(1, 24, 200), D, 7)
     W = torch.rand((D, M), generator=torch.Generator().manual_seed(8))
@@ -474,7 +478,8 @@ def test_norms_that_have_no_place_in_an_order(bmu, value):
 
 def test_batches_that_reach_further_than_the_first(bmu):
     """Batches share order and images: one whose lists reach further than the first one's, one of long lists only,
-    which needs the slabs in the order of the map, and a short one again."""
+    which needs the slabs in the order of the map, and a short one again (a few thousand documents; so many that
+    slabs are in the order of the norms, further down)."""
     D, M = 4096, 4096
     W = torch.rand((D, M), generator=torch.Generator().manual_seed(9)).cuda()
     r = np.random.default_rng(10)
@@ -549,3 +554,185 @@ def test_a_document_is_answered_alike_in_any_company(bmu):
     for k, (sb, sd) in enumerate(same):
         assert torch.equal(sb, ob) and torch.equal(sd, od), (k, int((sb != ob).sum()), int((sd != od).sum()))
     plan.close()
+
+
+# ---- ... with so many documents that slabs are in the order of the norms ----------------------------
+def order_of(ws, norms):
+    """What a search decided, from its workspace: None where its slabs followed the map, else (units in the order of the
+    norms, sets of documents swept in the order of the map beside it, documents evaluated whole).  Found by what stands in
+    front of it: the units of the smallest norm at even and at odd indices, and four words on those norms."""
+    off = (-ws.data_ptr()) % 256
+    words = ws[off:off + (ws.numel() - off) // 4 * 4].view(torch.int32)
+    floats = words.view(torch.float32)
+    finite = torch.where(torch.isfinite(norms), norms, torch.full_like(norms, float("inf")))
+    even, odd = 2 * int(finite[0::2].argmin()), 2 * int(finite[1::2].argmin()) + 1
+    found = (words[:-8] == even) & (words[1:-7] == odd) & (floats[4:-4] == norms[even]) & (floats[5:-3] == norms[odd])
+    (at,) = found.nonzero().flatten().tolist()
+    base = at - 16
+    return (int(words[base + 19]), int(words[base + 22]), int(words[38])) if int(words[base + 12]) else None
+
+
+def scratch(query, *sizes):
+    return torch.zeros(int(query(*sizes)) + 256, dtype=torch.uint8, device="cuda")
+
+
+def short_lists(n, D, seed, every=50, length=60, extra=()):
+    """n lists of 0 .. 23 ids, every 50th of 60 ids, and some given ones: CPU tensors."""
+    g = torch.Generator().manual_seed(seed)
+    lens = torch.randint(0, 24, (n,), generator=g)
+    if every:
+        lens[::every] = length
+    for at, m in extra:
+        lens[at] = m
+    return drawn(lens, D, seed)
+
+
+def drawn(lens, D, seed, s=0.05):
+    rowptr, colidx = synth.draw_corpus(lens.numel(), D, s, lens, seed, "cuda")
+    return rowptr.cpu(), colidx.cpu()
+
+
+@pytest.mark.parametrize("M,chunk,n,few_far", [(1024, 0, 40_000, False), (1027, 0, 40_000, False), (2304, 1024, 30_000, True),
+                                               (5000, 512, 12_000, False), (3331, 640, 24_000, True)])
+def test_many_documents_in_the_order_of_the_norms(bmu, M, chunk, n, few_far):
+    """Whole and ragged rows, last slabs that are not full, one launch and several; lists that reach far by the
+    hundred, whose sets are swept in the order of the map (or a handful, which are evaluated whole), one that
+    reaches all of the map and one that no sum holds.  Best and second-best unit, half precision, a plan."""
+    D = 4096
+    rowptr, colidx = short_lists(n, D, M, every=0 if few_far else 50, extra=((300, 700), (301, 1300)))
+    W = torch.rand((D, M), generator=torch.Generator().manual_seed(M)).half().float()
+    Wd, rp, ci, o = W.cuda(), rowptr.cuda(), colidx.cuda(), opts_of(bmu, chunk_neurons=chunk)
+    norms = bmu.bmu_codebook_norms(Wd)
+    args = (W.numpy(), rowptr.numpy(), colidx.numpy())
+    lib, by = bmu.load(), ctypes.byref(o)
+    ws = scratch(lib.bmu_search_workspace_bytes, D, M, n, ci.numel(), by)
+    ob, od = bmu.bmu_search_ws(Wd, rp, ci, norms=norms, opts=o, workspace=ws)
+    parity.compare(ob.cpu().numpy(), od.cpu().numpy(), *args)
+    kept, by_map, whole = order_of(ws, norms)
+    assert 0 < kept < M and (whole > 0 if few_far else by_map > 0), (kept, by_map, whole)
+    again = bmu.bmu_search_ws(Wd, rp, ci, norms=norms, opts=o, workspace=ws)
+    assert torch.equal(again[0], ob) and torch.equal(again[1], od)
+    ws = scratch(lib.bmu_search_top2_workspace_bytes, D, M, n, ci.numel(), by)
+    b1, d1, b2, d2 = bmu.bmu_search_top2_ws(Wd, rp, ci, norms=norms, opts=o, workspace=ws)
+    assert order_of(ws, norms)
+    assert torch.equal(b1, ob) and torch.equal(d1, od) and bool((b2 != b1).all())
+    np.testing.assert_allclose(d2.cpu().numpy(), oracle.bmu2(*args)[3], rtol=1e-6)
+    if M % 4 == 0:
+        plan = bmu.Plan(rp, ci, D, M, o)
+        pb, pd = plan.search(Wd, norms=norms)
+        assert order_of(plan.workspace, norms)
+        plan.close()
+        assert torch.equal(pb, ob) and torch.equal(pd, od)
+    if M % 256 == 0:
+        ws = scratch(lib.bmu_search_f16_workspace_bytes, D, M, n, ci.numel(), by)
+        hb, hd = bmu.bmu_search_f16_ws(Wd.half(), rp, ci, norms=norms, opts=o, workspace=ws)[:2]
+        assert order_of(ws, norms)
+        parity.compare(hb.cpu().numpy(), hd.cpu().numpy(), *args)
+
+
+@pytest.mark.parametrize("copies,step,ordered", [(2, 0.0, True), (40, 0.0, True), (200, 0.0, True), (700, 5e-8, True), (700, 0.0, False)])
+def test_equal_and_nearly_equal_units_by_norm(bmu, copies, step, ordered):
+    """Neighbours of the smallest norm: the lowest index wins, the next one is second.  700 units of nearly that norm lie
+    in the windows of all but the shortest lists, in 22 places where a document's list holds 16; 700 equal norms have no
+    order that sorting by counting finds, and the slabs follow the map."""
+    D, M, n = 4096, 8192, 12_000
+    rowptr, colidx = short_lists(n, D, 4, every=0)
+    W = torch.rand((D, M), generator=torch.Generator().manual_seed(5))
+    W[:, 7] = 0.98 * W[:, int((W ** 2).sum(0).argmin())]
+    where = 7 + torch.arange(copies)
+    W[:, where] = W[:, 7:8] * (1 + step * torch.arange(copies)[None, :])
+    Wd, rp, ci, o = W.cuda(), rowptr.cuda(), colidx.cuda(), opts_of(bmu)
+    norms = bmu.bmu_codebook_norms(Wd)
+    lib, by = bmu.load(), ctypes.byref(o)
+    ws = scratch(lib.bmu_search_workspace_bytes, D, M, n, ci.numel(), by)
+    ob, od = bmu.bmu_search_ws(Wd, rp, ci, norms=norms, opts=o, workspace=ws)
+    args = (W.numpy(), rowptr.numpy(), colidx.numpy())
+    parity.compare(ob.cpu().numpy(), od.cpu().numpy(), *args)
+    got = order_of(ws, norms)
+    assert bool(got) == ordered
+    if copies == 700 and ordered:
+        assert got[2] > n // 3                       # evaluated whole: their lists were too short
+    ws = scratch(lib.bmu_search_top2_workspace_bytes, D, M, n, ci.numel(), by)
+    b1, d1, b2, d2 = bmu.bmu_search_top2_ws(Wd, rp, ci, norms=norms, opts=o, workspace=ws)
+    assert bool(order_of(ws, norms)) == ordered
+    assert torch.equal(b1, ob) and torch.equal(d1, od) and bool((b2 != b1).all())
+    np.testing.assert_allclose(d2.cpu().numpy(), oracle.bmu2(*args)[3], rtol=1e-6)
+    if not step:
+        assert bool((b1 == 7).all()) and bool((b2 == 8).all()) and torch.equal(d1, d2)
+
+
+@pytest.mark.parametrize("value,ordered", [(float("inf"), True), (float("nan"), True), (float("-inf"), False)])
+def test_many_documents_and_norms_that_have_no_place(bmu, value, ordered):
+    """Some units at plus infinity or without a number as their norm never win, and the others are in order; one at
+    minus infinity always wins, and the slabs follow the map."""
+    D, M, n = 4096, 2050, 24_000
+    rowptr, colidx = short_lists(n, D, 7, every=0)
+    W = torch.rand((D, M), generator=torch.Generator().manual_seed(8))
+    Wd, rp, ci, o = W.cuda(), rowptr.cuda(), colidx.cuda(), opts_of(bmu)
+    norms = bmu.bmu_codebook_norms(Wd)
+    far = norms.argsort()[:1 if value < 0 else 5].sort().values
+    norms[far] = value
+    ws = scratch(bmu.load().bmu_search_workspace_bytes, D, M, n, ci.numel(), ctypes.byref(o))
+    ob, od = bmu.bmu_search_ws(Wd, rp, ci, norms=norms, opts=o, workspace=ws)
+    if value < 0:
+        assert bool((ob == far[0]).all()) and bool(torch.isinf(od).all())
+        return
+    assert bool(order_of(ws, norms)) == ordered
+    keep = torch.ones(M, dtype=torch.bool, device="cuda")
+    keep[far] = False
+    left = keep.nonzero().flatten()
+    rb, rd = bmu.bmu_search_ws(Wd[:, left].contiguous(), rp, ci, norms=norms[left].contiguous(), opts=o)
+    assert torch.equal(ob, left[rb.long()].int())
+    assert bool(((od - rd).abs() <= 1e-6 * rd.abs()).all())
+
+
+def test_many_batches_that_reach_further_than_the_first(bmu):
+    """Batches share order and images: lists that reach further than the first one's, long lists only, which need the
+    slabs in the order of the map, short ones again (order and images stand), and some that lower the steps of
+    the image, so that both images are made anew."""
+    D, M = 16384, 4096
+    W = torch.rand((D, M), generator=torch.Generator().manual_seed(9)).cuda()
+    norms = bmu.bmu_codebook_norms(W)
+    g = torch.Generator().manual_seed(10)
+    batches = []
+    for k, (n, lo, hi) in enumerate(((24_000, 20, 36), (20_000, 30, 60), (6_000, 300, 500), (24_500, 20, 36), (24_000, 20, 36), (23_000, 20, 40))):
+        lens = torch.randint(lo, hi, (n,), generator=g)
+        if k == 4:
+            lens[::100] = 800
+        batches.append(drawn(lens, D, 11 + k))
+    ordered, want = [], []
+    for rp, ci in batches:
+        assert bmu.bmu_describe_search(D, M, rp.numel() - 1, ci.numel()).two_stage
+        ws = scratch(bmu.load().bmu_search_workspace_bytes, D, M, rp.numel() - 1, ci.numel(), None)
+        want.append(bmu.bmu_search_ws(W, rp.cuda(), ci.cuda(), norms=norms, workspace=ws))
+        ordered.append(bool(order_of(ws, norms)))
+    assert ordered == [True, True, False, True, True, True]
+    outs = bmu.bmu_search_batches_host(W, [(rp.pin_memory(), ci.pin_memory()) for rp, ci in batches])
+    for (rp, ci), (ob, od), (rb, rd) in zip(batches, outs, want):
+        assert torch.equal(ob, rb.cpu()) and torch.equal(od, rd.cpu())
+        parity.compare(ob.numpy(), od.numpy(), W.cpu().numpy(), rp.numpy(), ci.numpy(), docs=np.arange(0, rp.numel() - 1, 97))
+
+
+@pytest.mark.parametrize("kind", ["by norm", "by map", "whole"])
+def test_captured_in_a_graph(bmu, kind):
+    """Launches that begin under the end of the one before stay in order when they are captured and replayed, in either
+    order of slabs and with documents evaluated whole, on other weights in the same buffers."""
+    D, M, n = 4096, 2304, 24_000
+    rowptr, colidx = short_lists(n, D, 14, every=0) if kind == "by norm" else \
+        drawn(torch.full((n,), 64, dtype=torch.int64), D, 14, 1.0)
+    rp, ci, o = rowptr.cuda(), colidx.cuda(), opts_of(bmu, chunk_neurons=1024)
+    W = synth.make_codebook(D, M, 73, kind="const" if kind == "whole" else "uniform").cuda()
+    other = synth.make_codebook(D, M, 74, kind="uniform").cuda()
+    ws = scratch(bmu.load().bmu_search_workspace_bytes, D, M, n, ci.numel(), ctypes.byref(o))
+    want = [bmu.bmu_search_ws(x, rp, ci, opts=o, workspace=ws) for x in (W, other)]
+    assert bool(order_of(ws, bmu.bmu_codebook_norms(other))) == (kind == "by norm")
+    buf, ob, od = W.clone(), torch.empty(n, dtype=torch.int32, device="cuda"), torch.empty(n, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        bmu.bmu_search_ws(buf, rp, ci, opts=o, workspace=ws, out_bmu=ob, out_dist=od)
+    for x, (wb, wd) in ((W, want[0]), (other, want[1]), (W, want[0])):
+        buf.copy_(x)
+        ob.fill_(-1)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(ob, wb) and torch.equal(od, wd)
