@@ -251,6 +251,12 @@ def scaled_traffic(rec, cfg, desc, opts, n_docs_per_launch):
     return fixed + per_doc * n_docs_per_launch
 
 
+def every_pair_summed(two_stage, M):
+    """A two-stage search of a map of 1,024 units or more may rule units out by their norms: which pairs of a document
+    and a unit were summed is then known on the device only, and no figure that counts them all is given."""
+    return not (two_stage and M >= 1024)
+
+
 def measure_roofs(bmu, dev):
     """On-chip ceilings of this GPU, measured now.  The L2 -> SM ceiling is the largest rate
     any committed microbenchmark reaches: loads alone, bulk copies alone, both together."""
@@ -392,6 +398,10 @@ def measure_config(bmu, cfg, args, dev, rank, world, roofs, peaks, steps, warmup
                  "head_mma_TFLOPs": mma_flops / launch_s / 1e12,
                  "head_mma_frac_of_bf16_peak" if parts == 2.0 else "head_mma_frac_of_twice_bf16_peak":
                  mma_flops / launch_s / 1e12 / (rate * peak16)}
+    summed = every_pair_summed(desc.two_stage, cfg.M)
+    if not summed:                              # left: what any search has to move, codebook, lists and results once
+        alg = {"hbm": ((4.0 * cfg.D * cfg.M + 4.0 * nnz + 24.0 * N) / (launch_s * n_chunks), peaks["hbm_gbs"] * 1e9, "B/s")}
+        extra = {"tail_share_of_updates": tail_share}
     bound = max(alg, key=lambda k: alg[k][0] / alg[k][1])
     ach, peak, unit = alg[bound]
     traffic = scaled_traffic(dram_traffic_record(), cfg, desc, opts, N)
@@ -404,18 +414,17 @@ def measure_config(bmu, cfg, args, dev, rank, world, roofs, peaks, steps, warmup
                            "profiles/dram_traffic_sweep_mma2.json (ncu on a small case, scaled "
                            "to this launch: codebook chunk once + the rest per document)"),
         "launch_ms": launch_s * 1e3, "launches_per_step": n_chunks * len(batches),
-        "units_per_launch": {"adds": adds, "union_rows_x_chunk": float(union_rows) * chunk},
+        "units_per_launch": {"adds": adds, "union_rows_x_chunk": float(union_rows) * chunk} if summed else None,
         "tile_reuse": reuse,
         "fractions": {k: v[0] / v[1] for k, v in alg.items()},
         **extra,
     }
-    if desc.two_stage:
-        # units that a norm rules out are counted all the same
-        roofline["counts"] = ("every (document, unit) pair; the two-stage search sums only those that the units' norms "
-                              "leave, a few per cent on this codebook: fractions are of the work of summing all")
+    if not summed:
+        roofline["counts"] = ("codebook, lists and results once; how many pairs of a document and a unit were summed, and what "
+                              "that moved, is known on the device only")
     frag = {
         "value": value, "ms_per_step": ms_per_step,
-        "updates_per_s": float(total_nnz) * cfg.M * world / (ms_per_step * 1e-3),
+        "updates_per_s": float(total_nnz) * cfg.M * world / (ms_per_step * 1e-3) if summed else None,
         "phases_ms": {"norms": norms_ms, "sweep_and_output": sweep_ms},
         "clocks": clocks, "gpu_launches": int(launches), "roofline": roofline,
         "search": {"kernel": desc.kernel, "head_rows": desc.two_stage or desc.head_rows,
@@ -609,7 +618,8 @@ def f16_codebook(bmu, cfg, W, rowptr, colidx, args):
     torch.cuda.synchronize(W.device)
     ms = e0.elapsed_time(e1) / args.steps
     return {"ms_per_step": ms, "value": n0 / (ms * 1e-3), "unit": UNIT,
-            "updates_per_s": nnz * float(M) / (ms * 1e-3), "dtype": "f16 storage, f32 sums",
+            "updates_per_s": nnz * float(M) / (ms * 1e-3) if every_pair_summed(o16.two_stage != 2, M) else None,
+            "dtype": "f16 storage, f32 sums",
             "api": "bmu_codebook_norms_f16 + bmu_search_f16_ws per step (rank 0's figure)"}
 
 

@@ -28,3 +28,9 @@ def test_bench_starts_its_own_ranks():
 def test_bench_single_rank_needs_no_launcher():
     rec = run_selfcheck(1)
     assert rec["n_gpus"] == 1 and rec["world_size"] == 1
+
+
+def test_figures_of_all_pairs_only_where_all_are_summed():
+    import bench
+    assert bench.every_pair_summed(0, 262144) and bench.every_pair_summed(1536, 1023)
+    assert not bench.every_pair_summed(1536, 1024)
