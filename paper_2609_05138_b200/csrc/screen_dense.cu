@@ -79,8 +79,9 @@ screen_dense_kernel(const VerifyArgs a)
     const bool whole = screen_whole(a.scalars);              // all documents, in the planned order
     const int64_t docs = whole ? a.N : (int64_t)*a.dense_count, warps = (int64_t)gridDim.x * X::WARPS;
     if (docs == 0) return;
-    // (few documents: pieces of fewer stretches, so that every warp has one or two)
-    const int64_t stretches = docs * ((a.M + X::UNITS - 1) / X::UNITS) / (2 * warps);
+    // Few documents: pieces of fewer stretches, so that every warp has four or more (two, eight, sixteen: 60,000 documents
+    // on fp16 256 x 256, 91 of them whole, 2,965, 2,957 and 2,984 us instead of 2,948).
+    const int64_t stretches = docs * ((a.M + X::UNITS - 1) / X::UNITS) / (4 * warps);
     const int piece = X::UNITS * (int)max((int64_t)1, min((int64_t)X::MOST, stretches));
     const int64_t pieces = (a.M + piece - 1) / piece;
     // the item: a document and the first unit of a piece; and so many of either to the next one
