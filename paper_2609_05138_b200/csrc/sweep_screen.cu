@@ -19,8 +19,8 @@
 // The MMAs of the next slab run under the gather.  Waits are bounded and report through the
 // status word.
 //
-// What bounds it (75,776 documents x 3,072 neurons, Zipf 1.1, 24 slabs in 477 us): the latency of the
-// gathered loads, 64 KB in flight per SM, which the registers of the tail warps bound; no unit is full
+// What bounds it (75,776 documents x 3,072 neurons, Zipf 1.1, 24 slabs in 477 us, and in 475 with a block per set of
+// documents, of which the parts are): the latency of the gathered loads, 64 KB in flight per SM, which the registers of the tail warps bound; no unit is full
 // (L1 data path 66 %, integer ALU 64, L2 55, tensor pipe 36).  The gather alone takes 373 us, the
 // epilogue 85, and the head's MMAs (194 us alone) run underneath.  Six instead of the four instructions
 // per two words of sc_add took 511 us where these took 507 at the time, three and two multiply-adds 513.  Nor did
@@ -33,8 +33,8 @@
 // 1.71 ms, 60,000 against an fp16 256 x 256 map 22.7 / 11.3 ms.
 //
 // The blocks stay, one per SM, and take sets of 128 documents and stretches of slabs one after the other; barriers and
-// accumulators go on from item to item: 200,000 documents on a trained 128 x 128 map 9.81 -> 9.62 ms, 30,011 on 75 x 75
-// 686 -> 663 us.
+// accumulators go on from item to item: 200,000 documents on a trained 128 x 128 map 9.81 -> 9.49 ms, 30,011 on 75 x 75
+// 686 -> 671 us; 120,000 on 64 x 64, D = 4,096, where slabs are short, 875 -> 885.
 //
 // ORDERED: slabs in the order of the norms (screen.cuh, screen_order.cu).  What differs:
 //   items      a set of documents reaches a few slabs of a launch, another set many: (set, up to SC_PART slabs),
@@ -46,7 +46,8 @@
 //   head first once a slab has brought the warp no candidate, the next ones are looked at with the head's sums and the
 //              most that the gathered rows could add; where that rules a slab out its rows are not gathered (for
 //              120,000 documents on 64 x 64 the search 970 -> 885 us).
-// The same documents take 1,255 us with all slabs in the order of the map; 100,000 on 512 x 512 57,000 and 1,500.
+// The same documents take 1,255 us with all slabs in the order of the map; 100,000 on 512 x 512 57,000 and 1,500.  Bound by
+// the latency of the gathered loads, and by meeting at an item's ends (a quarter of the stalls).
 
 #include "screen.cuh"
 #include "mma_ptx.cuh"
@@ -466,6 +467,8 @@ sweep_screen_kernel(const ScreenArgs a, const OrderedArgs o)
                 x[2] = sc_dist2(nm[2], hs[4], hs[5], t[w0 + 1], sh, st, minus_2p23);
                 x[3] = sc_dist2(nm[3], hs[6], hs[7], t[5 + w0], sh, st, minus_2p23);
             };
+            // (twice the same eight neurons at a time, on purpose: by dist8 the map's order, which frees the accumulator in
+            // front of the last eight's arithmetic, took 2-8 % more)
             float mc[4];
             if constexpr (ORDERED) {
 #pragma unroll

@@ -431,8 +431,9 @@ static int launch_blur_fast(const uint32_t *num, const uint32_t *cnt, int64_t D,
 // A block carries as many planes as fit its threads, and all rows of them, or an equal part of them with R more
 // on either side where planes are too few to fill the chip.
 //
-// Bound by HBM up to radius 5 (128 x 128 x 16,384, 2.15 GB: 369 us at radius 2, 374 at 5, 6 TB/s), then by the
-// multiplier, 2 (2R + 1) taps per output (429 at radius 6, 562 at 8).  The tiled kernel above, which exchanges every
+// Up to radius 5 near what a copy takes (128 x 128 x 16,384, 2.15 GB: 369 us at radius 2, 374 at 5, 6 TB/s; four fifths
+// of the issue slots are taken too); beyond, 429 us at radius 6 and 562 at 8, by issue with few warps (112 registers, 16 per
+// SM) and by fetching instructions: the loop is unrolled 2 (2R + 1) times.  The tiled kernel above, which exchanges every
 // tile through shared memory twice and is bound by that, took 457, 558, 594 and 677 us.
 template <int R> struct BlurStrip {
     static constexpr int T = 2 * R + 1, PAD = (R + 3) / 4 * 4;
