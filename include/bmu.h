@@ -180,9 +180,10 @@ BMU_API int bmu_codebook_norms(const float *W, int64_t D, int64_t M, float *norm
  * the split image of the frequent rows (4 * head_rows bytes per neuron) and the
  * compact chunk copy of the single-stage tensor-core sweep).  The two-stage form
  * keeps its id lists (2 bytes per listing), head masks (192 bytes per document),
- * candidate lists (288) and the smallest values of a launch (about 100) and the
- * chunk's 8-bit images there instead, 0.8 GB for 1,000,000 documents of 80 ids
- * against 16,384 x 4,096 weights (the single-stage arrays: 0.5 GB).  `nnz` is the
+ * candidate lists (288), the smallest values of a launch (about 100), the reach of
+ * documents and the order of units (20 and 28 bytes each) and the chunk's 8-bit images
+ * there instead, 0.9 GB for 1,000,000 documents of 80 ids against 16,384 x 4,096
+ * weights (the single-stage arrays: 0.5 GB).  `nnz` is the
  * length of colidx.
  * Never falls when N or nnz grow: a workspace for the largest batch serves all
  * smaller ones (the other workspace queries likewise).
