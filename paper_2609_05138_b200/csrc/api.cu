@@ -183,7 +183,9 @@ static int plan_order(const bmu_opts &o, bool tensor_core_sweep)
 //             D = 4,096, 30,000 documents of 64 ids: 244, two-stage 160; 256 units: 122 and 148)
 //   two-stage 90 + 0.0022 D + 0.009 M + 1.6e-6 D M + 0.002 N + U / 3.3e7
 // e.g. D = 4,096, M = 1,024: 4,000 documents 90 / 161 / 144 us, 10,000: 215 / 208 / 174; D = 16,384,
-// M = 4,096: 1,000 documents 92 / 454 / 269, 10,000: 761 / 757 / 450.  Two lines beside the model: from
+// M = 4,096: 1,000 documents 92 / 454 / 269, 10,000: 761 / 757 / 450 (with slabs by norm and blocks that stay, on an iid
+// codebook: 87 / 180 / 120, - / 211 / 155, 99 / 551 / 279, - / 734 / 426; the model has not been fitted again).  Two
+// lines beside the model: from
 // 1,024 documents and 600,000 listings on it is never the first, and below 1,024 documents never the second
 // (its warps would not fill the chip) unless two stages are ruled out and the sweep is large (2e10 updates).
 // There the first takes 60 + U / 6.1e6 (3.1e6) for more than a few hundred us, and two stages 0.2 us more
